@@ -280,11 +280,12 @@ typedef struct {
 
 /* Step 3b: K~ x = b~ by CG with the diagonal (= identity) preconditioner, binary64.
  * x_dev [device, dim] is written.  info may be NULL.  The whole iteration runs in one
- * cooperative launch (blocks over the block rows of K~, grid barriers between the
- * phases of an iteration); every barrier wait is bounded by the wait budget
- * (mor_set_wait_budget), and a wait that runs out ends the kernel with
- * MOR_ERR_TIMEOUT instead of hanging.  Where a cooperative launch is not possible the
- * same iteration runs as three launches per step. */
+ * launch: a small system in one thread-block cluster, a larger one cooperatively on
+ * every SM, where the blocks exchange their partial sums twice per iteration.  Every
+ * wait of such an exchange is bounded by the wait budget (mor_set_wait_budget), and a
+ * wait that runs out ends the kernel with MOR_ERR_TIMEOUT instead of hanging.  Where a
+ * cooperative launch is not possible the same iteration runs as three launches per
+ * step. */
 int mor_solve_reduced(const mor_reduced* h, double rtol, int32_t max_iter, void* stream,
                       double* x_dev, mor_solve_info* info);
 
@@ -312,20 +313,21 @@ int mor_solve_reduced(const mor_reduced* h, double rtol, int32_t max_iter, void*
  * That first call loads the module, which may allocate and synchronize inside the
  * CUDA runtime: make it once at initialisation, before any stream capture.  Later
  * calls on that device allocate nothing.
- * The call waits for its stream every 16 iterations to read the convergence flag, and
- * at the end to read the residual and energy.
+ * The solve is one launch (as in mor_solve_reduced); the call waits for its stream once,
+ * to read the flags, the residual and the energy.  Without cooperative launches it
+ * waits every 16 iterations to read the convergence flag.
  * Every call shares the one array and leaves its contents behind; the call clears the
  * state that must start at zero.  Calls whose GPU work overlaps (for example on two
  * streams, or two host threads) race on the array: serialise them.
- * Returns MOR_OK, MOR_ERR_NOT_CONVERGED (x holds the last iterate), MOR_ERR_ARG or
- * MOR_ERR_CUDA. */
+ * Returns MOR_OK, MOR_ERR_NOT_CONVERGED (x holds the last iterate), MOR_ERR_ARG,
+ * MOR_ERR_TIMEOUT (a wait ran out of its budget) or MOR_ERR_CUDA. */
 int mor_solve_reduced_noalloc(int32_t n_sub, int32_t kq, const int32_t* nbr_ptr_dev,
                               const int32_t* nbr_sub_dev, const int32_t* nbr_blk_dev,
                               const double* blocks_dev, const double* bt_dev, double rtol,
                               int32_t max_iter, void* stream, double* x_dev,
                               mor_solve_info* info);
 
-/* Budget of every bounded device-side wait (grid barriers of mor_solve_reduced, the
+/* Budget of every bounded device-side wait (the exchanges of the reduced solves, the
  * mbarrier waits of the tensor-core kernels), in seconds of the GPU's SM clock
  * (default 1 s; a wait normally lasts microseconds), between 1 ms and 3600 s
  * (MOR_ERR_ARG otherwise): a tensor-core kernel whose wait ran out waits once more, with

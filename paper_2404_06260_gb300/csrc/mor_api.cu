@@ -180,16 +180,26 @@ int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 // budget of the bounded device-side waits, seconds of SM clock
 double g_wait_budget_s = 1.0;
-long long wait_budget_cycles() {
+// the device's SM clock in kHz; asking the driver takes 0.4 ms, so each device is asked
+// once
+int sm_clock_khz() {
+  static std::array<std::atomic<int>, 64> known{};
   int dev = 0, khz = 0;
-  cudaGetDevice(&dev);
+  if (cudaGetDevice(&dev) != cudaSuccess) return 2000000;
+  if (dev >= 0 && dev < (int)known.size()) khz = known[dev].load(std::memory_order_relaxed);
+  if (khz > 0) return khz;
   cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev);
   if (khz <= 0) khz = 2000000;
-  return (long long)(g_wait_budget_s * 1e3 * (double)khz);
+  if (dev >= 0 && dev < (int)known.size()) known[dev].store(khz, std::memory_order_relaxed);
+  return khz;
 }
 int round_up4(int x) { return (x + 3) & ~3; }
 
 }  // namespace
+
+long long mor::wait_budget_cycles() {
+  return (long long)(g_wait_budget_s * 1e3 * (double)sm_clock_khz());
+}
 
 // error reporting for the other translation units (same thread-local message)
 int mor::set_error(int code, const std::string& msg) { return fail(code, msg); }
@@ -1748,61 +1758,79 @@ int mor_solve_reduced(const mor_reduced* h, double rtol, int32_t max_iter, void*
   cudaStream_t st = (cudaStream_t)stream;
   Allocs A;
   A.use_pool(st);
+  // r, p, q, and a zeroed tail: the partial sums of either iteration, the scalars and the
+  // flags
+  const size_t n_part = std::max(2 * (size_t)h->n_sd, 2 * (size_t)kRcgMaxGrid);
+  const size_t n_tail = n_part + 16;
+  double* ws;
+  TRY(A.alloc(&ws, 3 * (size_t)h->dim + n_tail, false, st));
+  double* tail = ws + 3 * (size_t)h->dim;
+  CK(cudaMemsetAsync(tail, 0, n_tail * sizeof(double), st));
   RcgState s{};
   s.x = x_dev;
-  TRY(A.alloc(&s.r, h->dim, false, st));
-  TRY(A.alloc(&s.p, h->dim, false, st));
-  TRY(A.alloc(&s.q, h->dim, false, st));
-  TRY(A.alloc(&s.part, (size_t)2 * h->n_sd, true, st));
-  TRY(A.alloc(&s.counter, 1, true, st));
-  TRY(A.alloc(&s.scal, 8, true, st));
-  TRY(A.alloc(&s.flag, 2, true, st));
-  int hf[2] = {0, 0};
-  unsigned* sync;
-  TRY(A.alloc(&sync, 4, true, st));
-  const int grid = launch_rcg_persistent(h->n_sd, h->kq, h->nbr_ptr, h->nbr_sd, h->nbr_blk,
-                                         h->blocks, h->bt, rtol * rtol, max_iter, s, sync,
-                                         wait_budget_cycles(), st);
-  if (grid > 0) {
-    unsigned hs[4] = {0, 0, 0, 0};
-    CK(cudaMemcpyAsync(hs, sync, sizeof(hs), cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(hf, s.flag, sizeof(hf), cudaMemcpyDeviceToHost, st));
+  s.r = ws;
+  s.p = ws + h->dim;
+  s.q = ws + 2 * (size_t)h->dim;
+  s.part = tail;
+  s.scal = tail + n_part;
+  s.flag = reinterpret_cast<int*>(s.scal + 8);
+  s.counter = s.flag + 4;
+  struct {
+    double sc[8];
+    int flag[4];
+  } out;
+  auto fetch = [&]() -> int {
+    CK(cudaMemcpyAsync(&out, s.scal, sizeof(out), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    if (hs[2] != 0)
-      return fail(MOR_ERR_TIMEOUT, "mor_solve_reduced: a grid-barrier wait ran out of its "
-                                   "budget (mor_set_wait_budget)");
+    return MOR_OK;
+  };
+  double E = 0.0;
+  auto launch = [&](bool cluster) {
+    return launch_rcg_solve(h->n_sd, h->kq, h->nbr_ptr, h->nbr_sd, h->nbr_blk,
+                            2 * (int64_t)h->n_pairs, h->blocks, h->bt, rtol * rtol, max_iter, s,
+                            s.part, wait_budget_cycles(), cluster, st);
+  };
+  RcgLaunch how = launch(true);
+  if (how != RcgLaunch::kNone) TRY(fetch());
+  if (how == RcgLaunch::kCluster && out.flag[2] == 2) {
+    CK(cudaMemsetAsync(s.flag, 0, 4 * sizeof(int), st));
+    how = launch(false);
+    if (how != RcgLaunch::kNone) TRY(fetch());
+  }
+  if (how != RcgLaunch::kNone) {
+    if (out.flag[2] != 0)
+      return fail(MOR_ERR_TIMEOUT, "mor_solve_reduced: an exchange between blocks ran out of "
+                                   "its budget (mor_set_wait_budget)");
+    E = out.sc[6];
   } else {
-    cudaGetLastError();  // no cooperative launch: three launches per step
+    cudaGetLastError();  // three launches per step
     launch_rcg_init(h->n_sd, h->kq, h->bt, s, st);
-    int it = 0;
-    while (it < max_iter) {
+    for (int it = 0; it < max_iter;) {
       int chunk = std::min(16, max_iter - it);
       for (int c = 0; c < chunk; ++c)
         launch_rcg_step(h->n_sd, h->kq, h->nbr_ptr, h->nbr_sd, h->nbr_blk, h->blocks,
                         rtol * rtol, s, st);
       it += chunk;
-      CK(cudaMemcpyAsync(hf, s.flag, sizeof(hf), cudaMemcpyDeviceToHost, st));
-      CK(cudaStreamSynchronize(st));
-      if (hf[0]) break;
+      TRY(fetch());
+      if (out.flag[0]) break;
     }
+    // energy b~^T x
+    std::vector<double> hx(h->dim), hb(h->dim);
+    CK(cudaMemcpyAsync(hx.data(), x_dev, h->dim * sizeof(double), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(hb.data(), h->bt, h->dim * sizeof(double), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    for (int64_t i = 0; i < h->dim; ++i) E += hb[i] * hx[i];
   }
   CK(cudaGetLastError());
-  double sc[8];
-  CK(cudaMemcpy(sc, s.scal, sizeof(sc), cudaMemcpyDeviceToHost));
-  // energy b~^T x
-  std::vector<double> hx(h->dim), hb(h->dim);
-  CK(cudaMemcpy(hx.data(), x_dev, h->dim * sizeof(double), cudaMemcpyDeviceToHost));
-  CK(cudaMemcpy(hb.data(), h->bt, h->dim * sizeof(double), cudaMemcpyDeviceToHost));
-  double E = 0.0;
-  for (int64_t i = 0; i < h->dim; ++i) E += hb[i] * hx[i];
+  const double* sc = out.sc;
+  const bool ok = out.flag[0] && sc[4] <= rtol * rtol * sc[1];
   if (info) {
-    info->iterations = hf[1];
-    info->converged = hf[0] && sc[4] <= rtol * rtol * sc[1];
+    info->iterations = out.flag[1];
+    info->converged = ok;
     info->rel_residual = sc[1] > 0 ? std::sqrt(sc[4] / sc[1]) : 0.0;
     info->energy = E;
   }
-  if (!(hf[0] && sc[4] <= rtol * rtol * sc[1]))
-    return fail(MOR_ERR_NOT_CONVERGED, "mor_solve_reduced: max_iter reached");
+  if (!ok) return fail(MOR_ERR_NOT_CONVERGED, "mor_solve_reduced: max_iter reached");
   return MOR_OK;
 }
 

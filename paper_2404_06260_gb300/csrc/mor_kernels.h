@@ -329,17 +329,27 @@ void launch_pair_blocks(int n_pairs, const int64_t* pair_ptr, const int32_t* uro
                         double* blocks, cudaStream_t st);
 struct RcgState {
   double *x, *r, *p, *q;    // dim
-  double* part;             // n_sd x 2
+  double* part;             // n_sd x 2 (three-launch iteration)
   int* counter;             // 1
-  double* scal;             // [0] rz, [1] bb, [2] alpha, [3] beta, [4] rr
-  int* flag;                // [0] done, [1] iterations
+  double* scal;             // [0] rz, [1] bb, [2] alpha, [3] beta, [4] rr, [6] b~.x
+  int* flag;                // [0] done, [1] iterations, [2] 1: a wait ran out, 2: not
+                            // fitting; [3] arrivals
 };
-// the reduced CG in one cooperative launch with bounded grid-barrier waits; returns the
-// grid size, or -1 when a cooperative launch is not possible.  sync: 3 zeroed words.
-int launch_rcg_persistent(int n_sd, int kq, const int32_t* nbr_ptr, const int32_t* nbr_sd,
-                          const int32_t* nbr_blk, const double* blocks, const double* bt,
-                          double tol2, int max_iter, const RcgState& s, unsigned* sync,
-                          long long budget, cudaStream_t st);
+// the reduced CG in one launch (one cluster, or cooperatively on every SM) with bounded
+// waits; p and q of s are the two halves of the double-buffered search direction, part
+// holds 2 * kRcgMaxGrid partial sums, flag is zeroed by the caller.  n_blocks: stored off-diagonal blocks (an estimate will do: it picks the launch shape).  kNone, with
+// nothing launched, where the device or the size does not allow it.  After kCluster
+// flag[2] = 2 says that the matrix did not fit into one cluster: launch again with
+// try_cluster = false.
+constexpr int kRcgMaxGrid = 512;
+enum class RcgLaunch { kNone, kCluster, kGrid };
+RcgLaunch launch_rcg_solve(int n_sd, int kq, const int32_t* nbr_ptr, const int32_t* nbr_sd,
+                           const int32_t* nbr_blk, int64_t n_blocks, const double* blocks,
+                           const double* bt, double tol2, int max_iter, const RcgState& s,
+                           double* part, long long budget, bool try_cluster,
+                           cudaStream_t st);
+// the budget of every bounded wait in SM clock cycles of the current device
+long long wait_budget_cycles();
 void launch_wait_unset_flag(unsigned* sync, long long budget, int* status, cudaStream_t st);
 void launch_rcg_init(int n_sd, int kq, const double* bt, const RcgState& s,
                      cudaStream_t st);

@@ -16,8 +16,8 @@ using namespace mor;
 namespace {
 
 // Limits of the fixed scratch array: the reduced vectors r, p, q (3 x kMaxDim binary64),
-// the per-subdomain partial sums (2 x kMaxSub), 8 scalars and a 3-int tail (ticket
-// counter, done flag, iteration count): 1,703,952 doubles = 13.6 MB.  The array is
+// the partial sums (2 x kMaxSub), 8 scalars and a tail of ints (done flag, iteration
+// count, wait status, arrivals, ticket counter): 1,703,952 doubles = 13.6 MB.  The array is
 // placed on a device when this file's device code is loaded there (with CUDA's default
 // lazy loading: at the first set-up below on that device) and stays until the process
 // exits.
@@ -28,6 +28,7 @@ constexpr int64_t kPartOff = 3 * kMaxDim;
 constexpr int64_t kScalOff = kPartOff + 2 * kMaxSub;
 constexpr int64_t kIntOff = kScalOff + 8;
 constexpr int64_t kScratchDoubles = kIntOff + 8;
+static_assert(kRcgMaxGrid <= kMaxSub, "partial sums of the one-launch solve");
 static_assert(kScratchDoubles == 1703952, "stated scratch size");
 
 static __device__ __align__(256) double g_solve_scratch[kScratchDoubles];
@@ -137,33 +138,63 @@ extern "C" int mor_solve_reduced_noalloc(int32_t n_sub, int32_t kq, const int32_
   s.q = base + kVecOff + 2 * dim;
   s.part = base + kPartOff;
   s.scal = base + kScalOff;
-  int* ints = reinterpret_cast<int*>(base + kIntOff);
-  s.counter = ints;
-  s.flag = ints + 1;
-  // the array keeps the previous call's contents: the ticket counter and the flags
-  // must start at zero
-  cudaError_t e = cudaMemsetAsync(ints, 0, 3 * sizeof(int), st);
+  s.flag = reinterpret_cast<int*>(base + kIntOff);
+  s.counter = s.flag + 4;
+  // the array keeps the previous call's contents: the flags and the counters must start
+  // at zero
+  cudaError_t e = cudaMemsetAsync(s.flag, 0, 8 * sizeof(int), st);
   if (e != cudaSuccess) return set_error(MOR_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
-  launch_rcg_init(n_sub, kq, bt_dev, s, st);
-  int hf[2] = {0, 0};
-  for (int it = 0; it < max_iter;) {
-    int chunk = max_iter - it < 16 ? max_iter - it : 16;
-    for (int c = 0; c < chunk; ++c)
-      launch_rcg_step(n_sub, kq, nbr_ptr_dev, nbr_sub_dev, nbr_blk_dev, blocks_dev,
-                      rtol * rtol, s, st);
-    it += chunk;
-    e = cudaMemcpyAsync(hf, s.flag, sizeof(hf), cudaMemcpyDeviceToHost, st);
+  struct {
+    double sc[8];
+    int flag[4];
+  } out;
+  auto fetch = [&]() {
+    e = cudaMemcpyAsync(&out, s.scal, sizeof(out), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return set_error(MOR_ERR_CUDA, std::string("reduced solve: ") + cudaGetErrorString(e));
-    if (hf[0]) break;
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) return (int)MOR_OK;
+    return set_error(MOR_ERR_CUDA, std::string("reduced solve: ") + cudaGetErrorString(e));
+  };
+  // the neighbour lists are on the device; for the launch shape, 9 neighbours per block
+  // row: the mean of small box partitions, whose inner boxes have 14
+  const int64_t n_blocks = (int64_t)n_sub * (n_sub - 1 < 9 ? n_sub - 1 : 9);
+  auto launch = [&](bool cluster) {
+    return launch_rcg_solve(n_sub, kq, nbr_ptr_dev, nbr_sub_dev, nbr_blk_dev, n_blocks,
+                            blocks_dev, bt_dev, rtol * rtol, max_iter, s,
+                            s.part, wait_budget_cycles(), cluster, st);
+  };
+  RcgLaunch how = launch(true);
+  if (how != RcgLaunch::kNone && (rc = fetch()) != MOR_OK) return rc;
+  if (how == RcgLaunch::kCluster && out.flag[2] == 2) {
+    e = cudaMemsetAsync(s.flag, 0, 4 * sizeof(int), st);
+    if (e != cudaSuccess) return set_error(MOR_ERR_CUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
+    how = launch(false);
+    if (how != RcgLaunch::kNone && (rc = fetch()) != MOR_OK) return rc;
   }
-  count_launch();
-  k_energy_dot<<<1, 256, 0, st>>>(dim, bt_dev, x_dev, s.scal + 6);
-  double sc[8];
-  e = cudaMemcpyAsync(sc, s.scal, sizeof(sc), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e == cudaSuccess) e = cudaGetLastError();
-  if (e != cudaSuccess) return set_error(MOR_ERR_CUDA, std::string("reduced solve: ") + cudaGetErrorString(e));
+  if (how != RcgLaunch::kNone) {
+    if (out.flag[2] != 0)
+      return set_error(MOR_ERR_TIMEOUT, "mor_solve_reduced_noalloc: an exchange between blocks "
+                                        "ran out of its budget (mor_set_wait_budget)");
+  } else {
+    cudaGetLastError();  // three launches per step
+    launch_rcg_init(n_sub, kq, bt_dev, s, st);
+    for (int it = 0; it < max_iter;) {
+      int chunk = max_iter - it < 16 ? max_iter - it : 16;
+      for (int c = 0; c < chunk; ++c)
+        launch_rcg_step(n_sub, kq, nbr_ptr_dev, nbr_sub_dev, nbr_blk_dev, blocks_dev,
+                        rtol * rtol, s, st);
+      it += chunk;
+      rc = fetch();
+      if (rc != MOR_OK) return rc;
+      if (out.flag[0]) break;
+    }
+    count_launch();
+    k_energy_dot<<<1, 256, 0, st>>>(dim, bt_dev, x_dev, s.scal + 6);
+    rc = fetch();
+    if (rc != MOR_OK) return rc;
+  }
+  const double* sc = out.sc;
+  const int* hf = out.flag;
   const bool ok = hf[0] && sc[4] <= rtol * rtol * sc[1];
   if (info) {
     info->iterations = hf[1];

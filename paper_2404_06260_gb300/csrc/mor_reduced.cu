@@ -5,6 +5,8 @@
 #include "mor_dev.cuh"
 #include "mor_kernels.h"
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 namespace mor {
@@ -187,97 +189,445 @@ __global__ void k_rcg_update_p(int kq, RcgState s) {
   }
 }
 
-// The whole reduced CG in one cooperative launch: blocks take block rows sd =
-// blockIdx.x, blockIdx.x + gridDim.x, ...; the three phases of an iteration (q = K~ p
-// with p.q; x and r update with r.r; p update) are separated by grid barriers with
-// bounded waits.  Every block forms the scalars itself from the same partial sums in
-// the same order (sum_parts), so all blocks take the same decisions; the arithmetic is
-// that of the three-kernel iteration.  sync[0] barrier count, sync[1] generation,
-// sync[2] error (a wait ran out).
-__global__ void __launch_bounds__(128)
-    k_rcg_persistent(int n_sd, int kq, const int32_t* __restrict__ nbr_ptr,
-                     const int32_t* __restrict__ nbr_sd, const int32_t* __restrict__ nbr_blk,
-                     const double* __restrict__ blocks, const double* __restrict__ bt,
-                     double tol2, int max_iter, RcgState s, unsigned* sync,
-                     long long budget) {
-  __shared__ double red[128];
-  unsigned* count = sync;
-  volatile unsigned* gen = sync + 1;
-  volatile int* err = reinterpret_cast<volatile int*>(sync + 2);
-  // x = 0, r = p = b~, ||b~||^2
-  for (int sd = blockIdx.x; sd < n_sd; sd += gridDim.x) {
-    double loc = 0.0;
-    for (int i = threadIdx.x; i < kq; i += blockDim.x) {
-      const int64_t g = (int64_t)sd * kq + i;
-      const double b = bt[g];
-      s.x[g] = 0.0;
-      s.r[g] = b;
-      s.p[g] = b;
-      loc += b * b;
-    }
-    const double t = block_sum128(loc, red);
-    if (threadIdx.x == 0) s.part[2 * sd] = t;
+// ---- the whole reduced CG in one launch ----
+// What bounds it: GB300 does 2 binary64 multiply-adds per SM and clock (a warp
+// instruction keeps its quarter of the SM busy for 64 clocks, and dependent steps are
+// about 100 clocks apart), and every iteration needs two sums over all rows.  So the
+// matrix is spread as far as the sums allow: up to kRcgClusterFma multiply-adds and
+// kRcgClusterDim rows one cluster of 8 CTAs keeps matrix and vectors in shared memory
+// and sums through distributed shared memory (k_rcg_cluster, about 1.5 us a sum); above,
+// every SM takes part and sums through global memory (k_rcg_grid, 3.5 us).  Whole calls
+// measured on both, cluster | every SM: 5 k multiply-adds 137 | 248 us, 28 k 221 | 346,
+// 50 k 267 | 370, 78 k 425 | 407, 80 k (more rows) 369 | 457, 109 k 500 | 480, 254 k
+// 511 | 494, hence the line.  Against three launches per step with one thread per row and
+// a host poll every 16 steps: 27 block rows of 12 (33 steps) 1,029 -> 224 us a call, 512 of
+// 36 (66 steps) 5.0 -> 1.9 ms.
+// Both: p = r + beta p is formed by every reader from r and its own copy of the last p,
+// which saves a third exchange; all CTAs sum the same partials in the same order and take
+// the same decisions.
+constexpr int kRcgCluster = 8;
+constexpr int kRcgClusterDim = 1024;       // rows: 4 lanes each, 512 threads a CTA
+constexpr double kRcgClusterFma = 100000.0;
+constexpr size_t kRcgClusterSmem = 200 * 1024;
+
+// sum over lanes xor lo, 2 lo, ..., hi / 2
+__device__ __forceinline__ double warp_sum(double v, int lo, int hi) {
+  for (int o = lo; o < hi; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// One cluster.  CTA c holds rows [dim c / G, dim (c + 1) / G) of K~'s off-diagonal part:
+// thread 4 i + h takes the entries h, h + 4, ... of the CTA's row i, value and column in
+// shared memory at [step][thread].  r and p of all rows are kept by every CTA: owners push
+// their new r into every CTA's copy together with their warps' partial sums, and one
+// cluster barrier makes both visible.  status 2: the entries do not fit (nothing done).
+template <int kSlots>
+struct RcgClusterSums {
+  double part[2][kRcgCluster * kSlots];
+  double res[4];
+};
+__global__ void __launch_bounds__(512)
+    k_rcg_cluster(int n_sd, int kq, const int32_t* __restrict__ nbr_ptr,
+                  const int32_t* __restrict__ nbr_sd, const int32_t* __restrict__ nbr_blk,
+                  const double* __restrict__ blocks, const double* __restrict__ bt,
+                  double tol2, int max_iter, int smem_entries, RcgState s) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  extern __shared__ __align__(16) unsigned char rcg_raw[];
+  __shared__ RcgClusterSums<16> sums;
+  __shared__ int s_steps[16], s_fit[kRcgCluster];
+  const int dim = n_sd * kq, G = gridDim.x, rank = blockIdx.x;
+  const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  const int nw = nth >> 5;
+  double* rf = reinterpret_cast<double*>(rcg_raw);
+  double* pf = rf + dim;
+  double* val = pf + dim;
+  uint16_t* col = reinterpret_cast<uint16_t*>(val + smem_entries);
+  const int row0 = (int)((int64_t)dim * rank / G), row1 = (int)((int64_t)dim * (rank + 1) / G);
+  const int i = row0 + (tid >> 2), h = tid & 3;
+  const bool mine = i < row1;
+  const int sd = mine ? i / kq : 0, il = i - sd * kq;
+  const int t0 = mine ? nbr_ptr[sd] : 0, ne = mine ? (nbr_ptr[sd + 1] - t0) * kq : 0;
+  int steps = ne > h ? (ne - h + 3) / 4 : 0;
+  steps = __reduce_max_sync(0xffffffffu, steps);  // of the warp
+  if (lane == 0) s_steps[warp] = steps;
+  __syncthreads();
+  int most = 0;
+  for (int w = 0; w < nw; ++w) most = max(most, s_steps[w]);
+  if (tid < G) *cl.map_shared_rank(&s_fit[rank], tid) = (int64_t)most * nth <= smem_entries;
+  cl.sync();
+  bool fit = true;
+  for (int g = 0; g < G; ++g) fit = fit && s_fit[g] != 0;
+  if (!fit) {
+    if (rank == 0 && tid == 0) s.flag[2] = 2;
+    return;
   }
-  if (!grid_barrier(count, gen, err, budget)) return;
-  const double bb = sum_parts(s.part, n_sd, 2, 0, red);
-  double rz = bb, rr = bb;
+  {
+    int t = t0, l = h;
+    for (int k = 0; k < steps; ++k) {
+      while (l >= kq && 4 * k + h < ne) {
+        l -= kq;
+        ++t;
+      }
+      double v = 0.0;
+      int c = 0;
+      if (4 * k + h < ne) {
+        v = blocks[((int64_t)nbr_blk[t] * kq + il) * kq + l];
+        c = nbr_sd[t] * kq + l;
+      }
+      val[k * nth + tid] = v;
+      col[k * nth + tid] = (uint16_t)c;
+      l += 4;
+    }
+  }
+  unsigned epoch = 0;
+  // v of the lanes with h = 0 summed over the cluster; warp 0 passes the sum to fin(sum, res)
+  auto exchange = [&](double v, auto fin) {
+    v = warp_sum(v, 4, 32);
+    double* slot = sums.part[epoch & 1u] + rank * nw + warp;
+    if (lane < G) *cl.map_shared_rank(slot, lane) = v;
+    cl.sync();
+    if (warp == 0) {
+      double t = 0.0;
+      for (int k = lane; k < G * nw; k += 32) t += sums.part[epoch & 1u][k];
+      t = warp_sum(t, 1, 32);
+      if (lane == 0) fin(t, sums.res);
+    }
+    ++epoch;
+    __syncthreads();
+  };
+  auto push_r = [&](double r) {
+    if (mine)
+      for (int g = h; g < G; g += 4) *cl.map_shared_rank(rf + i, g) = r;
+  };
+  double x = 0.0, r = mine ? bt[i] : 0.0;
+  const double b = r;
+  push_r(r);
+  exchange(r * r, [](double t, double* o) { o[0] = t; });
+  const double bb = sums.res[0];
+  double rz = bb, rr = bb, be = 0.0;
   int done = bb > 0.0 ? 0 : 1, it = 0;
   while (!done && it < max_iter) {
-    // q = K~ p (identity diagonal blocks) and p.q
-    for (int sd = blockIdx.x; sd < n_sd; sd += gridDim.x) {
-      double loc = 0.0;
-      for (int i = threadIdx.x; i < kq; i += blockDim.x) {
-        const int64_t g = (int64_t)sd * kq + i;
-        double acc = s.p[g];
-        for (int q = nbr_ptr[sd]; q < nbr_ptr[sd + 1]; ++q) {
-          const double* B = blocks + (int64_t)nbr_blk[q] * kq * kq + (int64_t)i * kq;
-          const double* pj = s.p + (int64_t)nbr_sd[q] * kq;
-          for (int l = 0; l < kq; ++l) acc += B[l] * pj[l];
-        }
-        s.q[g] = acc;
-        loc += s.p[g] * acc;
-      }
-      const double t = block_sum128(loc, red);
-      if (threadIdx.x == 0) s.part[2 * sd] = t;
-    }
-    if (!grid_barrier(count, gen, err, budget)) return;
-    const double pq = sum_parts(s.part, n_sd, 2, 0, red);
-    const double al = pq > 0.0 ? rz / pq : 0.0;
-    for (int sd = blockIdx.x; sd < n_sd; sd += gridDim.x) {
-      double loc = 0.0;
-      for (int i = threadIdx.x; i < kq; i += blockDim.x) {
-        const int64_t g = (int64_t)sd * kq + i;
-        s.x[g] += al * s.p[g];
-        const double r = s.r[g] - al * s.q[g];
-        s.r[g] = r;
-        loc += r * r;
-      }
-      const double t = block_sum128(loc, red);
-      if (threadIdx.x == 0) s.part[2 * sd + 1] = t;
-    }
-    if (!grid_barrier(count, gen, err, budget)) return;
-    rr = sum_parts(s.part, n_sd, 2, 1, red);
+    for (int j = tid; j < dim; j += nth) pf[j] = it ? fma(be, pf[j], rf[j]) : rf[j];
+    __syncthreads();
+    double q = 0.0;
+#pragma unroll 4
+    for (int k = 0; k < steps; ++k) q = fma(val[k * nth + tid], pf[col[k * nth + tid]], q);
+    q = warp_sum(q, 1, 4);
+    const double p = mine ? pf[i] : 0.0;
+    q += p;
+    exchange(p * q, [=](double pq, double* o) { o[0] = pq > 0.0 ? rz / pq : 0.0; });
+    const double al = sums.res[0];
+    x += al * p;
+    r -= al * q;
+    push_r(r);
+    exchange(r * r, [=](double t, double* o) {
+      o[1] = t;
+      o[2] = t / rz;
+      o[3] = t <= tol2 * bb || !(rz > 0.0) ? 1.0 : 0.0;
+    });
     ++it;
-    double be = 0.0;
-    if (rr <= tol2 * bb || !(rz > 0.0)) {
-      done = 1;
-    } else {
-      be = rr / rz;
+    rr = sums.res[1];
+    done = sums.res[3] != 0.0;
+    if (!done) {
+      be = sums.res[2];
       rz = rr;
     }
-    if (!done) {
-      for (int sd = blockIdx.x; sd < n_sd; sd += gridDim.x)
-        for (int i = threadIdx.x; i < kq; i += blockDim.x) {
-          const int64_t g = (int64_t)sd * kq + i;
-          s.p[g] = s.r[g] + be * s.p[g];
-        }
-      if (!grid_barrier(count, gen, err, budget)) return;
-    }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  if (mine && h == 0) s.x[i] = x;
+  exchange(b * x, [](double t, double* o) { o[0] = t; });
+  if (rank == 0 && tid == 0) {
     s.scal[0] = rz;
     s.scal[1] = bb;
     s.scal[4] = rr;
+    s.scal[6] = sums.res[0];
+    s.flag[0] = done;
+    s.flag[1] = it;
+  }
+  cl.sync();  // no CTA leaves while another may still push to it
+}
+
+// Every SM.  Units of four rows (rows 4w .. 4w + 3 of one block row) are dealt out in
+// contiguous runs of about equal work; a CTA keeps its rows of x, r, p and q in shared
+// memory and writes r and p (double-buffered) to global memory for its neighbours.  A warp
+// takes a unit's four rows at once: lanes run over the staged neighbour columns, and the
+// reduce-scatter over the lanes costs 6 additions for the four rows instead of 20.
+constexpr int kRcgThreads = 512;
+constexpr int kRcgCap = 3072;  // neighbour columns staged at a time
+constexpr size_t kRcgStageBytes = kRcgCap * (sizeof(double) + sizeof(int64_t));
+
+// part: 2 parities x gridDim.x partial sums; *count: arrivals since the launch (zeroed
+// before it).  A CTA rewrites a parity only after every CTA has arrived with the other one,
+// that is after every CTA has read this one.  One counter that one thread per CTA polls with
+// acquire loads took 5,000 clocks with both sums, against 9,000 for polled per-CTA slots
+// that carry the sum itself between two fences (152 CTAs).
+struct RcgXch {
+  double* part;
+  unsigned* count;
+  int* err;
+  long long budget;
+  unsigned epoch;
+  int n;        // threads with a value: those below n
+  double* red;  // 32 warp sums, [40] status, [41..] results
+};
+
+// v summed over all threads of all CTAs; one lane passes the sum to fin(sum, res), which
+// writes up to four results for every thread.  False when a wait ran out.  The CTA's earlier
+// global writes are visible to every CTA's later reads.
+template <class F>
+__device__ bool rcg_exchange(RcgXch& x, double v, F fin) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int G = gridDim.x;
+  double* red = x.red;
+  if (32 * warp < x.n) {
+    v = warp_sum(v, 1, 32);
+    if (lane == 0) red[warp] = v;
+  }
+  ++x.epoch;
+  __syncthreads();
+  if (warp == 0) {
+    double* P = x.part + (size_t)(x.epoch & 1u) * G;
+    int ok = 1;
+    if (lane == 0) {
+      double t = 0.0;
+      const int nw = (x.n + 31) >> 5;
+      for (int w = 0; w < nw; ++w) t += red[w];
+      __stcg(P + blockIdx.x, t);
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(x.count) : "memory");
+      const unsigned want = x.epoch * (unsigned)G;
+      const long long t0 = clock64();
+      unsigned c;
+      while (true) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(x.count) : "memory");
+        if ((int)(c - want) >= 0) break;
+        if (*(volatile int*)x.err) ok = 0;
+        if (clock64() - t0 > x.budget) {
+          atomicExch(x.err, 1);
+          ok = 0;
+        }
+        if (!ok) break;
+      }
+    }
+    __syncwarp();
+    double w[5], t = 0.0;
+    for (int g0 = lane; g0 < G; g0 += 160) {
+#pragma unroll
+      for (int k = 0; k < 5; ++k) w[k] = g0 + 32 * k < G ? __ldcg(P + g0 + 32 * k) : 0.0;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) t += w[k];
+    }
+    t = warp_sum(t, 1, 32);
+    if (lane == 0) {
+      red[40] = ok ? 1.0 : 0.0;
+      fin(t, red + 41);
+    }
+  }
+  __syncthreads();
+  return red[40] != 0.0;
+}
+
+// first row of unit u (upb units of four rows per block row of kq rows)
+__device__ __forceinline__ int64_t rcg_row(int u, int upb, int kq) {
+  return (int64_t)(u / upb) * kq + 4 * (u % upb);
+}
+
+// extra weight of a block row beside its neighbours: a quarter of the mean, so that no CTA
+// gets more than five times the mean number of units
+__host__ __device__ __forceinline__ int64_t rcg_base_weight(int64_t nnb, int64_t n_sd) {
+  return nnb / (4 * n_sd) + 1;
+}
+
+// first unit of CTA b's run: units weighted by their block row's neighbours plus a base
+// (weighted = 0: all alike)
+__device__ int rcg_first_unit(int b, int G, int n_sd, int upb, const int32_t* nbr_ptr,
+                              int weighted) {
+  const int64_t units = (int64_t)n_sd * upb;
+  if (!weighted || b == 0 || b == G) return (int)(units * b / G);
+  const int64_t base = rcg_base_weight(nbr_ptr[n_sd], n_sd);
+  const int64_t want = (nbr_ptr[n_sd] + base * n_sd) * upb * b / G;
+  int lo = 0, hi = n_sd - 1;  // the last block row whose units start at or before `want`
+  while (lo < hi) {
+    const int m = (lo + hi + 1) / 2;
+    if ((nbr_ptr[m] + base * m) * upb <= want)
+      lo = m;
+    else
+      hi = m - 1;
+  }
+  const int64_t w = nbr_ptr[lo + 1] - nbr_ptr[lo] + base;
+  const int64_t k = (want - (nbr_ptr[lo] + base * lo) * upb + w - 1) / w;
+  return (int)min(units, (int64_t)lo * upb + min(k, (int64_t)upb));
+}
+
+__global__ void __launch_bounds__(kRcgThreads)
+    k_rcg_grid(int n_sd, int kq, const int32_t* __restrict__ nbr_ptr,
+               const int32_t* __restrict__ nbr_sd, const int32_t* __restrict__ nbr_blk,
+               const double* __restrict__ blocks, const double* __restrict__ bt, double tol2,
+               int max_iter, int rows_max, int weighted, RcgState s, double* part,
+               long long budget) {
+  extern __shared__ __align__(16) unsigned char rcg_raw[];
+  double* xs = reinterpret_cast<double*>(rcg_raw);
+  double* rs = xs + rows_max;
+  double* ps = rs + rows_max;
+  double* qs = ps + rows_max;
+  double* pj = qs + rows_max;
+  int64_t* off = reinterpret_cast<int64_t*>(pj + kRcgCap);
+  __shared__ double red[48];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int upb = (kq + 3) / 4;
+  const int u0 = rcg_first_unit(blockIdx.x, gridDim.x, n_sd, upb, nbr_ptr, weighted);
+  const int u1 = rcg_first_unit(blockIdx.x + 1, gridDim.x, n_sd, upb, nbr_ptr, weighted);
+  const int64_t row0 = rcg_row(u0, upb, kq), row1 = rcg_row(u1, upb, kq);
+  const int rows = (int)(row1 - row0);
+  const int live = min(rows, kRcgThreads);
+  // the neighbour entries of the block rows this CTA touches
+  const int sd_lo = u0 / upb, sd_hi = u1 > u0 ? (u1 - 1) / upb + 1 : sd_lo;
+  const int t_lo = nbr_ptr[sd_lo], t_hi = nbr_ptr[sd_hi];
+  const int tcap = kRcgCap / kq;
+  const float inv_kq = 1.0f / (float)kq;
+  RcgXch x{part, reinterpret_cast<unsigned*>(s.flag + 3), s.flag + 2, budget, 0u, live, red};
+  const double* res = red + 41;
+  double loc = 0.0;
+  for (int i = tid; i < rows; i += kRcgThreads) {
+    const double b = bt[row0 + i];
+    xs[i] = 0.0;
+    rs[i] = b;
+    ps[i] = 0.0;
+    __stcg(s.r + row0 + i, b);
+    loc += b * b;
+  }
+  if (!rcg_exchange(x, loc, [](double t, double* o) { o[0] = t; })) return;
+  const double bb = res[0];
+  double rz = bb, rr = bb, be = 0.0;
+  int done = bb > 0.0 ? 0 : 1, it = 0;
+  while (!done && it < max_iter) {
+    // p = r + beta p on the own rows, q = p (the identity diagonal block)
+    double* pw = it & 1 ? s.q : s.p;
+    const double* pr = it & 1 ? s.p : s.q;
+    for (int i = tid; i < rows; i += kRcgThreads) {
+      const double p = it ? fma(be, ps[i], rs[i]) : rs[i];
+      ps[i] = p;
+      qs[i] = p;
+      __stcg(pw + row0 + i, p);
+    }
+    for (int t0 = t_lo; t0 < t_hi; t0 += tcap) {
+      const int t1 = min(t_hi, t0 + tcap);
+      __syncthreads();
+      const int ne = (t1 - t0) * kq;
+      for (int eb = tid; eb < ne; eb += 4 * kRcgThreads) {
+        double r[4], po[4];
+        int64_t o[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const int e = eb + m * kRcgThreads;
+          if (e >= ne) continue;
+          const int q = (int)(((float)e + 0.5f) * inv_kq), l = e - q * kq;  // e < 2^12
+          const int64_t j = (int64_t)nbr_sd[t0 + q] * kq + l;
+          o[m] = (int64_t)nbr_blk[t0 + q] * kq * kq + l;
+          r[m] = __ldcg(s.r + j);
+          po[m] = it ? __ldcg(pr + j) : 0.0;
+        }
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const int e = eb + m * kRcgThreads;
+          if (e >= ne) continue;
+          pj[e] = it ? fma(be, po[m], r[m]) : r[m];
+          off[e] = o[m];
+        }
+      }
+      __syncthreads();
+      for (int u = u0 + warp; u < u1; u += kRcgThreads / 32) {
+        const int sd = u / upb, i0 = 4 * (u % upb);
+        const int e0 = (max(nbr_ptr[sd], t0) - t0) * kq;
+        const int e1 = (min(nbr_ptr[sd + 1], t1) - t0) * kq;
+        if (e0 >= e1) continue;
+        // the rows of the unit; beyond kq (a last unit of fewer than four) row i0 again
+        const double* B = blocks + (int64_t)i0 * kq;
+        const int st1 = i0 + 1 < kq ? kq : 0, st2 = i0 + 2 < kq ? 2 * kq : 0,
+                  st3 = i0 + 3 < kq ? 3 * kq : 0;
+        double a[4] = {0.0, 0.0, 0.0, 0.0};
+        // two column steps per batch, the next batch's loads issued before this one's
+        // multiply-adds; lanes past the end read column e0 again, times 0
+        double v[2][4], p[2];
+        auto load = [&](int eb, double(&w)[2][4], double(&pv)[2]) {
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const int e = eb + lane + 32 * k;
+            if (eb + 32 * k >= e1) continue;  // the whole warp
+            pv[k] = e < e1 ? pj[e] : 0.0;
+            const double* Bo = B + off[e < e1 ? e : e0];
+            w[k][0] = __ldg(Bo);
+            w[k][1] = __ldg(Bo + st1);
+            w[k][2] = __ldg(Bo + st2);
+            w[k][3] = __ldg(Bo + st3);
+          }
+        };
+        load(e0, v, p);
+        for (int eb = e0; eb < e1; eb += 64) {
+          double w[2][4], pw2[2];
+          load(eb + 64, w, pw2);
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            if (eb + 32 * k < e1)
+#pragma unroll
+              for (int m = 0; m < 4; ++m) a[m] = fma(v[k][m], p[k], a[m]);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) v[k][m] = w[k][m];
+            p[k] = pw2[k];
+          }
+        }
+        // lanes with bit 4 take rows 2, 3, with bit 3 the odd row of the two
+        const bool h4 = lane & 16, h3 = lane & 8;
+        double c0 = h4 ? a[2] : a[0], c1 = h4 ? a[3] : a[1];
+        c0 += __shfl_xor_sync(0xffffffffu, h4 ? a[0] : a[2], 16);
+        c1 += __shfl_xor_sync(0xffffffffu, h4 ? a[1] : a[3], 16);
+        double c = h3 ? c1 : c0;
+        c += __shfl_xor_sync(0xffffffffu, h3 ? c0 : c1, 8);
+        c = warp_sum(c, 1, 8);
+        const int m = lane >> 3;
+        if ((lane & 7) == 0 && i0 + m < kq) qs[rcg_row(u, upb, kq) - row0 + m] += c;
+      }
+    }
+    __syncthreads();
+    loc = 0.0;
+    for (int i = tid; i < rows; i += kRcgThreads) loc += ps[i] * qs[i];
+    if (!rcg_exchange(
+            x, loc, [=](double pq, double* o) { o[0] = pq > 0.0 ? rz / pq : 0.0; }))
+      return;
+    const double al = res[0];
+    loc = 0.0;
+    for (int i = tid; i < rows; i += kRcgThreads) {
+      xs[i] += al * ps[i];
+      const double r = rs[i] - al * qs[i];
+      rs[i] = r;
+      __stcg(s.r + row0 + i, r);
+      loc += r * r;
+    }
+    if (!rcg_exchange(x, loc, [=](double t, double* o) {
+          o[0] = t;
+          o[1] = t / rz;
+          o[2] = t <= tol2 * bb || !(rz > 0.0) ? 1.0 : 0.0;
+        }))
+      return;
+    ++it;
+    rr = res[0];
+    done = res[2] != 0.0;
+    if (!done) {
+      be = res[1];
+      rz = rr;
+    }
+  }
+  // x and E = b~.x
+  loc = 0.0;
+  for (int i = tid; i < rows; i += kRcgThreads) {
+    s.x[row0 + i] = xs[i];
+    loc += bt[row0 + i] * xs[i];
+  }
+  if (!rcg_exchange(x, loc, [](double t, double* o) { o[0] = t; })) return;
+  if (blockIdx.x == 0 && tid == 0) {
+    s.scal[0] = rz;
+    s.scal[1] = bb;
+    s.scal[4] = rr;
+    s.scal[6] = res[0];
     s.flag[0] = done;
     s.flag[1] = it;
   }
@@ -335,28 +685,80 @@ void launch_rcg_step(int n_sd, int kq, const int32_t* nbr_ptr, const int32_t* nb
   k_rcg_update_p<<<n_sd, 128, 0, st>>>(kq, s);
 }
 
-int launch_rcg_persistent(int n_sd, int kq, const int32_t* nbr_ptr, const int32_t* nbr_sd,
-                          const int32_t* nbr_blk, const double* blocks, const double* bt,
-                          double tol2, int max_iter, const RcgState& s, unsigned* sync,
-                          long long budget, cudaStream_t st) {
-  int dev = 0, nsm = 0, per_sm = 0, coop = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return -1;
+RcgLaunch launch_rcg_solve(int n_sd, int kq, const int32_t* nbr_ptr, const int32_t* nbr_sd,
+                           const int32_t* nbr_blk, int64_t n_blocks, const double* blocks,
+                           const double* bt, double tol2, int max_iter, const RcgState& s,
+                           double* part, long long budget, bool try_cluster,
+                           cudaStream_t st) {
+  int dev = 0, nsm = 0, coop = 0, smem_max = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return RcgLaunch::kNone;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-  if (!coop) return -1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rcg_persistent, 128, 0) !=
-          cudaSuccess ||
-      per_sm < 1)
-    return -1;
-  int grid = std::min(n_sd, nsm * per_sm);
+  cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  const int64_t dim = (int64_t)n_sd * kq;
+  cudaLaunchAttribute at{};
+  cudaLaunchConfig_t cfg{};
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
   RcgState sc = s;
+  if (try_cluster && dim <= kRcgClusterDim &&
+      (double)n_blocks * kq * kq <= kRcgClusterFma && (size_t)smem_max >= kRcgClusterSmem + 8192) {
+    const int G = (int)std::min<int64_t>(kRcgCluster, dim);
+    const int rows = (int)((dim + G - 1) / G);
+    const int nth = (4 * rows + 31) / 32 * 32;
+    int entries = (int)((kRcgClusterSmem - 2 * sizeof(double) * (size_t)dim) /
+                        (sizeof(double) + sizeof(uint16_t)));
+    entries &= ~7;
+    const void* fn = (const void*)k_rcg_cluster;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kRcgClusterSmem) != cudaSuccess)
+      return RcgLaunch::kNone;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)G;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)G);
+    cfg.blockDim = dim3((unsigned)nth);
+    cfg.dynamicSmemBytes = kRcgClusterSmem;
+    void* args[] = {&n_sd, &kq, (void*)&nbr_ptr, (void*)&nbr_sd, (void*)&nbr_blk,
+                    (void*)&blocks, (void*)&bt, &tol2, &max_iter, &entries, &sc};
+    if (cudaLaunchKernelExC(&cfg, fn, args) == cudaSuccess) {
+      count_launch();
+      return RcgLaunch::kCluster;
+    }
+    cudaGetLastError();
+  }
+  const int64_t units = (int64_t)n_sd * ((kq + 3) / 4);
+  if (!coop || kq > kRcgCap || units > INT32_MAX || nsm < 1) return RcgLaunch::kNone;
+  const int G = (int)std::min<int64_t>(std::min(nsm, kRcgMaxGrid), units);
+  // weighted runs hold at most five times the mean number of units; where that does not
+  // fit in shared memory, runs of equal length
+  const int64_t mean = (units + G - 1) / G;
+  int weighted = 1;
+  int64_t rows = 4 * (5 * mean + 2);
+  const auto smem = [&](int64_t r) { return 4 * sizeof(double) * (size_t)r + kRcgStageBytes; };
+  const size_t cap = std::min<size_t>(200 * 1024, (size_t)smem_max);
+  if (smem(rows) > cap) {
+    weighted = 0;
+    rows = 4 * mean;
+  }
+  if (smem(rows) > cap) return RcgLaunch::kNone;
+  int rows_max = (int)rows;
+  const void* fn = (const void*)k_rcg_grid;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)smem(rows)) != cudaSuccess)
+    return RcgLaunch::kNone;
+  at.id = cudaLaunchAttributeCooperative;
+  at.val.cooperative = 1;
+  cfg.gridDim = dim3((unsigned)G);
+  cfg.blockDim = dim3(kRcgThreads);
+  cfg.dynamicSmemBytes = smem(rows);
   void* args[] = {&n_sd, &kq, (void*)&nbr_ptr, (void*)&nbr_sd, (void*)&nbr_blk,
-                  (void*)&blocks, (void*)&bt, &tol2, &max_iter, &sc, &sync, &budget};
+                  (void*)&blocks, (void*)&bt, &tol2, &max_iter, &rows_max, &weighted, &sc,
+                  &part, &budget};
+  if (cudaLaunchKernelExC(&cfg, fn, args) != cudaSuccess) return RcgLaunch::kNone;
   count_launch();
-  if (cudaLaunchCooperativeKernel((const void*)k_rcg_persistent, grid, 128, args, 0, st) !=
-      cudaSuccess)
-    return -1;
-  return grid;
+  return RcgLaunch::kGrid;
 }
 
 void launch_wait_unset_flag(unsigned* sync, long long budget, int* status, cudaStream_t st) {
