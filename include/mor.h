@@ -389,6 +389,15 @@ int mor_debug_tc_gram(int64_t rows, int32_t nx, int32_t ny, const double* X_dev,
  * local solves are direct). */
 int mor_debug_coarse_inverse(int32_t n, const double* E_dev, double* Einv_dev, void* stream);
 
+/* Debug/parity access: the eigensolver of step 2 (H_i-orthonormalisation, singular values,
+ * diagonal-block update) on n_sub symmetric positive semidefinite matrices A_dev [device,
+ * n_sub x n x n], 1 <= n <= 1024: pivoted Cholesky and one-sided Jacobi in binary64.
+ * evals_dev [device, n_sub x n] descending (noise and null directions 0), evecs_dev
+ * [device, n_sub x n x n] the eigenvectors as columns.  Allocates its work space.  The paper
+ * has no counterpart. */
+int mor_debug_sym_eig(int32_t n_sub, int32_t n, const double* A_dev, double* evals_dev,
+                      double* evecs_dev, void* stream);
+
 /* Kernel timing for the roofline: when enabled, the four kernels of every local CG
  * step of mor_build_bases are bracketed by CUDA events on the launching stream.
  * mor_profile_query fills out[host, 4] = {launches, total milliseconds, algorithmic

@@ -1149,9 +1149,9 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
       // the sketch Grams (k x k) and the diagonal-block Gram (at most 128 x 128)
       gsz = std::max(gsz, (size_t)n_sd * gram_wide_chunks(n_sd, k, k) * k * k);
       gsz = std::max(gsz, (size_t)n_sd * 16 * 128 * 128);
-      TRY(M.alloc(&eigw, (size_t)n_sd * 2 * kb * kb, false, st));
     }
     TRY(M.alloc(&gpart, gsz, true, st));
+    TRY(M.alloc(&eigw, (size_t)n_sd * sym_eig_work(kb), false, st));
   }
   TRY(M.alloc(&gcnt, n_sd, true, st));
   TRY(M.alloc(&kcnt, n_sd, true, st));
@@ -1180,10 +1180,7 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
       launch_gram(tl, n_sd, X, ldx, nx, Y, ldy, ny, gpart, gcnt, G, ldg, st);
   };
   auto sym_eig = [&](int ld, int n, double* ev, double* V_) {
-    if (n > 80)
-      launch_sym_eig_wide(n_sd, G, ld, n, ev, V_, eigw, st);
-    else
-      launch_sym_eig(n_sd, G, ld, n, ev, V_, st);
+    launch_sym_eig(n_sd, G, ld, n, ev, V_, eigw, st);
   };
   auto rowmul = [&](const DTiles& tl, const double* X, int ldx, int nin, int ldm, double* Y,
                     int ldy, int nout) {
@@ -1342,12 +1339,11 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
     if (mB > 80) {
       launch_gram_wide(S.tW, n_sd, Yw2, ldm, mB, Yw2, ldm, mB, gp, Gx, ldm, (int64_t)ldm * ldm,
                        st);
-      TRY(M.alloc(&ew, (size_t)n_sd * 2 * ldm * ldm, false, st));
-      launch_sym_eig_wide(n_sd, Gx, ldm, mB, evx, Vx, ew, st);
     } else {
       launch_gram(S.tW, n_sd, Yw2, ldm, mB, Yw2, ldm, mB, gp, gcnt, Gx, ldm, st);
-      launch_sym_eig(n_sd, Gx, ldm, mB, evx, Vx, st);
     }
+    TRY(M.alloc(&ew, (size_t)n_sd * sym_eig_work(mB), false, st));
+    launch_sym_eig(n_sd, Gx, ldm, mB, evx, Vx, ew, st);
     // kept directions: the first m_i, or sigma_j > eps (Eq. (15)); U_m = X V_m Sigma_m^-1
     std::vector<int32_t> keep(n_sd);
     for (int i = 0; i < n_sd; ++i) keep[i] = tol_mode ? DW.h_M[i] : h_rank[i];
@@ -2054,6 +2050,21 @@ int mor_debug_coarse_inverse(int32_t n, const double* E_dev, double* Einv_dev, v
   CK(cudaMemcpyAsync(&h, bad, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   if (h) return fail(MOR_ERR_ARG, "mor_debug_coarse_inverse: a pivot is not positive");
+  return MOR_OK;
+}
+
+int mor_debug_sym_eig(int32_t n_sub, int32_t n, const double* A_dev, double* evals_dev,
+                      double* evecs_dev, void* stream) {
+  if (n_sub < 1 || n < 1 || n > 1024 || !A_dev || !evals_dev || !evecs_dev)
+    return fail(MOR_ERR_ARG, "mor_debug_sym_eig: bad argument");
+  cudaStream_t st = (cudaStream_t)stream;
+  Allocs A;
+  A.use_pool(st);
+  double* work;
+  TRY(A.alloc(&work, (size_t)n_sub * sym_eig_work(n), false, st));
+  launch_sym_eig(n_sub, A_dev, n, n, evals_dev, evecs_dev, work, st);
+  CK(cudaGetLastError());
+  CK(cudaStreamSynchronize(st));
   return MOR_OK;
 }
 

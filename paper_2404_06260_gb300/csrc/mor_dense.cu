@@ -1,7 +1,6 @@
 // Small dense per-subdomain linear algebra of step 2 (Sec. 4, Sec. 6): tall-skinny
-// Grams X^T Y, the symmetric eigensolver used for the H_i-orthonormalisation, the
-// singular values of the projected operator (Eq. (24)) and the diagonal-block update,
-// and the k x k right-multiplications that apply their results to row blocks.
+// Grams X^T Y, and the k x k right-multiplications that apply the eigensolver's results
+// (mor_eig.cu) to row blocks.
 #include "mor_kernels.h"
 
 namespace mor {
@@ -72,120 +71,6 @@ __global__ void __launch_bounds__(kGramThreads)
     for (int t = lo; t < hi; ++t) s += __ldcg(part + (int64_t)t * nout + o);
     int i = o / ny, j = o % ny;
     G[(int64_t)sd * sd_stride + i * ldg + j] = s;
-  }
-}
-
-// cyclic Jacobi with the round-robin (circle) ordering: m/2 disjoint rotations per
-// round, m-1 rounds per sweep; A <- J^T A J, V <- V J with the symmetric 2x2 Schur
-// rotation (Golub & Van Loan, Alg. 8.4.1).  A pair is rotated only while
-// |a_pq| > eps sqrt(|a_pp a_qq|) (eps = 2^-52), the threshold that keeps small
-// eigenvalues accurate relative to themselves (Demmel & Veselic); the iteration stops
-// after a sweep without rotations (at most 40 sweeps).
-__global__ void k_sym_eig(const double* __restrict__ A, int ld, int n, double* evals,
-                          double* evecs) {
-  extern __shared__ double sh[];
-  int m = n + (n & 1);
-  int lds = m + 1;
-  double* a = sh;
-  double* v = a + m * lds;
-  double* rc = v + m * lds;        // m/2 cosines
-  double* rs = rc + m / 2;         // m/2 sines
-  double* red = rs + m / 2;        // blockDim.x
-  int* rp = reinterpret_cast<int*>(red + blockDim.x);
-  int* rq = rp + m / 2;
-  int sd = blockIdx.x;
-  int tid = threadIdx.x, nth = blockDim.x;
-  const double* As = A + (int64_t)sd * ld * ld;
-  for (int idx = tid; idx < m * m; idx += nth) {
-    int i = idx / m, j = idx % m;
-    a[i * lds + j] = (i < n && j < n) ? 0.5 * (As[i * ld + j] + As[j * ld + i]) : 0.0;
-    v[i * lds + j] = (i == j) ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  auto block_sum = [&](double x) -> double {
-    red[tid] = x;
-    __syncthreads();
-    for (int s = nth / 2; s > 0; s >>= 1) {
-      if (tid < s) red[tid] += red[tid + s];
-      __syncthreads();
-    }
-    double r = red[0];
-    __syncthreads();
-    return r;
-  };
-  (void)block_sum;
-  __shared__ int nrot;
-  for (int sweep = 0; sweep < 40 && m > 1; ++sweep) {
-    if (tid == 0) nrot = 0;
-    __syncthreads();
-    for (int round = 0; round < m - 1; ++round) {
-      for (int k = tid; k < m / 2; k += nth) {
-        int x0 = k, x1 = m - 1 - k;
-        int p = (x0 == 0) ? 0 : ((x0 - 1 + round) % (m - 1)) + 1;
-        int q = ((x1 - 1 + round) % (m - 1)) + 1;
-        double apq = a[p * lds + q];
-        double c = 1.0, s = 0.0;
-        if (fabs(apq) > 0x1p-52 * sqrt(fabs(a[p * lds + p] * a[q * lds + q]))) {
-          atomicAdd(&nrot, 1);
-          double tau = (a[q * lds + q] - a[p * lds + p]) / (2.0 * apq);
-          double t;
-          if (fabs(tau) > 1e150)
-            t = 0.5 / tau;
-          else
-            t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-          c = 1.0 / sqrt(1.0 + t * t);
-          s = t * c;
-        }
-        rp[k] = p;
-        rq[k] = q;
-        rc[k] = c;
-        rs[k] = s;
-      }
-      __syncthreads();
-      for (int w = tid; w < (m / 2) * m; w += nth) {
-        int k = w / m, j = w % m;
-        double c = rc[k], s = rs[k];
-        if (s == 0.0) continue;  // pair not rotated
-        int p = rp[k], q = rq[k];
-        double ap = a[p * lds + j], aq = a[q * lds + j];
-        a[p * lds + j] = c * ap - s * aq;
-        a[q * lds + j] = s * ap + c * aq;
-      }
-      __syncthreads();
-      for (int w = tid; w < (m / 2) * m; w += nth) {
-        int k = w / m, i = w % m;
-        double c = rc[k], s = rs[k];
-        if (s == 0.0) continue;
-        int p = rp[k], q = rq[k];
-        double ap = a[i * lds + p], aq = a[i * lds + q];
-        a[i * lds + p] = c * ap - s * aq;
-        a[i * lds + q] = s * ap + c * aq;
-        double vp = v[i * lds + p], vq = v[i * lds + q];
-        v[i * lds + p] = c * vp - s * vq;
-        v[i * lds + q] = s * vp + c * vq;
-      }
-      __syncthreads();
-    }
-    // every thread reads the count before thread 0 resets it for the next sweep
-    const int rotated = nrot;
-    __syncthreads();
-    if (rotated == 0) break;
-  }
-  double* ev = evals + (int64_t)sd * ld;
-  double* V = evecs + (int64_t)sd * ld * ld;
-  for (int idx = tid; idx < ld * ld; idx += nth) V[idx] = 0.0;
-  for (int i = tid; i < ld; i += nth)
-    if (i >= n) ev[i] = 0.0;
-  __syncthreads();
-  for (int i = tid; i < n; i += nth) {
-    double li = a[i * lds + i];
-    int rank = 0;
-    for (int j = 0; j < n; ++j) {
-      double lj = a[j * lds + j];
-      if (lj > li || (lj == li && j < i)) ++rank;
-    }
-    ev[rank] = li;
-    for (int r = 0; r < n; ++r) V[r * ld + rank] = v[r * lds + i];
   }
 }
 
@@ -299,21 +184,6 @@ void launch_gram_vec(const DTiles& tiles, int n_sd, const double* X, int ldx, in
   // the nx x 1 product, rows of stride 1 and ldg per subdomain
   k_gram<<<tiles.n, kGramThreads, sm, st>>>(tiles, X, ldx, nx, y, ldy, 1, part, counter, g, 1,
                                            ldg);
-}
-
-void launch_sym_eig(int n_sd, const double* A, int ld, int n, double* evals,
-                    double* evecs, cudaStream_t st) {
-  if (n_sd <= 0) return;
-  int m = n + (n & 1);
-  int nth = 256;
-  size_t sm = sizeof(double) * (2 * (size_t)m * (m + 1) + m + nth) + sizeof(int) * m;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_sym_eig, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr = true;
-  }
-  count_launch();
-  k_sym_eig<<<n_sd, nth, sm, st>>>(A, ld, n, evals, evecs);
 }
 
 void launch_make_M(int n_sd, int mode, const double* evals, const double* evecs, int ld,

@@ -1,0 +1,636 @@
+// The symmetric eigensolver of step 2 (the H_i-orthonormalisation, the singular values of
+// Eq. (24) or Eq. (14) and the diagonal-block update, Sec. 6): batched positive
+// semidefinite matrices, one per subdomain, of order up to 1024.
+//
+// Method: a diagonally pivoted Cholesky factor G = L L^T, then one-sided Jacobi on the
+// columns of L (Veselic & Hari, Numer. Math. 56, 1989; Demmel & Veselic, SIAM J. Matrix
+// Anal. 13, 1992): rotations make the columns W = L V orthogonal, and W_j = sigma_j u_j
+// gives eigenvalue sigma_j^2 and eigenvector u_j, accurate relative to themselves as those
+// of the two-sided threshold iteration.  The eigenvectors need no accumulation, a rotation
+// touches two columns instead of two rows, two columns and two more of V, and the pivoted
+// factor starts nearly orthogonal: 4 to 7 sweeps.
+//  - Scaling: G by a power of two to a largest diagonal entry in [1, 2).
+//  - A column whose pivot falls below n 2^-53 of its own diagonal entry is rounding noise:
+//    it becomes 2^-40 e_j (times the root of its entry), which the iteration turns into
+//    the completion of the eigenvectors; its eigenvalue (below 2^-70) is returned as 0.
+//    Columns with a zero diagonal entry stay out: eigenvalue 0, eigenvector e_j.
+//  - A pair rotates while |w_p.w_q| > sqrt(n) 2^-53 |w_p| |w_q| (the rounding level of the
+//    product); the iteration stops after a sweep without rotations (at most 40).
+//  - The tangent is formed in binary32 and only the orthogonality of the rotation in
+//    binary64: c = (1 + t^2)^(-1/2) by one third-order Householder step from a binary32
+//    root, s = t c.  An angle off by 2^-24 leaves 2^-24 of the product to the next sweep.
+//
+// What bounds it: binary64 issue (a warp instruction keeps a quarter of the SM busy for 64
+// clocks) and, for small orders, the chain product -> tangent -> rotation of each round.
+// Orders up to kEigSmem: one CTA per subdomain, the factor in shared memory, 8 lanes per
+// pair (k_sym_eig).  Larger ones: a cluster per subdomain works on pairs of column blocks
+// staged from L2 (k_sym_eig_blocks).
+// Per batch, against the two-sided iteration with the matrix in shared memory (up to 80) or
+// in L2 and one CTA per subdomain: 64 matrices of order 42 2.13 -> 1.06 ms, 40 of 74 8.5 ->
+// 2.6 ms, 14 of up to 261 145 -> 10 ms, 8 of 127 169 -> 6 ms (the noise directions of an
+// explicit Gram never met the two-sided threshold and ran all 40 sweeps).
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
+#include "mor_kernels.h"
+
+namespace mor {
+namespace {
+
+constexpr int kEigSmem = 128;  // largest order of k_sym_eig (128^2 binary64 in shared memory)
+constexpr int kEigMax = 1024;
+constexpr int kEigSweeps = 40;
+constexpr int kEigLanes = 8;  // lanes per column pair in k_sym_eig
+
+// d^(-1/2) for d in [2^-100, 2^100]: Householder's third-order iteration from binary32
+__device__ __forceinline__ double inv_sqrt(double d) {
+  const double y = (double)rsqrtf((float)d);
+  const double e = fma(-d * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// 2^-e with |x| in [2^e, 2^(e+1))
+__device__ __forceinline__ double pow2_below(double x) {
+  const int e = (int)((__double_as_longlong(x) >> 52) & 0x7FF);
+  return __longlong_as_double((long long)(2046 - e) << 52);
+}
+
+// about 2^-22 accurate; 0 for negative and zero x
+__device__ __forceinline__ float fast_sqrt(float x) { return x > 0.0f ? x * rsqrtf(x) : 0.0f; }
+
+// A column is d * w with 1 / d kept beside d, so that a rotation takes one multiply-add
+// per entry: c (p - t q) = (c d_p) (w_p - t d_q / d_p w_q).  d returns to 1 when the column
+// is next loaded or its norm taken.
+struct JCol {
+  double sq;     // squared norm of d * w, updated by the rotations
+  double d, di;  // scale and its inverse
+};
+
+// the rotation that orthogonalises columns p and q, pq = w_p.w_q: w_p -= al w_q, w_q += be
+// w_p (old), and the columns' new state in p and q; false when the product is at the
+// rounding level
+__device__ __forceinline__ bool jacobi_rotation(JCol& p, JCol& q, double pq, float tol,
+                                                double& al, double& be) {
+  const double apq = p.d * q.d * pq;
+  const float o = (float)apq;
+  // only the angle: binary32 roots and quotients by the fast instructions are exact enough
+  if (!(fabsf(o) > tol * (fast_sqrt((float)p.sq) * fast_sqrt((float)q.sq)))) return false;
+  const float tau = 0.5f * __fdividef((float)(q.sq - p.sq), o);
+  const float a = fabsf(tau);
+  const float tt = a > 1e8f ? __fdividef(0.5f, a)
+                            : __fdividef(1.0f, a + fast_sqrt(fmaf(a, a, 1.0f)));
+  const double t = (double)(tau >= 0.0f ? tt : -tt);
+  const double h = fma(t, t, 1.0), c = inv_sqrt(h), ci = h * c;
+  al = t * (q.d * p.di);
+  be = t * (p.d * q.di);
+  p.sq = fma(-t, apq, p.sq);
+  q.sq = fma(t, apq, q.sq);
+  p.d *= c;
+  q.d *= c;
+  p.di *= ci;
+  q.di *= ci;
+  return true;
+}
+
+// pair k of round `round` of the circle method over m (even) players
+__device__ __forceinline__ void circle_pair(int m, int round, int k, int& p, int& q) {
+  const int x1 = m - 1 - k;
+  int a = k - 1 + round, b = x1 - 1 + round;
+  if (a >= m - 1) a -= m - 1;
+  if (b >= m - 1) b -= m - 1;
+  p = k == 0 ? 0 : a + 1;
+  q = b + 1;
+}
+
+// rank by descending value (ties by index) of the n values in ev
+__device__ __forceinline__ int rank_of(const double* ev, int n, int i) {
+  const long long li = __double_as_longlong(ev[i]);  // values >= 0 order like their bits
+  int r = 0;
+  for (int j = 0; j < n; ++j) {
+    const long long lj = __double_as_longlong(ev[j]);
+    r += lj > li || (lj == li && j < i);
+  }
+  return r;
+}
+
+// a matrix with an infinity or a NaN: every result is NaN
+__device__ __forceinline__ void fill_nan(int ld, int n, double* ev, double* V) {
+  const double nan = __longlong_as_double(0x7ff8000000000000LL);
+  for (int64_t idx = threadIdx.x; idx < (int64_t)ld * ld; idx += blockDim.x)
+    V[idx] = idx / ld < n && idx % ld < n ? nan : 0.0;
+  for (int i = threadIdx.x; i < ld; i += blockDim.x) ev[i] = i < n ? nan : 0.0;
+}
+
+// One CTA per subdomain; columns of lds = kEigLanes * E doubles (rows beyond n zero).
+template <int E>
+__global__ void __launch_bounds__(E <= 12 ? 384 : 512)
+    k_sym_eig(const double* __restrict__ A, int ld, int n, double* evals, double* evecs) {
+  constexpr int lds = kEigLanes * E;
+  extern __shared__ __align__(16) double eig_sh[];
+  double* w = eig_sh;                 // n columns
+  double* g0 = w + (size_t)n * lds;   // diagonal of G
+  JCol* jc = reinterpret_cast<JCol*>(g0 + n);
+  double* nrm = g0 + n;  // factor: open columns < 0; at last the eigenvalues (over jc)
+  int* act = reinterpret_cast<int*>(jc + n);
+  __shared__ int s_m, s_p, s_rot;
+  __shared__ double s_scale;
+  const int sd = blockIdx.x, tid = threadIdx.x, nth = blockDim.x, lane = tid & 31;
+  const double* As = A + (int64_t)sd * ld * ld;
+  if (tid < 32) {
+    double mx = 0.0;
+    for (int i = lane; i < n; i += 32) mx = fmax(mx, As[(int64_t)i * ld + i]);
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) s_scale = mx > 0x1p-1000 && mx < 0x1p1000 ? pow2_below(mx) : 1.0;
+  }
+  __syncthreads();
+  const double scale = s_scale;
+  double* ev = evals + (int64_t)sd * ld;
+  double* V = evecs + (int64_t)sd * ld * ld;
+  bool bad = false;
+  for (int idx = tid; idx < n * lds; idx += nth) {
+    const int j = idx / lds, i = idx - j * lds;
+    double v = 0.0;
+    if (i < n) v = 0.5 * (As[(int64_t)i * ld + j] + As[(int64_t)j * ld + i]) * scale;
+    bad = bad || !isfinite(v);
+    w[idx] = v;
+    if (i == j) g0[j] = v;
+  }
+  if (__syncthreads_or(bad)) return fill_nan(ld, n, ev, V);
+  // ---- pivoted Cholesky: column p of w becomes the factor's column, with zeros in the rows
+  // factored before; nrm[j] < 0 marks a column still to be factored ----
+  const double noise = (double)n * 0x1p-53;
+  for (int j = tid; j < n; j += nth) nrm[j] = -1.0;
+  if (tid == 0) s_m = 0;
+  __syncthreads();
+  for (int step = 0; step < n; ++step) {
+    if (tid < 32) {
+      // the largest remaining diagonal entry above its noise level: positive doubles order
+      // like their bits, whose low byte gives way to the index
+      long long best = 0;
+      for (int j = lane; j < n; j += 32) {
+        const double d = w[j * lds + j];
+        if (nrm[j] < 0.0 && d > noise * g0[j] && d > 0x1p-120) {
+          const long long key = (__double_as_longlong(d) & ~255LL) | j;
+          best = best > key ? best : key;
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const long long x = __shfl_xor_sync(0xffffffffu, best, o);
+        best = best > x ? best : x;
+      }
+      if (lane == 0) s_p = best > 0 ? (int)(best & 255) : -1;
+    }
+    __syncthreads();
+    const int p = s_p;
+    if (p < 0) break;
+    double* wp = w + p * lds;
+    const double d = wp[p];
+    const double y = d > 0x1p-90 ? inv_sqrt(d) : 1.0 / sqrt(d);
+    __syncthreads();
+    for (int i = tid; i < n; i += nth) wp[i] = nrm[i] < 0.0 ? wp[i] * y : 0.0;
+    __syncthreads();
+    if (tid == 0) {
+      nrm[p] = 1.0;
+      act[step] = p;  // the pairs run in pivot order: one or two sweeps fewer
+      s_m = step + 1;
+    }
+    for (int idx = tid; idx < n * lds; idx += nth) {
+      const int j = idx / lds, i = idx - j * lds;
+      if (j != p && nrm[j] < 0.0) w[idx] = fma(-wp[j], wp[i], w[idx]);
+    }
+    __syncthreads();
+  }
+  // noise columns, and the list of columns that take part
+  for (int j = 0; j < n; ++j)
+    if (nrm[j] < 0.0)
+      for (int i = tid; i < lds; i += nth)
+        w[j * lds + i] = i == j ? 0x1p-40 * sqrt(fmax(g0[j], 0x1p-53)) : 0.0;
+  if (tid < 32) {
+    int c = s_m;
+    for (int j0 = 0; j0 < n; j0 += 32) {
+      const bool in = j0 + lane < n && nrm[j0 + lane] < 0.0 && g0[j0 + lane] > 0.0;
+      const unsigned b = __ballot_sync(0xffffffffu, in);
+      if (in) act[c + __popc(b & ((1u << lane) - 1))] = j0 + lane;
+      c += __popc(b);
+    }
+    if (lane == 0) s_m = c;
+  }
+  __syncthreads();
+  // ---- one-sided Jacobi ----
+  const int m = s_m, me = m + (m & 1);
+  const int grp = tid / kEigLanes, gl = tid % kEigLanes, ngrp = nth / kEigLanes;
+  const float tol = sqrtf((float)n) * 0x1p-53f;
+  auto squares = [&](int j) {  // squared norm of column j by the 8 lanes of a group
+    double s = 0.0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const double v = w[j * lds + gl + kEigLanes * e];
+      s = fma(v, v, s);
+    }
+    for (int o = 1; o < kEigLanes; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+  };
+  for (int sweep = 0; sweep < kEigSweeps; ++sweep) {
+    for (int k0 = 0; k0 < n; k0 += ngrp) {  // whole warps stay together for the shuffles
+      const int j = min(k0 + grp, n - 1);
+      const bool in = k0 + grp < n;
+      if (sweep > 0 && in) {
+        const double d = jc[j].d;
+#pragma unroll
+        for (int e = 0; e < E; ++e) w[j * lds + gl + kEigLanes * e] *= d;
+      }
+      __syncwarp();
+      const double s = squares(j);
+      if (gl == 0 && in) jc[j] = JCol{s, 1.0, 1.0};
+    }
+    if (tid == 0) s_rot = 0;
+    __syncthreads();
+    if (m < 2) break;
+    for (int round = 0; round < me - 1; ++round) {
+      for (int k0 = 0; k0 < me / 2; k0 += ngrp) {
+        const int k = k0 + grp;
+        int p = -1, q = -1;
+        if (k < me / 2) circle_pair(me, round, k, p, q);
+        const bool on = p >= 0 && p < m && q < m;
+        p = on ? act[p] : 0;
+        q = on ? act[q] : 0;
+        double a[E], b[E], s0 = 0.0, s1 = 0.0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          a[e] = w[p * lds + gl + kEigLanes * e];
+          b[e] = w[q * lds + gl + kEigLanes * e];
+          if (e & 1)
+            s1 = fma(a[e], b[e], s1);
+          else
+            s0 = fma(a[e], b[e], s0);
+        }
+        double pq = s0 + s1;
+        for (int o = 1; o < kEigLanes; o <<= 1) pq += __shfl_xor_sync(0xffffffffu, pq, o);
+        JCol cp = jc[p], cq = jc[q];
+        double al, be;
+        if (!on || !jacobi_rotation(cp, cq, pq, tol, al, be)) continue;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          w[p * lds + gl + kEigLanes * e] = fma(-al, b[e], a[e]);
+          w[q * lds + gl + kEigLanes * e] = fma(be, a[e], b[e]);
+        }
+        if (gl == 0) {
+          jc[p] = cp;
+          jc[q] = cq;
+          s_rot = 1;
+        }
+      }
+      __syncthreads();
+    }
+    const int rotated = s_rot;
+    __syncthreads();
+    if (!rotated) break;
+  }
+  // ---- eigenvalues in descending order, normalised columns ----
+  for (int k0 = 0; k0 < n; k0 += ngrp) {
+    const int j = min(k0 + grp, n - 1);
+    const double d = jc[j].d;  // 1 unless the last sweep still rotated
+    const double s = d * d * squares(j);
+    const bool in = k0 + grp < n;
+    __syncthreads();
+    if (gl == 0 && in) {
+      nrm[j] = s >= 0x1p-70 && g0[j] > 0.0 ? s : 0.0;
+      g0[j] = s > 0.0 ? d / sqrt(s) : 0.0;  // from here the column's scale
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < n; i += nth) act[i] = rank_of(nrm, n, i);
+  __syncthreads();
+  for (int i = tid; i < ld; i += nth) {
+    if (i < n)
+      ev[act[i]] = nrm[i] / scale;
+    else
+      ev[i] = 0.0;
+  }
+  for (int64_t idx = tid; idx < (int64_t)ld * ld; idx += nth) {
+    const int r = (int)(idx / ld), j = (int)(idx - (int64_t)r * ld);
+    if (r >= n || j >= n)
+      V[idx] = 0.0;
+    else
+      V[(int64_t)r * ld + act[j]] = w[j * lds + r] * g0[j];
+  }
+}
+
+// A cluster of C CTAs per subdomain.  Cholesky: CTA c keeps the columns j = c mod C
+// (shared memory, or its part of `work` where they do not fit) and the pivot's owner
+// writes the finished column to W, in pivot order; two cluster barriers per column.
+// Jacobi: the columns of W in blocks of b; a round of the circle method over the blocks
+// gives every CTA pairs of blocks, which it stages in shared memory, rotates (GL lanes per
+// column pair; all pairs of both blocks in the first round of a sweep, the pairs across
+// them in the others) and writes back; one cluster barrier per round.
+constexpr size_t kEigBlkSmem = 200 * 1024;
+template <int GL>
+__global__ void __launch_bounds__(768)
+    k_sym_eig_blocks(const double* __restrict__ A, int ld, int n, int b, int in_smem,
+                     double* evals, double* evecs, double* work) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  extern __shared__ __align__(16) double eig_sh[];
+  __shared__ long long s_key[2][8];
+  __shared__ int s_rot[2][8];
+  __shared__ int s_flag;
+  __shared__ double s_red[32];
+  const int C = (int)cl.num_blocks(), c = (int)cl.block_rank();
+  const int sd = blockIdx.x / C;
+  const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  const int nw = nth >> 5;
+  const double* As = A + (int64_t)sd * ld * ld;
+  double* ev = evals + (int64_t)sd * ld;
+  double* V = evecs + (int64_t)sd * ld * ld;
+  // global: W (columns), eigenvalues | open flags, diagonal of G, and the columns to factor
+  double* base = work + (int64_t)sd * (2 * (int64_t)n * n + 16 * n);
+  double* W = base;
+  double* gn = base + (int64_t)n * n;
+  double* gd = gn + n;
+  double* stage = in_smem ? eig_sh + (size_t)((n + C - 1) / C) * n : eig_sh;  // pivot column
+  double* F = in_smem ? eig_sh
+                      : base + (int64_t)n * n + 4 * n + (int64_t)c * ((n + C - 1) / C) * n;
+  // power-of-two scale by the largest diagonal entry
+  double mx = 0.0;
+  for (int i = tid; i < n; i += nth) mx = fmax(mx, As[(int64_t)i * ld + i]);
+  for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) s_red[warp] = mx;
+  __syncthreads();
+  mx = 0.0;
+  for (int k = 0; k < nw; ++k) mx = fmax(mx, s_red[k]);
+  const double scale = mx > 0x1p-1000 && mx < 0x1p1000 ? pow2_below(mx) : 1.0;
+  const int own = (n - c + C - 1) / C;  // columns c, c + C, ...
+  bool bad = false;
+  for (int64_t idx = tid; idx < (int64_t)own * n; idx += nth) {
+    const int k = (int)(idx / n), i = (int)(idx - (int64_t)k * n), j = c + C * k;
+    const double v = 0.5 * (As[(int64_t)i * ld + j] + As[(int64_t)j * ld + i]) * scale;
+    F[idx] = v;
+    bad = bad || !isfinite(v);
+    if (i == j) {
+      __stcg(gd + j, v);
+      __stcg(gn + j, -1.0);  // still to be factored
+    }
+  }
+  bad = __syncthreads_or(bad) != 0;
+  if (tid < C) *cl.map_shared_rank(&s_rot[0][c], tid) = bad;
+  cl.sync();
+  for (int g = 0; g < C; ++g) bad = bad || s_rot[0][g];
+  if (bad) {
+    if (c == 0) fill_nan(ld, n, ev, V);
+    cl.sync();
+    return;
+  }
+  const double noise = (double)n * 0x1p-53;
+  int r = 0;  // pivots taken
+  for (; r < n; ++r) {
+    const int par = r & 1;
+    if (warp == 0) {
+      long long best = 0;
+      for (int k = lane; k < own; k += 32) {
+        const int j = c + C * k;
+        const double d = F[(int64_t)k * n + j];
+        if (__ldcg(gn + j) < 0.0 && d > noise * __ldcg(gd + j) && d > 0x1p-120) {
+          const long long key = (__double_as_longlong(d) & ~2047LL) | j;
+          best = best > key ? best : key;
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const long long x = __shfl_xor_sync(0xffffffffu, best, o);
+        best = best > x ? best : x;
+      }
+      if (lane < C) *cl.map_shared_rank(&s_key[par][c], lane) = best;
+    }
+    cl.sync();
+    long long best = 0;
+    for (int g = 0; g < C; ++g) best = best > s_key[par][g] ? best : s_key[par][g];
+    if (best <= 0) break;
+    const int p = (int)(best & 2047);
+    if (p % C == c) {
+      const double* fp = F + (int64_t)(p / C) * n;
+      const double d = fp[p];
+      const double y = d > 0x1p-90 ? inv_sqrt(d) : 1.0 / sqrt(d);
+      for (int i = tid; i < n; i += nth)  // the rows factored before are zero
+        __stcg(W + (int64_t)r * n + i, __ldcg(gn + i) < 0.0 ? fp[i] * y : 0.0);
+    }
+    cl.sync();
+    if (p % C == c && tid == 0) __stcg(gn + p, 1.0);
+    for (int i = tid; i < n; i += nth) stage[i] = __ldcg(W + (int64_t)r * n + i);
+    __syncthreads();
+    // one warp per own column that is still open
+    for (int k = warp; k < own; k += nw) {
+      const int j = c + C * k;
+      if (j == p || !(__ldcg(gn + j) < 0.0)) continue;
+      const double lj = stage[j];
+      for (int i = lane; i < n; i += 32)
+        F[(int64_t)k * n + i] = fma(-lj, stage[i], F[(int64_t)k * n + i]);
+    }
+    __syncthreads();
+  }
+  // the columns left open, behind the pivots in index order
+  if (r < n)
+    for (int j = 0, at = r; j < n; ++j) {
+      if (!(__ldcg(gn + j) < 0.0)) continue;
+      if (at % C == c) {
+        const double v = 0x1p-40 * sqrt(fmax(__ldcg(gd + j), 0x1p-53));
+        for (int i = tid; i < n; i += nth) __stcg(W + (int64_t)at * n + i, i == j ? v : 0.0);
+      }
+      ++at;
+    }
+  cl.sync();
+  // ---- one-sided Jacobi on block pairs ----
+  const int nb = 2 * ((n + 2 * b - 1) / (2 * b));  // blocks (even), the last ones may be short
+  const float tol = sqrtf((float)n) * 0x1p-53f;
+  double* blk = eig_sh;                                       // 2 b columns of n
+  JCol* jc = reinterpret_cast<JCol*>(blk + (size_t)2 * b * n);
+  const int grp = tid / GL, gl = tid % GL, ngrp = nth / GL;
+  auto group_sum = [&](double v) {
+    for (int o = 1; o < GL; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+  for (int sweep = 0; sweep < kEigSweeps; ++sweep) {
+    if (tid == 0) s_flag = 0;
+    __syncthreads();
+    for (int round = 0; round < nb - 1; ++round) {
+      for (int k = c; k < nb / 2; k += C) {
+        int I, J;
+        circle_pair(nb, round, k, I, J);
+        const int i0 = min(n, I * b), ni = min(n, i0 + b) - i0;
+        const int j0 = min(n, J * b), nj = min(n, j0 + b) - j0;
+        __syncthreads();
+        for (int idx = tid; idx < ni * n; idx += nth)
+          blk[idx] = __ldcg(W + (int64_t)i0 * n + idx);
+        for (int idx = tid; idx < nj * n; idx += nth)
+          blk[b * n + idx] = __ldcg(W + (int64_t)j0 * n + idx);
+        __syncthreads();
+        // staged column x: x < b of block I, x - b of block J
+        auto present = [&](int x) { return x < b ? x < ni : x - b < nj; };
+        for (int x0 = 0; x0 < 2 * b; x0 += ngrp) {
+          const int x = x0 + grp;
+          const bool in = x < 2 * b && present(x);
+          double s = 0.0;
+          if (in)
+            for (int i = gl; i < n; i += GL) s = fma(blk[x * n + i], blk[x * n + i], s);
+          s = group_sum(s);
+          if (gl == 0 && in) jc[x] = JCol{s, 1.0, 1.0};
+        }
+        __syncthreads();
+        const bool all = round == 0;
+        const int rounds = all ? 2 * b - 1 : b;
+        bool rot = false;
+        for (int q = 0; q < rounds; ++q) {
+          for (int x0 = 0; x0 < b; x0 += ngrp) {
+            const int x = x0 + grp;
+            int u = 0, v = 0;
+            if (all) {
+              circle_pair(2 * b, q, x < b ? x : 0, u, v);
+            } else {
+              u = x;
+              v = x + q;
+              v = b + (v >= b ? v - b : v);
+            }
+            const bool on = x < b && present(u) && present(v);
+            double* wp = blk + (on ? u : 0) * n;
+            double* wq = blk + (on ? v : 0) * n;
+            double s0 = 0.0, s1 = 0.0;
+            int i = gl;
+            for (; i + GL < n; i += 2 * GL) {
+              s0 = fma(wp[i], wq[i], s0);
+              s1 = fma(wp[i + GL], wq[i + GL], s1);
+            }
+            if (i < n) s0 = fma(wp[i], wq[i], s0);
+            const double pq = group_sum(s0 + s1);
+            if (!on) continue;
+            JCol cp = jc[u], cq = jc[v];
+            double al, be;
+            if (!jacobi_rotation(cp, cq, pq, tol, al, be)) continue;
+#pragma unroll 4
+            for (i = gl; i < n; i += GL) {
+              const double x1 = wp[i], x2 = wq[i];
+              wp[i] = fma(-al, x2, x1);
+              wq[i] = fma(be, x1, x2);
+            }
+            if (gl == 0) {
+              jc[u] = cp;
+              jc[v] = cq;
+            }
+            rot = true;
+          }
+          __syncthreads();
+        }
+        if (rot) s_flag = 1;
+        for (int idx = tid; idx < ni * n; idx += nth)
+          __stcg(W + (int64_t)i0 * n + idx, blk[idx] * jc[idx / n].d);
+        for (int idx = tid; idx < nj * n; idx += nth)
+          __stcg(W + (int64_t)j0 * n + idx, blk[b * n + idx] * jc[b + idx / n].d);
+      }
+      cl.sync();
+    }
+    if (tid < C) *cl.map_shared_rank(&s_rot[sweep & 1][c], tid) = s_flag;
+    cl.sync();
+    int any = 0;
+    for (int g = 0; g < C; ++g) any |= s_rot[sweep & 1][g];
+    if (!any) break;
+  }
+  // ---- eigenvalues in descending order, normalised columns (CTA c: columns c, c + C, ...)
+  double* gs = gd + n;  // squared norms as they are
+  for (int k = warp; k < own; k += nw) {
+    const int j = c + C * k;
+    double s = 0.0;
+    for (int i = lane; i < n; i += 32) {
+      const double v = __ldcg(W + (int64_t)j * n + i);
+      s = fma(v, v, s);
+    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+      __stcg(gn + j, s >= 0x1p-70 ? s : 0.0);
+      __stcg(gs + j, s);
+    }
+  }
+  cl.sync();
+  double* evs = eig_sh;
+  for (int i = tid; i < n; i += nth) evs[i] = __ldcg(gn + i);
+  __syncthreads();
+  for (int k = warp; k < own; k += nw) {
+    const int j = c + C * k;
+    int rank = 0;
+    if (lane == 0) rank = rank_of(evs, n, j);
+    rank = __shfl_sync(0xffffffffu, rank, 0);
+    const double inv = 1.0 / sqrt(__ldcg(gs + j));
+    if (lane == 0) ev[rank] = evs[j] / scale;
+    for (int i = lane; i < n; i += 32)
+      V[(int64_t)i * ld + rank] = __ldcg(W + (int64_t)j * n + i) * inv;
+  }
+  if (c == 0) {
+    for (int i = n + tid; i < ld; i += nth) ev[i] = 0.0;
+    for (int64_t idx = tid; idx < (int64_t)ld * ld; idx += nth) {
+      const int i = (int)(idx / ld), j = (int)(idx - (int64_t)i * ld);
+      if (i >= n || j >= n) V[idx] = 0.0;
+    }
+  }
+  cl.sync();  // no CTA leaves while another may still write to it
+}
+
+template <int E>
+void launch_small(int n_sd, const double* A, int ld, int n, double* evals, double* evecs,
+                  cudaStream_t st) {
+  const int nth = std::max(64, (std::max(1, (n + 1) / 2) * kEigLanes + 31) / 32 * 32);
+  const size_t sm = sizeof(double) * ((size_t)n * kEigLanes * E + n) + sizeof(JCol) * n +
+                    sizeof(int) * n;
+  cudaFuncSetAttribute(k_sym_eig<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k_sym_eig<E><<<n_sd, nth, sm, st>>>(A, ld, n, evals, evecs);
+}
+
+}  // namespace
+
+// CTAs per subdomain: as many as fill the chip once, with at least 16 columns each; one up
+// to order 48, where the chain of a round counts and not its arithmetic (64 matrices of
+// order 42: 1.06 ms with one CTA each, 1.18 with two; 40 of 74: 3.6 with one, 2.6 with three)
+static int eig_ctas(int n_sd, int n) {
+  if (n <= 48) return 1;
+  return std::max(1, std::min({8, 152 / std::max(1, n_sd), n / 16}));
+}
+
+size_t sym_eig_work(int n) { return 2 * (size_t)n * n + 16 * (size_t)n; }
+
+void launch_sym_eig(int n_sd, const double* A, int ld, int n, double* evals, double* evecs,
+                    double* work, cudaStream_t st) {
+  if (n_sd <= 0 || n <= 0 || n > kEigMax) return;
+  count_launch();
+  int C = eig_ctas(n_sd, n);
+  if (n <= kEigSmem && C == 1) {
+    if (n <= 16) return launch_small<2>(n_sd, A, ld, n, evals, evecs, st);
+    if (n <= 32) return launch_small<4>(n_sd, A, ld, n, evals, evecs, st);
+    if (n <= 48) return launch_small<6>(n_sd, A, ld, n, evals, evecs, st);
+    if (n <= 64) return launch_small<8>(n_sd, A, ld, n, evals, evecs, st);
+    if (n <= 80) return launch_small<10>(n_sd, A, ld, n, evals, evecs, st);
+    if (n <= 96) return launch_small<12>(n_sd, A, ld, n, evals, evecs, st);
+    return launch_small<16>(n_sd, A, ld, n, evals, evecs, st);
+  }
+  const size_t col = sizeof(double) * (size_t)n + sizeof(JCol);  // a staged column
+  const int b = std::max(1, std::min((n + 2 * C - 1) / (2 * C), (int)(kEigBlkSmem / (2 * col))));
+  const size_t factor = sizeof(double) * (size_t)((n + C - 1) / C) * n;
+  int in_smem = factor <= kEigBlkSmem ? 1 : 0;
+  const size_t sm = std::max(2 * b * col, (in_smem ? factor : 0) + sizeof(double) * (size_t)n);
+  // a rotation's own arithmetic (about 25 binary64 instructions per warp) serves 32 / GL
+  // pairs, but its chain wants warps to hide behind: 16 lanes per pair, 8 from 26 pairs a
+  // CTA on (30 matrices of order 260: 52 -> 40 ms; 14 of 190: 10.6 ms against 14.2 with 8)
+  const int gl = b < 26 ? 16 : 8;
+  const int nth = std::min(768, std::max(256, (b * gl + 31) / 32 * 32));
+  auto fn = gl == 8 ? k_sym_eig_blocks<8> : k_sym_eig_blocks<16>;
+  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)C;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(n_sd * C));
+  cfg.blockDim = dim3((unsigned)nth);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, fn, A, ld, n, b, in_smem, evals, evecs, work);
+}
+
+}  // namespace mor

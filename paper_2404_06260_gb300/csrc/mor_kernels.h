@@ -243,11 +243,13 @@ void launch_gram(const DTiles& tiles, int n_sd, const double* X, int ldx, int nx
 void launch_gram_vec(const DTiles& tiles, int n_sd, const double* X, int ldx, int nx,
                      const double* y, int ldy, double* part, int* counter, double* g,
                      int ldg, cudaStream_t st);
-// symmetric eigensolver (cyclic Jacobi, parallel ordering) per subdomain on the
-// leading n x n block of A[sd] (stride ld); evals descending (n_sd x ld), evecs
-// columns (n_sd x ld x ld).
-void launch_sym_eig(int n_sd, const double* A, int ld, int n, double* evals,
-                    double* evecs, cudaStream_t st);
+// eigen-decomposition of the positive semidefinite leading n x n block (n <= 1024) of
+// A[sd] (stride ld), symmetrised (mor_eig.cu): evals descending (n_sd x ld, noise and null
+// directions 0), evecs orthonormal columns (n_sd x ld x ld), both zero beyond n.  work:
+// n_sd * sym_eig_work(n) doubles (none for n <= 160).
+size_t sym_eig_work(int n);
+void launch_sym_eig(int n_sd, const double* A, int ld, int n, double* evals, double* evecs,
+                    double* work, cudaStream_t st);
 // M[sd] from an eigen-decomposition: mode 0: V_j / sqrt(l_j) for l_j > rel * l_0 (else 0
 // column); mode 1: V_j for j < keep (or j < keep_sd[sd]); mode 2: V_j for l_j > rel
 // (absolute), j < keep and j < keep_sd[sd]; kept[sd] = number of nonzero columns.
@@ -260,14 +262,11 @@ void launch_rowmul(const DTiles& tiles, const double* X, int ldx, int nin, const
                    int ldm, double* Y, int ldy, int nout, cudaStream_t st);
 // dst[r, dc0 + c] = src[map[r], sc0 + c] (map null: r), c < ncols
 // wide-sketch versions (k up to 511 columns, mor_wide.cu): the Gram needs a partial
-// buffer of n_sd * gram_wide_chunks(n_sd, nx, ny) * nx * ny doubles, the eigensolver a
-// work buffer of n_sd * 2 * m * m doubles (m = n rounded up to even, n <= 1024)
+// buffer of n_sd * gram_wide_chunks(n_sd, nx, ny) * nx * ny doubles
 int gram_wide_chunks(int n_sd, int nx, int ny);
 void launch_gram_wide(const DTiles& tiles, int n_sd, const double* X, int ldx, int nx,
                       const double* Y, int ldy, int ny, double* part, double* G, int ldg,
                       int64_t sd_stride, cudaStream_t st);
-void launch_sym_eig_wide(int n_sd, const double* A, int ld, int n, double* evals,
-                         double* evecs, double* work, cudaStream_t st);
 void launch_rowmul_wide(const DTiles& tiles, const double* X, int ldx, int nin,
                         const double* M, int ldm, double* Y, int ldy, int nout,
                         cudaStream_t st);

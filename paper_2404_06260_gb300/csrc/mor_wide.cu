@@ -4,10 +4,6 @@
 // mor_dense.cu do not fit:
 //   - tall-skinny Grams X^T Y over the rows of each subdomain, 64 x 64 output tiles,
 //     split over row chunks and reduced in chunk order (deterministic);
-//   - the symmetric eigensolver: the same threshold cyclic Jacobi as the small kernel
-//     (round-robin ordering, Golub & Van Loan Alg. 8.4.1 rotations, Demmel-Veselic
-//     threshold) with the matrix and the eigenvectors in global memory, one block of
-//     1024 threads per subdomain;
 //   - row-block products X M_sd in 128-row x 64-column output tiles.
 // Everything is binary64.
 #include "mor_kernels.h"
@@ -84,104 +80,6 @@ __global__ void k_gram_wide_reduce(int S, int nx, int ny, const double* __restri
     for (int s = 0; s < S; ++s) acc += part[(int64_t)(sd * S + s) * n + o];
     const int i = (int)(o / ny), j = (int)(o % ny);
     G[(int64_t)sd * sd_stride + (int64_t)i * ldg + j] = acc;
-  }
-}
-
-// threshold cyclic Jacobi of the symmetric part of A_sd (n x n, leading dimension ld),
-// a and v are m x m work arrays per subdomain (m = n rounded up to even, n <= 1024).
-// evals descending, evecs[r * ld + rank] the matching eigenvectors, zero beyond n.
-constexpr int kEigThreads = 1024;
-__global__ void __launch_bounds__(kEigThreads)
-    k_sym_eig_wide(const double* __restrict__ A, int ld, int n, double* evals, double* evecs,
-                   double* work) {
-  __shared__ double rc[512], rs[512];
-  __shared__ int rp[512], rq[512];
-  __shared__ int nrot;
-  const int m = n + (n & 1);
-  const int sd = blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
-  double* a = work + (int64_t)sd * 2 * m * m;
-  double* v = a + (int64_t)m * m;
-  const double* As = A + (int64_t)sd * ld * ld;
-  for (int idx = tid; idx < m * m; idx += nth) {
-    const int i = idx / m, j = idx % m;
-    a[idx] = (i < n && j < n) ? 0.5 * (As[i * ld + j] + As[j * ld + i]) : 0.0;
-    v[idx] = (i == j) ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  for (int sweep = 0; sweep < 40 && m > 1; ++sweep) {
-    if (tid == 0) nrot = 0;
-    __syncthreads();
-    for (int round = 0; round < m - 1; ++round) {
-      for (int k = tid; k < m / 2; k += nth) {
-        const int x0 = k, x1 = m - 1 - k;
-        const int p = (x0 == 0) ? 0 : ((x0 - 1 + round) % (m - 1)) + 1;
-        const int q = ((x1 - 1 + round) % (m - 1)) + 1;
-        const double apq = a[(int64_t)p * m + q];
-        const double app = a[(int64_t)p * m + p], aqq = a[(int64_t)q * m + q];
-        double c = 1.0, s = 0.0;
-        if (fabs(apq) > 0x1p-52 * sqrt(fabs(app * aqq))) {
-          atomicAdd(&nrot, 1);
-          const double tau = (aqq - app) / (2.0 * apq);
-          double t;
-          if (fabs(tau) > 1e150)
-            t = 0.5 / tau;
-          else
-            t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-          c = 1.0 / sqrt(1.0 + t * t);
-          s = t * c;
-        }
-        rp[k] = p;
-        rq[k] = q;
-        rc[k] = c;
-        rs[k] = s;
-      }
-      __syncthreads();
-      // rows p, q of A: A <- J^T A
-      for (int w = tid; w < (m / 2) * m; w += nth) {
-        const int k = w / m, j = w % m;
-        const double c = rc[k], s = rs[k];
-        if (s == 0.0) continue;
-        const int64_t p = rp[k], q = rq[k];
-        const double ap = a[p * m + j], aq = a[q * m + j];
-        a[p * m + j] = c * ap - s * aq;
-        a[q * m + j] = s * ap + c * aq;
-      }
-      __syncthreads();
-      // columns p, q of A and V: A <- A J, V <- V J
-      for (int w = tid; w < (m / 2) * m; w += nth) {
-        const int k = w % (m / 2), i = w / (m / 2);
-        const double c = rc[k], s = rs[k];
-        if (s == 0.0) continue;
-        const int p = rp[k], q = rq[k];
-        const int64_t ri = (int64_t)i * m;
-        const double ap = a[ri + p], aq = a[ri + q];
-        a[ri + p] = c * ap - s * aq;
-        a[ri + q] = s * ap + c * aq;
-        const double vp = v[ri + p], vq = v[ri + q];
-        v[ri + p] = c * vp - s * vq;
-        v[ri + q] = s * vp + c * vq;
-      }
-      __syncthreads();
-    }
-    const int rotated = nrot;
-    __syncthreads();
-    if (rotated == 0) break;
-  }
-  double* ev = evals + (int64_t)sd * ld;
-  double* V = evecs + (int64_t)sd * ld * ld;
-  for (int64_t idx = tid; idx < (int64_t)ld * ld; idx += nth) V[idx] = 0.0;
-  for (int i = tid; i < ld; i += nth)
-    if (i >= n) ev[i] = 0.0;
-  __syncthreads();
-  for (int i = tid; i < n; i += nth) {
-    const double li = a[(int64_t)i * m + i];
-    int rank = 0;
-    for (int j = 0; j < n; ++j) {
-      const double lj = a[(int64_t)j * m + j];
-      if (lj > li || (lj == li && j < i)) ++rank;
-    }
-    ev[rank] = li;
-    for (int r = 0; r < n; ++r) V[(int64_t)r * ld + rank] = v[(int64_t)r * m + i];
   }
 }
 
@@ -264,13 +162,6 @@ void launch_gram_wide(const DTiles& tiles, int n_sd, const double* X, int ldx, i
   const int64_t n = (int64_t)nx * ny;
   const int bx = (int)((n + 255) / 256 < 64 ? (n + 255) / 256 : 64);
   k_gram_wide_reduce<<<dim3(bx, n_sd), 256, 0, st>>>(S, nx, ny, part, G, ldg, sd_stride);
-}
-
-void launch_sym_eig_wide(int n_sd, const double* A, int ld, int n, double* evals,
-                         double* evecs, double* work, cudaStream_t st) {
-  if (n_sd <= 0) return;
-  count_launch();
-  k_sym_eig_wide<<<n_sd, kEigThreads, 0, st>>>(A, ld, n, evals, evecs, work);
 }
 
 void launch_rowmul_wide(const DTiles& tiles, const double* X, int ldx, int nin,

@@ -92,6 +92,7 @@ _sig("mor_debug_wait_timeout", _i32, _dbl, ctypes.POINTER(_i32))
 _sig("mor_energy_norm", _i32, _P, _P, _P, ctypes.POINTER(_dbl), _P)
 _sig("mor_debug_tc_gram", _i32, _i64, _i32, _i32, _P, _P, _P, _P)
 _sig("mor_debug_coarse_inverse", _i32, _i32, _P, _P, _P)
+_sig("mor_debug_sym_eig", _i32, _i32, _i32, _P, _P, _P, _P)
 _sig("mor_debug_sketch_rhs", _i32, _P, ctypes.POINTER(BasisOpts), _i32, _P, _P)
 _sig("mor_profile_enable", _i32, _i32)
 _sig("mor_profile_reset", _i32)
@@ -113,7 +114,7 @@ EXPORTED = ["mor_build_subdomains", "mor_build_subdomains_host",
             "mor_solve_reduced_noalloc", "mor_set_wait_budget", "mor_debug_wait_timeout",
             "mor_lift",
             "mor_energy_norm", "mor_debug_sketch_rhs", "mor_debug_plan_check",
-            "mor_debug_tc_gram", "mor_debug_coarse_inverse",
+            "mor_debug_tc_gram", "mor_debug_coarse_inverse", "mor_debug_sym_eig",
             "mor_profile_enable",
             "mor_profile_reset", "mor_profile_query", "mor_kernel_launches", "mor_autotune",
             "mor_autotune_report", "mor_free_subdomains",
@@ -406,6 +407,17 @@ def coarse_inverse(E, stream=None):
     _check(_lib.mor_debug_coarse_inverse(int(E.shape[0]), _P(E.data_ptr()), _P(out.data_ptr()),
                                          _stream(stream)))
     return out
+
+
+def sym_eig(A, stream=None):
+    """Eigenvalues (descending) and eigenvectors of positive semidefinite matrices
+    (mor_debug_sym_eig); A a binary64 CUDA tensor n_sub x n x n."""
+    assert A.is_cuda and A.dtype == torch.float64 and A.dim() == 3 and A.shape[1] == A.shape[2]
+    A = A.contiguous()
+    ev, V = torch.empty(A.shape[:2], dtype=A.dtype, device=A.device), torch.empty_like(A)
+    _check(_lib.mor_debug_sym_eig(int(A.shape[0]), int(A.shape[1]), _P(A.data_ptr()),
+                                  _P(ev.data_ptr()), _P(V.data_ptr()), _stream(stream)))
+    return ev, V
 
 
 def profile(on: bool):
