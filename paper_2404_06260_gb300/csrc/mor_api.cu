@@ -963,10 +963,10 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
       for (int set = 0; set < 2; ++set) {
         const DTiles& tl = set == 0 ? S.tP_I : S.tP_all;
         const Mat& Am = set == 0 ? A_II : Hp;
-        int32_t *nca, *tfirst, *tcount;
+        int32_t *nca, *tbase, *tcount;
         int64_t *toff, *eoff;
         TRY(M.upload(&nca, ap.nca[set], st));
-        TRY(M.upload(&tfirst, ap.tfirst[set], st));
+        TRY(M.upload(&tbase, ap.tbase[set], st));
         TRY(M.upload(&tcount, ap.tcount[set], st));
         TRY(M.upload(&toff, ap.toff[set], st));
         TRY(M.upload(&eoff, ap.eoff[set], st));
@@ -993,7 +993,7 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
           c.aloc = aloc;
           c.aoff = aoff;
           c.nca = nca;
-          c.tfirst = tfirst;
+          c.tbase = tbase;
           c.tcount = tcount;
           c.toff = toff;
           c.eoff = eoff;
@@ -1032,6 +1032,9 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
           __nv_bfloat16* rcb;
           TRY(M.upload(&rcb_off, h_rc, st));
           TRY(M.alloc(&rcb, (size_t)std::max<int64_t>(h_rc[n_sd], 1) * 2 * NP * 32, true, st));
+          float* rcf;
+          TRY(M.alloc(&rcf, (size_t)n_agg * kp, true, st));
+          B.co32[set].rcf = rcf;
           B.co32[set].rcb = rcb;
           B.co32[set].rcb_off = rcb_off;
           B.co32[set].etc = etc;
@@ -1105,6 +1108,10 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
   TRY(M.alloc(&B.cs.done, (size_t)n_sd * kp, true, st));
   TRY(M.alloc(&B.cs.part1, (size_t)mt * kp, true, st));
   TRY(M.alloc(&B.cs.part2, (size_t)mt * kp, true, st));
+  TRY(M.alloc(&B.cs.gpart, (size_t)3 * mt * kp, false, st));
+  TRY(M.alloc(&B.cs.gcount, mt, true, st));
+  B.rs.gpart = B.cs.gpart;
+  B.rs.gcount = B.cs.gcount;
   TRY(M.alloc(&B.cs.counter, n_sd, true, st));
   TRY(M.alloc(&B.cs.iters, n_sd, true, st));
   TRY(M.alloc(&B.cs.active, n_sd, true, st));

@@ -84,6 +84,8 @@ struct CgState {
                                     // beta, gam (binary32 kernels load them as packs)
   int* done;                        // n_sd x kp
   double *part1, *part2;            // n_tiles x kp
+  double* gpart;                    // 3 x n_tiles x kp: sums of groups of tiles
+  int* gcount;                      // n_tiles: tickets of the groups
   int* counter;                     // n_sd
   int* iters;                       // n_sd
   int* active;                      // n_sd: active columns after the last update
@@ -104,14 +106,15 @@ struct CgState {
 // preconditioner is D^{-1} alone.
 constexpr int kMaxSlots = 32;  // aggregates meeting one row tile (host-enforced)
 constexpr int kMaxAgg = 1024;  // aggregates per subdomain and matrix (host-enforced)
-constexpr int kCoarseRowsMin = 256;  // fewest rows of E^{-1} per block of the SIMT coarse product
+constexpr int kCoarseRowsMin = 256;  // fewest rows of E^{-1} per row block of the SIMT product
 template <typename T>
 struct Coarse {
   const int32_t* aloc = nullptr;    // per P row: aggregate index within its subdomain
   const int32_t* aoff = nullptr;    // per subdomain: first global aggregate id
   const int32_t* nca = nullptr;     // per subdomain: aggregates of this matrix (<= kMaxAgg)
-  const int32_t* tfirst = nullptr;  // per global aggregate: first tile holding its rows
-  const int32_t* tcount = nullptr;  // per global aggregate: tiles holding its rows
+  const int32_t* tbase = nullptr;   // per global aggregate: its first row of cpart
+  const int32_t* tcount = nullptr;  // per global aggregate: tiles holding its rows, each with
+                                    // one of its consecutive rows of cpart
   const int64_t* toff = nullptr;    // per tile: first row of its partials (n_tiles + 1)
   const int64_t* eoff = nullptr;    // per subdomain: offset of its nca x nca block
   const T* einv = nullptr;          // E^{-1} blocks, symmetric, row-major
@@ -127,6 +130,7 @@ struct Coarse {
   // r_c of every step as bf16 high and low planes, 2 x NP x 32 per 32-aggregate block
   // (NP = kp rounded up to 16), the first block of each subdomain at rcb_off[sd]
   __nv_bfloat16* rcb = nullptr;
+  float* rcf = nullptr;  // r_c of every step, global aggregates x kp
   const int64_t* rcb_off = nullptr;
   int* tc_err = nullptr;
   long long tc_budget = 0;
@@ -170,6 +174,8 @@ struct RefineState {
   double *obb, *orr, *scale;  // n_sd x kp
   double* oaa;                // n_sd x kp: || |A| |x| + |b| ||^2 at the last refresh
   double *part, *part2, *part3;  // n_tiles x kp
+  double* gpart;              // 3 x n_tiles x kp
+  int* gcount;                // n_tiles
   int* counter;               // n_sd
   int* active;                // n_sd
   int* nfloor;                // n_sd: columns stopped by the attainable-accuracy test

@@ -850,7 +850,7 @@ void build_aggregates(const HostPlan& hp, int target_rows, int max_agg, AggPlan&
     const HostTiles& T = set == 0 ? hp.tP_I : hp.tP_all;
     const size_t nt = T.sd.size();
     ap.toff[set].assign(nt + 1, 0);
-    ap.tfirst[set].assign(n_agg, 0);
+    ap.tbase[set].assign(n_agg, 0);
     ap.tcount[set].assign(n_agg, 0);
     for (size_t t = 0; t < nt; ++t) {
       const int sd = T.sd[t];
@@ -860,7 +860,8 @@ void build_aggregates(const HostPlan& hp, int target_rows, int max_agg, AggPlan&
       ap.toff[set][t + 1] = ap.toff[set][t] + ns;
       for (int a = a0; a <= a1; ++a) {
         int64_t ga = ap.aoff[sd] + a;
-        if (ap.tcount[set][ga]++ == 0) ap.tfirst[set][ga] = (int32_t)t;
+        if (ap.tcount[set][ga]++ == 0)
+          ap.tbase[set][ga] = (int32_t)(ap.toff[set][t] + (a - a0));
       }
     }
     ap.eoff[set].assign(n_sd + 1, 0);

@@ -110,7 +110,9 @@ struct AggPlan {
   std::vector<int32_t> aoff;        // n_sd + 1: global id of the first aggregate
   std::vector<int32_t> nca[2];      // per subdomain: aggregates of set 0 / 1
   std::vector<int64_t> toff[2];     // per tile + 1: partial rows of the tile
-  std::vector<int32_t> tfirst[2], tcount[2];  // per global aggregate
+  // per global aggregate: its first partial row and the tiles holding its rows (its partial
+  // rows are consecutive: it is the last of one tile and the first of the next)
+  std::vector<int32_t> tbase[2], tcount[2];
   std::vector<int64_t> eoff[2];     // n_sd + 1: offsets of the nca x nca blocks
   int max_slots = 0;                // most aggregates meeting one tile
 };

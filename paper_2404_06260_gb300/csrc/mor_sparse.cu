@@ -10,6 +10,7 @@
 #include "mor_kernels.h"
 #include "mor_tc.cuh"
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -57,7 +58,7 @@ struct alignas(16) Slot2 {
   int32_t c[2];
 };
 
-// shared memory layout: red[nth * N] of T, scratch[nth] doubles, sums[2*kp] doubles,
+// shared memory layout: red[nth * N] of T, scratch[nth] doubles, sums[3*kp] doubles,
 // then the staged sliced-ELL tile: slots[((W + 1) / 2) * kTileRows] pair records,
 // pair-major (record h of row rr at h * kTileRows + rr)
 template <typename T>
@@ -77,14 +78,14 @@ __device__ __forceinline__ Smem<T> smem_layout(const Geo& g, int kp, int W) {
   o += align16(16 * (size_t)g.nth);
   s.scratch = reinterpret_cast<double*>(raw + o);
   s.sums = s.scratch + g.nth;
-  o += align16(sizeof(double) * ((size_t)g.nth + 2 * kp));
+  o += align16(sizeof(double) * ((size_t)g.nth + 3 * kp));
   s.slots = reinterpret_cast<Slot2<T>*>(raw + o);
   return s;
 }
 template <typename T>
 __host__ __device__ __forceinline__ size_t smem_bytes(int nch, int rb, int kp, int W) {
   size_t nth = (size_t)nch * rb;
-  return align16(16 * nth) + align16(sizeof(double) * (nth + 2 * kp)) +
+  return align16(16 * nth) + align16(sizeof(double) * (nth + 3 * kp)) +
          sizeof(Slot2<T>) * (size_t)kTileRows * ((W + 1) / 2);
 }
 
@@ -107,33 +108,43 @@ __device__ void block_colsum(const Geo& g, const T (&acc)[N], T* red, double* ou
     for (int e = 0; e < N; ++e) out[g.tx * N + e] = (double)red[g.tx * N + e];
 }
 
-__device__ __forceinline__ bool last_block(const Geo& g, int* counter, int sd, int nblk) {
+// true in the last of n blocks to come here (for every thread); the counter returns to
+// zero.  One thread's acquire-release ticket behind the block barrier orders the blocks'
+// earlier writes before the last block's later reads (which pass by L1: __ldcg).
+__device__ __forceinline__ bool take_ticket(const Geo& g, int* counter, int n) {
   __shared__ int is_last;
-  __threadfence();
   __syncthreads();
   if (g.tid == 0) {
-    int prev = atomicAdd(counter + sd, 1);
-    is_last = (prev == nblk - 1);
-    if (is_last) counter[sd] = 0;
+    int prev;
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;"
+                 : "=r"(prev)
+                 : "l"(counter)
+                 : "memory");
+    is_last = prev == n - 1;
+    if (is_last) *counter = 0;
   }
   __syncthreads();
-  if (is_last) __threadfence();
-  return is_last;
+  return is_last != 0;
 }
 
-// sums[c] = sum over tiles lo..hi-1 of part[t*kp + c], fixed order.  Columns are taken
+// sums[c] = sum over rows lo..hi-1 of part[t*kp + c], fixed order.  Columns are taken
 // in groups of at most nth; within a group S = nth / group threads share a column.
-__device__ void sd_colsums(const Geo& g, const double* part, int kp, int lo, int hi,
-                           double* scratch, double* sums) {
+__device__ void rows_colsum(const Geo& g, const double* part, int kp, int lo, int hi,
+                            double* scratch, double* sums) {
   for (int c0 = 0; c0 < kp; c0 += g.nth) {
     const int cw = min(kp - c0, g.nth);
     const int S = g.nth / cw;
     const int c = c0 + g.tid % cw, sidx = g.tid / cw;
     double acc = 0.0;
-    if (sidx < S) {
-#pragma unroll 4
-      for (int t = lo + sidx; t < hi; t += S) acc += __ldcg(part + (int64_t)t * kp + c);
-    }
+    if (sidx < S)
+      for (int t = lo + sidx; t < hi; t += 4 * S) {
+        double v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          v[u] = t + u * S < hi ? __ldcg(part + (int64_t)(t + u * S) * kp + c) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc += v[u];
+      }
     scratch[g.tid] = acc;
     __syncthreads();
     for (int cc = g.tid; cc < cw; cc += g.nth) {
@@ -143,6 +154,42 @@ __device__ void sd_colsums(const Geo& g, const double* part, int kp, int lo, int
     }
     __syncthreads();
   }
+}
+
+// The column sums of a subdomain's tiles lo..hi-1 (part[q][t*kp + c], this block wrote tile
+// `tile`) into sums[q*kp + c], q < NS; true in the one block that ends up with them.  Two
+// levels, in a fixed order: the last block of every kRedGroup tiles adds those to a group
+// sum, the last group adds the groups.  One block adding a subdomain's 170 to 250 tiles
+// alone was a tail of 10 us per sum behind every kernel (binary64 additions at 2 per clock
+// behind a dozen dependent loads); the two short ones take 4.  Few tiles: one level.
+constexpr int kRedGroup = 16;
+template <int NS>
+__device__ bool tile_sums(const Geo& g, const double* const (&part)[NS], double* gpart,
+                          int* gcount, int* count, int kp, int tile, int lo, int hi,
+                          double* scratch, double* sums) {
+  const int nt = hi - lo;
+  if (nt <= kRedGroup + kRedGroup / 2) {
+    if (!take_ticket(g, count, nt)) return false;
+#pragma unroll
+    for (int q = 0; q < NS; ++q) rows_colsum(g, part[q], kp, lo, hi, scratch, sums + q * kp);
+    return true;
+  }
+  const int ng = (nt + kRedGroup - 1) / kRedGroup, gi = (tile - lo) / kRedGroup;
+  const int g0 = lo + gi * kRedGroup, g1 = min(hi, g0 + kRedGroup);
+  if (!take_ticket(g, gcount + lo + gi, g1 - g0)) return false;
+  // group sums of a subdomain: rows (lo + gi) NS .. of gpart, NS rows per group
+  double* gp = gpart + (int64_t)lo * NS * kp;
+#pragma unroll
+  for (int q = 0; q < NS; ++q) {
+    rows_colsum(g, part[q], kp, g0, g1, scratch, sums + q * kp);
+    for (int c = g.tid; c < kp; c += g.nth)
+      __stcg(gp + ((int64_t)q * ng + gi) * kp + c, sums[q * kp + c]);
+  }
+  if (!take_ticket(g, count, ng)) return false;
+#pragma unroll
+  for (int q = 0; q < NS; ++q)
+    rows_colsum(g, gp + (int64_t)q * ng * kp, kp, 0, ng, scratch, sums + q * kp);
+  return true;
 }
 
 // CG coefficients: binary64 state with a binary32 copy
@@ -358,9 +405,10 @@ __global__ void __launch_bounds__(TH, 1536 / TH)
     for (int e = 0; e < N; ++e) acc[e] += pv.v[e] * qv.v[e];
   }
   block_colsum<T, N>(g, acc, sm.red, s.part1 + (int64_t)tile * kp);
-  const int lo = tl.lo[sd], hi = tl.hi[sd];
-  if (!last_block(g, s.counter, sd, hi - lo)) return;
-  sd_colsums(g, s.part1, kp, lo, hi, sm.scratch, sm.sums);
+  const double* const parts[1] = {s.part1};
+  if (!tile_sums<1>(g, parts, s.gpart, s.gcount, s.counter + sd, kp, tile, tl.lo[sd], tl.hi[sd],
+                    sm.scratch, sm.sums))
+    return;
   for (int c = g.tid; c < kp; c += g.nth) {
     int i = sd * kp + c;
     double a = 0.0;
@@ -422,15 +470,18 @@ __global__ void k_residual64(DTiles tl, EllView<double> A, const double* __restr
     __syncthreads();
     block_colsum<double, N>(g, aca, sm.red, s.part2 + (int64_t)tile * kp);
   }
-  const int lo = tl.lo[sd], hi = tl.hi[sd];
-  if (!last_block(g, s.counter, sd, hi - lo)) return;
-  sd_colsums(g, s.part, kp, lo, hi, sm.scratch, sm.sums);
   if constexpr (kFloor) {
-    sd_colsums(g, s.part2, kp, lo, hi, sm.scratch, sm.sums + kp);
-    for (int c = g.tid; c < kp; c += g.nth) s.oaa[sd * kp + c] = sm.sums[kp + c];
-    __syncthreads();
+    const double* const parts[3] = {s.part, s.part3, s.part2};
+    if (!tile_sums<3>(g, parts, s.gpart, s.gcount, s.counter + sd, kp, tile, tl.lo[sd],
+                      tl.hi[sd], sm.scratch, sm.sums))
+      return;
+    for (int c = g.tid; c < kp; c += g.nth) s.oaa[sd * kp + c] = sm.sums[2 * kp + c];
+  } else {
+    const double* const parts[2] = {s.part, s.part3};
+    if (!tile_sums<2>(g, parts, s.gpart, s.gcount, s.counter + sd, kp, tile, tl.lo[sd],
+                      tl.hi[sd], sm.scratch, sm.sums))
+      return;
   }
-  sd_colsums(g, s.part3, kp, lo, hi, sm.scratch, sm.sums + kp);
   for (int c = g.tid; c < kp; c += g.nth) s.xx[sd * kp + c] = sm.sums[kp + c];
   __shared__ int cnt, nfl, nnear;
   __shared__ double bref;
@@ -574,10 +625,10 @@ __global__ void k_cg_init(DTiles tl, const T* __restrict__ b, T* x, T* r,
   block_colsum<T, N>(g, arz, sm.red, s.part1 + (int64_t)tile * kp);
   __syncthreads();
   block_colsum<T, N>(g, arr, sm.red, s.part2 + (int64_t)tile * kp);
-  int lo = tl.lo[sd], hi = tl.hi[sd];
-  if (!last_block(g, s.counter, sd, hi - lo)) return;
-  sd_colsums(g, s.part1, kp, lo, hi, sm.scratch, sm.sums);
-  sd_colsums(g, s.part2, kp, lo, hi, sm.scratch, sm.sums + kp);
+  const double* const parts[2] = {s.part1, s.part2};
+  if (!tile_sums<2>(g, parts, s.gpart, s.gcount, s.counter + sd, kp, tile, tl.lo[sd], tl.hi[sd],
+                    sm.scratch, sm.sums))
+    return;
   __shared__ double bref;
   if (g.tid == 0) {
     double m = 0.0;
@@ -655,10 +706,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 4)
   block_colsum<T, N>(g, arr, sm.red, s.part1 + (int64_t)tile * kp);
   __syncthreads();
   block_colsum<T, N>(g, arz, sm.red, s.part2 + (int64_t)tile * kp);
-  int lo = tl.lo[sd], hi = tl.hi[sd];
-  if (!last_block(g, s.counter, sd, hi - lo)) return;
-  sd_colsums(g, s.part1, kp, lo, hi, sm.scratch, sm.sums);
-  sd_colsums(g, s.part2, kp, lo, hi, sm.scratch, sm.sums + kp);
+  const double* const parts[2] = {s.part1, s.part2};
+  if (!tile_sums<2>(g, parts, s.gpart, s.gcount, s.counter + sd, kp, tile, tl.lo[sd], tl.hi[sd],
+                    sm.scratch, sm.sums))
+    return;
   for (int c = g.tid; c < kp; c += g.nth) {
     int i = sd * kp + c;
     s.rr[i] = sm.sums[c];
@@ -680,9 +731,9 @@ __device__ void coarse_finish(const Geo& g, const DTiles& tl, int sd, int kp, in
   const int nchunk = (kp + cw - 1) / cw;
   // the subdomain's columns: open packs before the update (the sparse product and the
   // x/r update of this step worked on them), the test and beta, open packs after
-  __shared__ int open_pre, open_post, chunks_open;
+  __shared__ int open_pre, open_post, chunks_open, open_cols;
   const bool count = s.work && mode == kCoarseStep;
-  if (g.tid == 0) open_pre = open_post = chunks_open = 0;
+  if (g.tid == 0) open_pre = open_post = chunks_open = open_cols = 0;
   __syncthreads();
   if (count) {
     for (int pk = g.tid; pk * PN < kp; pk += g.nth) {
@@ -695,68 +746,158 @@ __device__ void coarse_finish(const Geo& g, const DTiles& tl, int sd, int kp, in
       for (int j = 0; j < cw && ch * cw + j < kp; ++j) open = open || !s.done[sd * kp + ch * cw + j];
       if (open) atomicAdd(&chunks_open, 1);
     }
+    __syncthreads();
   }
-  __syncthreads();
+  int open = 0;
   for (int c = g.tid; c < kp; c += g.nth) {
     const int i = sd * kp + c;
+    const double rzf = s.rzf[i], rr = s.rr[i], bb = s.bb[i], rz = s.rz[i];
+    int done = s.done[i];
     double cd = 0.0;
     if (co.dpart)
-      for (int r = 0; r < nrb; ++r) cd += __ldcg(co.dpart + ((int64_t)sd * nrb + r) * kp + c);
-    const double rzn = s.rzf[i] + cd;
+      for (int r0 = 0; r0 < nrb; r0 += 4) {
+        double v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          v[u] = r0 + u < nrb ? __ldcg(co.dpart + ((int64_t)sd * nrb + r0 + u) * kp + c) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) cd += v[u];
+      }
+    const double rzn = rzf + cd;
     if (mode == kCoarseStep) {
       double be = 0.0;
-      if (!s.done[i]) {
-        if (s.rr[i] <= tol2 * s.bb[i] || !(s.rz[i] > 0.0)) {
-          s.done[i] = 1;
+      if (!done) {
+        if (rr <= tol2 * bb || !(rz > 0.0)) {
+          s.done[i] = done = 1;
         } else {
-          be = rzn / s.rz[i];
+          be = rzn / rz;
           s.rz[i] = rzn;
         }
       }
       set_coef(s.beta, s.beta32, i, be);
       set_coef(s.gam, s.gam32, i, 1.0);
+      open += !done;
     } else {
       s.rz[i] = rzn;
     }
   }
   if (mode != kCoarseStep) return;
+  if (open) atomicAdd(&open_cols, open);
   __syncthreads();
   if (count) {
     for (int pk = g.tid; pk * PN < kp; pk += g.nth) {
-      bool open = false;
-      for (int e = 0; e < PN; ++e) open = open || !s.done[sd * kp + pk * PN + e];
-      if (open) atomicAdd(&open_post, 1);
+      bool op = false;
+      for (int e = 0; e < PN; ++e) op = op || !s.done[sd * kp + pk * PN + e];
+      if (op) atomicAdd(&open_post, 1);
     }
     __syncthreads();
     if (g.tid == 0) {
       // work counts of the algorithmic-bytes model
       const int nsd = tl.n_sd;
       const unsigned long long rows = (unsigned long long)s.sd_rows[sd];
-      const unsigned long long nc = co.aloc ? (unsigned long long)co.nca[sd] : 0ull;
+      const unsigned long long nc = co.tbase ? (unsigned long long)co.nca[sd] : 0ull;
       atomicAdd(s.work + sd, (unsigned long long)s.sd_nnz[sd]);
       atomicAdd(s.work + nsd + sd, (unsigned long long)open_pre * rows);
       atomicAdd(s.work + 2 * nsd + sd, (unsigned long long)open_post * rows);
       if (nc) atomicAdd(s.work + 3 * nsd + sd, (unsigned long long)chunks_open * nc * nc);
     }
   }
-  count_active(g, s.done, sd, kp, s.active);
-  if (g.tid == 0 && s.active[sd] > 0) s.iters[sd] += 1;
+  if (g.tid == 0) {
+    s.active[sd] = open_cols;
+    if (open_cols > 0) s.iters[sd] += 1;
+  }
 }
 
-// Coarse level of one subdomain in SIMT arithmetic (grid: x = row block x column chunk,
-// y = subdomain).  Block (rb, chunk) forms r_c = Z^T r for the chunk's kCoarseCols
-// columns from the tile partials, then rows [rb R, (rb + 1) R) of y_c = E^{-1} r_c
-// (stored for the p update), R = kCoarseThreads kCoarseRpt with kCoarseRpt rows per
-// thread (1 up to 256 aggregates, else 2), and their part of r_c.y_c.  The last block
-// of the subdomain (atomic ticket) adds the parts in row-block order, r.M^{-1}r = fine
-// part + r_c.y_c, and in mode STEP takes the convergence test on the recursive residual
-// and beta = (r.z)_new / (r.z)_old; INIT / REPLACE: rz only (beta and gam come from the
-// init / replacement kernel).  Without a coarse level y_c = 0.  The blocks of one row
-// block are adjacent in the grid, so the chunks read its E^{-1} rows from L2 after the
-// first.
+// r_c pack (aggregate ga, N columns from column c): the partials of an aggregate are
+// consecutive rows of cpart, one per tile that holds some of its rows
+template <typename T>
+__device__ __forceinline__ Pack<T> restrict_pack(const Coarse<T>& co, int ga, int kp, int c) {
+  const int64_t b0 = co.tbase[ga];
+  const int tn = co.tcount[ga];
+  Pack<T> v = ld(co.cpart + b0 * kp + c);
+  for (int t = 1; t < tn; ++t) {
+    const Pack<T> pv = ld(co.cpart + (b0 + t) * kp + c);
+#pragma unroll
+    for (int e = 0; e < Pack<T>::N; ++e) v.v[e] += pv.v[e];
+  }
+  return v;
+}
+
+// Coarse level of one subdomain in SIMT arithmetic, up to kCoarseSmallMax aggregates
+// (block (column chunk, sd), kCoarseSmallCols columns): r_c = Z^T r for the chunk, y_c =
+// E^{-1} r_c with one thread per (row, column), the chunk's part of r_c.y_c; the last chunk
+// of the subdomain (atomic ticket) finishes.  A binary64 multiply-add occupies its quarter
+// of the SM for 64 clocks per warp, so the products are spread over as many warps and
+// blocks as there are: 16 columns per thread and one row per thread took 69 us a launch for
+// 27 subdomains of 52 aggregates and 32 columns, 20 us now.
+constexpr int kCoarseSmallMax = 256;
+constexpr int kCoarseSmallCols = 4;
 constexpr int kCoarseThreads = 256;
+template <typename T>
+__global__ void __launch_bounds__(kCoarseThreads)
+    k_cg_coarse_small(DTiles tl, int kp, double tol2, int mode, CgState s, Coarse<T> co) {
+  constexpr int CW = kCoarseSmallCols, PN = Pack<T>::N;
+  __shared__ __align__(16) T rc[kCoarseSmallMax * CW];
+  __shared__ double red[(kCoarseThreads / 32) * CW];
+  Geo g = geo();
+  const int sd = blockIdx.y, c0 = blockIdx.x * CW;
+  if (s.active[sd] == 0) return;
+  bool open = false;  // a chunk whose columns have all converged needs no coarse product
+#pragma unroll
+  for (int j = 0; j < CW; ++j) open = !s.done[sd * kp + c0 + j] || open;
+  const int n = co.tbase && open ? co.nca[sd] : 0;
+  const int j = g.tid % CW, lane = g.tid & 31;
+  double dl = 0.0;
+  if (n > 0) {
+    const int a0 = co.aoff[sd];
+    for (int idx = g.tid; idx < n * (CW / PN); idx += g.nth) {
+      const int a = idx / (CW / PN), pk = idx - a * (CW / PN);
+      st(rc + a * CW + pk * PN, restrict_pack(co, a0 + a, kp, c0 + pk * PN));
+    }
+    __syncthreads();
+    const T* Eb = co.einv + co.eoff[sd];
+    for (int a = g.tid / CW; a < n; a += kCoarseThreads / CW) {
+      // E^{-1} is symmetric: row a is read as column a (eight rows per warp: one sector or two)
+      T acc0 = T(0), acc1 = T(0);
+      int b = 0;
+      for (; b + 8 <= n; b += 8) {
+        T e[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) e[u] = Eb[(int64_t)(b + u) * n + a];
+#pragma unroll
+        for (int u = 0; u < 8; u += 2) {
+          acc0 += e[u] * rc[(b + u) * CW + j];
+          acc1 += e[u + 1] * rc[(b + u + 1) * CW + j];
+        }
+      }
+      for (; b < n; ++b) acc0 += Eb[(int64_t)b * n + a] * rc[b * CW + j];
+      const T y = acc0 + acc1;
+      co.yc[(int64_t)(a0 + a) * kp + c0 + j] = y;
+      dl += (double)y * (double)rc[a * CW + j];
+    }
+  }
+  for (int o = CW; o < 32; o <<= 1) dl += __shfl_xor_sync(0xffffffffu, dl, o);
+  if (lane < CW) red[(g.tid >> 5) * CW + lane] = dl;
+  __syncthreads();
+  if (g.tid < CW && co.dpart) {
+    double t = 0.0;
+    for (int w = 0; w < kCoarseThreads / 32; ++w) t += red[w * CW + g.tid];
+    __stcg(co.dpart + (int64_t)sd * kp + c0 + g.tid, t);
+  }
+  if (!take_ticket(g, s.counter + sd, gridDim.x)) return;
+  coarse_finish<T>(g, tl, sd, kp, CW, 1, tol2, mode, s, co);
+}
+
+// Coarse level of one subdomain in SIMT arithmetic, above kCoarseSmallMax aggregates
+// (grid: x = row block x column chunk, y = subdomain).  Block (rb, chunk) forms r_c = Z^T r
+// for the chunk's kCoarseCols columns from the tile partials, then rows [rb R, (rb + 1) R) of
+// y_c = E^{-1} r_c (stored for the p update), R = kCoarseThreads kCoarseRpt with kCoarseRpt
+// rows per thread, and their part of r_c.y_c.  The last block of the subdomain (atomic
+// ticket) adds the parts in row-block order and finishes.  The blocks of one row block are
+// adjacent in the grid, so the chunks read its E^{-1} rows from L2 after the first.
+constexpr int kCoarseRpt = 2;  // rows of y_c per thread
 constexpr size_t kCoarseRedBytes = sizeof(double) * (kCoarseThreads / 32) * kCoarseCols;
-template <typename T, int kCoarseRpt>  // rows of y_c per thread
+template <typename T>
 __global__ void __launch_bounds__(kCoarseThreads)
     k_cg_coarse(DTiles tl, int kp, double tol2, int mode, CgState s, Coarse<T> co) {
   constexpr int kCoarseRows = kCoarseThreads * kCoarseRpt;
@@ -766,44 +907,33 @@ __global__ void __launch_bounds__(kCoarseThreads)
   extern __shared__ __align__(16) unsigned char raw[];
   T* rc = reinterpret_cast<T*>(raw);  // round_up(n, 8) x CW
   // rc holds round_up(n_max, 8) rows (the product reads whole groups of 8)
-  const int n_max8 = co.aloc ? (co.n_max + 7) & ~7 : 0;
+  const int n_max8 = (co.n_max + 7) & ~7;
   double* red = reinterpret_cast<double*>(raw + align16(sizeof(T) * n_max8 * CW));
   const int sd = blockIdx.y;
   const int nchunk = (kp + CW - 1) / CW;
   const int chunk = blockIdx.x % nchunk, rbk = blockIdx.x / nchunk;
   const int nrb = gridDim.x / nchunk;
   const int c0 = chunk * CW, ncol = min(CW, kp - c0);
-  const int cw = CW;
   if (s.active[sd] == 0) return;
   // a chunk whose columns have all converged needs no coarse product
   bool chunk_open = false;
-  for (int j = 0; j < ncol; ++j) chunk_open = chunk_open || !s.done[sd * kp + c0 + j];
-  const int n = (co.aloc && chunk_open) ? co.nca[sd] : 0;
+  for (int j = 0; j < ncol; ++j) chunk_open = !s.done[sd * kp + c0 + j] || chunk_open;
+  const int n = chunk_open ? co.nca[sd] : 0;
   const int a_lo = rbk * kCoarseRows, a_hi = min(n, a_lo + kCoarseRows);
   double dl[CW];
 #pragma unroll
   for (int j = 0; j < CW; ++j) dl[j] = 0.0;
   if (a_lo < n) {
     const int a0 = co.aoff[sd];
-    // r_c = Z^T r: one (aggregate, pack) pair per thread step, summed over the tiles
-    // holding the aggregate (kp and c0 are multiples of the pack width).  Rows
-    // n .. round_up(n, 8) are zero: the product runs in steps of 8.
+    // r_c = Z^T r: one (aggregate, pack) pair per thread step (kp and c0 are multiples of
+    // the pack width).  Rows n .. round_up(n, 8) are zero: the product runs in steps of 8.
     const int n8 = (n + 7) & ~7, cwp = CW / PN;
     for (int idx = g.tid; idx < n8 * cwp; idx += g.nth) {
       const int a = idx / cwp, pk = idx - a * cwp;
       Pack<T> v;
 #pragma unroll
       for (int e = 0; e < PN; ++e) v.v[e] = T(0);
-      if (a < n && pk * PN < ncol) {
-        const int ga = a0 + a;
-        const int t0 = co.tfirst[ga], tn = co.tcount[ga];
-        for (int t = t0; t < t0 + tn; ++t) {
-          const int slot = a - co.aloc[tl.r0[t]];
-          Pack<T> pv = ld(co.cpart + (co.toff[t] + slot) * kp + c0 + pk * PN);
-#pragma unroll
-          for (int e = 0; e < PN; ++e) v.v[e] += pv.v[e];
-        }
-      }
+      if (a < n && pk * PN < ncol) v = restrict_pack(co, a0 + a, kp, c0 + pk * PN);
       st(rc + a * CW + pk * PN, v);
     }
     __syncthreads();
@@ -870,131 +1000,122 @@ __global__ void __launch_bounds__(kCoarseThreads)
       if (lane == 0) red[wid * CW + j] = v;
     }
     __syncthreads();
-    if (g.tid < ncol && co.dpart) {
+    if (g.tid < ncol) {
       double t = 0.0;
       for (int w = 0; w < g.nth / 32; ++w) t += red[w * CW + g.tid];
       co.dpart[((int64_t)sd * nrb + rbk) * kp + c0 + g.tid] = t;
     }
   }
-  if (!last_block(g, s.counter, sd, gridDim.x)) return;
-  coarse_finish<T>(g, tl, sd, kp, cw, nrb, tol2, mode, s, co);
+  if (!take_ticket(g, s.counter + sd, gridDim.x)) return;
+  coarse_finish<T>(g, tl, sd, kp, CW, nrb, tol2, mode, s, co);
 }
 
 // The coarse product of the binary32 path on the tensor cores, y_c = E^{-1} r_c for
 // every column (NP = kp rounded up to 16, at most 128), in two kernels.
-// k_coarse_rc_pack forms r_c = Z^T r per 32-aggregate block from the tile partials and
-// stores it as bf16 high and low planes in the K-major operand layout (row = column of
-// r_c).  k_cg_coarse_tc then runs block (m, sd): rows [128 m, 128 m + 128) of y_c as
-// one tcgen05 MMA tile with its FP32 accumulator in TMEM, A = E^{-1} (launch_coarse_tc_
-// pack) and B = r_c streamed through kTcStages shared-memory stages by cp.async, and
-// three products hi.hi + hi.lo + lo.hi per block (about 16 significant bits of each
-// factor; the dropped lo.lo term is below 2^-16 of a product, under the binary32
-// accumulation error of a 1,000-term sum).  One thread issues the MMAs and commits them
-// to the stage's mbarrier; a stage is refilled once its MMAs are done, and every wait
-// is bounded (a timeout sets co.tc_err and ends the block after its MMAs drain).  The
-// epilogue reads the accumulator rows (tcgen05.ld, one row per thread), stores y_c and
-// this block's part of r_c.y_c; the last block of the subdomain finishes as in
-// k_cg_coarse.
+// k_coarse_rc_pack forms r_c = Z^T r per 32-aggregate block from the tile partials, keeps
+// it in binary32 and as bf16 high and low planes in the K-major operand layout (row =
+// column of r_c).  k_cg_coarse_tc then runs a cluster of KS CTAs per 128 rows of y_c: CTA
+// k takes every KS-th part of the aggregates and accumulates its products in TMEM
+// (tcgen05, A = E^{-1} from launch_coarse_tc_pack, B = r_c, three products hi.hi + hi.lo +
+// lo.hi per block: about 16 significant bits of each factor; the dropped lo.lo term is
+// below 2^-16 of a product, under the binary32 accumulation error of a 1,000-term sum).
+// One thread streams the operand blocks (whole and contiguous) through kTcStages stages
+// with bulk copies, another issues the MMAs; stages are handed over by mbarriers alone.
+// The CTAs' accumulators then go to shared memory, and every CTA adds the cluster's for its
+// share of the columns (distributed shared memory, in order), stores y_c and forms r_c.y_c
+// in binary64; the last block of the subdomain finishes.  Every wait is bounded (a timeout
+// sets co.tc_err; the CTA still waits for its own copies and MMAs, keeps to the cluster's
+// barriers and leaves).
+// What bounds it: latency.  One CTA over all of K with cp.async, two block barriers and one
+// wait per 32 aggregates took 1.2 us per block, and r_c.y_c 10 us of shuffled binary64
+// additions: 53 us a step (with the packing) however few subdomains, 26 us now; 64 subdomains
+// of up to 1,000 aggregates 76 -> 51 us.
 constexpr int kTcThreads = 128;  // one thread per accumulator row (TMEM lane)
 constexpr int kTcStages = 4;
+constexpr int kTcTileLd = kCoarseTcM + 1;  // padded row of the accumulator tile
 __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16& h, __nv_bfloat16& l) {
   h = __float2bfloat16_rn(v);
   l = __float2bfloat16_rn(v - __bfloat162float(h));
 }
-// r_c pack (aggregate a of subdomain sd, columns 4 pk .. 4 pk + 3), zero outside n, kp
-__device__ __forceinline__ Pack<float> restrict_pack(const DTiles& tl, const Coarse<float>& co,
-                                                     int a0, int n, int kp, int a, int pk) {
+
+// block (kb, sd): r_c of aggregates 32 kb .. 32 kb + 31 into co.rcf and co.rcb, one thread
+// per (aggregate, 4 columns)
+constexpr int kRcThreads = 128;
+__global__ void __launch_bounds__(kRcThreads)
+    k_coarse_rc_pack(int kp, int NP, CgState s, Coarse<float> co) {
+  const int sd = blockIdx.y, kb = blockIdx.x;
+  if (s.active[sd] == 0) return;
+  const int n = co.nca[sd];
+  if (kb * tc::kKB >= n) return;
+  const int npk = NP / 4;
+  const int idx = blockIdx.z * kRcThreads + threadIdx.x;
+  if (idx >= tc::kKB * npk) return;
+  const int a0 = co.aoff[sd];
+  __nv_bfloat16* bh = co.rcb + (co.rcb_off[sd] + kb) * (int64_t)(2 * NP * tc::kKB);
+  __nv_bfloat16* bl = bh + NP * tc::kKB;
+  const int k = idx / npk, pk = idx - k * npk;
+  const int a = kb * tc::kKB + k;
   Pack<float> v;
 #pragma unroll
   for (int e = 0; e < 4; ++e) v.v[e] = 0.0f;
   if (a < n && 4 * pk < kp) {
-    const int ga = a0 + a;
-    const int t0 = co.tfirst[ga], tn = co.tcount[ga];
-    for (int t = t0; t < t0 + tn; ++t) {
-      const int slot = a - co.aloc[tl.r0[t]];
-      const Pack<float> pv = ld(co.cpart + (co.toff[t] + slot) * kp + 4 * pk);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) v.v[e] += pv.v[e];
-    }
+    v = restrict_pack(co, a0 + a, kp, 4 * pk);
+    st(co.rcf + (int64_t)(a0 + a) * kp + 4 * pk, v);
   }
-  return v;
-}
-// an open column of subdomain sd (the coarse product is skipped without one)
-__device__ __forceinline__ bool any_open_column(const CgState& s, int sd, int kp) {
-  bool open = false;
-  for (int c = 0; c < kp; ++c) open = open || !s.done[sd * kp + c];
-  return open;
-}
-
-// block (kb, sd): r_c of aggregates 32 kb .. 32 kb + 31 into co.rcb at co.rcb_off[sd] + kb
-__global__ void __launch_bounds__(kTcThreads)
-    k_coarse_rc_pack(DTiles tl, int kp, int NP, CgState s, Coarse<float> co) {
-  const int sd = blockIdx.y, kb = blockIdx.x;
-  if (s.active[sd] == 0 || !any_open_column(s, sd, kp)) return;
-  const int n = co.nca[sd];
-  if (kb * tc::kKB >= n) return;
-  const int a0 = co.aoff[sd];
-  __nv_bfloat16* bh = co.rcb + (co.rcb_off[sd] + kb) * (int64_t)(2 * NP * tc::kKB);
-  __nv_bfloat16* bl = bh + NP * tc::kKB;
-  const int npk = NP / 4;
-  for (int idx = threadIdx.x; idx < tc::kKB * npk; idx += blockDim.x) {
-    const int k = idx / npk, pk = idx - k * npk;
-    const Pack<float> v = restrict_pack(tl, co, a0, n, kp, kb * tc::kKB + k, pk);
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      __nv_bfloat16 h, l;
-      split_bf16(v.v[e], h, l);
-      const uint32_t o = tc::kmajor(4 * pk + e, k) >> 1;
-      bh[o] = h;
-      bl[o] = l;
-    }
+  for (int e = 0; e < 4; ++e) {
+    __nv_bfloat16 h, l;
+    split_bf16(v.v[e], h, l);
+    const uint32_t o = tc::kmajor(4 * pk + e, k) >> 1;
+    bh[o] = h;
+    bl[o] = l;
   }
 }
 
-__device__ __forceinline__ void cp_async16(uint32_t saddr, const void* g) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(g) : "memory");
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes,
+                                          uint32_t mbar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+          "r"(dst),
+      "l"(src), "r"(bytes), "r"(mbar)
+      : "memory");
 }
 
 __global__ void __launch_bounds__(kTcThreads)
     k_cg_coarse_tc(DTiles tl, int kp, int NP, double tol2, int mode, CgState s,
                    Coarse<float> co) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
   constexpr int KB = tc::kKB;
   constexpr int A_PLANE = kCoarseTcM * KB * 2;  // bytes
   extern __shared__ __align__(128) unsigned char smem[];
   const int B_PLANE = NP * KB * 2;
   const int STAGE = 2 * A_PLANE + 2 * B_PLANE;  // A hi, A lo, B hi, B lo
-  double* red = reinterpret_cast<double*>(smem + kTcStages * STAGE);  // 4 warps x NP
+  float* tile = reinterpret_cast<float*>(smem);  // after the MMAs: NP x kTcTileLd
   __shared__ uint32_t tmem_base;
-  __shared__ __align__(8) uint64_t mbar[kTcStages];
-  __shared__ int s_ok;
+  __shared__ __align__(8) uint64_t full[kTcStages], empty[kTcStages], ready;
+  __shared__ double red[kTcThreads * 4];
   Geo g = geo();
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int sd = blockIdx.y, mt = blockIdx.x, nmt = gridDim.x;
-  if (s.active[sd] == 0) return;
-  const int n = (co.aloc && any_open_column(s, sd, kp)) ? co.nca[sd] : 0;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int KS = (int)cl.num_blocks(), ks = (int)cl.block_rank();
+  const int sd = blockIdx.y, mt = blockIdx.x / KS, nmt = gridDim.x / KS;
+  if (s.active[sd] == 0) return;  // the whole cluster
+  const int n = co.nca[sd];
   const int a_lo = mt * kCoarseTcM;
-  for (int c = tid; c < 4 * NP; c += kTcThreads) red[c] = 0.0;
+  const int npk = NP / 4 / KS;  // packs of this CTA's share of the columns
+  const int c_lo = ks * npk * 4;
   if (a_lo < n) {
     const int a0 = co.aoff[sd];
     const int nkb = (n + KB - 1) / KB;
-    const unsigned char* Ag =
-        reinterpret_cast<const unsigned char*>(co.etc + (co.etc_off[sd] + (int64_t)mt * nkb) * 1024);
-    const unsigned char* Bg =
-        reinterpret_cast<const unsigned char*>(co.rcb + co.rcb_off[sd] * (int64_t)(2 * NP * KB));
+    const int kb0 = nkb * ks / KS, nblk = nkb * (ks + 1) / KS - kb0;
+    const unsigned char* Ag = reinterpret_cast<const unsigned char*>(
+        co.etc + (co.etc_off[sd] + (int64_t)mt * nkb + kb0) * 1024);
+    const unsigned char* Bg = reinterpret_cast<const unsigned char*>(
+        co.rcb + (co.rcb_off[sd] + kb0) * (int64_t)(2 * NP * KB));
     const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
-    // block kb's operands into stage stg: 16-byte asynchronous copies, one group
-    auto issue = [&](int kb, int stg) {
-      if (kb < nkb) {
-        const uint32_t sa = s0 + (uint32_t)(stg * STAGE);
-        const unsigned char* ga = Ag + (int64_t)kb * (2 * A_PLANE);
-        for (int i = tid; i < 2 * A_PLANE / 16; i += kTcThreads)
-          cp_async16(sa + 16 * i, ga + 16 * i);
-        const unsigned char* gb = Bg + (int64_t)kb * (2 * B_PLANE);
-        for (int i = tid; i < 2 * B_PLANE / 16; i += kTcThreads)
-          cp_async16(sa + 2 * A_PLANE + 16 * i, gb + 16 * i);
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-    };
+    const uint32_t mfull = (uint32_t)__cvta_generic_to_shared(full);
+    const uint32_t mempty = (uint32_t)__cvta_generic_to_shared(empty);
+    const uint32_t mready = (uint32_t)__cvta_generic_to_shared(&ready);
     uint32_t ncols = 32;
     while (ncols < (uint32_t)NP) ncols <<= 1;
     if (warp == 0) {
@@ -1005,143 +1126,137 @@ __global__ void __launch_bounds__(kTcThreads)
     }
     if (tid == 0) {
       for (int q = 0; q < kTcStages; ++q) {
-        const uint32_t mq = (uint32_t)__cvta_generic_to_shared(&mbar[q]);
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mq), "r"(1));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mfull + 8 * q));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mempty + 8 * q));
       }
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mready));
       asm volatile("fence.mbarrier_init.release.cluster;");
-      s_ok = 1;
     }
-    for (int q = 0; q < kTcStages - 1; ++q) issue(q, q);
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tbase = tmem_base;
-    const uint32_t idesc = tc::instr_desc(kCoarseTcM, NP);
-    uint32_t ph = 0;  // bit q: parity of the next completion of stage q's mbarrier
     bool ok = true;
-    int last = -1;  // stage of the last committed MMAs
-    for (int kb = 0; kb < nkb && ok; ++kb) {
-      const int stg = kb % kTcStages;
-      // block kb's copies are done (at most kTcStages - 2 newer groups pending)
-      asm volatile("cp.async.wait_group %0;" ::"n"(kTcStages - 2) : "memory");
-      asm volatile("fence.proxy.async.shared::cta;");
-      asm volatile("tcgen05.fence::before_thread_sync;");
-      __syncthreads();
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      if (tid == 0) {
-        const uint32_t sa = s0 + (uint32_t)(stg * STAGE);
+    if (tid == 32) {
+      // operand blocks kb0 .. kb0 + nblk - 1 into the stages in turn
+      int i = 0;
+      for (; i < nblk && ok; ++i) {
+        const int q = i % kTcStages;
+        if (i >= kTcStages)
+          ok = tc::mbar_wait(mempty + 8 * q, (uint32_t)(i / kTcStages - 1) & 1u, co.tc_budget);
+        if (!ok) break;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mfull + 8 * q),
+                     "r"((uint32_t)STAGE)
+                     : "memory");
+        bulk_copy(s0 + q * STAGE, Ag + (int64_t)i * (2 * A_PLANE), 2 * A_PLANE, mfull + 8 * q);
+        bulk_copy(s0 + q * STAGE + 2 * A_PLANE, Bg + (int64_t)i * (2 * B_PLANE), 2 * B_PLANE,
+                  mfull + 8 * q);
+      }
+      // after a timeout: the copies in flight still land in this CTA's shared memory
+      if (!ok)
+        for (int j = i > kTcStages ? i - kTcStages : 0; j < i; ++j)
+          tc::mbar_wait(mfull + 8 * (j % kTcStages), (uint32_t)(j / kTcStages) & 1u,
+                        co.tc_budget);
+    } else if (tid == 0) {
+      const uint32_t idesc = tc::instr_desc(kCoarseTcM, NP);
+      for (int i = 0; i < nblk; ++i) {
+        const int q = i % kTcStages;
+        ok = tc::mbar_wait(mfull + 8 * q, (uint32_t)(i / kTcStages) & 1u, co.tc_budget);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        const uint32_t sa = s0 + (uint32_t)(q * STAGE);
         const int pa[3] = {0, 0, 1}, pb[3] = {0, 1, 0};  // hi.hi, hi.lo, lo.hi
 #pragma unroll
-        for (int q = 0; q < 3; ++q)
+        for (int x = 0; x < 3; ++x)
 #pragma unroll
-          for (int ks = 0; ks < KB / 16; ++ks) {
+          for (int k = 0; k < KB / 16; ++k) {
             const uint64_t ad =
-                tc::smem_desc(sa + (uint32_t)(pa[q] * A_PLANE + ks * 256), 128, (KB / 8) * 128);
+                tc::smem_desc(sa + (uint32_t)(pa[x] * A_PLANE + k * 256), 128, (KB / 8) * 128);
             const uint64_t bd = tc::smem_desc(
-                sa + (uint32_t)(2 * A_PLANE + pb[q] * B_PLANE + ks * 256), 128, (KB / 8) * 128);
-            const uint32_t en = (kb == 0 && q == 0 && ks == 0) ? 0u : 1u;
+                sa + (uint32_t)(2 * A_PLANE + pb[x] * B_PLANE + k * 256), 128, (KB / 8) * 128);
+            const uint32_t en = (i == 0 && x == 0 && k == 0) ? 0u : 1u;
             asm volatile(
                 "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tbase),
                 "l"(ad), "l"(bd), "r"(idesc), "r"(en));
           }
-        const uint32_t mq = (uint32_t)__cvta_generic_to_shared(&mbar[stg]);
         asm volatile(
             "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                mq));
+                mempty + 8 * q));
       }
-      __syncwarp();
-      last = stg;
-      // refill the stage of block kb - 1 (block kb + kTcStages - 1) once its MMAs are done
-      if (kb >= 1) {
-        const int ps = (kb - 1) % kTcStages;
-        const uint32_t mq = (uint32_t)__cvta_generic_to_shared(&mbar[ps]);
-        if (tc::mbar_wait(mq, (ph >> ps) & 1u, co.tc_budget)) {
-          ph ^= 1u << ps;
-        } else {
-          atomicExch(co.tc_err, 1);
-          s_ok = 0;
-        }
-      }
-      issue(kb + kTcStages - 1, (kb + kTcStages - 1) % kTcStages);
-      __syncthreads();
-      ok = s_ok != 0;
+      // every MMA issued so far (none where the aggregates are fewer than the CTAs)
+      if (nblk > 0)
+        asm volatile(
+            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                mready));
+      else
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mready) : "memory");
     }
-    // the last block's MMAs (the others were waited for before their refills)
-    if (ok && last >= 0) {
-      const uint32_t mq = (uint32_t)__cvta_generic_to_shared(&mbar[last]);
-      if (tc::mbar_wait(mq, (ph >> last) & 1u, co.tc_budget)) {
-        ph ^= 1u << last;
-      } else {
-        atomicExch(co.tc_err, 1);
-        s_ok = 0;
-      }
+    __syncwarp();
+    // the MMAs are done: their stages may be overwritten
+    if (!tc::mbar_wait(mready, 0, co.tc_budget)) {
+      ok = false;
+      tc::mbar_wait(mready, 0, co.tc_budget);
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (!ok) atomicExch(co.tc_err, 1);
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
-    ok = s_ok != 0;
-    if (ok) {
-      // epilogue: row a of the tile is TMEM lane a = thread tid; eight columns per load
-      const int a = a_lo + tid;
-      for (int c0 = 0; c0 < NP; c0 += 8) {
-        uint32_t r[8];
-        const uint32_t ta = tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
-              "=r"(r[6]), "=r"(r[7])
-            : "r"(ta));
-        asm volatile("tcgen05.wait::ld.sync.aligned;");
-        double dl[8];
+    // row a of the accumulator is TMEM lane a = thread tid; eight columns per load
+    for (int c = 0; c < NP; c += 8) {
+      uint32_t r[8];
+      const uint32_t ta = tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)c;
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+            "=r"(r[7])
+          : "r"(ta));
+      asm volatile("tcgen05.wait::ld.sync.aligned;");
 #pragma unroll
-        for (int e = 0; e < 8; ++e) dl[e] = 0.0;
-        if (a < n) {
-          float* yo = co.yc + (int64_t)(a0 + a) * kp;
-#pragma unroll
-          for (int h = 0; h < 8; h += 4) {
-            const Pack<float> rp = restrict_pack(tl, co, a0, n, kp, a, (c0 + h) / 4);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int c = c0 + h + e;
-              const float y = __uint_as_float(r[h + e]);
-              if (c < kp) yo[c] = y;
-              dl[h + e] = (double)y * (double)rp.v[e];
-            }
-          }
-        }
-        // rows summed within the warp (fixed shuffle tree), one partial per warp
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          double v = dl[e];
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-          if (lane == 0) red[warp * NP + c0 + e] = v;
-        }
-      }
-    } else if (last >= 0) {
-      // a wait ran out: wait once more (bounded) for the stages' pending MMAs, so that
-      // they drain before the TMEM is released
-      for (int q = 0; q < kTcStages; ++q) {
-        const uint32_t mq = (uint32_t)__cvta_generic_to_shared(&mbar[q]);
-        tc::mbar_wait(mq, (ph >> q) & 1u, co.tc_budget);
-      }
+      for (int e = 0; e < 8; ++e)
+        tile[(c + e) * kTcTileLd + tid] = nblk > 0 ? __uint_as_float(r[e]) : 0.0f;
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
+    if (KS > 1)
+      cl.sync();
+    else
+      __syncthreads();
     if (warp == 0)
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase),
                    "r"(ncols));
+    // y_c and r_c.y_c for this CTA's columns: thread (pack tx, rows ty, ty + RB, ...)
+    const int RB = kTcThreads / npk, tx = tid % npk, ty = tid / npk;
+    const int c = c_lo + 4 * tx;
+    double dl[4] = {0.0, 0.0, 0.0, 0.0};
+    if (ty < RB && c < kp)
+      for (int r = ty; r < kCoarseTcM && a_lo + r < n; r += RB) {
+        const int64_t at = (int64_t)(a0 + a_lo + r) * kp + c;
+        const Pack<float> rv = ld(co.rcf + at);
+        Pack<float> y;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          y.v[e] = 0.0f;
+          for (int k = 0; k < KS; ++k)
+            y.v[e] += *(KS > 1 ? cl.map_shared_rank(tile + (c + e) * kTcTileLd + r, k)
+                               : tile + (c + e) * kTcTileLd + r);
+          dl[e] += (double)y.v[e] * (double)rv.v[e];
+        }
+        st(co.yc + at, y);
+      }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) red[tid * 4 + e] = dl[e];
+    __syncthreads();
+    for (int x = tid; x < 4 * npk && c_lo + x < kp; x += kTcThreads) {
+      double t = 0.0;
+      for (int q = 0; q < RB; ++q) t += red[(q * npk + x / 4) * 4 + (x & 3)];
+      __stcg(co.dpart + ((int64_t)sd * nmt + mt) * kp + c_lo + x, t);
+    }
+    if (KS > 1) cl.sync();  // no CTA leaves while another reads its accumulators
+  } else {
+    for (int x = tid; x < 4 * npk && c_lo + x < kp; x += kTcThreads)
+      __stcg(co.dpart + ((int64_t)sd * nmt + mt) * kp + c_lo + x, 0.0);
   }
-  __syncthreads();
-  // this block's part of r_c.y_c per column, warps in order
-  for (int c = tid; c < kp; c += kTcThreads) {
-    double t = 0.0;
-    for (int w = 0; w < kTcThreads / 32; ++w) t += red[w * NP + c];
-    co.dpart[((int64_t)sd * nmt + mt) * kp + c] = t;
-  }
-  if (!last_block(g, s.counter, sd, nmt)) return;
+  if (!take_ticket(g, s.counter + sd, gridDim.x)) return;
   coarse_finish<float>(g, tl, sd, kp, kp, nmt, tol2, mode, s, co);
 }
 
@@ -1191,9 +1306,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 4)
     st(p + o, pv);
   }
   block_colsum<T, N>(g, apr, sm.red, s.part1 + (int64_t)tile * kp);
-  int lo = tl.lo[sd], hi = tl.hi[sd];
-  if (!last_block(g, s.counter, sd, hi - lo)) return;
-  sd_colsums(g, s.part1, kp, lo, hi, sm.scratch, sm.sums);
+  const double* const parts[1] = {s.part1};
+  if (!tile_sums<1>(g, parts, s.gpart, s.gcount, s.counter + sd, kp, tile, tl.lo[sd], tl.hi[sd],
+                    sm.scratch, sm.sums))
+    return;
   for (int c = g.tid; c < kp; c += g.nth) s.pr[sd * kp + c] = sm.sums[c];
 }
 
@@ -1272,9 +1388,10 @@ __global__ void k_cg_replace(DTiles tl, const double* __restrict__ r64, T* __res
     slots_store(g, cs, nsl, kp, co.cpart + co.toff[tile] * kp);
   }
   block_colsum<T, N>(g, arz, sm.red, s.part1 + (int64_t)tile * kp);
-  int lo = tl.lo[sd], hi = tl.hi[sd];
-  if (!last_block(g, s.counter, sd, hi - lo)) return;
-  sd_colsums(g, s.part1, kp, lo, hi, sm.scratch, sm.sums);
+  const double* const parts[1] = {s.part1};
+  if (!tile_sums<1>(g, parts, s.gpart, s.gcount, s.counter + sd, kp, tile, tl.lo[sd], tl.hi[sd],
+                    sm.scratch, sm.sums))
+    return;
   for (int c = g.tid; c < kp; c += g.nth) {
     int i = sd * kp + c;
     // reopened, or the recursion drifted from the true residual (a stale direction
@@ -1374,52 +1491,68 @@ void launch_coarse_then_p(const DTiles& tiles, int n_sd, const T* r, T* p, const
   static bool attr = false;
   if (!attr) {
     const int mx = (int)(align16(sizeof(T) * kMaxAgg * kCoarseCols) + kCoarseRedBytes);
-    cudaFuncSetAttribute((const void*)k_cg_coarse<T, 1>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    cudaFuncSetAttribute((const void*)k_cg_coarse<T, 2>,
+    cudaFuncSetAttribute((const void*)k_cg_coarse<T>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
     attr = true;
   }
-  const int n_max = co.aloc ? co.n_max : 0;
+  const int n_max = co.tbase ? co.n_max : 0;
   dim3 bl = block_of<T>(kp);
-  count_launch(2);
+  bool done = false;
   if constexpr (sizeof(T) == 4) {
     if (co.etc) {
-      // tensor-core product: one block per 128 rows of y_c and subdomain, every column
+      // tensor-core product: a cluster per 128 rows of y_c and subdomain, every column
       const int NP = (kp + 15) & ~15;
-      const size_t smt = (size_t)kTcStages * (2 * (kCoarseTcM * tc::kKB * 2) +
-                                              2 * NP * tc::kKB * 2) +
-                         sizeof(double) * 4 * NP;
+      const int nmt = std::max(1, (n_max + kCoarseTcM - 1) / kCoarseTcM);
+      const int nkb = std::max(1, (n_max + tc::kKB - 1) / tc::kKB);
+      // split the aggregates over 2 or 4 CTAs while the grid stays within two blocks per SM
+      int KS = 1;
+      while (KS < 4 && 2 * KS * nmt * n_sd <= 2 * 152 && 4 * KS <= nkb) KS *= 2;
+      const size_t smt = std::max((size_t)kTcStages * (2 * (kCoarseTcM * tc::kKB * 2) +
+                                                       2 * NP * tc::kKB * 2),
+                                  sizeof(float) * kTcTileLd * (size_t)NP);
       static bool attr_tc = false;
       if (!attr_tc) {
         cudaFuncSetAttribute((const void*)k_cg_coarse_tc,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         attr_tc = true;
       }
-      const int nmt = std::max(1, (n_max + kCoarseTcM - 1) / kCoarseTcM);
-      const int nkb = std::max(1, (n_max + tc::kKB - 1) / tc::kKB);
-      count_launch();
-      k_coarse_rc_pack<<<dim3(nkb, n_sd), kTcThreads, 0, st>>>(tiles, kp, NP, s, co);
-      k_cg_coarse_tc<<<dim3(nmt, n_sd), kTcThreads, smt, st>>>(tiles, kp, NP, tol2, mode, s,
-                                                                co);
-      if (ev_mid) cudaEventRecord(*ev_mid, st);
-      k_cg_update_p<T><<<tiles.n, bl, smem_bytes<T>(bl.x, bl.y, kp, 0), st>>>(tiles, r, p,
-                                                                             dinv, kp, s, co);
-      return;
+      count_launch(2);
+      const int per = tc::kKB * (NP / 4);
+      k_coarse_rc_pack<<<dim3(nkb, n_sd, (per + kRcThreads - 1) / kRcThreads), kRcThreads, 0,
+                         st>>>(kp, NP, s, co);
+      cudaLaunchAttribute at{};
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = (unsigned)KS;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg{};
+      cfg.gridDim = dim3(nmt * KS, n_sd);
+      cfg.blockDim = dim3(kTcThreads);
+      cfg.dynamicSmemBytes = smt;
+      cfg.stream = st;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      cudaLaunchKernelEx(&cfg, k_cg_coarse_tc, tiles, kp, NP, tol2, mode, s, co);
+      done = true;
     }
   }
-  const size_t sm = align16(sizeof(T) * ((n_max + 7) & ~7) * kCoarseCols) + kCoarseRedBytes;
-  const int rows = n_max > kCoarseThreads ? 2 * kCoarseThreads : kCoarseThreads;
-  const int nrb = std::max(1, (n_max + rows - 1) / rows);
-  const int nchunk = (kp + kCoarseCols - 1) / kCoarseCols;
-  dim3 grid(nrb * nchunk, n_sd);
-  if (rows > kCoarseThreads)
-    k_cg_coarse<T, 2><<<grid, kCoarseThreads, sm, st>>>(tiles, kp, tol2, mode, s, co);
-  else
-    k_cg_coarse<T, 1><<<grid, kCoarseThreads, sm, st>>>(tiles, kp, tol2, mode, s, co);
+  if (!done) {
+    count_launch();
+    if (n_max <= kCoarseSmallMax) {
+      k_cg_coarse_small<T><<<dim3(kp / kCoarseSmallCols, n_sd), kCoarseThreads, 0, st>>>(
+          tiles, kp, tol2, mode, s, co);
+    } else {
+      const size_t sm = align16(sizeof(T) * ((n_max + 7) & ~7) * kCoarseCols) + kCoarseRedBytes;
+      const int rows = kCoarseRpt * kCoarseThreads;
+      const int nrb = (n_max + rows - 1) / rows;
+      const int nchunk = (kp + kCoarseCols - 1) / kCoarseCols;
+      k_cg_coarse<T><<<dim3(nrb * nchunk, n_sd), kCoarseThreads, sm, st>>>(tiles, kp, tol2, mode,
+                                                                          s, co);
+    }
+  }
   if (ev_mid) cudaEventRecord(*ev_mid, st);
-  k_cg_update_p<T><<<tiles.n, bl, smem_bytes<T>(bl.x, bl.y, kp, 0), st>>>(tiles, r, p, dinv,
-                                                                         kp, s, co);
+  count_launch();
+  k_cg_update_p<T><<<tiles.n, bl, smem_bytes<T>(bl.x, bl.y, kp, 0), st>>>(tiles, r, p, dinv, kp,
+                                                                         s, co);
 }
 
 template <typename T>
