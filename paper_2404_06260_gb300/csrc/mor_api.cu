@@ -561,10 +561,11 @@ struct Build {
     if (h_poll) cudaFreeHost(h_poll);
   }
 
-  // sum of active[] over the subdomains (and of second[] into h_poll[1])
-  int poll(const int* active, const int* second = nullptr) {
-    launch_count_active(n_sd, active, d_poll, st, second);
-    CK(cudaMemcpyAsync(h_poll, d_poll, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
+  // sum of active[] over the subdomains (of second[] into h_poll[1], the row tiles of the
+  // subdomains with active > 0 into h_poll[2])
+  int poll(const DTiles& tl, const int* active, const int* second = nullptr) {
+    launch_count_active(tl, active, d_poll, st, second);
+    CK(cudaMemcpyAsync(h_poll, d_poll, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     return h_poll[0];
   }
@@ -616,12 +617,12 @@ struct Build {
     launch_zero_rows(tl, x64, kp, st);
     launch_residual64(tl, A.e64(), b64, x64, vR64, kp, nc, ncn, rtol2, 1, false, anorm[set],
                       rs, st);
-    if (poll(rs.active) == 0) return MOR_OK;
+    if (poll(tl, rs.active) == 0) return MOR_OK;
     launch_cast<T>(tl, vR64, b, kp, st);
     launch_cg_init<T>(tl, b, x, r, p, dinvT, kp, nc, ncn, cs, co, st);
     const int check = 8;
     const int every = std::max(check, o->replace_every / check * check);
-    int it = 0;
+    int it = 0, open_tiles = tl.n;
     while (true) {
       int chunk = std::min(check, o->max_iter - it);
       for (int c = 0; c < chunk; ++c) {
@@ -632,23 +633,26 @@ struct Build {
               Prof::Pending{sizeof(T) == 4 ? 0 : 1, {pb[0], pb[1], pb[2], pb[3]},
                             g_prof.used - 1});
         }
-        launch_cg_step<T>(tl, AT, x, r, p, q, dinvT, kp, rtol2, cs, co, st, ev);
+        launch_cg_step<T>(tl, AT, x, r, p, q, dinvT, kp, rtol2, open_tiles, cs, co, st, ev);
       }
       it += chunk;
-      int act = poll(cs.active);
+      int act = poll(tl, cs.active);
+      open_tiles = h_poll[2];
       if (act == 0 || it % every == 0 || it >= o->max_iter) {
         launch_accum_reset<T>(tl, x, x64, kp, st);
         launch_residual64(tl, A.e64(), b64, x64, vR64, kp, nc, ncn, rtol2, 0, false,
                           anorm[set], rs, st);
         ++sweeps;
-        int ract = poll(rs.active, rs.nnear);
+        int ract = poll(tl, rs.active, rs.nnear);
+        int rs_tiles = h_poll[2];
         if (ract > 0 && h_poll[1] > 0) {
           // some open column is within reach of the rounding level: measure the exact
           // reference || |A| |x| + |b| || and test again
           launch_residual64(tl, A.e64(), b64, x64, vR64, kp, nc, ncn, rtol2, 0, true,
                             anorm[set], rs, st);
           ++sweeps;
-          ract = poll(rs.active);
+          ract = poll(tl, rs.active);
+          rs_tiles = h_poll[2];
         }
         if (debug) {
           std::vector<double> orr((size_t)n_sd * kp), obb((size_t)n_sd * kp);
@@ -685,6 +689,7 @@ struct Build {
           break;
         }
         launch_cg_replace<T>(tl, vR64, r, p, dinvT, kp, o->drift_restart, cs, rs, co, st);
+        open_tiles = rs_tiles;
       }
     }
     iters[which] += it;
@@ -858,8 +863,8 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
   const int64_t nEllW = ceil_div(nW, 32) * 32 * WW;
   const int64_t nEllO = ceil_div(nO, 32) * 32 * WW;
 
-  CK(cudaMallocHost((void**)&B.h_poll, 2 * sizeof(int)));
-  TRY(M.alloc(&B.d_poll, 2, true, st));
+  CK(cudaMallocHost((void**)&B.h_poll, 3 * sizeof(int)));
+  TRY(M.alloc(&B.d_poll, 3, true, st));
   int* d_err;
   TRY(M.alloc(&d_err, 1, true, st));
 

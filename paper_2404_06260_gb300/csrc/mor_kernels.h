@@ -158,14 +158,16 @@ template <typename T>
 void launch_cg_init(const DTiles& tiles, const T* b, T* x, T* r, T* p, const T* dinv,
                     int kp, int nc, int ncn, const CgState& s, const Coarse<T>& co,
                     cudaStream_t st);
-// ev (null or 5 events) is recorded before the sparse product and after each of the
+// open_tiles: row tiles of the subdomains still open (it picks the block size).  ev (null or
+// 5 events) is recorded before the sparse product and after each of the
 // four kernels of the step.
 template <typename T>
 void launch_cg_step(const DTiles& tiles, const EllView<T>& A, T* x, T* r, T* p, T* q,
-                    const T* dinv, int kp, double tol2, const CgState& s,
+                    const T* dinv, int kp, double tol2, int open_tiles, const CgState& s,
                     const Coarse<T>& co, cudaStream_t st, const cudaEvent_t* ev = nullptr);
-// out[0] = sum of active[0..n_sd), out[1] = sum of second (0 if null); out has 2 ints
-void launch_count_active(int n_sd, const int* active, int* out, cudaStream_t st,
+// out[0] = sum of active[0..n_sd), out[1] = sum of second (0 if null), out[2] = row tiles of
+// the subdomains with active > 0
+void launch_count_active(const DTiles& tiles, const int* active, int* out, cudaStream_t st,
                          const int* second = nullptr);
 
 // binary64 residual: r64 = b64 - A64 x64 with per-column norms; scale = 1/||r64|| for

@@ -127,29 +127,37 @@ __device__ __forceinline__ bool take_ticket(const Geo& g, int* counter, int n) {
   return is_last != 0;
 }
 
-// sums[c] = sum over rows lo..hi-1 of part[t*kp + c], fixed order.  Columns are taken
-// in groups of at most nth; within a group S = nth / group threads share a column.
-__device__ void rows_colsum(const Geo& g, const double* part, int kp, int lo, int hi,
+// sums[q*kp + c] = sum over rows lo..hi-1 of part[q][t*kp + c], q < NS, in a fixed order: S
+// threads share a column (at most 4: their sums are then added one after the other, and a
+// binary64 addition takes 66 clocks), eight loads in flight each
+template <int NS>
+__device__ void rows_colsum(const Geo& g, const double* const (&part)[NS], int kp, int lo, int hi,
                             double* scratch, double* sums) {
-  for (int c0 = 0; c0 < kp; c0 += g.nth) {
-    const int cw = min(kp - c0, g.nth);
-    const int S = g.nth / cw;
-    const int c = c0 + g.tid % cw, sidx = g.tid / cw;
+  const int cols = NS * kp;
+  for (int c0 = 0; c0 < cols; c0 += g.nth) {
+    const int cw = min(cols - c0, g.nth);
+    const int S = min(4, g.nth / cw);
+    const int sidx = g.tid / cw, x = c0 + g.tid - sidx * cw;
     double acc = 0.0;
-    if (sidx < S)
-      for (int t = lo + sidx; t < hi; t += 4 * S) {
-        double v[4];
+    if (sidx < S) {
+      const int q = x / kp, c = x - q * kp;
+      const double* P = part[0];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          v[u] = t + u * S < hi ? __ldcg(part + (int64_t)(t + u * S) * kp + c) : 0.0;
+      for (int u = 1; u < NS; ++u) P = q == u ? part[u] : P;
+      for (int t = lo + sidx; t < hi; t += 8 * S) {
+        double v[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) acc += v[u];
+        for (int u = 0; u < 8; ++u)
+          v[u] = t + u * S < hi ? __ldcg(P + (int64_t)(t + u * S) * kp + c) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc += v[u];
       }
+    }
     scratch[g.tid] = acc;
     __syncthreads();
     for (int cc = g.tid; cc < cw; cc += g.nth) {
-      double s = 0.0;
-      for (int q = 0; q < S; ++q) s += scratch[q * cw + cc];
+      double s = scratch[cc];
+      for (int q = 1; q < S; ++q) s += scratch[q * cw + cc];
       sums[c0 + cc] = s;
     }
     __syncthreads();
@@ -168,27 +176,26 @@ __device__ bool tile_sums(const Geo& g, const double* const (&part)[NS], double*
                           int* gcount, int* count, int kp, int tile, int lo, int hi,
                           double* scratch, double* sums) {
   const int nt = hi - lo;
-  if (nt <= kRedGroup + kRedGroup / 2) {
+  if (nt <= 2 * kRedGroup) {
     if (!take_ticket(g, count, nt)) return false;
-#pragma unroll
-    for (int q = 0; q < NS; ++q) rows_colsum(g, part[q], kp, lo, hi, scratch, sums + q * kp);
+    rows_colsum<NS>(g, part, kp, lo, hi, scratch, sums);
     return true;
   }
   const int ng = (nt + kRedGroup - 1) / kRedGroup, gi = (tile - lo) / kRedGroup;
   const int g0 = lo + gi * kRedGroup, g1 = min(hi, g0 + kRedGroup);
   if (!take_ticket(g, gcount + lo + gi, g1 - g0)) return false;
-  // group sums of a subdomain: rows (lo + gi) NS .. of gpart, NS rows per group
+  // group sums of a subdomain: NS blocks of ng rows from row lo NS of gpart
   double* gp = gpart + (int64_t)lo * NS * kp;
-#pragma unroll
-  for (int q = 0; q < NS; ++q) {
-    rows_colsum(g, part[q], kp, g0, g1, scratch, sums + q * kp);
-    for (int c = g.tid; c < kp; c += g.nth)
-      __stcg(gp + ((int64_t)q * ng + gi) * kp + c, sums[q * kp + c]);
+  rows_colsum<NS>(g, part, kp, g0, g1, scratch, sums);
+  for (int x = g.tid; x < NS * kp; x += g.nth) {
+    const int q = x / kp, c = x - q * kp;
+    __stcg(gp + ((int64_t)q * ng + gi) * kp + c, sums[x]);
   }
   if (!take_ticket(g, count, ng)) return false;
+  const double* gparts[NS];
 #pragma unroll
-  for (int q = 0; q < NS; ++q)
-    rows_colsum(g, gp + (int64_t)q * ng * kp, kp, 0, ng, scratch, sums + q * kp);
+  for (int q = 0; q < NS; ++q) gparts[q] = gp + (int64_t)q * ng * kp;
+  rows_colsum<NS>(g, gparts, kp, 0, ng, scratch, sums);
   return true;
 }
 
@@ -380,7 +387,7 @@ __device__ __forceinline__ void spmm_row_res(int rr, int w, int tx, const Slot2<
 // at most TH threads per block; 40 registers leave room for 1536 threads per SM (six
 // blocks of 256, twelve of 128).  R: records gathered per batch (spmm_row)
 template <typename T, int R = 1, int TH = 256>
-__global__ void __launch_bounds__(TH, 1536 / TH)
+__global__ void __launch_bounds__(TH, TH <= 256 ? 1536 / TH : 1)
     k_cg_spmm_pq(DTiles tl, EllView<T> A, const T* __restrict__ p, T* __restrict__ q, int kp,
                  CgState s) {
   constexpr int N = Pack<T>::N;
@@ -532,49 +539,103 @@ __global__ void k_residual64(DTiles tl, EllView<double> A, const double* __restr
 }
 
 // ---------------------------------------------------------------------------------
-// Restriction r_c = Z^T r on a row tile: aggregates are contiguous runs of rows, so the
-// rows of one thread (increasing) change aggregate rarely; each thread keeps a running
-// sum and adds it to the tile's slot (aggregate - aggregate of the first row) in shared
-// memory when its aggregate changes.  The tile's slots then go to cpart in order.
-template <typename T>
-__device__ __forceinline__ T* slot_smem(const Geo& g, int kp) {
-  extern __shared__ __align__(16) unsigned char raw[];
-  return reinterpret_cast<T*>(raw + align16(smem_bytes<T>(g.nch, g.rb, kp, 0)));
+// Restriction r_c = Z^T r on a row tile.  Aggregates are contiguous runs of rows, so the
+// tile's rows go to shared memory (SB rows at a time) and one thread per (aggregate, pack)
+// adds the run in row order: a fixed order, and no atomics.  (Every thread adding its
+// rows to the aggregates' slots by shared-memory atomics, one flush per row as the threads'
+// rows lie 23 apart, made the x/r update of the 64^3 workload 217 us a launch, now 203.)
+constexpr size_t kRestrictWhole = 32 * 1024;  // a whole tile of r up to this, else equal
+constexpr size_t kRestrictBytes = 24 * 1024;  // parts of at most this (or RB rows)
+__host__ __device__ __forceinline__ int restrict_rows(int rb, int kp, size_t tsz) {
+  const size_t tile = (size_t)kTileRows * kp * tsz;
+  if (tile <= kRestrictWhole) return kTileRows;
+  const int parts = (int)((tile + kRestrictBytes - 1) / kRestrictBytes);
+  const int rows = ((kTileRows + parts - 1) / parts + rb - 1) / rb * rb;
+  return rows < kTileRows ? rows : kTileRows;
 }
-size_t slot_smem_bytes(size_t base, int kp, size_t tsz) {
-  return align16(base) + (size_t)kMaxSlots * kp * tsz;
-}
-
 template <typename T>
-struct RestrictAcc {
+struct TileRestrict {
   static constexpr int N = Pack<T>::N;
-  int cur = -1;
-  T acc[N];
-  __device__ __forceinline__ void flush(T* cs, int kp, int tx) {
-    if (cur >= 0)
-#pragma unroll
-      for (int e = 0; e < N; ++e) atomicAdd(&cs[cur * kp + tx * N + e], acc[e]);
-  }
-  __device__ __forceinline__ void add(T* cs, int kp, int tx, int slot, const Pack<T>& v) {
-    if (slot != cur) {
-      flush(cs, kp, tx);
-      cur = slot;
-#pragma unroll
-      for (int e = 0; e < N; ++e) acc[e] = T(0);
+  T* buf;    // SB rows x kp
+  T* cs;     // kMaxSlots x kp: sums of the aggregates (tiles of more than SB rows)
+  int* run;  // kMaxSlots + 1: first row (in the tile) of each aggregate
+  int a0, nsl, SB;
+  __device__ __forceinline__ void begin(const Geo& g, int kp, size_t base, int r0, int nrows,
+                                        const int32_t* aloc) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    SB = restrict_rows(g.rb, kp, sizeof(T));
+    size_t o = align16(base);
+    buf = reinterpret_cast<T*>(raw + o);
+    o += align16(sizeof(T) * (size_t)SB * kp);
+    cs = reinterpret_cast<T*>(raw + o);
+    if (SB < nrows) o += align16(sizeof(T) * (size_t)kMaxSlots * kp);
+    run = reinterpret_cast<int*>(raw + o);
+    a0 = aloc[r0];
+    nsl = aloc[r0 + nrows - 1] - a0 + 1;
+    for (int rr = g.tid; rr < nrows; rr += g.nth) {
+      const int a = aloc[r0 + rr];
+      if (rr == 0 || a != aloc[r0 + rr - 1]) run[a - a0] = rr;
     }
+    if (g.tid == 0) run[nsl] = nrows;
+  }
+  __device__ __forceinline__ void put(int rr, int kp, int tx, const Pack<T>& v) {
+    st(buf + rr * kp + tx * N, v);
+  }
+  // rows [s0, s0 + SB) are in buf (and visible): add them; the last step stores to dst.
+  // S threads share an (aggregate, pack) where there are more threads than pairs, each a
+  // stretch of the run, their sums meeting in red (one pack per thread)
+  __device__ __forceinline__ void add(const Geo& g, int kp, int s0, int nrows, T* red, T* dst) {
+    const int s1 = min(nrows, s0 + SB);
+    const int items = nsl * g.nch, S = max(1, g.nth / items);
+    for (int idx = g.tid; idx < items * S; idx += g.nth) {
+      const int it = idx % items, sg = idx / items;
+      const int sl = it / g.nch, pk = it - sl * g.nch;
+      const int r0 = max(run[sl], s0), len = max(0, min(run[sl + 1], s1) - r0);
+      const int lo = r0 + len * sg / S, hi = r0 + len * (sg + 1) / S;
+      Pack<T> acc;
 #pragma unroll
-    for (int e = 0; e < N; ++e) acc[e] += v.v[e];
+      for (int e = 0; e < N; ++e) acc.v[e] = T(0);
+#pragma unroll 4
+      for (int rr = lo; rr < hi; ++rr) {
+        const Pack<T> v = ld(buf + (rr - s0) * kp + pk * N);
+#pragma unroll
+        for (int e = 0; e < N; ++e) acc.v[e] += v.v[e];
+      }
+      if (S == 1)
+        finish(kp, s0, s1 == nrows, sl, pk, acc, dst);
+      else
+        st(red + g.tid * N, acc);
+    }
+    if (S == 1) return;
+    __syncthreads();
+    if (g.tid < items) {
+      Pack<T> acc = ld(red + g.tid * N);
+      for (int sg = 1; sg < S; ++sg) {
+        const Pack<T> v = ld(red + (sg * items + g.tid) * N);
+#pragma unroll
+        for (int e = 0; e < N; ++e) acc.v[e] += v.v[e];
+      }
+      const int sl = g.tid / g.nch;
+      finish(kp, s0, s1 == nrows, sl, g.tid - sl * g.nch, acc, dst);
+    }
+    __syncthreads();
+  }
+  __device__ __forceinline__ void finish(int kp, int s0, bool last, int sl, int pk, Pack<T> acc,
+                                         T* dst) {
+    if (s0 > 0) {
+      const Pack<T> v = ld(cs + sl * kp + pk * N);
+#pragma unroll
+      for (int e = 0; e < N; ++e) acc.v[e] = v.v[e] + acc.v[e];
+    }
+    st((last ? dst + (int64_t)sl * kp : cs + sl * kp) + pk * N, acc);
   }
 };
-
 template <typename T>
-__device__ __forceinline__ void slots_zero(const Geo& g, T* cs, int nsl, int kp) {
-  for (int i = g.tid; i < nsl * kp; i += g.nth) cs[i] = T(0);
-}
-template <typename T>
-__device__ __forceinline__ void slots_store(const Geo& g, const T* cs, int nsl, int kp,
-                                            T* dst) {
-  for (int i = g.tid; i < nsl * kp; i += g.nth) dst[i] = cs[i];
+size_t restrict_smem_bytes(int rb, int kp) {
+  const int SB = restrict_rows(rb, kp, sizeof(T));
+  return align16(sizeof(T) * (size_t)SB * kp) +
+         (SB < kTileRows ? align16(sizeof(T) * (size_t)kMaxSlots * kp) : 0) +
+         align16(sizeof(int) * (kMaxSlots + 1));
 }
 
 // x = 0, r = b, the fine r.z = b.D^{-1}b, ||b||^2 and the restriction of b; the coarse
@@ -589,38 +650,36 @@ __global__ void k_cg_init(DTiles tl, const T* __restrict__ b, T* x, T* r,
   int tile = blockIdx.x, sd = tl.sd[tile];
   int r0 = tl.r0[tile], r1 = tl.r1[tile];
   const bool coarse = co.aloc != nullptr;
-  T* cs = slot_smem<T>(g, kp);
-  int a0 = 0, nsl = 0;
-  if (coarse) {
-    a0 = co.aloc[r0];
-    nsl = co.aloc[r1 - 1] - a0 + 1;
-    slots_zero(g, cs, nsl, kp);
-    __syncthreads();
-  }
-  RestrictAcc<T> ra;
+  const int nrows = r1 - r0;
+  TileRestrict<T> tr;
+  if (coarse) tr.begin(g, kp, smem_bytes<T>(g.nch, g.rb, kp, 0), r0, nrows, co.aloc);
+  const int step = coarse ? tr.SB : nrows;
   T arz[N], arr[N];
 #pragma unroll
   for (int e = 0; e < N; ++e) arz[e] = arr[e] = T(0);
   Pack<T> zero;
 #pragma unroll
   for (int e = 0; e < N; ++e) zero.v[e] = T(0);
-  for (int64_t row = r0 + g.ty; row < r1; row += g.rb) {
-    int64_t o = row * kp + g.tx * N;
-    Pack<T> bv = ld(b + o);
-    T d = dinv[row];
+  for (int s0 = 0; s0 < nrows; s0 += step) {
+    for (int rr = s0 + g.ty; rr < min(nrows, s0 + step); rr += g.rb) {
+      const int64_t row = r0 + rr;
+      int64_t o = row * kp + g.tx * N;
+      Pack<T> bv = ld(b + o);
+      T d = dinv[row];
 #pragma unroll
-    for (int e = 0; e < N; ++e) {
-      arz[e] += bv.v[e] * (d * bv.v[e]);
-      arr[e] += bv.v[e] * bv.v[e];
+      for (int e = 0; e < N; ++e) {
+        arz[e] += bv.v[e] * (d * bv.v[e]);
+        arr[e] += bv.v[e] * bv.v[e];
+      }
+      if (coarse) tr.put(rr - s0, kp, g.tx, bv);
+      st(x + o, zero);
+      st(r + o, bv);
     }
-    if (coarse) ra.add(cs, kp, g.tx, co.aloc[row] - a0, bv);
-    st(x + o, zero);
-    st(r + o, bv);
-  }
-  if (coarse) {
-    ra.flush(cs, kp, g.tx);
-    __syncthreads();
-    slots_store(g, cs, nsl, kp, co.cpart + co.toff[tile] * kp);
+    if (coarse) {
+      __syncthreads();
+      tr.add(g, kp, s0, nrows, sm.red, co.cpart + co.toff[tile] * kp);
+      if (s0 + step < nrows) __syncthreads();
+    }
   }
   block_colsum<T, N>(g, arz, sm.red, s.part1 + (int64_t)tile * kp);
   __syncthreads();
@@ -654,9 +713,10 @@ __global__ void k_cg_init(DTiles tl, const T* __restrict__ b, T* x, T* r,
 
 // x += alpha p, r -= alpha q; ||r||^2, the fine r.z = r.D^{-1}r and the restriction of
 // the new r; the coarse kernel (STEP) completes r.M^{-1}r, beta and the done flags.
-// 48 registers (binary32) leave room for five blocks per SM; six cost spills.
-template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 4)
+// TH = 256: 48 registers (binary32) leave room for five blocks per SM; six cost spills.
+// TH = 1024: light loads (light_threads)
+template <typename T, int TH>
+__global__ void __launch_bounds__(TH, TH == 256 ? (sizeof(T) == 4 ? 5 : 4) : 1)
     k_cg_update_xr(DTiles tl, T* x, T* r, const T* __restrict__ p, const T* __restrict__ q,
                    const T* __restrict__ dinv, int kp, CgState s, Coarse<T> co) {
   constexpr int N = Pack<T>::N;
@@ -664,18 +724,12 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 4)
   Smem<T> sm = smem_layout<T>(g, kp, 0);
   int tile = blockIdx.x, sd = tl.sd[tile];
   if (s.active[sd] == 0) return;
-  int r0 = tl.r0[tile], r1 = tl.r1[tile];
+  const int r0 = tl.r0[tile], nrows = tl.r1[tile] - r0;
   const bool coarse = co.aloc != nullptr;
-  T* cs = slot_smem<T>(g, kp);
-  int a0 = 0, nsl = 0;
-  if (coarse) {
-    a0 = co.aloc[r0];
-    nsl = co.aloc[r1 - 1] - a0 + 1;
-    slots_zero(g, cs, nsl, kp);
-    __syncthreads();
-  }
-  RestrictAcc<T> ra;
-  const int64_t rend = pack_done<T>(s, sd, kp, g.tx) ? r0 : r1;
+  TileRestrict<T> tr;
+  if (coarse) tr.begin(g, kp, smem_bytes<T>(g.nch, g.rb, kp, 0), r0, nrows, co.aloc);
+  const int step = coarse ? tr.SB : nrows;
+  const bool skip = pack_done<T>(s, sd, kp, g.tx);
   const Pack<T> alp = coef_pack<T>(s.alpha, s.alpha32, sd, kp, g.tx);
   T al[N];
 #pragma unroll
@@ -683,25 +737,35 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 4)
   T arr[N], arz[N];
 #pragma unroll
   for (int e = 0; e < N; ++e) arr[e] = arz[e] = T(0);
-  for (int64_t row = r0 + g.ty; row < rend; row += g.rb) {
-    int64_t o = row * kp + g.tx * N;
-    Pack<T> xv = ld(x + o), rv = ld(r + o), pv = ld(p + o), qv = ld(q + o);
-    T d = dinv[row];
+  for (int s0 = 0; s0 < nrows; s0 += step) {
+    for (int rr = s0 + g.ty; rr < min(nrows, s0 + step); rr += g.rb) {
+      const int64_t row = r0 + rr;
+      const int64_t o = row * kp + g.tx * N;
+      Pack<T> rv;
+      if (skip) {
 #pragma unroll
-    for (int e = 0; e < N; ++e) {
-      xv.v[e] += al[e] * pv.v[e];
-      rv.v[e] -= al[e] * qv.v[e];
-      arr[e] += rv.v[e] * rv.v[e];
-      arz[e] += rv.v[e] * (d * rv.v[e]);
+        for (int e = 0; e < N; ++e) rv.v[e] = T(0);
+      } else {
+        Pack<T> xv = ld(x + o), pv = ld(p + o), qv = ld(q + o);
+        rv = ld(r + o);
+        T d = dinv[row];
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+          xv.v[e] += al[e] * pv.v[e];
+          rv.v[e] -= al[e] * qv.v[e];
+          arr[e] += rv.v[e] * rv.v[e];
+          arz[e] += rv.v[e] * (d * rv.v[e]);
+        }
+        st(x + o, xv);
+        st(r + o, rv);
+      }
+      if (coarse) tr.put(rr - s0, kp, g.tx, rv);
     }
-    if (coarse) ra.add(cs, kp, g.tx, co.aloc[row] - a0, rv);
-    st(x + o, xv);
-    st(r + o, rv);
-  }
-  if (coarse) {
-    ra.flush(cs, kp, g.tx);
-    __syncthreads();
-    slots_store(g, cs, nsl, kp, co.cpart + co.toff[tile] * kp);
+    if (coarse) {
+      __syncthreads();
+      tr.add(g, kp, s0, nrows, sm.red, co.cpart + co.toff[tile] * kp);
+      if (s0 + step < nrows) __syncthreads();
+    }
   }
   block_colsum<T, N>(g, arr, sm.red, s.part1 + (int64_t)tile * kp);
   __syncthreads();
@@ -1262,8 +1326,8 @@ __global__ void __launch_bounds__(kTcThreads)
 
 // p = gam (D^{-1} r + Z y_c) + beta p (p is not read where beta = 0), and p.r of the
 // new direction for the next step length
-template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 4)
+template <typename T, int TH>
+__global__ void __launch_bounds__(TH, TH == 256 ? (sizeof(T) == 4 ? 6 : 4) : 1)
     k_cg_update_p(DTiles tl, const T* __restrict__ r, T* p, const T* __restrict__ dinv, int kp,
                   CgState s, Coarse<T> co) {
   constexpr int N = Pack<T>::N;
@@ -1313,25 +1377,25 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 4)
   for (int c = g.tid; c < kp; c += g.nth) s.pr[sd * kp + c] = sm.sums[c];
 }
 
-// out[0] = sum of active, out[1] = sum of second (if not null)
-__global__ void k_count_active(int n_sd, const int* active, const int* second, int* out) {
-  __shared__ int tot, tot2;
-  if (threadIdx.x == 0) tot = tot2 = 0;
+// out[0] = sum of active, out[1] = sum of second (if not null), out[2] = row tiles of the
+// subdomains with active > 0
+__global__ void k_count_active(DTiles tl, const int* active, const int* second, int* out) {
+  __shared__ int tot[3];
+  if (threadIdx.x < 3) tot[threadIdx.x] = 0;
   __syncthreads();
-  int a = 0, b = 0;
-  for (int i = threadIdx.x; i < n_sd; i += blockDim.x) {
-    a += active[i];
+  int a = 0, b = 0, t = 0;
+  for (int i = threadIdx.x; i < tl.n_sd; i += blockDim.x) {
+    const int ac = active[i];
+    a += ac;
     if (second) b += second[i];
+    if (ac > 0) t += tl.hi[i] - tl.lo[i];
   }
-  atomicAdd(&tot, a);
-  atomicAdd(&tot2, b);
+  atomicAdd(&tot[0], a);
+  atomicAdd(&tot[1], b);
+  atomicAdd(&tot[2], t);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    out[0] = tot;
-    out[1] = tot2;
-  }
+  if (threadIdx.x < 3) out[threadIdx.x] = tot[threadIdx.x];
 }
-
 
 __global__ void k_zero_rows(DTiles tl, double* x, int kp) {
   Geo g = geo();
@@ -1358,34 +1422,32 @@ __global__ void k_cg_replace(DTiles tl, const double* __restrict__ r64, T* __res
   int tile = blockIdx.x, sd = tl.sd[tile];
   int r0 = tl.r0[tile], r1 = tl.r1[tile];
   const bool coarse = co.aloc != nullptr;
-  T* cs = slot_smem<T>(g, kp);
-  int a0 = 0, nsl = 0;
-  if (coarse) {
-    a0 = co.aloc[r0];
-    nsl = co.aloc[r1 - 1] - a0 + 1;
-    slots_zero(g, cs, nsl, kp);
-    __syncthreads();
-  }
-  RestrictAcc<T> ra;
+  const int nrows = r1 - r0;
+  TileRestrict<T> tr;
+  if (coarse) tr.begin(g, kp, smem_bytes<T>(g.nch, g.rb, kp, 0), r0, nrows, co.aloc);
+  const int step = coarse ? tr.SB : nrows;
   T arz[N];
 #pragma unroll
   for (int e = 0; e < N; ++e) arz[e] = T(0);
-  for (int64_t row = r0 + g.ty; row < r1; row += g.rb) {
-    int64_t o = row * kp + g.tx * N;
-    Pack<T> rv;
-    T d = dinv[row];
+  for (int s0 = 0; s0 < nrows; s0 += step) {
+    for (int rr = s0 + g.ty; rr < min(nrows, s0 + step); rr += g.rb) {
+      const int64_t row = r0 + rr;
+      int64_t o = row * kp + g.tx * N;
+      Pack<T> rv;
+      T d = dinv[row];
 #pragma unroll
-    for (int e = 0; e < N; ++e) {
-      rv.v[e] = (T)r64[o + e];
-      arz[e] += rv.v[e] * (d * rv.v[e]);
+      for (int e = 0; e < N; ++e) {
+        rv.v[e] = (T)r64[o + e];
+        arz[e] += rv.v[e] * (d * rv.v[e]);
+      }
+      if (coarse) tr.put(rr - s0, kp, g.tx, rv);
+      st(rT + o, rv);
     }
-    if (coarse) ra.add(cs, kp, g.tx, co.aloc[row] - a0, rv);
-    st(rT + o, rv);
-  }
-  if (coarse) {
-    ra.flush(cs, kp, g.tx);
-    __syncthreads();
-    slots_store(g, cs, nsl, kp, co.cpart + co.toff[tile] * kp);
+    if (coarse) {
+      __syncthreads();
+      tr.add(g, kp, s0, nrows, sm.red, co.cpart + co.toff[tile] * kp);
+      if (s0 + step < nrows) __syncthreads();
+    }
   }
   block_colsum<T, N>(g, arz, sm.red, s.part1 + (int64_t)tile * kp);
   const double* const parts[1] = {s.part1};
@@ -1453,9 +1515,21 @@ __global__ void k_cast(DTiles tl, const double* __restrict__ src, T* __restrict_
 template <typename T>
 dim3 block_of(int kp, int threads = 256) {
   int nch = kp / Pack<T>::N;
-  int rb = threads / nch;
+  int rb = std::min(threads / nch, kTileRows);
   if (rb < 1) rb = 1;
   return dim3(nch, rb);
+}
+
+// Threads per block of a step's tile kernels by the row tiles of the subdomains still
+// open.  A full chip wants blocks of 256 (registers, several blocks per SM).  With no more
+// tiles than SMs a step is as long as one block, whose threads take their rows one after
+// the other: blocks of 1024 shorten that chain (16^3 workload, 113 tiles: 18.4 -> 17.6 ms;
+// blocks of 512 up to 456 tiles: no change).  Binary64 steps are bound by their arithmetic,
+// of which larger blocks have more (block_colsum; 21 -> 27 ms): 256 always.
+template <typename T>
+int light_threads(int open_tiles) {
+  if (sizeof(T) == 8) return 256;
+  return open_tiles <= 152 ? 1024 : 256;
 }
 
 }  // namespace
@@ -1481,13 +1555,13 @@ void launch_spmm(const DTiles& tiles, const EllView<T>& A, const T* X, T* Y, int
 
 template <typename T>
 size_t slot_kernel_smem(dim3 bl, int kp) {
-  return slot_smem_bytes(smem_bytes<T>(bl.x, bl.y, kp, 0), kp, sizeof(T));
+  return align16(smem_bytes<T>(bl.x, bl.y, kp, 0)) + restrict_smem_bytes<T>(bl.y, kp);
 }
 
 template <typename T>
 void launch_coarse_then_p(const DTiles& tiles, int n_sd, const T* r, T* p, const T* dinv,
-                          int kp, double tol2, int mode, const CgState& s, const Coarse<T>& co,
-                          cudaStream_t st, const cudaEvent_t* ev_mid) {
+                          int kp, double tol2, int mode, int open_tiles, const CgState& s,
+                          const Coarse<T>& co, cudaStream_t st, const cudaEvent_t* ev_mid) {
   static bool attr = false;
   if (!attr) {
     const int mx = (int)(align16(sizeof(T) * kMaxAgg * kCoarseCols) + kCoarseRedBytes);
@@ -1496,7 +1570,6 @@ void launch_coarse_then_p(const DTiles& tiles, int n_sd, const T* r, T* p, const
     attr = true;
   }
   const int n_max = co.tbase ? co.n_max : 0;
-  dim3 bl = block_of<T>(kp);
   bool done = false;
   if constexpr (sizeof(T) == 4) {
     if (co.etc) {
@@ -1551,8 +1624,11 @@ void launch_coarse_then_p(const DTiles& tiles, int n_sd, const T* r, T* p, const
   }
   if (ev_mid) cudaEventRecord(*ev_mid, st);
   count_launch();
-  k_cg_update_p<T><<<tiles.n, bl, smem_bytes<T>(bl.x, bl.y, kp, 0), st>>>(tiles, r, p, dinv, kp,
-                                                                         s, co);
+  const int th = light_threads<T>(open_tiles);
+  const dim3 bl = block_of<T>(kp, th);
+  const size_t sm = smem_bytes<T>(bl.x, bl.y, kp, 0);
+  auto fn = th == 1024 ? k_cg_update_p<T, 1024> : k_cg_update_p<T, 256>;
+  fn<<<tiles.n, bl, sm, st>>>(tiles, r, p, dinv, kp, s, co);
 }
 
 template <typename T>
@@ -1569,8 +1645,8 @@ void launch_cg_init(const DTiles& tiles, const T* b, T* x, T* r, T* p, const T* 
   count_launch();
   k_cg_init<T><<<tiles.n, bl, slot_kernel_smem<T>(bl, kp), st>>>(tiles, b, x, r, dinv, kp, nc,
                                                                   ncn, s, co);
-  launch_coarse_then_p<T>(tiles, tiles.n_sd, r, p, dinv, kp, 0.0, kCoarseInit, s, co, st,
-                          nullptr);
+  launch_coarse_then_p<T>(tiles, tiles.n_sd, r, p, dinv, kp, 0.0, kCoarseInit,
+                          tiles.n, s, co, st, nullptr);
 }
 
 // ---- autotuner of the sparse product: four launch configurations of k_cg_spmm_pq
@@ -1643,8 +1719,8 @@ int spmm_variant(const DTiles& tiles, const EllView<T>& A, const T* p, T* q, int
 
 template <typename T>
 void launch_cg_step(const DTiles& tiles, const EllView<T>& A, T* x, T* r, T* p, T* q,
-                    const T* dinv, int kp, double tol2, const CgState& s, const Coarse<T>& co,
-                    cudaStream_t st, const cudaEvent_t* ev) {
+                    const T* dinv, int kp, double tol2, int open_tiles, const CgState& s,
+                    const Coarse<T>& co, cudaStream_t st, const cudaEvent_t* ev) {
   if (tiles.n <= 0) return;
   static bool attr = false;
   if (!attr) {
@@ -1652,27 +1728,34 @@ void launch_cg_step(const DTiles& tiles, const EllView<T>& A, T* x, T* r, T* p, 
     set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 2, 256>);
     set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 1, 128>);
     set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 2, 128>);
-    set_smem_attr<T>((const void*)k_cg_update_xr<T>);
+    set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 2, 1024>);
+    set_smem_attr<T>((const void*)k_cg_update_xr<T, 256>);
+    set_smem_attr<T>((const void*)k_cg_update_xr<T, 1024>);
     attr = true;
   }
-  dim3 bl = block_of<T>(kp);
+  const int th = light_threads<T>(open_tiles);
+  const dim3 bl = block_of<T>(kp, th);
   const int variant = spmm_variant<T>(tiles, A, p, q, kp, s, st);
   count_launch(2);
   if (ev) cudaEventRecord(ev[0], st);
-  launch_spmm_pq_variant<T>(variant, tiles, A, p, q, kp, s, st);
+  if (th == 256) {
+    launch_spmm_pq_variant<T>(variant, tiles, A, p, q, kp, s, st);
+  } else {
+    k_cg_spmm_pq<T, 2, 1024><<<tiles.n, bl, smem_bytes<T>(bl.x, bl.y, kp, A.W), st>>>(tiles, A, p, q, kp, s);
+  }
   if (ev) cudaEventRecord(ev[1], st);
-  k_cg_update_xr<T><<<tiles.n, bl, slot_kernel_smem<T>(bl, kp), st>>>(tiles, x, r, p, q, dinv,
-                                                                       kp, s, co);
+  auto fn = th == 1024 ? k_cg_update_xr<T, 1024> : k_cg_update_xr<T, 256>;
+  fn<<<tiles.n, bl, slot_kernel_smem<T>(bl, kp), st>>>(tiles, x, r, p, q, dinv, kp, s, co);
   if (ev) cudaEventRecord(ev[2], st);
-  launch_coarse_then_p<T>(tiles, tiles.n_sd, r, p, dinv, kp, tol2, kCoarseStep, s, co, st,
-                          ev ? &ev[3] : nullptr);
+  launch_coarse_then_p<T>(tiles, tiles.n_sd, r, p, dinv, kp, tol2, kCoarseStep, open_tiles, s, co,
+                          st, ev ? &ev[3] : nullptr);
   if (ev) cudaEventRecord(ev[4], st);
 }
 
-void launch_count_active(int n_sd, const int* active, int* out, cudaStream_t st,
+void launch_count_active(const DTiles& tiles, const int* active, int* out, cudaStream_t st,
                          const int* second) {
   count_launch();
-  k_count_active<<<1, 256, 0, st>>>(n_sd, active, second, out);
+  k_count_active<<<1, 256, 0, st>>>(tiles, active, second, out);
 }
 
 void launch_residual64(const DTiles& tiles, const EllView<double>& A, const double* b64,
@@ -1711,8 +1794,8 @@ void launch_cg_replace(const DTiles& tiles, const double* r64, T* rT, T* pT, con
   count_launch();
   k_cg_replace<T><<<tiles.n, bl, slot_kernel_smem<T>(bl, kp), st>>>(
       tiles, r64, rT, dinv, kp, drift * drift, s, rs, co);
-  launch_coarse_then_p<T>(tiles, tiles.n_sd, rT, pT, dinv, kp, 0.0, kCoarseReplace, s, co, st,
-                          nullptr);
+  launch_coarse_then_p<T>(tiles, tiles.n_sd, rT, pT, dinv, kp, 0.0, kCoarseReplace,
+                          tiles.n, s, co, st, nullptr);
 }
 
 template <typename T>
@@ -1785,10 +1868,11 @@ template void launch_cg_init<double>(const DTiles&, const double*, double*, doub
                                      const double*, int, int, int, const CgState&,
                                      const Coarse<double>&, cudaStream_t);
 template void launch_cg_step<float>(const DTiles&, const EllView<float>&, float*, float*,
-                                    float*, float*, const float*, int, double, const CgState&,
-                                    const Coarse<float>&, cudaStream_t, const cudaEvent_t*);
+                                    float*, float*, const float*, int, double, int,
+                                    const CgState&, const Coarse<float>&, cudaStream_t,
+                                    const cudaEvent_t*);
 template void launch_cg_step<double>(const DTiles&, const EllView<double>&, double*, double*,
-                                     double*, double*, const double*, int, double,
+                                     double*, double*, const double*, int, double, int,
                                      const CgState&, const Coarse<double>&, cudaStream_t,
                                      const cudaEvent_t*);
 void autotune_enable(bool on) {
