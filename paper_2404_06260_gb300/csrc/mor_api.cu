@@ -551,7 +551,7 @@ struct Build {
   int* d_poll = nullptr;
   // workspace
   double *vR64 = nullptr;
-  void *xT = nullptr, *rT = nullptr, *pT = nullptr, *qT = nullptr, *bT = nullptr;
+  void *xT = nullptr, *rT = nullptr, *pT = nullptr, *qT = nullptr;
   CgState cs{};
   RefineState rs{};
   int64_t iters[4] = {0, 0, 0, 0};
@@ -605,7 +605,6 @@ struct Build {
     T* r = (T*)rT;
     T* p = (T*)pT;
     T* q = (T*)qT;
-    T* b = (T*)bT;
     double rtol2 = rtol * rtol;
     double pb[4] = {0, 0, 0, 0};
     // bytes come from the device work counters (cs.work), attributed when the build
@@ -614,12 +613,9 @@ struct Build {
     // recursively updated residual replaced by the binary64 residual b - A x64 every
     // replace_every iterations and whenever the recursion reports convergence
     // (residual replacement keeps the search directions, so no Krylov restart)
-    launch_zero_rows(tl, x64, kp, st);
-    launch_residual64(tl, A.e64(), b64, x64, vR64, kp, nc, ncn, rtol2, 1, false, anorm[set],
-                      rs, st);
+    launch_cg_start<T>(tl, b64, x64, x, r, p, dinvT, kp, nc, ncn, rtol2, cs, rs, co, st);
     if (poll(tl, rs.active) == 0) return MOR_OK;
-    launch_cast<T>(tl, vR64, b, kp, st);
-    launch_cg_init<T>(tl, b, x, r, p, dinvT, kp, nc, ncn, cs, co, st);
+    bool seen = false;  // a residual sweep of this solve has marked what it settled
     const int check = 8;
     const int every = std::max(check, o->replace_every / check * check);
     int it = 0, open_tiles = tl.n;
@@ -639,17 +635,18 @@ struct Build {
       int act = poll(tl, cs.active);
       open_tiles = h_poll[2];
       if (act == 0 || it % every == 0 || it >= o->max_iter) {
-        launch_accum_reset<T>(tl, x, x64, kp, st);
-        launch_residual64(tl, A.e64(), b64, x64, vR64, kp, nc, ncn, rtol2, 0, false,
-                          anorm[set], rs, st);
+        launch_accum_reset<T>(tl, x, x64, kp, seen, rs, st);
+        launch_residual64(tl, A.e64(), b64, x64, vR64, kp, nc, rtol2, seen, false, anorm[set],
+                          rs, st);
+        seen = true;
         ++sweeps;
         int ract = poll(tl, rs.active, rs.nnear);
         int rs_tiles = h_poll[2];
         if (ract > 0 && h_poll[1] > 0) {
           // some open column is within reach of the rounding level: measure the exact
           // reference || |A| |x| + |b| || and test again
-          launch_residual64(tl, A.e64(), b64, x64, vR64, kp, nc, ncn, rtol2, 0, true,
-                            anorm[set], rs, st);
+          launch_residual64(tl, A.e64(), b64, x64, vR64, kp, nc, rtol2, seen, true, anorm[set],
+                            rs, st);
           ++sweeps;
           ract = poll(tl, rs.active);
           rs_tiles = h_poll[2];
@@ -1073,17 +1070,15 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
   TRY(M.alloc(&vX, nP * kp, true, st));
   TRY(M.alloc(&B.vR64, nP * kp, true, st));
   {
-    unsigned char *a, *b, *c, *d, *e;
+    unsigned char *a, *b, *c, *d;
     TRY(M.alloc(&a, nP * kp * tsz, true, st));
     TRY(M.alloc(&b, nP * kp * tsz, true, st));
     TRY(M.alloc(&c, nP * kp * tsz, true, st));
     TRY(M.alloc(&d, nP * kp * tsz, true, st));
-    TRY(M.alloc(&e, nP * kp * tsz, true, st));
     B.xT = a;
     B.rT = b;
     B.pT = c;
     B.qT = d;
-    B.bT = e;
   }
   int mt = S.max_tiles;
   TRY(M.alloc(&B.cs.rz, (size_t)n_sd * kp, true, st));

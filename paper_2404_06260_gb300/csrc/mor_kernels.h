@@ -154,10 +154,6 @@ void launch_spmm(const DTiles& tiles, const EllView<T>& A, const T* X, T* Y, int
 // the fine r.z and the restriction, coarse solve with beta, p update).  Columns
 // c < ncn of a subdomain measure convergence against the largest ||b_c|| among them
 // (block-normwise); the others against their own ||b_c||.
-template <typename T>
-void launch_cg_init(const DTiles& tiles, const T* b, T* x, T* r, T* p, const T* dinv,
-                    int kp, int nc, int ncn, const CgState& s, const Coarse<T>& co,
-                    cudaStream_t st);
 // open_tiles: row tiles of the subdomains still open (it picks the block size).  ev (null or
 // 5 events) is recorded before the sparse product and after each of the
 // four kernels of the step.
@@ -187,15 +183,22 @@ struct RefineState {
 // a binary64 residual below kResidualFloor * 2^-53 * || |A| |x| + |b| ||_2 is rounding
 // noise of its own evaluation; launch_residual64 stops such columns
 constexpr double kResidualFloor = 4.0;
+// x64 = 0, xT = 0, rT = (T) b64, pT = M^{-1} rT, the references and the first test of the
+// binary64 convergence test (of the residual b64) and the CG state
+template <typename T>
+void launch_cg_start(const DTiles& tiles, const double* b64, double* x64, T* x, T* r, T* p,
+                     const T* dinv, int kp, int nc, int ncn, double rtol2, const CgState& s,
+                     const RefineState& rs, const Coarse<T>& co, cudaStream_t st);
 // r64 = b - A x64 per column, the binary64 convergence test (rtol, or the rounding level
-// of the residual itself), done flags in s.scale; first = 1 also fixes the references
-// from b (x64 = 0).  floor_ref = true refreshes the rounding-level reference
-// || |A| |x| + |b| || (one extra binary64 add per product).  s.nnear counts the open
-// columns whose residual is within the rounding level of the bound
-// anorm[sd] ||x|| + ||b|| (anorm = max row sum of |A|; ||x|| of this sweep).
+// of the residual itself), done flags in s.scale.  seen: this solve has had a sweep; the
+// subdomains and 16-byte packs that met the test then are skipped (their x64 has not
+// changed).  floor_ref = true refreshes the rounding-level reference || |A| |x| + |b| ||
+// (one extra binary64 add per product).  s.nnear counts the open columns whose residual is
+// within the rounding level of the bound anorm[sd] ||x|| + ||b|| (anorm = max row sum of
+// |A|; ||x|| of this sweep).
 void launch_residual64(const DTiles& tiles, const EllView<double>& A, const double* b64,
-                       const double* x64, double* r64, int kp, int nc, int ncn, double rtol2,
-                       int first, bool floor_ref, const double* anorm, const RefineState& s,
+                       const double* x64, double* r64, int kp, int nc, double rtol2, bool seen,
+                       bool floor_ref, const double* anorm, const RefineState& s,
                        cudaStream_t st);
 // out[sd] += stored entries in the rows of the tiles of sd (out zeroed by the caller)
 void launch_count_sd_nnz(const DTiles& tiles, const EllView<double>& A, int64_t* out,
@@ -203,7 +206,6 @@ void launch_count_sd_nnz(const DTiles& tiles, const EllView<double>& A, int64_t*
 // anorm[sd] = max over the rows of tiles in sd of sum_j |a_ij| (anorm zeroed by caller)
 void launch_row_abs_max(const DTiles& tiles, const EllView<double>& A, double* anorm,
                         cudaStream_t st);
-void launch_zero_rows(const DTiles& tiles, double* x, int kp, cudaStream_t st);
 // residual replacement of the CG recursion: rT = (T) r64, rz recomputed, done flags from
 // the binary64 convergence test of launch_residual64 (scale == 0 means converged);
 // reopened columns restart with pT = M^{-1} rT
@@ -234,12 +236,10 @@ constexpr int kCoarseTcM = 128;  // rows of y_c per tensor-core block (the MMA M
 void launch_coarse_tc_pack(int n_sd, int blocks_max, const int32_t* nca, const int64_t* eoff,
                            const float* einv, const int64_t* etc_off, uint4* out,
                            cudaStream_t st);
-// x64 += xT, xT = 0
+// x64 += xT, xT = 0 (seen as in launch_residual64)
 template <typename T>
-void launch_accum_reset(const DTiles& tiles, T* xT, double* x64, int kp, cudaStream_t st);
-// dst = (T) src on the rows of tiles
-template <typename T>
-void launch_cast(const DTiles& tiles, const double* src, T* dst, int kp, cudaStream_t st);
+void launch_accum_reset(const DTiles& tiles, T* xT, double* x64, int kp, bool seen,
+                        const RefineState& rs, cudaStream_t st);
 
 // ---------------- dense per-subdomain kernels (mor_dense.cu) ----------------
 // G[sd] = X^T Y over the rows of tiles: nx x ny with row stride ldg and subdomain

@@ -91,7 +91,8 @@ __host__ __device__ __forceinline__ size_t smem_bytes(int nch, int rb, int kp, i
 
 // column sums over ty of per-thread N-wide accumulators -> out[tx*N + e] (double)
 template <typename T, int N>
-__device__ void block_colsum(const Geo& g, const T (&acc)[N], T* red, double* out) {
+__device__ void block_colsum(const Geo& g, const T (&acc)[N], T* red, double* out,
+                             bool write = true) {
 #pragma unroll
   for (int e = 0; e < N; ++e) red[g.tid * N + e] = acc[e];
   __syncthreads();
@@ -103,7 +104,7 @@ __device__ void block_colsum(const Geo& g, const T (&acc)[N], T* red, double* ou
       for (int e = 0; e < N; ++e) red[g.tid * N + e] += red[(g.tid + s * g.nch) * N + e];
     __syncthreads();
   }
-  if (g.ty == 0)
+  if (g.ty == 0 && write)
 #pragma unroll
     for (int e = 0; e < N; ++e) out[g.tx * N + e] = (double)red[g.tx * N + e];
 }
@@ -432,20 +433,33 @@ __global__ void __launch_bounds__(TH, TH <= 256 ? 1536 / TH : 1)
   }
 }
 
+// the N columns of pack tx met the binary64 test in the last sweep of this solve (seen: there
+// was one): their x64 has not changed since, nor have their residual and its sums
+template <int N>
+__device__ __forceinline__ bool pack_settled(const RefineState& s, int sd, int kp, int tx,
+                                             int seen) {
+  bool all = seen != 0;
+#pragma unroll
+  for (int e = 0; e < N; ++e) all = s.scale[sd * kp + tx * N + e] == 0.0 && all;
+  return all;
+}
+
 template <bool kFloor>
 __global__ void k_residual64(DTiles tl, EllView<double> A, const double* __restrict__ b,
                              const double* __restrict__ x, double* __restrict__ r, int kp,
-                             int nc, int ncn, double rtol2, int first, RefineState s,
+                             int nc, double rtol2, int seen, RefineState s,
                              const double* __restrict__ anorm) {
   constexpr int N = 2;
   Geo g = geo();
   Smem<double> sm = smem_layout<double>(g, kp, A.W);
   const int tile = blockIdx.x, sd = tl.sd[tile];
+  if (seen && s.active[sd] == 0) return;  // settled in the last sweep
   const int r0 = tl.r0[tile], r1 = tl.r1[tile];
   stage_tile(g, r0, r1 - r0, A, sm.slots);
   __syncthreads();
+  const bool settled = pack_settled<N>(s, sd, kp, g.tx, seen);
   double acc[N] = {0.0, 0.0}, aca[N] = {0.0, 0.0}, axx[N] = {0.0, 0.0};
-  for (int rr = g.ty; rr < r1 - r0; rr += g.rb) {
+  for (int rr = g.ty; rr < (settled ? 0 : r1 - r0); rr += g.rb) {
     int64_t row = r0 + rr;
     Pack<double> ax, aabs;
     {
@@ -470,9 +484,10 @@ __global__ void k_residual64(DTiles tl, EllView<double> A, const double* __restr
     }
     st(r + o, rv);
   }
-  block_colsum<double, N>(g, acc, sm.red, s.part + (int64_t)tile * kp);
+  // a settled pack keeps the last sweep's sums
+  block_colsum<double, N>(g, acc, sm.red, s.part + (int64_t)tile * kp, !settled);
   __syncthreads();
-  block_colsum<double, N>(g, axx, sm.red, s.part3 + (int64_t)tile * kp);
+  block_colsum<double, N>(g, axx, sm.red, s.part3 + (int64_t)tile * kp, !settled);
   if constexpr (kFloor) {
     __syncthreads();
     block_colsum<double, N>(g, aca, sm.red, s.part2 + (int64_t)tile * kp);
@@ -482,7 +497,9 @@ __global__ void k_residual64(DTiles tl, EllView<double> A, const double* __restr
     if (!tile_sums<3>(g, parts, s.gpart, s.gcount, s.counter + sd, kp, tile, tl.lo[sd],
                       tl.hi[sd], sm.scratch, sm.sums))
       return;
-    for (int c = g.tid; c < kp; c += g.nth) s.oaa[sd * kp + c] = sm.sums[2 * kp + c];
+    // (a settled pack's part2 holds zeros: its reference stays)
+    for (int c = g.tid; c < kp; c += g.nth)
+      if (sm.sums[2 * kp + c] > 0.0) s.oaa[sd * kp + c] = sm.sums[2 * kp + c];
   } else {
     const double* const parts[2] = {s.part, s.part3};
     if (!tile_sums<2>(g, parts, s.gpart, s.gcount, s.counter + sd, kp, tile, tl.lo[sd],
@@ -491,16 +508,7 @@ __global__ void k_residual64(DTiles tl, EllView<double> A, const double* __restr
   }
   for (int c = g.tid; c < kp; c += g.nth) s.xx[sd * kp + c] = sm.sums[kp + c];
   __shared__ int cnt, nfl, nnear;
-  __shared__ double bref;
-  if (g.tid == 0) {
-    cnt = 0;
-    nfl = 0;
-    nnear = 0;
-    double m = 0.0;
-    if (first)
-      for (int c = 0; c < ncn; ++c) m = fmax(m, sm.sums[c]);
-    bref = m;
-  }
+  if (g.tid == 0) cnt = nfl = nnear = 0;
   __syncthreads();
   // attainable accuracy: the rounding error of the binary64 residual of a binary64 x is
   // about u || |A| |x| + |b| ||_2 (u = 2^-53); a residual below kResidualFloor times that
@@ -511,10 +519,6 @@ __global__ void k_residual64(DTiles tl, EllView<double> A, const double* __restr
   for (int c = g.tid; c < kp; c += g.nth) {
     int i = sd * kp + c;
     double rr = sm.sums[c];
-    if (first) {
-      s.obb[i] = (c < ncn) ? bref : rr;
-      s.oaa[i] = 0.0;
-    }
     s.orr[i] = rr;
     bool by_rtol = rr <= rtol2 * s.obb[i];
     bool by_floor = rr <= fl2 * s.oaa[i];
@@ -525,7 +529,7 @@ __global__ void k_residual64(DTiles tl, EllView<double> A, const double* __restr
     // || |A| |x| + |b| || <= ||A||_inf ||x|| + ||b|| (A symmetric): a column above
     // that bound's rounding level cannot stop on the floor test, so the reference
     // needs refreshing only when some open column is below it
-    if (!done && !first) {
+    if (!done) {
       double bnd = anorm[sd] * sqrt(s.xx[i]) + sqrt(s.obb[i]);
       if (rr <= fl2 * bnd * bnd) atomicAdd(&nnear, 1);
     }
@@ -630,6 +634,12 @@ struct TileRestrict {
     st((last ? dst + (int64_t)sl * kp : cs + sl * kp) + pk * N, acc);
   }
 };
+// k_cg_start has a binary64 column-sum area behind the usual layout
+template <typename T>
+__host__ __device__ __forceinline__ size_t start_smem_base(int nch, int rb, int kp) {
+  return align16(smem_bytes<T>(nch, rb, kp, 0)) +
+         sizeof(double) * Pack<T>::N * (size_t)nch * rb;
+}
 template <typename T>
 size_t restrict_smem_bytes(int rb, int kp) {
   const int SB = restrict_rows(rb, kp, sizeof(T));
@@ -638,12 +648,16 @@ size_t restrict_smem_bytes(int rb, int kp) {
          align16(sizeof(int) * (kMaxSlots + 1));
 }
 
-// x = 0, r = b, the fine r.z = b.D^{-1}b, ||b||^2 and the restriction of b; the coarse
-// kernel (INIT) then sets rz and the p update forms p = M^{-1} b
+// Start of a solve with x = 0, in one pass over b: x64 = 0, xT = 0, rT = (T) b, the binary64
+// norms that fix the references of the convergence test (RefineState, as k_residual64 leaves
+// it for a residual b), the fine r.z = b.D^{-1}b, ||b||^2 and the restriction of b; the
+// coarse kernel (INIT) then sets rz and the p update forms p = M^{-1} b.  One read of b and
+// three writes instead of a zero fill, a residual sweep A 0, a cast and an init pass: the
+// sweep alone was a full binary64 product: 2.35 ms of the 64^3 workload's solve, 0.32 now.
 template <typename T>
-__global__ void k_cg_init(DTiles tl, const T* __restrict__ b, T* x, T* r,
-                          const T* __restrict__ dinv, int kp, int nc, int ncn, CgState s,
-                          Coarse<T> co) {
+__global__ void k_cg_start(DTiles tl, const double* __restrict__ b64, double* x64, T* x, T* r,
+                           const T* __restrict__ dinv, int kp, int nc, int ncn, double rtol2,
+                           CgState s, RefineState rs, Coarse<T> co) {
   constexpr int N = Pack<T>::N;
   Geo g = geo();
   Smem<T> sm = smem_layout<T>(g, kp, 0);
@@ -652,20 +666,35 @@ __global__ void k_cg_init(DTiles tl, const T* __restrict__ b, T* x, T* r,
   const bool coarse = co.aloc != nullptr;
   const int nrows = r1 - r0;
   TileRestrict<T> tr;
-  if (coarse) tr.begin(g, kp, smem_bytes<T>(g.nch, g.rb, kp, 0), r0, nrows, co.aloc);
+  if (coarse) tr.begin(g, kp, start_smem_base<T>(g.nch, g.rb, kp), r0, nrows, co.aloc);
   const int step = coarse ? tr.SB : nrows;
   T arz[N], arr[N];
+  double ab[N];
 #pragma unroll
-  for (int e = 0; e < N; ++e) arz[e] = arr[e] = T(0);
+  for (int e = 0; e < N; ++e) {
+    arz[e] = arr[e] = T(0);
+    ab[e] = 0.0;
+  }
   Pack<T> zero;
 #pragma unroll
   for (int e = 0; e < N; ++e) zero.v[e] = T(0);
+  const Pack<double> zero64{{0.0, 0.0}};
   for (int s0 = 0; s0 < nrows; s0 += step) {
     for (int rr = s0 + g.ty; rr < min(nrows, s0 + step); rr += g.rb) {
       const int64_t row = r0 + rr;
-      int64_t o = row * kp + g.tx * N;
-      Pack<T> bv = ld(b + o);
-      T d = dinv[row];
+      const int64_t o = row * kp + g.tx * N;
+      Pack<T> bv;
+      const T d = dinv[row];
+#pragma unroll
+      for (int h = 0; h < N; h += 2) {
+        const Pack<double> v = ld(b64 + o + h);
+        st(x64 + o + h, zero64);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          ab[h + e] += v.v[e] * v.v[e];
+          bv.v[h + e] = (T)v.v[e];
+        }
+      }
 #pragma unroll
       for (int e = 0; e < N; ++e) {
         arz[e] += bv.v[e] * (d * bv.v[e]);
@@ -684,21 +713,42 @@ __global__ void k_cg_init(DTiles tl, const T* __restrict__ b, T* x, T* r,
   block_colsum<T, N>(g, arz, sm.red, s.part1 + (int64_t)tile * kp);
   __syncthreads();
   block_colsum<T, N>(g, arr, sm.red, s.part2 + (int64_t)tile * kp);
-  const double* const parts[2] = {s.part1, s.part2};
-  if (!tile_sums<2>(g, parts, s.gpart, s.gcount, s.counter + sd, kp, tile, tl.lo[sd], tl.hi[sd],
+  __syncthreads();
+  double* red64;
+  {
+    extern __shared__ __align__(16) unsigned char raw[];
+    red64 = reinterpret_cast<double*>(raw + align16(smem_bytes<T>(g.nch, g.rb, kp, 0)));
+  }
+  block_colsum<double, N>(g, ab, red64, rs.part + (int64_t)tile * kp);
+  const double* const parts[3] = {rs.part, s.part1, s.part2};
+  if (!tile_sums<3>(g, parts, s.gpart, s.gcount, s.counter + sd, kp, tile, tl.lo[sd], tl.hi[sd],
                     sm.scratch, sm.sums))
     return;
-  __shared__ double bref;
+  __shared__ double bref, bref64;
+  __shared__ int open64;
   if (g.tid == 0) {
-    double m = 0.0;
-    for (int c = 0; c < ncn; ++c) m = fmax(m, sm.sums[kp + c]);
+    double m = 0.0, m64 = 0.0;
+    for (int c = 0; c < ncn; ++c) {
+      m = fmax(m, sm.sums[2 * kp + c]);
+      m64 = fmax(m64, sm.sums[c]);
+    }
     bref = m;
+    bref64 = m64;
+    open64 = 0;
   }
   __syncthreads();
   for (int c = g.tid; c < kp; c += g.nth) {
     int i = sd * kp + c;
-    double bb = sm.sums[kp + c];
-    s.rzf[i] = sm.sums[c];
+    const double rr = sm.sums[c], obb = c < ncn ? bref64 : rr;
+    const bool done = c >= nc || !(obb > 0.0) || rr <= rtol2 * obb || rr <= 0.0;
+    rs.obb[i] = obb;
+    rs.oaa[i] = 0.0;
+    rs.orr[i] = rr;
+    rs.xx[i] = 0.0;
+    rs.scale[i] = done ? 0.0 : 1.0 / sqrt(rr);
+    if (!done) atomicAdd(&open64, 1);
+    const double bb = sm.sums[2 * kp + c];
+    s.rzf[i] = sm.sums[kp + c];
     s.bb[i] = (c < ncn) ? bref : bb;
     s.rr[i] = bb;
     s.done[i] = (c >= nc || !(bb > 0.0)) ? 1 : 0;
@@ -706,8 +756,12 @@ __global__ void k_cg_init(DTiles tl, const T* __restrict__ b, T* x, T* r,
     set_coef(s.beta, s.beta32, i, 0.0);
     set_coef(s.gam, s.gam32, i, 1.0);
   }
-  if (g.tid == 0) s.iters[sd] = 0;
   __syncthreads();
+  if (g.tid == 0) {
+    s.iters[sd] = 0;
+    rs.active[sd] = open64;
+    rs.nfloor[sd] = rs.nnear[sd] = 0;
+  }
   count_active(g, s.done, sd, kp, s.active);
 }
 
@@ -1397,14 +1451,6 @@ __global__ void k_count_active(DTiles tl, const int* active, const int* second, 
   if (threadIdx.x < 3) out[threadIdx.x] = tot[threadIdx.x];
 }
 
-__global__ void k_zero_rows(DTiles tl, double* x, int kp) {
-  Geo g = geo();
-  int tile = blockIdx.x;
-  int r0 = tl.r0[tile], r1 = tl.r1[tile];
-  for (int64_t row = r0 + g.ty; row < r1; row += g.rb)
-    for (int c = g.tx; c < kp; c += g.nch) x[row * kp + c] = 0.0;
-}
-
 // residual replacement: rT = (T) r64 (the true residual), the fine r.z and the
 // restriction of it, each column's done flag from the binary64 convergence test
 // (scale == 0).  Columns the recursion had declared converged but the binary64 test
@@ -1420,12 +1466,15 @@ __global__ void k_cg_replace(DTiles tl, const double* __restrict__ r64, T* __res
   Geo g = geo();
   Smem<T> sm = smem_layout<T>(g, kp, 0);
   int tile = blockIdx.x, sd = tl.sd[tile];
+  // closed in both tests: nothing of this subdomain is read again
+  if (s.active[sd] == 0 && rs.active[sd] == 0) return;
   int r0 = tl.r0[tile], r1 = tl.r1[tile];
   const bool coarse = co.aloc != nullptr;
   const int nrows = r1 - r0;
   TileRestrict<T> tr;
   if (coarse) tr.begin(g, kp, smem_bytes<T>(g.nch, g.rb, kp, 0), r0, nrows, co.aloc);
   const int step = coarse ? tr.SB : nrows;
+  const bool settled = pack_settled<N>(rs, sd, kp, g.tx, 1);
   T arz[N];
 #pragma unroll
   for (int e = 0; e < N; ++e) arz[e] = T(0);
@@ -1434,14 +1483,22 @@ __global__ void k_cg_replace(DTiles tl, const double* __restrict__ r64, T* __res
       const int64_t row = r0 + rr;
       int64_t o = row * kp + g.tx * N;
       Pack<T> rv;
-      T d = dinv[row];
+      if (settled) {
 #pragma unroll
-      for (int e = 0; e < N; ++e) {
-        rv.v[e] = (T)r64[o + e];
-        arz[e] += rv.v[e] * (d * rv.v[e]);
+        for (int e = 0; e < N; ++e) rv.v[e] = T(0);
+      } else {
+        T d = dinv[row];
+#pragma unroll
+        for (int h = 0; h < N; h += 2) {
+          const Pack<double> v = ld(r64 + o + h);
+          rv.v[h] = (T)v.v[0];
+          rv.v[h + 1] = (T)v.v[1];
+        }
+#pragma unroll
+        for (int e = 0; e < N; ++e) arz[e] += rv.v[e] * (d * rv.v[e]);
+        st(rT + o, rv);
       }
       if (coarse) tr.put(rr - s0, kp, g.tx, rv);
-      st(rT + o, rv);
     }
     if (coarse) {
       __syncthreads();
@@ -1471,18 +1528,45 @@ __global__ void k_cg_replace(DTiles tl, const double* __restrict__ r64, T* __res
   count_active(g, s.done, sd, kp, s.active);
 }
 
-// x64 += xT; xT = 0
+// x64 += xT; xT = 0 (settled packs: xT is zero)
 template <typename T>
-__global__ void k_accum_reset(DTiles tl, T* __restrict__ xT, double* __restrict__ x64, int kp) {
+__global__ void __launch_bounds__(256)
+    k_accum_reset(DTiles tl, T* __restrict__ xT, double* __restrict__ x64, int kp, int seen,
+                  RefineState rs) {
+  constexpr int N = Pack<T>::N;
   Geo g = geo();
-  int tile = blockIdx.x;
-  int r0 = tl.r0[tile], r1 = tl.r1[tile];
-  for (int64_t row = r0 + g.ty; row < r1; row += g.rb)
-    for (int c = g.tx; c < kp; c += g.nch) {
-      int64_t o = row * kp + c;
-      x64[o] += (double)xT[o];
-      xT[o] = T(0);
+  const int tile = blockIdx.x, sd = tl.sd[tile];
+  if (seen && rs.active[sd] == 0) return;
+  if (pack_settled<N>(rs, sd, kp, g.tx, seen)) return;
+  Pack<T> zero;
+#pragma unroll
+  for (int e = 0; e < N; ++e) zero.v[e] = T(0);
+  const int r1 = tl.r1[tile];
+  for (int row = tl.r0[tile] + g.ty; row < r1; row += 2 * g.rb) {
+    // both rows' loads before the first store
+    Pack<T> v[2];
+    Pack<double> y[2][N / 2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int64_t o = (int64_t)(row + u * g.rb) * kp + g.tx * N;
+      if (row + u * g.rb >= r1) continue;
+      v[u] = ld(xT + o);
+#pragma unroll
+      for (int h = 0; h < N / 2; ++h) y[u][h] = ld(x64 + o + 2 * h);
     }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int64_t o = (int64_t)(row + u * g.rb) * kp + g.tx * N;
+      if (row + u * g.rb >= r1) continue;
+#pragma unroll
+      for (int h = 0; h < N / 2; ++h) {
+        y[u][h].v[0] += (double)v[u].v[2 * h];
+        y[u][h].v[1] += (double)v[u].v[2 * h + 1];
+        st(x64 + o + 2 * h, y[u][h]);
+      }
+      st(xT + o, zero);
+    }
+  }
 }
 
 // per subdomain: max over its rows of sum_j |a_ij| (nonnegative doubles order like
@@ -1500,16 +1584,6 @@ __global__ void k_row_abs_max(DTiles tl, EllView<double> A, unsigned long long* 
   }
   for (int o = 16; o > 0; o >>= 1) sum = fmax(sum, __shfl_xor_sync(0xFFFFFFFFu, sum, o));
   if ((threadIdx.x & 31) == 0) atomicMax(out + sd, (unsigned long long)__double_as_longlong(sum));
-}
-
-// rT = (T) src
-template <typename T>
-__global__ void k_cast(DTiles tl, const double* __restrict__ src, T* __restrict__ dst, int kp) {
-  Geo g = geo();
-  int tile = blockIdx.x;
-  int r0 = tl.r0[tile], r1 = tl.r1[tile];
-  for (int64_t row = r0 + g.ty; row < r1; row += g.rb)
-    for (int c = g.tx; c < kp; c += g.nch) dst[row * kp + c] = (T)src[row * kp + c];
 }
 
 template <typename T>
@@ -1632,21 +1706,22 @@ void launch_coarse_then_p(const DTiles& tiles, int n_sd, const T* r, T* p, const
 }
 
 template <typename T>
-void launch_cg_init(const DTiles& tiles, const T* b, T* x, T* r, T* p, const T* dinv,
-                    int kp, int nc, int ncn, const CgState& s, const Coarse<T>& co,
-                    cudaStream_t st) {
+void launch_cg_start(const DTiles& tiles, const double* b64, double* x64, T* x, T* r, T* p,
+                     const T* dinv, int kp, int nc, int ncn, double rtol2, const CgState& s,
+                     const RefineState& rs, const Coarse<T>& co, cudaStream_t st) {
   if (tiles.n <= 0) return;
   static bool attr = false;
   if (!attr) {
-    set_smem_attr<T>((const void*)k_cg_init<T>);
+    set_smem_attr<T>((const void*)k_cg_start<T>);
     attr = true;
   }
   dim3 bl = block_of<T>(kp);
+  const size_t sm = align16(start_smem_base<T>(bl.x, bl.y, kp)) + restrict_smem_bytes<T>(bl.y, kp);
   count_launch();
-  k_cg_init<T><<<tiles.n, bl, slot_kernel_smem<T>(bl, kp), st>>>(tiles, b, x, r, dinv, kp, nc,
-                                                                  ncn, s, co);
-  launch_coarse_then_p<T>(tiles, tiles.n_sd, r, p, dinv, kp, 0.0, kCoarseInit,
-                          tiles.n, s, co, st, nullptr);
+  k_cg_start<T><<<tiles.n, bl, sm, st>>>(tiles, b64, x64, x, r, dinv, kp, nc, ncn, rtol2, s, rs,
+                                         co);
+  launch_coarse_then_p<T>(tiles, tiles.n_sd, r, p, dinv, kp, 0.0, kCoarseInit, tiles.n, s, co, st,
+                          nullptr);
 }
 
 // ---- autotuner of the sparse product: four launch configurations of k_cg_spmm_pq
@@ -1759,8 +1834,8 @@ void launch_count_active(const DTiles& tiles, const int* active, int* out, cudaS
 }
 
 void launch_residual64(const DTiles& tiles, const EllView<double>& A, const double* b64,
-                       const double* x64, double* r64, int kp, int nc, int ncn, double rtol2,
-                       int first, bool floor_ref, const double* anorm, const RefineState& s,
+                       const double* x64, double* r64, int kp, int nc, double rtol2, bool seen,
+                       bool floor_ref, const double* anorm, const RefineState& s,
                        cudaStream_t st) {
   if (tiles.n <= 0) return;
   static bool attr = false;
@@ -1772,12 +1847,8 @@ void launch_residual64(const DTiles& tiles, const EllView<double>& A, const doub
   dim3 bl = block_of<double>(kp);
   size_t sm = smem_bytes<double>(bl.x, bl.y, kp, A.W);
   count_launch();
-  if (floor_ref && !first)
-    k_residual64<true><<<tiles.n, bl, sm, st>>>(tiles, A, b64, x64, r64, kp, nc, ncn, rtol2,
-                                                first, s, anorm);
-  else
-    k_residual64<false><<<tiles.n, bl, sm, st>>>(tiles, A, b64, x64, r64, kp, nc, ncn, rtol2,
-                                                 first, s, anorm);
+  auto fn = floor_ref ? k_residual64<true> : k_residual64<false>;
+  fn<<<tiles.n, bl, sm, st>>>(tiles, A, b64, x64, r64, kp, nc, rtol2, seen ? 1 : 0, s, anorm);
 }
 
 template <typename T>
@@ -1799,10 +1870,11 @@ void launch_cg_replace(const DTiles& tiles, const double* r64, T* rT, T* pT, con
 }
 
 template <typename T>
-void launch_accum_reset(const DTiles& tiles, T* xT, double* x64, int kp, cudaStream_t st) {
+void launch_accum_reset(const DTiles& tiles, T* xT, double* x64, int kp, bool seen,
+                        const RefineState& rs, cudaStream_t st) {
   if (tiles.n <= 0) return;
   count_launch();
-  k_accum_reset<T><<<tiles.n, dim3(32, 8), 0, st>>>(tiles, xT, x64, kp);
+  k_accum_reset<T><<<tiles.n, block_of<T>(kp), 0, st>>>(tiles, xT, x64, kp, seen ? 1 : 0, rs);
 }
 
 // out[sd] += stored entries of the rows of each tile of sd (one thread per row)
@@ -1832,13 +1904,6 @@ void launch_row_abs_max(const DTiles& tiles, const EllView<double>& A, double* o
   k_row_abs_max<<<tiles.n, kTileRows, 0, st>>>(tiles, A, (unsigned long long*)out);
 }
 
-template <typename T>
-void launch_cast(const DTiles& tiles, const double* src, T* dst, int kp, cudaStream_t st) {
-  if (tiles.n <= 0) return;
-  count_launch();
-  k_cast<T><<<tiles.n, dim3(32, 8), 0, st>>>(tiles, src, dst, kp);
-}
-
 template void launch_cg_replace<float>(const DTiles&, const double*, float*, float*,
                                        const float*, int, double, const CgState&,
                                        const RefineState&, const Coarse<float>&, cudaStream_t);
@@ -1846,27 +1911,22 @@ template void launch_cg_replace<double>(const DTiles&, const double*, double*, d
                                         const double*, int, double, const CgState&,
                                         const RefineState&, const Coarse<double>&,
                                         cudaStream_t);
-template void launch_accum_reset<float>(const DTiles&, float*, double*, int, cudaStream_t);
-template void launch_accum_reset<double>(const DTiles&, double*, double*, int, cudaStream_t);
-template void launch_cast<float>(const DTiles&, const double*, float*, int, cudaStream_t);
-template void launch_cast<double>(const DTiles&, const double*, double*, int, cudaStream_t);
-
-void launch_zero_rows(const DTiles& tiles, double* x, int kp, cudaStream_t st) {
-  if (tiles.n <= 0) return;
-  count_launch();
-  k_zero_rows<<<tiles.n, dim3(32, 8), 0, st>>>(tiles, x, kp);
-}
-
+template void launch_accum_reset<float>(const DTiles&, float*, double*, int, bool,
+                                        const RefineState&, cudaStream_t);
+template void launch_accum_reset<double>(const DTiles&, double*, double*, int, bool,
+                                         const RefineState&, cudaStream_t);
 template void launch_spmm<float>(const DTiles&, const EllView<float>&, const float*, float*,
                                  int, cudaStream_t);
 template void launch_spmm<double>(const DTiles&, const EllView<double>&, const double*,
                                   double*, int, cudaStream_t);
-template void launch_cg_init<float>(const DTiles&, const float*, float*, float*, float*,
-                                    const float*, int, int, int, const CgState&,
-                                    const Coarse<float>&, cudaStream_t);
-template void launch_cg_init<double>(const DTiles&, const double*, double*, double*, double*,
-                                     const double*, int, int, int, const CgState&,
-                                     const Coarse<double>&, cudaStream_t);
+template void launch_cg_start<float>(const DTiles&, const double*, double*, float*, float*,
+                                     float*, const float*, int, int, int, double,
+                                     const CgState&, const RefineState&, const Coarse<float>&,
+                                     cudaStream_t);
+template void launch_cg_start<double>(const DTiles&, const double*, double*, double*, double*,
+                                      double*, const double*, int, int, int, double,
+                                      const CgState&, const RefineState&, const Coarse<double>&,
+                                      cudaStream_t);
 template void launch_cg_step<float>(const DTiles&, const EllView<float>&, float*, float*,
                                     float*, float*, const float*, int, double, int,
                                     const CgState&, const Coarse<float>&, cudaStream_t,
