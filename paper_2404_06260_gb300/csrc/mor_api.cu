@@ -562,10 +562,11 @@ struct Build {
   }
 
   // sum of active[] over the subdomains (of second[] into h_poll[1], the row tiles of the
-  // subdomains with active > 0 into h_poll[2])
+  // subdomains with active > 0 into h_poll[2], the steps of the last resident launch into
+  // h_poll[3])
   int poll(const DTiles& tl, const int* active, const int* second = nullptr) {
     launch_count_active(tl, active, d_poll, st, second);
-    CK(cudaMemcpyAsync(h_poll, d_poll, 3 * sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemcpyAsync(h_poll, d_poll, 4 * sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     return h_poll[0];
   }
@@ -575,6 +576,7 @@ struct Build {
   int32_t* sd_rows[2] = {nullptr, nullptr};
   int64_t* sd_nnz[2] = {nullptr, nullptr};
 
+  int n_rows[2] = {0, 0};  // per matrix set: rows of the largest subdomain
   // coarse levels of the two-level preconditioner: [0] A_II (I tiles), [1] H^+ (all P
   // tiles)
   Coarse<float> co32[2];
@@ -619,8 +621,20 @@ struct Build {
     const int check = 8;
     const int every = std::max(check, o->replace_every / check * check);
     int it = 0, open_tiles = tl.n;
+    // the kernel times of the roofline are those of the streaming kernels
+    const ResidentPlan rp =
+        g_prof.on ? ResidentPlan() : resident_plan<T>(n_sd, n_rows[set], AT.W, co.n_max, kp);
     while (true) {
-      int chunk = std::min(check, o->max_iter - it);
+      int act = 0;
+      if (rp.S > 0) {
+        // the steps up to the next replacement in one launch (the tuner keeps to its
+        // contract: every shape the process meets has an entry)
+        if (it == 0) tune_spmm<T>(tl, AT, p, q, kp, cs, st);
+        CK(cudaMemsetAsync(d_poll + 3, 0, sizeof(int), st));
+        launch_cg_resident<T>(rp, tl, AT, x, r, p, dinvT, kp, rtol2,
+                              std::min(every, o->max_iter - it), cs, co, d_poll + 3, st);
+      }
+      int chunk = rp.S > 0 ? 0 : std::min(check, o->max_iter - it);
       for (int c = 0; c < chunk; ++c) {
         const cudaEvent_t* ev = nullptr;
         if (g_prof.on) {
@@ -632,9 +646,11 @@ struct Build {
         launch_cg_step<T>(tl, AT, x, r, p, q, dinvT, kp, rtol2, open_tiles, cs, co, st, ev);
       }
       it += chunk;
-      int act = poll(tl, cs.active);
-      open_tiles = h_poll[2];
-      if (act == 0 || it % every == 0 || it >= o->max_iter) {
+      if (rp.S == 0) {
+        act = poll(tl, cs.active);
+        open_tiles = h_poll[2];
+      }
+      if (rp.S > 0 || act == 0 || it % every == 0 || it >= o->max_iter) {
         launch_accum_reset<T>(tl, x, x64, kp, seen, rs, st);
         launch_residual64(tl, A.e64(), b64, x64, vR64, kp, nc, rtol2, seen, false, anorm[set],
                           rs, st);
@@ -642,6 +658,8 @@ struct Build {
         ++sweeps;
         int ract = poll(tl, rs.active, rs.nnear);
         int rs_tiles = h_poll[2];
+        // (no step at all: every column of the recursion is closed, count the interval)
+        if (rp.S > 0) it += h_poll[3] > 0 ? h_poll[3] : every;
         if (ract > 0 && h_poll[1] > 0) {
           // some open column is within reach of the rounding level: measure the exact
           // reference || |A| |x| + |b| || and test again
@@ -860,8 +878,8 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
   const int64_t nEllW = ceil_div(nW, 32) * 32 * WW;
   const int64_t nEllO = ceil_div(nO, 32) * 32 * WW;
 
-  CK(cudaMallocHost((void**)&B.h_poll, 3 * sizeof(int)));
-  TRY(M.alloc(&B.d_poll, 3, true, st));
+  CK(cudaMallocHost((void**)&B.h_poll, 4 * sizeof(int)));
+  TRY(M.alloc(&B.d_poll, 4, true, st));
   int* d_err;
   TRY(M.alloc(&d_err, 1, true, st));
 
@@ -1060,6 +1078,11 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
   // ---- paper-literal weights: dense H^+ factor, R_BB (Lemma 4.1) ----
   DenseWeights DW;
   if (dense) TRY(dense_weights(hp, S.p_sd, M, Hp.e64(), DW, st));
+
+  for (int i = 0; i < n_sd; ++i) {
+    B.n_rows[0] = std::max(B.n_rows[0], hp.nI[i]);
+    B.n_rows[1] = std::max(B.n_rows[1], hp.nI[i] + hp.nB[i]);
+  }
 
   // ---- solver workspace ----
   size_t tsz = B.mixed ? sizeof(float) : sizeof(double);

@@ -161,6 +161,25 @@ template <typename T>
 void launch_cg_step(const DTiles& tiles, const EllView<T>& A, T* x, T* r, T* p, T* q,
                     const T* dinv, int kp, double tol2, int open_tiles, const CgState& s,
                     const Coarse<T>& co, cudaStream_t st, const cudaEvent_t* ev = nullptr);
+// the autotuner's choice for a product it has not met (its first meeting with a precision,
+// column count and slot width, on data that the next step forms anew: q, the step length)
+template <typename T>
+void tune_spmm(const DTiles& tiles, const EllView<T>& A, const T* p, T* q, int kp,
+               const CgState& s, cudaStream_t st);
+// Small subdomains: up to `steps` CG steps in one launch with the data on chip
+// (mor_resident.cu).  resident_plan: S = 0 where the largest subdomain (n_max rows, nc_max
+// aggregates, slot stride W) does not fit.  Zeroes s.active and fills it with the open
+// columns; steps_run takes the largest number of steps (zeroed by the caller).
+struct ResidentPlan {
+  int S = 0;
+  size_t smem = 0;
+};
+template <typename T>
+ResidentPlan resident_plan(int n_sd, int n_max, int W, int nc_max, int kp);
+template <typename T>
+void launch_cg_resident(const ResidentPlan& rp, const DTiles& tiles, const EllView<T>& A, T* x,
+                        const T* r, T* p, const T* dinv, int kp, double tol2, int steps,
+                        const CgState& s, const Coarse<T>& co, int* steps_run, cudaStream_t st);
 // out[0] = sum of active[0..n_sd), out[1] = sum of second (0 if null), out[2] = row tiles of
 // the subdomains with active > 0
 void launch_count_active(const DTiles& tiles, const int* active, int* out, cudaStream_t st,

@@ -1793,6 +1793,16 @@ int spmm_variant(const DTiles& tiles, const EllView<T>& A, const T* p, T* q, int
 }
 
 template <typename T>
+void tune_spmm(const DTiles& tiles, const EllView<T>& A, const T* p, T* q, int kp,
+               const CgState& s, cudaStream_t st) {
+  if (tiles.n > 0) spmm_variant<T>(tiles, A, p, q, kp, s, st);
+}
+template void tune_spmm<float>(const DTiles&, const EllView<float>&, const float*, float*, int,
+                               const CgState&, cudaStream_t);
+template void tune_spmm<double>(const DTiles&, const EllView<double>&, const double*, double*,
+                                int, const CgState&, cudaStream_t);
+
+template <typename T>
 void launch_cg_step(const DTiles& tiles, const EllView<T>& A, T* x, T* r, T* p, T* q,
                     const T* dinv, int kp, double tol2, int open_tiles, const CgState& s,
                     const Coarse<T>& co, cudaStream_t st, const cudaEvent_t* ev) {
