@@ -891,12 +891,15 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
   TRY(M.alloc(&valA_W, nEllW, true, st));
   TRY(M.alloc(&valH_W, nEllW, true, st));
   TRY(M.alloc(&loadW, nW, true, st));
-  launch_assemble(nP, S.incP_ptr, S.incP_tet, S.incP_code, WP, S.xyz, S.tets, S.kappa,
-                  o.h1_weighted, valA_P,
-                  valH_P, loadP, d_err, st);
-  launch_assemble(nW, S.incW_ptr, S.incW_tet, S.incW_code, WW, S.xyz, S.tets, S.kappa,
-                  o.h1_weighted, valA_W,
-                  valH_W, loadW, d_err, st);
+  // per element: its stiffness for the assembly, then the factor of its H1 matrix for the
+  // sketch in the same place
+  double* elem;
+  TRY(M.alloc(&elem, (size_t)hp.n_tets * kElemDoubles, false, st));
+  launch_elem_stiff(hp.n_tets, S.xyz, S.tets, elem, st);
+  launch_assemble(nP, S.incP_ptr, S.incP_tet, S.incP_code, WP, elem, S.kappa, o.h1_weighted,
+                  valA_P, valH_P, loadP, d_err, st);
+  launch_assemble(nW, S.incW_ptr, S.incW_tet, S.incW_code, WW, elem, S.kappa, o.h1_weighted,
+                  valA_W, valH_W, loadW, d_err, st);
 
   // ---- extraction of the blocks used by the solves ----
   auto make_mat = [&](Mat& mt, int64_t n_rows, int W, bool f32) -> int {
@@ -1240,8 +1243,7 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
   const double rt_sketch = o.sketch_rtol > 0.0 ? o.sketch_rtol : o.cg_rtol;
 
   // ---- sketch: W = ((H^+)^{-1} L xi)_B ----
-  float2* lsplit;
-  TRY(M.alloc(&lsplit, (size_t)hp.n_tets * 10, false, st));
+  float2* lsplit = reinterpret_cast<float2*>(elem);
   launch_elem_chol(hp.n_tets, S.xyz, S.tets, S.kappa, o.h1_weighted, lsplit, st);
   int32_t *d_ksd, *d_msd, *d_msel;
   TRY(M.upload(&d_ksd, h_k, st));

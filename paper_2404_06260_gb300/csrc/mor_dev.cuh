@@ -146,13 +146,23 @@ __device__ __forceinline__ void box_muller(uint32_t x1, uint32_t x2, float& z0, 
 }
 
 // four standard normals xi_T[0..3] for (element T, column j, subdomain i): counter
-// (T, j, i, 0), key = seed
+// (T, j, i, 0), key = seed; z[2] and z[3] only where `last` asks for them (the normals
+// past z[last] stay unset)
 __device__ __forceinline__ void field_normals(uint32_t T, uint32_t j, uint32_t i,
-                                              uint64_t seed, float z[4]) {
+                                              uint64_t seed, float z[4], int last) {
   uint32_t c[4] = {T, j, i, 0u};
   philox4x32_10(c, (uint32_t)(seed & 0xFFFFFFFFull), (uint32_t)(seed >> 32));
   box_muller(c[0], c[1], z[0], z[1]);
-  box_muller(c[2], c[3], z[2], z[3]);
+  if (last >= 2) box_muller(c[2], c[3], z[2], z[3]);
+}
+
+__device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
+
+// x != 0 by its bits: a binary64 compare costs as much as a multiply-add
+__device__ __forceinline__ bool nonzero(float x) { return x != 0.0f; }
+__device__ __forceinline__ bool nonzero(double x) {
+  return (__double2loint(x) | (__double2hiint(x) << 1)) != 0;
 }
 
 // Bounded wait of one thread until *gen differs from `seen` (any flag that another block

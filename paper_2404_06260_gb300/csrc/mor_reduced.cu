@@ -12,54 +12,101 @@
 namespace mor {
 namespace {
 
-constexpr int kPairThreads = 512;
-constexpr int kPairPerThread = 32;  // 512 * 32 >= 128 * 128
-constexpr int kPairChunk = 32;
-
+// K~_ij = sum over the entries (u, v) of pair (i, j) of a_uv Q[u]^T Q[v].  The entries come
+// sorted by u, so a row of Q_i meets the few rows of Q_j it is coupled with first: w_u =
+// sum_v a_uv Q[v], then K~_ij = sum_u Q[u]^T w_u.  Bound by binary64 issue; that takes
+// kq + kq^2 / (entries per u, three to four) multiply-adds per entry where the plain sum
+// took 2 kq^2 operations.  A block takes `rows` of the kq rows of one pair's block: enough
+// blocks for every SM where the pairs are few.  56^3 in 343 subdomains (28 columns) 700 -> 141
+// us, 48^3 in 40 (68 columns) 6.2 -> 0.39 ms, 16^3 in 8 (12 columns) 39 -> 11 us.
+constexpr int kPairThreads = 256;
+constexpr int kPairOut = 16;      // outputs per thread: rows * kq <= 256 * 16
+constexpr int kPairEntries = 128;  // entries per chunk
+constexpr int kPairGroups = 32;    // rows u per pass
 __global__ void __launch_bounds__(kPairThreads)
     k_pair_blocks(const int64_t* __restrict__ pair_ptr, const int32_t* __restrict__ urow,
                   const int32_t* __restrict__ vrow, const double* __restrict__ aval,
-                  const double* __restrict__ Q, int kq, double* blocks) {
+                  const double* __restrict__ Q, int kq, int rows, double* blocks) {
   extern __shared__ double sh[];
-  double* Qu = sh;
-  double* Qv = Qu + kPairChunk * kq;
-  double* av = Qv + kPairChunk * kq;
-  int p = blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
-  int64_t e0 = pair_ptr[p], e1 = pair_ptr[p + 1];
-  int nout = kq * kq;
-  double acc[kPairPerThread];
+  double* Wv = sh;                      // [kPairGroups][kq]
+  double* Qu = Wv + kPairGroups * kq;   // [kPairGroups][rows]
+  __shared__ double av[kPairEntries];
+  __shared__ int32_t vr[kPairEntries], gu[kPairEntries];
+  __shared__ int gs[kPairEntries + 1], wcnt[kPairEntries / 32];
+  const int p = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const int i0 = blockIdx.y * rows, ni = min(rows, kq - i0);
+  const int64_t e0 = pair_ptr[p], e1 = pair_ptr[p + 1];
+  const int nout = ni * kq;
+  double acc[kPairOut];
 #pragma unroll
-  for (int m = 0; m < kPairPerThread; ++m) acc[m] = 0.0;
-  for (int64_t base = e0; base < e1; base += kPairChunk) {
-    int ne = (int)min((int64_t)kPairChunk, e1 - base);
-    for (int idx = tid; idx < ne * kq; idx += nth) {
-      int ee = idx / kq, c = idx % kq;
-      Qu[ee * kq + c] = Q[(int64_t)urow[base + ee] * kq + c];
-      Qv[ee * kq + c] = Q[(int64_t)vrow[base + ee] * kq + c];
+  for (int m = 0; m < kPairOut; ++m) acc[m] = 0.0;
+  for (int64_t base = e0; base < e1; base += kPairEntries) {
+    const int ne = (int)min((int64_t)kPairEntries, e1 - base);
+    // rows u of the chunk: gu[g], entries gs[g] to gs[g + 1]
+    bool head = false;
+    int32_t u = 0;
+    if (tid < ne) {
+      u = urow[base + tid];
+      head = tid == 0 || urow[base + tid - 1] != u;
+      vr[tid] = vrow[base + tid];
+      av[tid] = aval[base + tid];
     }
-    for (int ee = tid; ee < ne; ee += nth) av[ee] = aval[base + ee];
+    const unsigned hb = __ballot_sync(0xFFFFFFFFu, head);
+    if (lane == 0 && wp < kPairEntries / 32) wcnt[wp] = __popc(hb);
     __syncthreads();
+    int ng = 0, before = 0;
 #pragma unroll
-    for (int m = 0; m < kPairPerThread; ++m) {
-      int o = tid + m * nth;
-      if (o < nout) {
-        int i = o / kq, j = o % kq;
-        double s = 0.0;
-        for (int ee = 0; ee < ne; ++ee) s += av[ee] * Qu[ee * kq + i] * Qv[ee * kq + j];
-        acc[m] += s;
+    for (int w = 0; w < kPairEntries / 32; ++w) {
+      if (w < wp) before += wcnt[w];
+      ng += wcnt[w];
+    }
+    if (head) {
+      const int g = before + __popc(hb & ((1u << lane) - 1u));
+      gu[g] = u;
+      gs[g] = tid;
+    }
+    if (tid == 0) gs[ng] = ne;
+    __syncthreads();
+    for (int g0 = 0; g0 < ng; g0 += kPairGroups) {
+      const int nb = min(kPairGroups, ng - g0);
+      for (int idx = tid; idx < nb * kq; idx += kPairThreads) {
+        const int g = idx / kq, j = idx - g * kq;
+        double w = 0.0;
+        for (int e = gs[g0 + g]; e < gs[g0 + g + 1]; ++e) w += av[e] * Q[(int64_t)vr[e] * kq + j];
+        Wv[idx] = w;
       }
-    }
-    __syncthreads();
-  }
-  double* Bij = blocks + (int64_t)(2 * p) * nout;
-  double* Bji = blocks + (int64_t)(2 * p + 1) * nout;
+      for (int idx = tid; idx < nb * ni; idx += kPairThreads) {
+        const int g = idx / ni, i = idx - g * ni;
+        Qu[idx] = Q[(int64_t)gu[g0 + g] * kq + i0 + i];
+      }
+      __syncthreads();
 #pragma unroll
-  for (int m = 0; m < kPairPerThread; ++m) {
-    int o = tid + m * nth;
+      for (int m = 0; m < kPairOut; ++m) {
+        const int o = tid + m * kPairThreads;
+        if (o < nout) {
+          const int i = o / kq, j = o - i * kq;
+          double s0 = 0.0, s1 = 0.0;
+          int g = 0;
+          for (; g + 1 < nb; g += 2) {
+            s0 += Qu[g * ni + i] * Wv[g * kq + j];
+            s1 += Qu[(g + 1) * ni + i] * Wv[(g + 1) * kq + j];
+          }
+          if (g < nb) s0 += Qu[g * ni + i] * Wv[g * kq + j];
+          acc[m] += s0 + s1;
+        }
+      }
+      __syncthreads();
+    }
+  }
+  double* Bij = blocks + (int64_t)(2 * p) * kq * kq;
+  double* Bji = blocks + (int64_t)(2 * p + 1) * kq * kq;
+#pragma unroll
+  for (int m = 0; m < kPairOut; ++m) {
+    const int o = tid + m * kPairThreads;
     if (o < nout) {
-      int i = o / kq, j = o % kq;
-      Bij[i * kq + j] = acc[m];
-      Bji[j * kq + i] = acc[m];
+      const int i = o / kq, j = o - i * kq;
+      Bij[(i0 + i) * kq + j] = acc[m];
+      Bji[j * kq + i0 + i] = acc[m];
     }
   }
 }
@@ -657,15 +704,15 @@ void launch_pair_blocks(int n_pairs, const int64_t* pair_ptr, const int32_t* uro
                         const int32_t* vrow, const double* aval, const double* Q, int kq,
                         double* blocks, cudaStream_t st) {
   if (n_pairs <= 0) return;
-  size_t sm = sizeof(double) * (2 * (size_t)kPairChunk * kq + kPairChunk);
-  static bool attr = false;
-  if (!attr) {  // kq up to 128: 66 KB
-    cudaFuncSetAttribute(k_pair_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         100 * 1024);
-    attr = true;
-  }
+  // rows per block: what the accumulators hold, fewer while the blocks do not fill the SMs
+  // four times over, eight at least (each slice repeats the w_u, three multiply-adds per entry and
+  // column: with four rows a slice spends nearly half its time on them)
+  int rows = std::min(kq, kPairThreads * kPairOut / kq);
+  while (rows > 8 && (int64_t)n_pairs * ((kq + rows - 1) / rows) < 4 * 152) rows = (rows + 1) / 2;
+  const size_t sm = sizeof(double) * (size_t)kPairGroups * (kq + rows);  // kq <= 128: 40 KB
   count_launch();
-  k_pair_blocks<<<n_pairs, kPairThreads, sm, st>>>(pair_ptr, urow, vrow, aval, Q, kq, blocks);
+  k_pair_blocks<<<dim3(n_pairs, (kq + rows - 1) / rows), kPairThreads, sm, st>>>(
+      pair_ptr, urow, vrow, aval, Q, kq, rows, blocks);
 }
 
 void launch_rcg_init(int n_sd, int kq, const double* bt, const RcgState& s,
