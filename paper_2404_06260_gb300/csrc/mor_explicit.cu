@@ -4,12 +4,12 @@
 //
 //   - k_ell_to_dense: scatter a sliced-ELL block into a dense per-subdomain matrix
 //     (row-major, leading dimension = its order) with caller-given local indices;
-//   - k_potrf_diag / k_potrf_update: right-looking blocked Cholesky A = L L^T in place,
+//   - k_potrf_diag / _panel / _update: right-looking blocked Cholesky A = L L^T in place,
 //     64-column panels, batched over subdomains of different orders (Golub & Van Loan
 //     Alg. 4.2.2 by blocks);
 //   - k_transpose_block: copy of a square block, transposed (the triangular solves
 //     walk columns of a factor as contiguous rows of its transpose);
-//   - k_trsv_cols: one vector per block: forward (L x = b) or backward (U x = b)
+//   - k_trsv_cols: two vectors per warp: forward (L x = b) or backward (U x = b)
 //     substitution, column-oriented;
 //   - k_trsv_rows: one row per warp: x R = y with R upper (row-major), for
 //     X = Y R_BB^{-1};
@@ -56,51 +56,130 @@ __global__ void k_ell_to_dense(int64_t n_rows, const int32_t* __restrict__ row_s
   }
 }
 
-// diagonal block j0 of every subdomain's matrix (order n[sd]) factored in shared
-// memory, then the panel below it solved against it: rows i >= j0 + nb satisfy
-// L[i, j0:j0+nb] L_dd^T = A[i, j0:j0+nb].  A non-positive pivot sets *bad.
+// b / d from r = 1 / d rounded: the quotient b r with one correction step, faithful to the
+// last bit; the reciprocal of a pivot is formed once for all the entries it divides
+__device__ __forceinline__ double div_by(double b, double d, double r) {
+  const double q = b * r;
+  return fma(fma(-d, q, b), r, q);
+}
+
+// Diagonal block j0 of every subdomain's matrix (order n[sd]), nb columns: factored as
+// L D L^T in registers (lower triangle, one multiply-add per entry and column), the square
+// roots of the pivots at the end, in parallel.  A non-positive pivot sets *bad.  A chain of
+// nb steps: a square root in front of every division and the update's index arithmetic
+// made a step 4,500 clocks.  8 blocks of 64: 46 us, with the panel below 81 instead of 300.
+constexpr int kPotrfOwn = (kNB * (kNB + 1) / 2 + 255) / 256;  // entries per thread
 __global__ void __launch_bounds__(256)
     k_potrf_diag(double* D, const int64_t* __restrict__ doff, const int32_t* __restrict__ nn,
                  int j0, int* bad) {
-  __shared__ double a[kNB][kNB + 1];
+  __shared__ double col[2][kNB], colp[kNB];  // column c, and column c / a_cc
+  __shared__ double rs[kNB];                 // 1 / sqrt of the pivots
   const int sd = blockIdx.x, n = nn[sd];
   if (j0 >= n) return;
   const int nb = min(kNB, n - j0);
-  double* A = D + doff[sd];
-  const int tid = threadIdx.x, nth = blockDim.x;
-  for (int idx = tid; idx < nb * nb; idx += nth) {
-    const int r = idx / nb, c = idx % nb;
-    a[r][c] = (c <= r) ? A[(int64_t)(j0 + r) * n + j0 + c] : 0.0;
+  double* A = D + doff[sd] + (int64_t)j0 * n + j0;
+  const int tid = threadIdx.x;
+  double a[kPotrfOwn];
+  int ri[kPotrfOwn], ci[kPotrfOwn];  // entry (ri, ci), ci <= ri; ci = -1: none
+#pragma unroll
+  for (int m = 0; m < kPotrfOwn; ++m) {
+    const int idx = tid + m * 256;
+    a[m] = 0.0;
+    ri[m] = ci[m] = -1;
+    if (idx < nb * (nb + 1) / 2) {
+      // columns from the last to the first: the entries of the columns still to come are
+      // the first ones, and whole warps run out of work as the factorisation proceeds
+      int c = (int)((sqrtf(8.0f * (float)idx + 1.0f) - 1.0f) * 0.5f);
+      while ((c + 1) * (c + 2) / 2 <= idx) ++c;
+      while (c * (c + 1) / 2 > idx) --c;
+      ci[m] = nb - 1 - c;
+      ri[m] = ci[m] + idx - c * (c + 1) / 2;
+      a[m] = A[(int64_t)ri[m] * n + ci[m]];
+      if (ci[m] == 0) col[0][ri[m]] = a[m];
+    }
+  }
+  for (int c = 0; c < nb; ++c) {
+    __syncthreads();
+    const double* cc = col[c & 1];
+    double* cn = col[(c + 1) & 1];
+    if (tid >= c && tid < nb) {
+      double d = cc[c];
+      if (!(d > 0.0)) {
+        if (tid == c) atomicExch(bad, 1);
+        d = 1.0;
+      }
+      const double r = 1.0 / d;
+      colp[tid] = div_by(cc[tid], d, r);
+      if (tid == c) rs[c] = d;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < kPotrfOwn; ++m)
+      if (ci[m] > c) {
+        a[m] -= cc[ri[m]] * colp[ci[m]];
+        if (ci[m] == c + 1) cn[ri[m]] = a[m];
+      }
   }
   __syncthreads();
-  for (int c = 0; c < nb; ++c) {
-    const double d2 = a[c][c];
-    const double d = d2 > 0.0 ? sqrt(d2) : 1.0;
-    if (!(d2 > 0.0) && tid == 0) atomicExch(bad, 1);
-    __syncthreads();
-    for (int r = c + 1 + tid; r < nb; r += nth) a[r][c] /= d;
-    if (tid == 0) a[c][c] = d;
-    __syncthreads();
-    const int m = nb - c - 1;
-    for (int idx = tid; idx < m * m; idx += nth) {
-      const int r = c + 1 + idx / m, s = c + 1 + idx % m;
-      if (s <= r) a[r][s] -= a[r][c] * a[s][c];
+  // rs holds the pivots d; L_rc = a_rc / sqrt(d_c)
+  if (tid < nb) {
+    const double l = sqrt(rs[tid]);
+    colp[tid] = l;
+    rs[tid] = 1.0 / l;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int m = 0; m < kPotrfOwn; ++m)
+    if (ci[m] >= 0) {
+      const int r = ri[m], c = ci[m];
+      A[(int64_t)r * n + c] = r == c ? colp[c] : div_by(a[m], colp[c], rs[c]);
+      if (r != c) A[(int64_t)c * n + r] = 0.0;
     }
-    __syncthreads();
+}
+
+// The panel below diagonal block j0: rows i >= j0 + nb satisfy L[i, j0:j0+nb] L_dd^T =
+// A[i, j0:j0+nb].  32 rows per block, four lanes per row, each with every fourth column in
+// registers: x_c comes by shuffle and its multiply-adds on the columns behind it are
+// independent.  grid (n_sd, row chunks).  One thread per row and one block per subdomain
+// cost most of 300 us a panel; 35 now (8 subdomains of order up to 340).
+constexpr int kPanelRows = 32;
+__global__ void __launch_bounds__(4 * kPanelRows)
+    k_potrf_panel(double* D, const int64_t* __restrict__ doff, const int32_t* __restrict__ nn,
+                  int j0) {
+  __shared__ double Lt[kNB][kNB + 4];  // Lt[c][s] = L_dd[s][c]
+  __shared__ double rc[kNB];
+  const int sd = blockIdx.x, n = nn[sd];
+  const int i0 = j0 + kNB + blockIdx.y * kPanelRows;
+  if (i0 >= n) return;  // rows below: the block has kNB columns
+  double* A = D + doff[sd];
+  const int tid = threadIdx.x, h = tid & 3;
+  for (int idx = tid; idx < kNB * kNB; idx += 4 * kPanelRows) {
+    const int s = idx / kNB, c = idx % kNB;
+    Lt[c][s] = A[(int64_t)(j0 + s) * n + j0 + c];
   }
-  for (int idx = tid; idx < nb * nb; idx += nth) {
-    const int r = idx / nb, c = idx % nb;
-    A[(int64_t)(j0 + r) * n + j0 + c] = (c <= r) ? a[r][c] : 0.0;
-  }
-  // panel: forward substitution of each row against L_dd^T
-  for (int i = j0 + nb + tid; i < n; i += nth) {
-    double* row = A + (int64_t)i * n + j0;
-    for (int c = 0; c < nb; ++c) {
-      double s = row[c];
-      for (int q = 0; q < c; ++q) s -= row[q] * a[c][q];
-      row[c] = s / a[c][c];
+  __syncthreads();
+  if (tid < kNB) rc[tid] = 1.0 / Lt[tid][tid];
+  const int i = i0 + (tid >> 2);
+  double* row = A + (int64_t)min(i, n - 1) * n + j0;
+  double x[kNB / 4];
+#pragma unroll
+  for (int q = 0; q < kNB / 4; ++q) x[q] = i < n ? row[4 * q + h] : 0.0;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < kNB / 4; ++q)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int c = 4 * q + e;
+      double v = div_by(x[q], Lt[c][c], rc[c]);
+      v = __shfl_sync(0xFFFFFFFFu, v, e, 4);
+      if (h == e) x[q] = v;
+      if (h > e) x[q] = fma(-v, Lt[c][4 * q + h], x[q]);
+#pragma unroll
+      for (int p = q + 1; p < kNB / 4; ++p) x[p] = fma(-v, Lt[c][4 * p + h], x[p]);
     }
-  }
+  if (i < n)
+#pragma unroll
+    for (int q = 0; q < kNB / 4; ++q) row[4 * q + h] = x[q];
 }
 
 // trailing update of panel j0: A[I, J] -= P_I P_J^T for the 64 x 64 tiles I >= J of the
@@ -179,38 +258,62 @@ __global__ void k_transpose_block(const double* __restrict__ In, const int64_t* 
   }
 }
 
-// one vector per block: x = F^{-1} b with F triangular of order n[sd], given through T
-// whose row j is column j of F (contiguous).  forward (F lower): x_j = b_j / F_jj, then
-// b_l -= F_lj x_j for l > j; backward (F upper): the same for l < j from the last row.
-// The vector is column `col` of rows [roff[sd], roff[sd] + n) of X (leading dimension
-// ldx), solved in place.  grid (n_sd, columns).
-__global__ void __launch_bounds__(256)
+// Two vectors per warp: x = F^{-1} b with F triangular of order n[sd], given through T whose
+// row j is column j of F (contiguous).  forward (F lower): x_j = b_j / F_jj, then b_l -=
+// F_lj x_j for l > j; backward (F upper): the same for l < j from the last row.  The vectors
+// are columns `col` of rows [roff[sd], roff[sd] + n) of X (leading dimension ldx), solved in
+// place, staged in shared memory beside the reciprocals of the diagonal.  Bound by binary64
+// issue: with one vector per block its eight warps each repeated the division of every step,
+// 8 of its 9 operations: 1.14 -> 0.25 ms a solve (8 subdomains of order about 250, 100
+// to 160 vectors each).  grid (n_sd, columns / (2 warps)).
+__global__ void __launch_bounds__(128)
     k_trsv_cols(const double* __restrict__ Tm, const int64_t* __restrict__ toff,
                 const int32_t* __restrict__ nn, const int32_t* __restrict__ tld,
                 const int32_t* __restrict__ tsh, double* X, const int64_t* __restrict__ roff,
-                int ldx, const int32_t* __restrict__ ncol, int forward) {
-  extern __shared__ double b[];
-  const int sd = blockIdx.x, col = blockIdx.y;
-  if (col >= ncol[sd]) return;
-  const int n = nn[sd], ld = tld[sd], sh = tsh[sd];
-  const double* T = Tm + toff[sd] + (int64_t)sh * ld + sh;
-  double* x = X + roff[sd] * ldx + col;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) b[i] = x[(int64_t)i * ldx];
-  __syncthreads();
-  for (int s = 0; s < n; ++s) {
-    const int j = forward ? s : n - 1 - s;
-    const double* tj = T + (int64_t)j * ld;
-    const double xj = b[j] / tj[j];
-    if (forward) {
-      for (int l = j + 1 + threadIdx.x; l < n; l += blockDim.x) b[l] -= tj[l] * xj;
-    } else {
-      for (int l = threadIdx.x; l < j; l += blockDim.x) b[l] -= tj[l] * xj;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) b[j] = xj;
-    __syncthreads();
+                int ldx, const int32_t* __restrict__ ncol, int forward, int n_max) {
+  extern __shared__ double sh[];
+  const int sd = blockIdx.x, nw = blockDim.x / 32, lane = threadIdx.x & 31;
+  const int col0 = blockIdx.y * 2 * nw;
+  if (col0 >= ncol[sd]) return;
+  const int n = nn[sd], ld = tld[sd], shift = tsh[sd];
+  const double* T = Tm + toff[sd] + (int64_t)shift * ld + shift;
+  double* rd = sh;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) rd[i] = 1.0 / T[(int64_t)i * ld + i];
+  const int nv = min(2 * nw, ncol[sd] - col0);
+  double* x = X + roff[sd] * ldx + col0;
+  for (int idx = threadIdx.x; idx < n * nv; idx += blockDim.x) {
+    const int i = idx / nv, v = idx - i * nv;
+    sh[(int64_t)(1 + v) * n_max + i] = x[(int64_t)i * ldx + v];
   }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) x[(int64_t)i * ldx] = b[i];
+  __syncthreads();
+  const int v0 = 2 * (threadIdx.x / 32);
+  if (v0 < nv) {
+    double* b0 = sh + (int64_t)(1 + v0) * n_max;
+    double* b1 = v0 + 1 < nv ? b0 + n_max : b0;  // an odd last vector runs alone
+    const bool two = v0 + 1 < nv;
+    for (int s = 0; s < n; ++s) {
+      const int j = forward ? s : n - 1 - s;
+      const double* tj = T + (int64_t)j * ld;
+      // odd lanes divide for the second vector
+      const double xv = div_by((lane & 1) ? b1[j] : b0[j], tj[j], rd[j]);
+      const double x0 = __shfl_sync(0xFFFFFFFFu, xv, 0);
+      const double x1 = __shfl_sync(0xFFFFFFFFu, xv, 1);
+      const int l0 = forward ? j + 1 : 0, l1 = forward ? n : j;
+      for (int l = l0 + lane; l < l1; l += 32) {
+        const double t = tj[l];
+        b0[l] = fma(-t, x0, b0[l]);
+        if (two) b1[l] = fma(-t, x1, b1[l]);
+      }
+      if (lane == 0) b0[j] = x0;
+      if (two && lane == 1) b1[j] = x1;
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < n * nv; idx += blockDim.x) {
+    const int i = idx / nv, v = idx - i * nv;
+    x[(int64_t)i * ldx + v] = sh[(int64_t)(1 + v) * n_max + i];
+  }
 }
 
 // one row per warp: the row y (length m[sd]) of X (rows [roff[sd], roff[sd] + rows[sd]),
@@ -315,7 +418,9 @@ void launch_potrf(int n_sd, int n_max, double* D, const int64_t* doff, const int
     k_potrf_diag<<<n_sd, 256, 0, st>>>(D, doff, nn, j0, bad);
     const int T = (n_max - j0 - kNB + kNB - 1) / kNB;
     if (T > 0) {
-      count_launch();
+      count_launch(2);
+      k_potrf_panel<<<dim3(n_sd, (n_max - j0 - kNB + kPanelRows - 1) / kPanelRows),
+                      4 * kPanelRows, 0, st>>>(D, doff, nn, j0);
       k_potrf_update<<<dim3(n_sd, T * (T + 1) / 2), dim3(16, 16), sm, st>>>(D, doff, nn, j0);
     }
   }
@@ -339,12 +444,17 @@ void launch_trsv_cols(int n_sd, int n_max, int ncol_max, const double* T, const 
   if (n_sd <= 0 || ncol_max <= 0) return;
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_trsv_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_trsv_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     attr = true;
   }
+  // two vectors per warp and the reciprocals in 220 KB: four warps up to order 3,128, one at
+  // the largest (6,144)
+  int nw = 4;
+  while (nw > 1 && sizeof(double) * (1 + 2 * nw) * (size_t)n_max > 220 * 1024) --nw;
   count_launch();
-  k_trsv_cols<<<dim3(n_sd, ncol_max), 256, sizeof(double) * n_max, st>>>(
-      T, toff, nn, tld, tsh, X, roff, ldx, ncol, forward);
+  k_trsv_cols<<<dim3(n_sd, (ncol_max + 2 * nw - 1) / (2 * nw)), 32 * nw,
+                sizeof(double) * (1 + 2 * nw) * (size_t)n_max, st>>>(
+      T, toff, nn, tld, tsh, X, roff, ldx, ncol, forward, n_max);
 }
 
 void launch_trsv_rows(const double* R, const int64_t* roff_r, const int32_t* mm, double* X,
