@@ -1395,13 +1395,15 @@ __global__ void __launch_bounds__(TH, TH == 256 ? (sizeof(T) == 4 ? 6 : 4) : 1)
   const int64_t a0 = coarse ? co.aoff[sd] : 0;
   const Pack<T> bep = coef_pack<T>(s.beta, s.beta32, sd, kp, g.tx);
   const Pack<T> gap = coef_pack<T>(s.gam, s.gam32, sd, kp, g.tx);
-  T be[N], ga[N];
+  T be[N];
+  bool hasp[N], hasz[N];  // beta != 0; gam is 0 or 1
   bool needp = false;
 #pragma unroll
   for (int e = 0; e < N; ++e) {
     be[e] = bep.v[e];
-    ga[e] = gap.v[e];
-    needp = needp || be[e] != T(0);
+    hasp[e] = nonzero(be[e]);
+    hasz[e] = nonzero(gap.v[e]);
+    needp = needp || hasp[e];
   }
   T apr[N];
 #pragma unroll
@@ -1412,14 +1414,15 @@ __global__ void __launch_bounds__(TH, TH == 256 ? (sizeof(T) == 4 ? 6 : 4) : 1)
     if (needp) pv = ld(p + o);
     if (coarse) yv = ld(co.yc + (a0 + co.aloc[row]) * kp + g.tx * N);
     T d = dinv[row];
+    // three multiply-adds per element: choices of 0 by select, not by a product (a binary64
+    // operation or compare holds its quarter of the SM for 64 clocks per warp)
 #pragma unroll
     for (int e = 0; e < N; ++e) {
-      T z = d * rv.v[e];
-      if (coarse) z += yv.v[e];
-      T v = ga[e] * z;
-      if (be[e] != T(0)) v += be[e] * pv.v[e];
+      T z = coarse ? fma_t(d, rv.v[e], yv.v[e]) : d * rv.v[e];
+      z = hasz[e] ? z : T(0);
+      const T v = fma_t(be[e], hasp[e] ? pv.v[e] : T(0), z);
       pv.v[e] = v;
-      apr[e] += v * rv.v[e];
+      apr[e] = fma_t(v, rv.v[e], apr[e]);
     }
     st(p + o, pv);
   }
