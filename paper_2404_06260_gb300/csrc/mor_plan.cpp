@@ -820,8 +820,11 @@ void build_aggregates(const HostPlan& hp, int target_rows, int max_agg, AggPlan&
   ap.aoff.assign(n_sd + 1, 0);
   ap.nca[0].assign(n_sd, 0);
   ap.nca[1].assign(n_sd, 0);
-  std::vector<int> sI, sB;
-  for (int i = 0; i < n_sd; ++i) {
+  // subdomains in parallel where a thread's share outweighs its start
+  const int nthr = (int)std::min<int64_t>(std::max(1u, std::thread::hardware_concurrency()),
+                                          1 + hp.nP / 50000);
+  auto cut = [&](int i, int) {
+    std::vector<int> sI, sB;
     const int nI = hp.nI[i], nB = hp.nB[i];
     const uint32_t* cI = hp.p_code.data() + hp.Poff[i];
     const uint32_t* cB = cI + nI;
@@ -843,8 +846,12 @@ void build_aggregates(const HostPlan& hp, int target_rows, int max_agg, AggPlan&
     }
     ap.nca[0][i] = (int32_t)sI.size();
     ap.nca[1][i] = (int32_t)(sI.size() + sB.size());
-    ap.aoff[i + 1] = ap.aoff[i] + ap.nca[1][i];
-  }
+  };
+  if (nthr > 1)
+    parallel_for(n_sd, nthr, cut);
+  else
+    for (int i = 0; i < n_sd; ++i) cut(i, 0);
+  for (int i = 0; i < n_sd; ++i) ap.aoff[i + 1] = ap.aoff[i] + ap.nca[1][i];
   const int64_t n_agg = ap.aoff[n_sd];
   for (int set = 0; set < 2; ++set) {
     const HostTiles& T = set == 0 ? hp.tP_I : hp.tP_all;
