@@ -410,8 +410,9 @@ int mor_debug_sym_eig(int32_t n_sub, int32_t n, const double* A_dev, double* eva
  * every stored nonzero (value + column index) of an active subdomain's sparse
  * product, and every element of an open pack the kernel must read or write once (the
  * coarse kernel: its E^{-1} blocks once per open 16-column chunk); diagonal,
- * aggregate-index and coarse-correction reads are not counted.  Process-wide state,
- * not thread-safe. */
+ * aggregate-index and coarse-correction reads are not counted.  While enabled, small
+ * subdomains take these four kernels too instead of the on-chip iteration.  Process-wide
+ * state, not thread-safe. */
 int mor_profile_enable(int32_t on);
 int mor_profile_reset(void);
 int mor_profile_query(int32_t family, double* out);
