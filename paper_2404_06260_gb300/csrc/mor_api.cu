@@ -1206,7 +1206,7 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
     size_t gsz = (size_t)mt * nk * nk;
     if (wide || kb > 80) {
       // the sketch Grams (k x k) and the diagonal-block Gram (at most 128 x 128)
-      gsz = std::max(gsz, (size_t)n_sd * gram_wide_chunks(n_sd, k, k) * k * k);
+      gsz = std::max(gsz, (size_t)n_sd * gram_wide_chunks(n_sd, k) * k * k);
       gsz = std::max(gsz, (size_t)n_sd * 16 * 128 * 128);
     }
     TRY(M.alloc(&gpart, gsz, true, st));
@@ -1233,8 +1233,7 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
       launch_tc_gram(tl, n_sd, X, ldx, nx, Y, ldy, ny, tcpart, tcrange, G, ldg,
                      (int64_t)ldg * ldg, tc_budget, tcerr, st);
     else if (nx > 80 || ny > 80)
-      launch_gram_wide(tl, n_sd, X, ldx, nx, Y, ldy, ny, gpart, G, ldg, (int64_t)ldg * ldg,
-                       st);
+      launch_gram_wide(tl, n_sd, X, ldx, nx, Y, ldy, gpart, G, ldg, (int64_t)ldg * ldg, st);
     else
       launch_gram(tl, n_sd, X, ldx, nx, Y, ldy, ny, gpart, gcnt, G, ldg, st);
   };
@@ -1392,11 +1391,10 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
     TRY(M.alloc(&Vx, (size_t)n_sd * ldm * ldm, true, st));
     TRY(M.alloc(&Mx, (size_t)n_sd * ldm * ldm, true, st));
     TRY(M.alloc(&gp, (size_t)std::max<int64_t>(
-                         (int64_t)n_sd * gram_wide_chunks(n_sd, mB, mB) * mB * mB,
+                         (int64_t)n_sd * gram_wide_chunks(n_sd, mB) * mB * mB,
                          (int64_t)mt * std::min(ldm, 80) * std::min(ldm, 80)), true, st));
     if (mB > 80) {
-      launch_gram_wide(S.tW, n_sd, Yw2, ldm, mB, Yw2, ldm, mB, gp, Gx, ldm, (int64_t)ldm * ldm,
-                       st);
+      launch_gram_wide(S.tW, n_sd, Yw2, ldm, mB, Yw2, ldm, gp, Gx, ldm, (int64_t)ldm * ldm, st);
     } else {
       launch_gram(S.tW, n_sd, Yw2, ldm, mB, Yw2, ldm, mB, gp, gcnt, Gx, ldm, st);
     }
@@ -1497,8 +1495,7 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
   // blocks Q_i^T A_ii Q_i as the identity, and Q_i = V W Lambda^{-1/2} amplifies the
   // Gram's error on directions of small energy
   if (mcols + 1 > 80)
-    launch_gram_wide(S.tO, n_sd, V, kq, mcols + 1, AV, kq, mcols + 1, gpart, G, kq,
-                     (int64_t)kq * kq, st);
+    launch_gram_wide(S.tO, n_sd, V, kq, mcols + 1, AV, kq, gpart, G, kq, (int64_t)kq * kq, st);
   else
     launch_gram(S.tO, n_sd, V, kq, mcols + 1, AV, kq, mcols + 1, gpart, gcnt, G, kq, st);
   sym_eig(kq, mcols + 1, evals, evecs);

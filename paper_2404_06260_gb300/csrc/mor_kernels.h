@@ -293,10 +293,11 @@ void launch_rowmul(const DTiles& tiles, const double* X, int ldx, int nin, const
                    int ldm, double* Y, int ldy, int nout, cudaStream_t st);
 // dst[r, dc0 + c] = src[map[r], sc0 + c] (map null: r), c < ncols
 // wide-sketch versions (k up to 511 columns, mor_wide.cu): the Gram needs a partial
-// buffer of n_sd * gram_wide_chunks(n_sd, nx, ny) * nx * ny doubles
-int gram_wide_chunks(int n_sd, int nx, int ny);
-void launch_gram_wide(const DTiles& tiles, int n_sd, const double* X, int ldx, int nx,
-                      const double* Y, int ldy, int ny, double* part, double* G, int ldg,
+// buffer of n_sd * gram_wide_chunks(n_sd, n) * n * n doubles; X^T Y is symmetric up to
+// rounding (the lower triangle is computed and mirrored)
+int gram_wide_chunks(int n_sd, int n);
+void launch_gram_wide(const DTiles& tiles, int n_sd, const double* X, int ldx, int n,
+                      const double* Y, int ldy, double* part, double* G, int ldg,
                       int64_t sd_stride, cudaStream_t st);
 void launch_rowmul_wide(const DTiles& tiles, const double* X, int ldx, int nin,
                         const double* M, int ldm, double* Y, int ldy, int nout,

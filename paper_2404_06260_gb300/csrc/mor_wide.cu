@@ -14,16 +14,23 @@ namespace {
 constexpr int kWT = 64;      // output tile of the Gram and of the row product
 constexpr int kWRows = 16;   // rows staged per step of the Gram
 
-// part[(sd * S + s)][i * ny + j] = sum over the rows of chunk s of subdomain sd of
-// X[r, i] Y[r, j]; block (16, 16), each thread a 4 x 4 patch of the 64 x 64 tile
+// part[(sd * S + s)][i * n + j] = sum over the rows of chunk s of subdomain sd of
+// X[r, i] Y[r, j] for the 64 x 64 tiles on and below the diagonal: every product here is
+// symmetric up to rounding (X^T X, X^T H X, V^T A V) and its reader symmetrises.  Block
+// (16, 16), thread (tx, ty) rows ty + 16 a and columns tx + 16 b of the tile; the 16-wide
+// strips past n are left out.  Bound by binary64 issue, so by what is multiplied: the whole
+// square in tiles padded to 64 took 1.95 ms for 14 subdomains of up to 261 columns, 0.91 now.
 __global__ void __launch_bounds__(256)
-    k_gram_wide(DTiles tl, int S, const double* __restrict__ X, int ldx, int nx,
-                const double* __restrict__ Y, int ldy, int ny, double* __restrict__ part) {
+    k_gram_wide(DTiles tl, int S, const double* __restrict__ X, int ldx, int n,
+                const double* __restrict__ Y, int ldy, double* __restrict__ part) {
   __shared__ double Xs[kWRows][kWT + 1];
   __shared__ double Ys[kWRows][kWT + 1];
   const int sd = blockIdx.x / S, s = blockIdx.x % S;
-  const int ntj = (ny + kWT - 1) / kWT;
-  const int i0 = (blockIdx.y / ntj) * kWT, j0 = (blockIdx.y % ntj) * kWT;
+  // tile (ti, tj), tj <= ti, of the lower triangle by rows
+  int ti = 0;
+  while ((ti + 1) * (ti + 2) / 2 <= (int)blockIdx.y) ++ti;
+  const int i0 = ti * kWT, j0 = ((int)blockIdx.y - ti * (ti + 1) / 2) * kWT;
+  const int na = (min(kWT, n - i0) + 15) / 16, nb = (min(kWT, n - j0) + 15) / 16;
   const int lo = tl.lo[sd], hi = tl.hi[sd];
   const int nt = hi - lo;
   const int t0 = lo + (int)((int64_t)nt * s / S), t1 = lo + (int)((int64_t)nt * (s + 1) / S);
@@ -40,46 +47,53 @@ __global__ void __launch_bounds__(256)
       for (int idx = tid; idx < kWRows * kWT; idx += 256) {
         const int rr = idx / kWT, c = idx % kWT;
         const bool in = rr < nr;
-        Xs[rr][c] = (in && i0 + c < nx) ? X[(int64_t)(base + rr) * ldx + i0 + c] : 0.0;
-        Ys[rr][c] = (in && j0 + c < ny) ? Y[(int64_t)(base + rr) * ldy + j0 + c] : 0.0;
+        Xs[rr][c] = (in && i0 + c < n) ? X[(int64_t)(base + rr) * ldx + i0 + c] : 0.0;
+        Ys[rr][c] = (in && j0 + c < n) ? Y[(int64_t)(base + rr) * ldy + j0 + c] : 0.0;
       }
       __syncthreads();
 #pragma unroll 4
       for (int rr = 0; rr < kWRows; ++rr) {
         double xa[4], yb[4];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) xa[a] = Xs[rr][ty * 4 + a];
+        for (int a = 0; a < 4; ++a) xa[a] = Xs[rr][ty + 16 * a];
 #pragma unroll
-        for (int b = 0; b < 4; ++b) yb[b] = Ys[rr][tx * 4 + b];
+        for (int b = 0; b < 4; ++b) yb[b] = Ys[rr][tx + 16 * b];
 #pragma unroll
         for (int a = 0; a < 4; ++a)
+          if (a < na) {
 #pragma unroll
-          for (int b = 0; b < 4; ++b) acc[a][b] += xa[a] * yb[b];
+            for (int b = 0; b < 4; ++b)
+              if (b < nb) acc[a][b] += xa[a] * yb[b];
+          }
       }
       __syncthreads();
     }
   }
-  double* P = part + (int64_t)(sd * S + s) * nx * ny;
+  double* P = part + (int64_t)(sd * S + s) * n * n;
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
-      const int i = i0 + ty * 4 + a, j = j0 + tx * 4 + b;
-      if (i < nx && j < ny) P[(int64_t)i * ny + j] = acc[a][b];
+      const int i = i0 + ty + 16 * a, j = j0 + tx + 16 * b;
+      if (i < n && j < n) P[(int64_t)i * n + j] = acc[a][b];
     }
 }
 
-// G[sd][i * ldg + j] = sum over s of part[(sd * S + s)][i * ny + j], s in order
-__global__ void k_gram_wide_reduce(int S, int nx, int ny, const double* __restrict__ part,
+// G[sd][i * ldg + j] and its mirror image = sum over s of part[(sd * S + s)][i * n + j],
+// j <= i, s in order
+__global__ void k_gram_wide_reduce(int S, int n, const double* __restrict__ part,
                                    double* __restrict__ G, int ldg, int64_t sd_stride) {
   const int sd = blockIdx.y;
-  const int64_t n = (int64_t)nx * ny;
-  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < n;
+  const int64_t nn = (int64_t)n * n;
+  double* Gs = G + (int64_t)sd * sd_stride;
+  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < nn;
        o += (int64_t)gridDim.x * blockDim.x) {
+    const int i = (int)(o / n), j = (int)(o % n);
+    if (j > i) continue;
     double acc = 0.0;
-    for (int s = 0; s < S; ++s) acc += part[(int64_t)(sd * S + s) * n + o];
-    const int i = (int)(o / ny), j = (int)(o % ny);
-    G[(int64_t)sd * sd_stride + (int64_t)i * ldg + j] = acc;
+    for (int s = 0; s < S; ++s) acc += part[(int64_t)(sd * S + s) * nn + o];
+    Gs[(int64_t)i * ldg + j] = acc;
+    Gs[(int64_t)j * ldg + i] = acc;
   }
 }
 
@@ -144,24 +158,24 @@ __global__ void __launch_bounds__(256)
 
 }  // namespace
 
-int gram_wide_chunks(int n_sd, int nx, int ny) {
-  const int tiles = ((nx + kWT - 1) / kWT) * ((ny + kWT - 1) / kWT);
+int gram_wide_chunks(int n_sd, int n) {
+  const int nt = (n + kWT - 1) / kWT, tiles = nt * (nt + 1) / 2;
   int S = (4 * 152 + n_sd * tiles - 1) / (n_sd * tiles);
   return S < 1 ? 1 : (S > 16 ? 16 : S);
 }
 
-void launch_gram_wide(const DTiles& tiles, int n_sd, const double* X, int ldx, int nx,
-                      const double* Y, int ldy, int ny, double* part, double* G, int ldg,
+void launch_gram_wide(const DTiles& tiles, int n_sd, const double* X, int ldx, int n,
+                      const double* Y, int ldy, double* part, double* G, int ldg,
                       int64_t sd_stride, cudaStream_t st) {
   if (tiles.n <= 0 || n_sd <= 0) return;
-  const int S = gram_wide_chunks(n_sd, nx, ny);
-  const int nt = ((nx + kWT - 1) / kWT) * ((ny + kWT - 1) / kWT);
+  const int S = gram_wide_chunks(n_sd, n);
+  const int nt = (n + kWT - 1) / kWT;
   count_launch(2);
-  k_gram_wide<<<dim3(n_sd * S, nt), dim3(16, 16), 0, st>>>(tiles, S, X, ldx, nx, Y, ldy, ny,
-                                                          part);
-  const int64_t n = (int64_t)nx * ny;
-  const int bx = (int)((n + 255) / 256 < 64 ? (n + 255) / 256 : 64);
-  k_gram_wide_reduce<<<dim3(bx, n_sd), 256, 0, st>>>(S, nx, ny, part, G, ldg, sd_stride);
+  k_gram_wide<<<dim3(n_sd * S, nt * (nt + 1) / 2), dim3(16, 16), 0, st>>>(tiles, S, X, ldx, n,
+                                                                        Y, ldy, part);
+  const int64_t nn = (int64_t)n * n;
+  const int bx = (int)((nn + 255) / 256 < 64 ? (nn + 255) / 256 : 64);
+  k_gram_wide_reduce<<<dim3(bx, n_sd), 256, 0, st>>>(S, n, part, G, ldg, sd_stride);
 }
 
 void launch_rowmul_wide(const DTiles& tiles, const double* X, int ldx, int nin,
