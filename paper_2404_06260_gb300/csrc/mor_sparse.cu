@@ -768,9 +768,9 @@ __global__ void k_cg_start(DTiles tl, const double* __restrict__ b64, double* x6
 // x += alpha p, r -= alpha q; ||r||^2, the fine r.z = r.D^{-1}r and the restriction of
 // the new r; the coarse kernel (STEP) completes r.M^{-1}r, beta and the done flags.
 // TH = 256: 48 registers (binary32) leave room for five blocks per SM; six cost spills.
-// TH = 1024: light loads (light_threads)
-template <typename T, int TH>
-__global__ void __launch_bounds__(TH, TH == 256 ? (sizeof(T) == 4 ? 5 : 4) : 1)
+// TH = 1024: light loads (light_threads).  R rows in flight per thread (wide_rows)
+template <typename T, int TH, int R = 1>
+__global__ void __launch_bounds__(TH, TH == 256 ? (R == 2 ? 3 : sizeof(T) == 4 ? 5 : 4) : 1)
     k_cg_update_xr(DTiles tl, T* x, T* r, const T* __restrict__ p, const T* __restrict__ q,
                    const T* __restrict__ dinv, int kp, CgState s, Coarse<T> co) {
   constexpr int N = Pack<T>::N;
@@ -792,28 +792,40 @@ __global__ void __launch_bounds__(TH, TH == 256 ? (sizeof(T) == 4 ? 5 : 4) : 1)
 #pragma unroll
   for (int e = 0; e < N; ++e) arr[e] = arz[e] = T(0);
   for (int s0 = 0; s0 < nrows; s0 += step) {
-    for (int rr = s0 + g.ty; rr < min(nrows, s0 + step); rr += g.rb) {
-      const int64_t row = r0 + rr;
-      const int64_t o = row * kp + g.tx * N;
-      Pack<T> rv;
-      if (skip) {
+    const int send = min(nrows, s0 + step);
+    for (int rb = s0 + g.ty; rb < send; rb += R * g.rb) {
+      Pack<T> xv[R], pv[R], qv[R], rv[R];
+      T d[R];
 #pragma unroll
-        for (int e = 0; e < N; ++e) rv.v[e] = T(0);
-      } else {
-        Pack<T> xv = ld(x + o), pv = ld(p + o), qv = ld(q + o);
-        rv = ld(r + o);
-        T d = dinv[row];
+      for (int u = 0; u < R; ++u) {
+        const int64_t row = r0 + rb + u * g.rb, o = row * kp + g.tx * N;
+        if (skip || rb + u * g.rb >= send) {
 #pragma unroll
-        for (int e = 0; e < N; ++e) {
-          xv.v[e] += al[e] * pv.v[e];
-          rv.v[e] -= al[e] * qv.v[e];
-          arr[e] += rv.v[e] * rv.v[e];
-          arz[e] += rv.v[e] * (d * rv.v[e]);
+          for (int e = 0; e < N; ++e) rv[u].v[e] = T(0);
+          continue;
         }
-        st(x + o, xv);
-        st(r + o, rv);
+        xv[u] = ld(x + o), pv[u] = ld(p + o), qv[u] = ld(q + o);
+        rv[u] = ld(r + o);
+        d[u] = dinv[row];
       }
-      if (coarse) tr.put(rr - s0, kp, g.tx, rv);
+#pragma unroll
+      for (int u = 0; u < R; ++u) {
+        const int rr = rb + u * g.rb;
+        if (rr >= send) continue;
+        const int64_t o = (int64_t)(r0 + rr) * kp + g.tx * N;
+        if (!skip) {
+#pragma unroll
+          for (int e = 0; e < N; ++e) {
+            xv[u].v[e] += al[e] * pv[u].v[e];
+            rv[u].v[e] -= al[e] * qv[u].v[e];
+            arr[e] += rv[u].v[e] * rv[u].v[e];
+            arz[e] += rv[u].v[e] * (d[u] * rv[u].v[e]);
+          }
+          st(x + o, xv[u]);
+          st(r + o, rv[u]);
+        }
+        if (coarse) tr.put(rr - s0, kp, g.tx, rv[u]);
+      }
     }
     if (coarse) {
       __syncthreads();
@@ -942,38 +954,91 @@ __device__ __forceinline__ Pack<T> restrict_pack(const Coarse<T>& co, int ga, in
 }
 
 // Coarse level of one subdomain in SIMT arithmetic, up to kCoarseSmallMax aggregates
-// (block (column chunk, sd), kCoarseSmallCols columns): r_c = Z^T r for the chunk, y_c =
-// E^{-1} r_c with one thread per (row, column), the chunk's part of r_c.y_c; the last chunk
-// of the subdomain (atomic ticket) finishes.  A binary64 multiply-add occupies its quarter
-// of the SM for 64 clocks per warp, so the products are spread over as many warps and
-// blocks as there are: 16 columns per thread and one row per thread took 69 us a launch for
-// 27 subdomains of 52 aggregates and 32 columns, 20 us now.
+// (block (column chunk, sd), CW columns): r_c = Z^T r for the chunk, y_c = E^{-1} r_c, the
+// chunk's part of r_c.y_c; the last chunk of the subdomain (atomic ticket) finishes.
+//  - Binary64: one thread per (row, column).  A multiply-add occupies its quarter of the SM
+//    for 64 clocks per warp, so the products are spread over as many warps and blocks as
+//    there are: 16 columns per thread took 69 us a launch for 27 subdomains of 52
+//    aggregates and 32 columns, 20 us now.
+//  - Binary32: one thread per row and all CW columns.  Bound by the loads: an element of
+//    E^{-1}, read coalesced, feeds CW multiply-adds, and a block of 8 columns reads E^{-1}
+//    half as often as one of 4.  14 subdomains of up to 200
+//    aggregates, 264 columns: 34 -> 23 us against one thread per (row, column).
 constexpr int kCoarseSmallMax = 256;
-constexpr int kCoarseSmallCols = 4;
 constexpr int kCoarseThreads = 256;
-template <typename T>
+template <typename T, int CW>
 __global__ void __launch_bounds__(kCoarseThreads)
     k_cg_coarse_small(DTiles tl, int kp, double tol2, int mode, CgState s, Coarse<T> co) {
-  constexpr int CW = kCoarseSmallCols, PN = Pack<T>::N;
+  constexpr int PN = Pack<T>::N;
   __shared__ __align__(16) T rc[kCoarseSmallMax * CW];
   __shared__ double red[(kCoarseThreads / 32) * CW];
   Geo g = geo();
-  const int sd = blockIdx.y, c0 = blockIdx.x * CW;
+  const int sd = blockIdx.y, c0 = blockIdx.x * CW, ncol = min(CW, kp - c0);
   if (s.active[sd] == 0) return;
   bool open = false;  // a chunk whose columns have all converged needs no coarse product
 #pragma unroll
-  for (int j = 0; j < CW; ++j) open = !s.done[sd * kp + c0 + j] || open;
+  for (int j = 0; j < CW; ++j) open = (j < ncol && !s.done[sd * kp + c0 + j]) || open;
   const int n = co.tbase && open ? co.nca[sd] : 0;
   const int j = g.tid % CW, lane = g.tid & 31;
-  double dl = 0.0;
+  const int a0 = n > 0 ? co.aoff[sd] : 0;
+  const T* Eb = n > 0 ? co.einv + co.eoff[sd] : nullptr;
   if (n > 0) {
-    const int a0 = co.aoff[sd];
     for (int idx = g.tid; idx < n * (CW / PN); idx += g.nth) {
       const int a = idx / (CW / PN), pk = idx - a * (CW / PN);
-      st(rc + a * CW + pk * PN, restrict_pack(co, a0 + a, kp, c0 + pk * PN));
+      Pack<T> v;
+#pragma unroll
+      for (int e = 0; e < PN; ++e) v.v[e] = T(0);
+      if (pk * PN < ncol) v = restrict_pack(co, a0 + a, kp, c0 + pk * PN);
+      st(rc + a * CW + pk * PN, v);
     }
     __syncthreads();
-    const T* Eb = co.einv + co.eoff[sd];
+  }
+  if constexpr (sizeof(T) == 4) {
+    double dl[CW];
+#pragma unroll
+    for (int c = 0; c < CW; ++c) dl[c] = 0.0;
+    const int a = g.tid;
+    if (a < n) {
+      T y[CW];
+#pragma unroll
+      for (int c = 0; c < CW; ++c) y[c] = T(0);
+#pragma unroll 8
+      for (int b = 0; b < n; ++b) {
+        const T e = Eb[(int64_t)b * n + a];  // symmetric: column a as row a
+#pragma unroll
+        for (int pk = 0; pk < CW / PN; ++pk) {
+          const Pack<T> v = ld(rc + b * CW + pk * PN);
+#pragma unroll
+          for (int c = 0; c < PN; ++c) y[pk * PN + c] += e * v.v[c];
+        }
+      }
+#pragma unroll
+      for (int pk = 0; pk < CW / PN; ++pk) {
+        Pack<T> yv;
+#pragma unroll
+        for (int c = 0; c < PN; ++c) {
+          yv.v[c] = y[pk * PN + c];
+          dl[pk * PN + c] = (double)yv.v[c] * (double)rc[a * CW + pk * PN + c];
+        }
+        if (pk * PN < ncol) st(co.yc + (int64_t)(a0 + a) * kp + c0 + pk * PN, yv);
+      }
+    }
+    // the warp's CW sums: halves of the columns change sides until a lane holds one
+    int c = 0, o = 16;
+#pragma unroll
+    for (int h = CW / 2; h >= 1; h /= 2, o /= 2) {
+      const bool up = (lane & o) != 0;
+      c += up ? h : 0;
+#pragma unroll
+      for (int i = 0; i < h; ++i) {
+        const double give = up ? dl[i] : dl[i + h], keep = up ? dl[i + h] : dl[i];
+        dl[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+    }
+    for (; o >= 1; o /= 2) dl[0] += __shfl_xor_sync(0xffffffffu, dl[0], o);
+    if ((lane & (32 / CW - 1)) == 0) red[(g.tid >> 5) * CW + c] = dl[0];
+  } else {
+    double dl = 0.0;
     for (int a = g.tid / CW; a < n; a += kCoarseThreads / CW) {
       // E^{-1} is symmetric: row a is read as column a (eight rows per warp: one sector or two)
       T acc0 = T(0), acc1 = T(0);
@@ -993,11 +1058,11 @@ __global__ void __launch_bounds__(kCoarseThreads)
       co.yc[(int64_t)(a0 + a) * kp + c0 + j] = y;
       dl += (double)y * (double)rc[a * CW + j];
     }
+    for (int o = CW; o < 32; o <<= 1) dl += __shfl_xor_sync(0xffffffffu, dl, o);
+    if (lane < CW) red[(g.tid >> 5) * CW + lane] = dl;
   }
-  for (int o = CW; o < 32; o <<= 1) dl += __shfl_xor_sync(0xffffffffu, dl, o);
-  if (lane < CW) red[(g.tid >> 5) * CW + lane] = dl;
   __syncthreads();
-  if (g.tid < CW && co.dpart) {
+  if (g.tid < ncol && co.dpart) {
     double t = 0.0;
     for (int w = 0; w < kCoarseThreads / 32; ++w) t += red[w * CW + g.tid];
     __stcg(co.dpart + (int64_t)sd * kp + c0 + g.tid, t);
@@ -1380,8 +1445,8 @@ __global__ void __launch_bounds__(kTcThreads)
 
 // p = gam (D^{-1} r + Z y_c) + beta p (p is not read where beta = 0), and p.r of the
 // new direction for the next step length
-template <typename T, int TH>
-__global__ void __launch_bounds__(TH, TH == 256 ? (sizeof(T) == 4 ? 6 : 4) : 1)
+template <typename T, int TH, int R = 1>
+__global__ void __launch_bounds__(TH, TH == 256 ? (sizeof(T) == 4 && R == 1 ? 6 : 4) : 1)
     k_cg_update_p(DTiles tl, const T* __restrict__ r, T* p, const T* __restrict__ dinv, int kp,
                   CgState s, Coarse<T> co) {
   constexpr int N = Pack<T>::N;
@@ -1408,23 +1473,34 @@ __global__ void __launch_bounds__(TH, TH == 256 ? (sizeof(T) == 4 ? 6 : 4) : 1)
   T apr[N];
 #pragma unroll
   for (int e = 0; e < N; ++e) apr[e] = T(0);
-  for (int64_t row = r0 + g.ty; row < rend; row += g.rb) {
-    int64_t o = row * kp + g.tx * N;
-    Pack<T> rv = ld(r + o), pv, yv;
-    if (needp) pv = ld(p + o);
-    if (coarse) yv = ld(co.yc + (a0 + co.aloc[row]) * kp + g.tx * N);
-    T d = dinv[row];
+  for (int64_t rowb = r0 + g.ty; rowb < rend; rowb += R * g.rb) {
+    Pack<T> rv[R], pv[R], yv[R];
+    T d[R];
+#pragma unroll
+    for (int u = 0; u < R; ++u) {
+      const int64_t row = rowb + u * g.rb, o = row * kp + g.tx * N;
+      if (row >= rend) continue;
+      rv[u] = ld(r + o);
+      if (needp) pv[u] = ld(p + o);
+      if (coarse) yv[u] = ld(co.yc + (a0 + co.aloc[row]) * kp + g.tx * N);
+      d[u] = dinv[row];
+    }
     // three multiply-adds per element: choices of 0 by select, not by a product (a binary64
     // operation or compare holds its quarter of the SM for 64 clocks per warp)
 #pragma unroll
-    for (int e = 0; e < N; ++e) {
-      T z = coarse ? fma_t(d, rv.v[e], yv.v[e]) : d * rv.v[e];
-      z = hasz[e] ? z : T(0);
-      const T v = fma_t(be[e], hasp[e] ? pv.v[e] : T(0), z);
-      pv.v[e] = v;
-      apr[e] = fma_t(v, rv.v[e], apr[e]);
+    for (int u = 0; u < R; ++u) {
+      const int64_t row = rowb + u * g.rb;
+      if (row >= rend) continue;
+#pragma unroll
+      for (int e = 0; e < N; ++e) {
+        T z = coarse ? fma_t(d[u], rv[u].v[e], yv[u].v[e]) : d[u] * rv[u].v[e];
+        z = hasz[e] ? z : T(0);
+        const T v = fma_t(be[e], hasp[e] ? pv[u].v[e] : T(0), z);
+        pv[u].v[e] = v;
+        apr[e] = fma_t(v, rv[u].v[e], apr[e]);
+      }
+      st(p + row * kp + g.tx * N, pv[u]);
     }
-    st(p + o, pv);
   }
   block_colsum<T, N>(g, apr, sm.red, s.part1 + (int64_t)tile * kp);
   const double* const parts[1] = {s.part1};
@@ -1630,6 +1706,15 @@ void launch_spmm(const DTiles& tiles, const EllView<T>& A, const T* X, T* Y, int
   k_spmm<T><<<tiles.n, bl, smem_bytes<T>(bl.x, bl.y, kp, A.W), st>>>(tiles, A, X, Y, kp);
 }
 
+// Two rows in flight per thread in the updates where a block holds up to eight (more than 28
+// packs of columns): its threads walk 16 or more rows one after another (wide sketches on
+// 25^3: x/r update 47 -> 40 us, p update 26 -> 22).  With 11 packs and 23 rows a block
+// (64^3) the x/r update already runs at 98 % of the copy bandwidth, in 48 registers.
+template <typename T>
+bool wide_rows(dim3 bl) {
+  return sizeof(T) == 4 && bl.y <= 8;
+}
+
 template <typename T>
 size_t slot_kernel_smem(dim3 bl, int kp) {
   return align16(smem_bytes<T>(bl.x, bl.y, kp, 0)) + restrict_smem_bytes<T>(bl.y, kp);
@@ -1688,8 +1773,11 @@ void launch_coarse_then_p(const DTiles& tiles, int n_sd, const T* r, T* p, const
   if (!done) {
     count_launch();
     if (n_max <= kCoarseSmallMax) {
-      k_cg_coarse_small<T><<<dim3(kp / kCoarseSmallCols, n_sd), kCoarseThreads, 0, st>>>(
-          tiles, kp, tol2, mode, s, co);
+      // 8 columns a block while that leaves two blocks per SM
+      const bool wide = sizeof(T) == 4 && (kp + 7) / 8 * n_sd >= 2 * 152;
+      const int cw = wide ? 8 : 4;
+      auto fn = wide ? k_cg_coarse_small<T, sizeof(T) == 4 ? 8 : 4> : k_cg_coarse_small<T, 4>;
+      fn<<<dim3((kp + cw - 1) / cw, n_sd), kCoarseThreads, 0, st>>>(tiles, kp, tol2, mode, s, co);
     } else {
       const size_t sm = align16(sizeof(T) * ((n_max + 7) & ~7) * kCoarseCols) + kCoarseRedBytes;
       const int rows = kCoarseRpt * kCoarseThreads;
@@ -1704,7 +1792,8 @@ void launch_coarse_then_p(const DTiles& tiles, int n_sd, const T* r, T* p, const
   const int th = light_threads<T>(open_tiles);
   const dim3 bl = block_of<T>(kp, th);
   const size_t sm = smem_bytes<T>(bl.x, bl.y, kp, 0);
-  auto fn = th == 1024 ? k_cg_update_p<T, 1024> : k_cg_update_p<T, 256>;
+  auto fn = th == 1024 ? k_cg_update_p<T, 1024>
+            : wide_rows<T>(bl) ? k_cg_update_p<T, 256, 2> : k_cg_update_p<T, 256>;
   fn<<<tiles.n, bl, sm, st>>>(tiles, r, p, dinv, kp, s, co);
 }
 
@@ -1818,6 +1907,7 @@ void launch_cg_step(const DTiles& tiles, const EllView<T>& A, T* x, T* r, T* p, 
     set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 2, 128>);
     set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 2, 1024>);
     set_smem_attr<T>((const void*)k_cg_update_xr<T, 256>);
+    set_smem_attr<T>((const void*)k_cg_update_xr<T, 256, 2>);
     set_smem_attr<T>((const void*)k_cg_update_xr<T, 1024>);
     attr = true;
   }
@@ -1832,7 +1922,8 @@ void launch_cg_step(const DTiles& tiles, const EllView<T>& A, T* x, T* r, T* p, 
     k_cg_spmm_pq<T, 2, 1024><<<tiles.n, bl, smem_bytes<T>(bl.x, bl.y, kp, A.W), st>>>(tiles, A, p, q, kp, s);
   }
   if (ev) cudaEventRecord(ev[1], st);
-  auto fn = th == 1024 ? k_cg_update_xr<T, 1024> : k_cg_update_xr<T, 256>;
+  auto fn = th == 1024 ? k_cg_update_xr<T, 1024>
+            : wide_rows<T>(bl) ? k_cg_update_xr<T, 256, 2> : k_cg_update_xr<T, 256>;
   fn<<<tiles.n, bl, slot_kernel_smem<T>(bl, kp), st>>>(tiles, x, r, p, q, dinv, kp, s, co);
   if (ev) cudaEventRecord(ev[2], st);
   launch_coarse_then_p<T>(tiles, tiles.n_sd, r, p, dinv, kp, tol2, kCoarseStep, open_tiles, s, co,

@@ -61,3 +61,15 @@ def test_without_a_coarse_level(mor):
     E0, _, _ = _run(mor, sd, rank=6, oversample=4, precision="mixed", coarse_rows=0)
     E1, _, _ = _run(mor, sd, rank=6, oversample=4, precision="fp64", cg_rtol=1e-10)
     assert abs(E0 - E1) <= 1e-6 * E1
+
+
+# 130 to 222 columns: the SIMT product takes four or eight columns a block (an odd last chunk
+# of four), the updates two rows a thread from 196 columns on, the Grams strips of 16
+@pytest.mark.parametrize("n,parts,hops,rank,over", [
+    (15, 3, 3, 100, 29), (15, 3, 3, 60, 161), (14, 2, 3, 60, 141), (15, 3, 3, 40, 89)])
+def test_wide_columns(mor, n, parts, hops, rank, over):
+    sd = _plan(mor, n, parts, hops)
+    E0, it0, s0 = _run(mor, sd, precision="mixed", rank=rank, oversample=over)
+    E1, it1, s1 = _run(mor, sd, precision="fp64", cg_rtol=1e-10, rank=rank, oversample=over)
+    assert abs(E0 - E1) <= 1e-6 * E1
+    assert np.abs(s0 - s1).max() <= 1e-6 * s1.max()
