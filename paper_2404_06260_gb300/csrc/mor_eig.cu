@@ -27,7 +27,7 @@
 // staged from L2 (k_sym_eig_blocks).
 // Per batch, against the two-sided iteration with the matrix in shared memory (up to 80) or
 // in L2 and one CTA per subdomain: 64 matrices of order 42 2.13 -> 1.06 ms, 40 of 74 8.5 ->
-// 2.6 ms, 14 of up to 261 145 -> 10 ms, 8 of 127 169 -> 6 ms (the noise directions of an
+// 2.0 ms, 14 of 203 145 -> 8 ms, 8 of 127 169 -> 5.4 ms (the noise directions of an
 // explicit Gram never met the two-sided threshold and ran all 40 sweeps).
 #include <cooperative_groups.h>
 
@@ -67,30 +67,44 @@ struct JCol {
   double d, di;  // scale and its inverse
 };
 
-// the rotation that orthogonalises columns p and q, pq = w_p.w_q: w_p -= al w_q, w_q += be
-// w_p (old), and the columns' new state in p and q; false when the product is at the
-// rounding level
-__device__ __forceinline__ bool jacobi_rotation(JCol& p, JCol& q, double pq, float tol,
-                                                double& al, double& be) {
-  const double apq = p.d * q.d * pq;
+// The rotation that orthogonalises columns p and q, in two parts around the tangent, the one
+// thing that waits for the product pq = w_p.w_q: w_p -= t rq w_q, w_q += t rp w_p (old).
+struct JPair {
+  double dd;       // d_p d_q
+  double diff;     // |q|^2 - |p|^2
+  double rp, rq;   // d_p / d_q, d_q / d_p
+  float level;     // |d_p d_q pq| above which the pair rotates
+};
+__device__ __forceinline__ JPair jacobi_prepare(const JCol& p, const JCol& q, float tol) {
+  JPair s;
+  s.dd = p.d * q.d;
+  s.diff = q.sq - p.sq;
+  s.rp = p.d * q.di;
+  s.rq = q.d * p.di;
+  s.level = tol * (fast_sqrt((float)p.sq) * fast_sqrt((float)q.sq));
+  return s;
+}
+// the tangent, 0 when the product is at the rounding level (only the angle: binary32 roots
+// and quotients by the fast instructions are exact enough); apq = d_p d_q pq
+__device__ __forceinline__ double jacobi_tangent(const JPair& s, double pq, double& apq) {
+  apq = s.dd * pq;
   const float o = (float)apq;
-  // only the angle: binary32 roots and quotients by the fast instructions are exact enough
-  if (!(fabsf(o) > tol * (fast_sqrt((float)p.sq) * fast_sqrt((float)q.sq)))) return false;
-  const float tau = 0.5f * __fdividef((float)(q.sq - p.sq), o);
+  if (!(fabsf(o) > s.level)) return 0.0;
+  const float tau = 0.5f * __fdividef((float)s.diff, o);
   const float a = fabsf(tau);
   const float tt = a > 1e8f ? __fdividef(0.5f, a)
                             : __fdividef(1.0f, a + fast_sqrt(fmaf(a, a, 1.0f)));
-  const double t = (double)(tau >= 0.0f ? tt : -tt);
+  return (double)(tau >= 0.0f ? tt : -tt);
+}
+// the columns' state after the rotation
+__device__ __forceinline__ void jacobi_finish(JCol& p, JCol& q, double t, double apq) {
   const double h = fma(t, t, 1.0), c = inv_sqrt(h), ci = h * c;
-  al = t * (q.d * p.di);
-  be = t * (p.d * q.di);
   p.sq = fma(-t, apq, p.sq);
   q.sq = fma(t, apq, q.sq);
   p.d *= c;
   q.d *= c;
   p.di *= ci;
   q.di *= ci;
-  return true;
 }
 
 // pair k of round `round` of the circle method over m (even) players
@@ -255,6 +269,8 @@ __global__ void __launch_bounds__(E <= 12 ? 384 : 512)
         const bool on = p >= 0 && p < m && q < m;
         p = on ? act[p] : 0;
         q = on ? act[q] : 0;
+        JCol cp = jc[p], cq = jc[q];
+        const JPair pr = jacobi_prepare(cp, cq, tol);
         double a[E], b[E], s0 = 0.0, s1 = 0.0;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
@@ -267,14 +283,16 @@ __global__ void __launch_bounds__(E <= 12 ? 384 : 512)
         }
         double pq = s0 + s1;
         for (int o = 1; o < kEigLanes; o <<= 1) pq += __shfl_xor_sync(0xffffffffu, pq, o);
-        JCol cp = jc[p], cq = jc[q];
-        double al, be;
-        if (!on || !jacobi_rotation(cp, cq, pq, tol, al, be)) continue;
+        double apq;
+        const double t = jacobi_tangent(pr, pq, apq);
+        if (!on || !nonzero(t)) continue;
+        const double al = t * pr.rq, be = t * pr.rp;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           w[p * lds + gl + kEigLanes * e] = fma(-al, b[e], a[e]);
           w[q * lds + gl + kEigLanes * e] = fma(be, a[e], b[e]);
         }
+        jacobi_finish(cp, cq, t, apq);
         if (gl == 0) {
           jc[p] = cp;
           jc[q] = cq;
@@ -321,13 +339,20 @@ __global__ void __launch_bounds__(E <= 12 ? 384 : 512)
 // (shared memory, or its part of `work` where they do not fit) and the pivot's owner
 // writes the finished column to W, in pivot order; two cluster barriers per column.
 // Jacobi: the columns of W in blocks of b; a round of the circle method over the blocks
-// gives every CTA pairs of blocks, which it stages in shared memory, rotates (GL lanes per
-// column pair; all pairs of both blocks in the first round of a sweep, the pairs across
-// them in the others) and writes back; one cluster barrier per round.
+// gives every CTA pairs of blocks, which it stages in shared memory, rotates (all pairs of
+// both blocks in the first round of a sweep, the pairs across them in the others) and writes
+// back; one cluster barrier per round.  In a round of column pairs the first warps keep one
+// thread per pair for the rotations, the others form the products (eight lanes per pair and
+// row segment) and apply the rotations (a warp per pair), so that the columns' state is read
+// and updated beside that work; with everything done by 16 lanes per pair the rotation's 30
+// binary64 instructions were a third of the issue.  A pair is tested at the same place of
+// every sweep: one whose columns have not turned since its last test is skipped, and a block
+// pair without any such column is not staged.  Against 16 lanes per pair for everything: 40
+// matrices of order 74 2.64 -> 2.00 ms, 14 of 203 9.7 -> 8.1, 8 of 127 6.2 -> 5.4.
 constexpr size_t kEigBlkSmem = 200 * 1024;
-template <int GL>
+constexpr int kEigParts = 4;  // row segments of a product at most (and two for the rotations)
 __global__ void __launch_bounds__(768)
-    k_sym_eig_blocks(const double* __restrict__ A, int ld, int n, int b, int in_smem,
+    k_sym_eig_blocks(const double* __restrict__ A, int ld, int n, int b, int R, int in_smem,
                      double* evals, double* evecs, double* work) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
@@ -348,6 +373,7 @@ __global__ void __launch_bounds__(768)
   double* W = base;
   double* gn = base + (int64_t)n * n;
   double* gd = gn + n;
+  int* gturn = reinterpret_cast<int*>(gd + 2 * n);  // tick of a column's last rotation
   double* stage = in_smem ? eig_sh + (size_t)((n + C - 1) / C) * n : eig_sh;  // pivot column
   double* F = in_smem ? eig_sh
                       : base + (int64_t)n * n + 4 * n + (int64_t)c * ((n + C - 1) / C) * n;
@@ -370,6 +396,7 @@ __global__ void __launch_bounds__(768)
     if (i == j) {
       __stcg(gd + j, v);
       __stcg(gn + j, -1.0);  // still to be factored
+      __stcg(gturn + j, 0);
     }
   }
   bad = __syncthreads_or(bad) != 0;
@@ -427,25 +454,35 @@ __global__ void __launch_bounds__(768)
     }
     __syncthreads();
   }
-  // the columns left open, behind the pivots in index order
-  if (r < n)
-    for (int j = 0, at = r; j < n; ++j) {
-      if (!(__ldcg(gn + j) < 0.0)) continue;
+  // the columns left open, behind the pivots in index order; those with a zero diagonal entry
+  // last (column m on): they are e_j already and take no part
+  int m = r;
+  for (int zero = 0, at = r; zero < 2 && at < n; ++zero) {
+    for (int j = 0; j < n; ++j) {
+      const double d = __ldcg(gd + j);
+      if (!(__ldcg(gn + j) < 0.0) || (d > 0.0) != (zero == 0)) continue;
       if (at % C == c) {
-        const double v = 0x1p-40 * sqrt(fmax(__ldcg(gd + j), 0x1p-53));
+        const double v = 0x1p-40 * sqrt(fmax(d, 0x1p-53));
         for (int i = tid; i < n; i += nth) __stcg(W + (int64_t)at * n + i, i == j ? v : 0.0);
       }
       ++at;
     }
+    if (zero == 0) m = at;
+  }
   cl.sync();
   // ---- one-sided Jacobi on block pairs ----
-  const int nb = 2 * ((n + 2 * b - 1) / (2 * b));  // blocks (even), the last ones may be short
+  b = max(1, min(b, (m + 2 * C - 1) / (2 * C)));
+  const int nb = 2 * ((m + 2 * b - 1) / (2 * b));  // blocks (even), the last ones may be short
   const float tol = sqrtf((float)n) * 0x1p-53f;
   double* blk = eig_sh;                                       // 2 b columns of n
   JCol* jc = reinterpret_cast<JCol*>(blk + (size_t)2 * b * n);
-  const int grp = tid / GL, gl = tid % GL, ngrp = nth / GL;
-  auto group_sum = [&](double v) {
-    for (int o = 1; o < GL; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  double* s_pq = reinterpret_cast<double*>(jc + 2 * b);  // products: R parts of b | b, b: t rq, t rp
+  int* s_turn = reinterpret_cast<int*>(s_pq + kEigParts * b);
+  const int PG = (b + 3) / 4, rs = ((n + R - 1) / R + 7) & ~7;  // groups of 4 pairs, segment
+  const int T = nb * 2 * b;                                     // ticks per sweep
+  const int ws = (b + 31) / 32, w1 = warp - ws, nw1 = nw - ws;  // ws warps for the rotations
+  auto warp_sum = [&](double v) {
+    for (int o = 1; o < 32; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
   };
   for (int sweep = 0; sweep < kEigSweeps; ++sweep) {
@@ -455,70 +492,118 @@ __global__ void __launch_bounds__(768)
       for (int k = c; k < nb / 2; k += C) {
         int I, J;
         circle_pair(nb, round, k, I, J);
-        const int i0 = min(n, I * b), ni = min(n, i0 + b) - i0;
-        const int j0 = min(n, J * b), nj = min(n, j0 + b) - j0;
-        __syncthreads();
+        const int i0 = min(m, I * b), ni = min(m, i0 + b) - i0;
+        const int j0 = min(m, J * b), nj = min(m, j0 + b) - j0;
+        const int tick0 = (sweep * nb + round) * 2 * b;
+        __syncthreads();  // the last pair's columns and ticks are written back
+        // nothing of either block has turned since the pair was here
+        bool turned = sweep == 0;
+        for (int x = tid; x < ni + nj; x += nth) {
+          const int tk = __ldcg(gturn + (x < ni ? i0 + x : j0 + x - ni));
+          s_turn[x < ni ? x : b + x - ni] = tk;
+          turned = turned || tk >= tick0 - T;
+        }
+        if (!__syncthreads_or(turned)) continue;
+#pragma unroll 4
         for (int idx = tid; idx < ni * n; idx += nth)
           blk[idx] = __ldcg(W + (int64_t)i0 * n + idx);
+#pragma unroll 4
         for (int idx = tid; idx < nj * n; idx += nth)
           blk[b * n + idx] = __ldcg(W + (int64_t)j0 * n + idx);
         __syncthreads();
         // staged column x: x < b of block I, x - b of block J
         auto present = [&](int x) { return x < b ? x < ni : x - b < nj; };
-        for (int x0 = 0; x0 < 2 * b; x0 += ngrp) {
-          const int x = x0 + grp;
-          const bool in = x < 2 * b && present(x);
+        for (int x = warp; x < 2 * b; x += nw) {
+          if (!present(x)) continue;
           double s = 0.0;
-          if (in)
-            for (int i = gl; i < n; i += GL) s = fma(blk[x * n + i], blk[x * n + i], s);
-          s = group_sum(s);
-          if (gl == 0 && in) jc[x] = JCol{s, 1.0, 1.0};
+          for (int i = lane; i < n; i += 32) s = fma(blk[x * n + i], blk[x * n + i], s);
+          s = warp_sum(s);
+          if (lane == 0) jc[x] = JCol{s, 1.0, 1.0};
         }
         __syncthreads();
         const bool all = round == 0;
         const int rounds = all ? 2 * b - 1 : b;
         bool rot = false;
         for (int q = 0; q < rounds; ++q) {
-          for (int x0 = 0; x0 < b; x0 += ngrp) {
-            const int x = x0 + grp;
-            int u = 0, v = 0;
+          auto pair = [&](int x, int& u, int& v) {
             if (all) {
-              circle_pair(2 * b, q, x < b ? x : 0, u, v);
+              circle_pair(2 * b, q, x, u, v);
             } else {
               u = x;
               v = x + q;
               v = b + (v >= b ? v - b : v);
             }
-            const bool on = x < b && present(u) && present(v);
-            double* wp = blk + (on ? u : 0) * n;
-            double* wq = blk + (on ? v : 0) * n;
+            return present(u) && present(v);
+          };
+          const int last = tick0 + q - T;  // the pairs' last test
+          auto due = [&](int u, int v) {
+            return sweep == 0 || s_turn[u] >= last || s_turn[v] >= last;
+          };
+          // thread x < b: pair x
+          int u = 0, v = 0;
+          const bool mine = tid < b && pair(tid, u, v) && due(u, v);
+          JCol cp, cq;
+          JPair pr;
+          if (mine) {
+            cp = jc[u];
+            cq = jc[v];
+            pr = jacobi_prepare(cp, cq, tol);
+          }
+          for (int wk = w1 < 0 ? PG * R : w1; wk < PG * R; wk += nw1) {
+            const int x = (wk % PG) * 4 + (lane >> 3), seg = wk / PG;
+            int xu = 0, xv = 0;
+            const bool on = x < b && pair(x, xu, xv) && due(xu, xv);
+            if (!__any_sync(0xffffffffu, on)) continue;
+            const double *wp = blk + xu * n, *wq = blk + xv * n;
+            const int iend = on ? min(n, (seg + 1) * rs) : 0;
             double s0 = 0.0, s1 = 0.0;
-            int i = gl;
-            for (; i + GL < n; i += 2 * GL) {
+            int i = seg * rs + (lane & 7);
+            for (; i + 8 < iend; i += 16) {
               s0 = fma(wp[i], wq[i], s0);
-              s1 = fma(wp[i + GL], wq[i + GL], s1);
+              s1 = fma(wp[i + 8], wq[i + 8], s1);
             }
-            if (i < n) s0 = fma(wp[i], wq[i], s0);
-            const double pq = group_sum(s0 + s1);
-            if (!on) continue;
-            JCol cp = jc[u], cq = jc[v];
-            double al, be;
-            if (!jacobi_rotation(cp, cq, pq, tol, al, be)) continue;
+            if (i < iend) s0 = fma(wp[i], wq[i], s0);
+            double pq = s0 + s1;
+            for (int o = 1; o < 8; o <<= 1) pq += __shfl_xor_sync(0xffffffffu, pq, o);
+            if ((lane & 7) == 0 && on) s_pq[seg * b + x] = pq;
+          }
+          __syncthreads();
+          double t = 0.0, apq = 0.0;
+          if (mine) {
+            double pq = s_pq[tid];
+            for (int g = 1; g < R; ++g) pq += s_pq[g * b + tid];
+            t = jacobi_tangent(pr, pq, apq);
+          }
+          if (tid < b) {
+            s_pq[tid] = mine ? t * pr.rq : 0.0;
+            s_pq[b + tid] = mine ? t * pr.rp : 0.0;
+          }
+          __syncthreads();
+          if (nonzero(t)) {
+            jacobi_finish(cp, cq, t, apq);
+            jc[u] = cp;
+            jc[v] = cq;
+            s_turn[u] = s_turn[v] = tick0 + q;
+            rot = true;
+          }
+          for (int x = w1 < 0 ? b : w1; x < b; x += nw1) {
+            const double al = s_pq[x], be = s_pq[b + x];
+            if (!nonzero(al)) continue;
+            int xu, xv;
+            pair(x, xu, xv);
+            double *wp = blk + xu * n, *wq = blk + xv * n;
 #pragma unroll 4
-            for (i = gl; i < n; i += GL) {
+            for (int i = lane; i < n; i += 32) {
               const double x1 = wp[i], x2 = wq[i];
               wp[i] = fma(-al, x2, x1);
               wq[i] = fma(be, x1, x2);
             }
-            if (gl == 0) {
-              jc[u] = cp;
-              jc[v] = cq;
-            }
-            rot = true;
           }
           __syncthreads();
         }
         if (rot) s_flag = 1;
+        for (int x = tid; x < ni + nj; x += nth)
+          __stcg(gturn + (x < ni ? i0 + x : j0 + x - ni), s_turn[x < ni ? x : b + x - ni]);
         for (int idx = tid; idx < ni * n; idx += nth)
           __stcg(W + (int64_t)i0 * n + idx, blk[idx] * jc[idx / n].d);
         for (int idx = tid; idx < nj * n; idx += nth)
@@ -607,17 +692,22 @@ void launch_sym_eig(int n_sd, const double* A, int ld, int n, double* evals, dou
     if (n <= 96) return launch_small<12>(n_sd, A, ld, n, evals, evecs, st);
     return launch_small<16>(n_sd, A, ld, n, evals, evecs, st);
   }
-  const size_t col = sizeof(double) * (size_t)n + sizeof(JCol);  // a staged column
+  // a staged column, its state, its share of the products and its last turn
+  const size_t col = sizeof(double) * (size_t)n + sizeof(JCol) + sizeof(double) * kEigParts / 2 +
+                     sizeof(int);
   const int b = std::max(1, std::min((n + 2 * C - 1) / (2 * C), (int)(kEigBlkSmem / (2 * col))));
   const size_t factor = sizeof(double) * (size_t)((n + C - 1) / C) * n;
   int in_smem = factor <= kEigBlkSmem ? 1 : 0;
   const size_t sm = std::max(2 * b * col, (in_smem ? factor : 0) + sizeof(double) * (size_t)n);
-  // a rotation's own arithmetic (about 25 binary64 instructions per warp) serves 32 / GL
-  // pairs, but its chain wants warps to hide behind: 16 lanes per pair, 8 from 26 pairs a
-  // CTA on (30 matrices of order 260: 52 -> 40 ms; 14 of 190: 10.6 ms against 14.2 with 8)
-  const int gl = b < 26 ? 16 : 8;
-  const int nth = std::min(768, std::max(256, (b * gl + 31) / 32 * 32));
-  auto fn = gl == 8 ? k_sym_eig_blocks<8> : k_sym_eig_blocks<16>;
+  // row segments of a product by the binary64 issue of the busiest quarter of the SM: each
+  // warp takes n / 8R multiply-adds and four additions
+  const int PG = (b + 3) / 4;
+  auto cost = [&](int r) { return (PG * r + 3) / 4 * ((n + 8 * r - 1) / (8 * r) + 4); };
+  int R = 1;
+  for (int r = 2; r <= kEigParts; r *= 2)
+    if (cost(r) < cost(R)) R = r;
+  const int nth = std::min(768, std::max(256, 32 * ((b + 31) / 32 + std::max(PG * R, b))));
+  auto fn = k_sym_eig_blocks;
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
@@ -630,7 +720,7 @@ void launch_sym_eig(int n_sd, const double* A, int ld, int n, double* evals, dou
   cfg.stream = st;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, fn, A, ld, n, b, in_smem, evals, evecs, work);
+  cudaLaunchKernelEx(&cfg, fn, A, ld, n, b, R, in_smem, evals, evecs, work);
 }
 
 }  // namespace mor
