@@ -400,6 +400,15 @@ ResidentPlan resident_plan(int n_sd, int n_max, int W, int nc_max, int kp) {
   // more CTAs per subdomain while the chip is not full and a CTA keeps a warp's worth of rows
   // per warp
   while (2 * S <= kResCluster && 2 * S * tasks <= 152 && n_max / (2 * S) >= NT / 2) S *= 2;
+  // Clusters beyond what the chip holds at once run in waves, each with its own chain of
+  // steps, while a streaming step has one fixed cost for all subdomains.  Builds, streaming
+  // against on chip: binary64 at S = 8 and 5.7 waves 35.4 and 29.2 ms, 11.4 waves 42.1 and
+  // 47.6; S = 4, 6.7 waves 47.6 and 43.0, 13.5 waves 61.5 and 70.5; S = 2, 13.5 waves 39.9
+  // and 38.6, 22 waves 61.9 and 67.9.  Binary32 at S = 8 and 5.7 waves 21.5 and 16.8 ms, 11.4
+  // waves 26.6 and 28.2; S = 4, 13.5 waves 35.2 and 29.1, 22 waves 51.5 and 51.6; S = 2, 23
+  // waves 57.8 and 45.9, 37 waves 89.3 and 86.7
+  const double waves = (double)S * tasks / 152.0;
+  if (sizeof(T) == 8 ? waves * std::min(S, 5) > 30.0 : waves * S > 48.0) return rp;
   rp.S = S;
   rp.smem = res_smem<T>(n_max, (n_max + S - 1) / S, W, nc_max, S);
   return rp;
@@ -410,8 +419,9 @@ void launch_cg_resident(const ResidentPlan& rp, const DTiles& tiles, const EllVi
                         const T* r, T* p, const T* dinv, int kp, double tol2, int steps,
                         const CgState& s, const Coarse<T>& co, int* steps_run, cudaStream_t st) {
   cudaMemsetAsync(s.active, 0, sizeof(int) * (size_t)tiles.n_sd, st);
+  // (one limit for every shape: threads may launch different ones at the same time)
   cudaFuncSetAttribute((const void*)k_cg_resident<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)rp.smem);
+                       (int)ResThreads<T>::smem);
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
   at.val.clusterDim.x = (unsigned)rp.S;
