@@ -660,10 +660,13 @@ template <int E>
 void launch_small(int n_sd, const double* A, int ld, int n, double* evals, double* evecs,
                   cudaStream_t st) {
   const int nth = std::max(64, (std::max(1, (n + 1) / 2) * kEigLanes + 31) / 32 * 32);
-  const size_t sm = sizeof(double) * ((size_t)n * kEigLanes * E + n) + sizeof(JCol) * n +
-                    sizeof(int) * n;
-  cudaFuncSetAttribute(k_sym_eig<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_sym_eig<E><<<n_sd, nth, sm, st>>>(A, ld, n, evals, evecs);
+  auto smem = [](int m) {
+    return sizeof(double) * ((size_t)m * kEigLanes * E + m) + sizeof(JCol) * m + sizeof(int) * m;
+  };
+  // (one limit for every order: threads may launch different ones at the same time)
+  cudaFuncSetAttribute(k_sym_eig<E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)smem(kEigLanes * E));
+  k_sym_eig<E><<<n_sd, nth, smem(n), st>>>(A, ld, n, evals, evecs);
 }
 
 }  // namespace
@@ -708,7 +711,9 @@ void launch_sym_eig(int n_sd, const double* A, int ld, int n, double* evals, dou
     if (cost(r) < cost(R)) R = r;
   const int nth = std::min(768, std::max(256, 32 * ((b + 31) / 32 + std::max(PG * R, b))));
   auto fn = k_sym_eig_blocks;
-  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  // one limit for every order, as above: the factor or the blocks, and a column
+  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)(kEigBlkSmem + sizeof(double) * kEigMax));
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
   at.val.clusterDim.x = (unsigned)C;

@@ -792,8 +792,9 @@ RcgLaunch launch_rcg_solve(int n_sd, int kq, const int32_t* nbr_ptr, const int32
   if (smem(rows) > cap) return RcgLaunch::kNone;
   int rows_max = (int)rows;
   const void* fn = (const void*)k_rcg_grid;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem(rows)) != cudaSuccess)
+  // (one limit for every size: threads may launch different ones at the same time)
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) !=
+      cudaSuccess)
     return RcgLaunch::kNone;
   at.id = cudaLaunchAttributeCooperative;
   at.val.cooperative = 1;

@@ -1708,8 +1708,7 @@ void launch_spmm(const DTiles& tiles, const EllView<T>& A, const T* X, T* Y, int
 
 // Two rows in flight per thread in the updates where a block holds up to eight (more than 28
 // packs of columns): its threads walk 16 or more rows one after another (wide sketches on
-// 25^3: x/r update 47 -> 40 us, p update 26 -> 22).  With 11 packs and 23 rows a block
-// (64^3) the x/r update already runs at 98 % of the copy bandwidth, in 48 registers.
+// 25^3: x/r update 47 -> 40 us, p update 26 -> 22).
 template <typename T>
 bool wide_rows(dim3 bl) {
   return sizeof(T) == 4 && bl.y <= 8;
