@@ -193,7 +193,8 @@ typedef struct {
                           off by at most about 2^-28 rows max|X_i| max|Y_j|), and the
                           coarse-level product E^{-1} r_c of the local solves for up to
                           128 columns (bf16 high and low parts of both factors, three
-                          products, FP32 accumulators); 2 also
+                          products, FP32 accumulators; small subdomains, whose solves
+                          run on chip, keep it in binary32); 2 also
                           forms the interface blocks of Eq. (23) there, whose error is
                           then relative to the largest a_e-weighted entry of a column
                           (at 1e4 coefficient contrast it moves x^T K~ x away from the
