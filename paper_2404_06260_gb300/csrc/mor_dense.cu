@@ -1,6 +1,8 @@
 // Small dense per-subdomain linear algebra of step 2 (Sec. 4, Sec. 6): tall-skinny
 // Grams X^T Y, and the k x k right-multiplications that apply the eigensolver's results
 // (mor_eig.cu) to row blocks.
+#include <algorithm>
+
 #include "mor_kernels.h"
 
 namespace mor {
@@ -74,6 +76,9 @@ __global__ void __launch_bounds__(kGramThreads)
   }
 }
 
+// grid (subdomain, part of the rows).  The roots once per column and block: one per entry, in
+// one block per subdomain, took 149 us for 14 subdomains of up to 203 columns, 22 now.
+constexpr int kMakeMMax = 1024;
 __global__ void k_make_M(int mode, const double* __restrict__ evals,
                          const double* __restrict__ evecs, int ld, int n, double rel, int keep,
                          double* M, int* kept, const int32_t* __restrict__ keep_sd) {
@@ -91,13 +96,19 @@ __global__ void k_make_M(int mode, const double* __restrict__ evals,
     return j < kmax && ev[j] > rel;
   };
   const bool scaled = mode == 0 || mode >= 3;
-  for (int idx = threadIdx.x; idx < ld * ld; idx += blockDim.x) {
+  __shared__ double root[kMakeMMax];  // 0: column not taken
+  for (int j = threadIdx.x; j < n; j += blockDim.x)
+    root[j] = !take(j) ? 0.0 : scaled ? sqrt(ev[j]) : 1.0;
+  __syncthreads();
+  const int la = (int)((int64_t)ld * blockIdx.y / gridDim.y);
+  const int lb = (int)((int64_t)ld * (blockIdx.y + 1) / gridDim.y);
+  for (int idx = la * ld + threadIdx.x; idx < lb * ld; idx += blockDim.x) {
     int l = idx / ld, j = idx % ld;
     double val = 0.0;
-    if (l < n && j < n && take(j)) val = scaled ? V[l * ld + j] / sqrt(ev[j]) : V[l * ld + j];
+    if (l < n && j < n && nonzero(root[j])) val = scaled ? V[l * ld + j] / root[j] : V[l * ld + j];
     Ms[idx] = val;
   }
-  if (threadIdx.x == 0 && kept) {
+  if (threadIdx.x == 0 && blockIdx.y == 0 && kept) {
     int c = 0;
     for (int j = 0; j < n; ++j) c += take(j) ? 1 : 0;
     kept[sd] = c;
@@ -191,7 +202,8 @@ void launch_make_M(int n_sd, int mode, const double* evals, const double* evecs,
                    const int32_t* keep_sd) {
   if (n_sd <= 0) return;
   count_launch();
-  k_make_M<<<n_sd, 256, 0, st>>>(mode, evals, evecs, ld, n, rel, keep, M, kept, keep_sd);
+  const int parts = std::max(1, std::min(16, ld / 16));
+  k_make_M<<<dim3(n_sd, parts), 256, 0, st>>>(mode, evals, evecs, ld, n, rel, keep, M, kept, keep_sd);
 }
 
 void launch_rowmul(const DTiles& tiles, const double* X, int ldx, int nin, const double* M,
