@@ -356,6 +356,7 @@ __global__ void __launch_bounds__(768)
                      double* evals, double* evecs, double* work) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
+  cl.barrier_arrive();  // waited for before the first store to another CTA's shared memory
   extern __shared__ __align__(16) double eig_sh[];
   __shared__ long long s_key[2][8];
   __shared__ int s_rot[2][8];
@@ -400,6 +401,7 @@ __global__ void __launch_bounds__(768)
     }
   }
   bad = __syncthreads_or(bad) != 0;
+  cl.barrier_wait();  // every CTA of the cluster has started
   if (tid < C) *cl.map_shared_rank(&s_rot[0][c], tid) = bad;
   cl.sync();
   for (int g = 0; g < C; ++g) bad = bad || s_rot[0][g];

@@ -280,6 +280,7 @@ __global__ void __launch_bounds__(512)
                   double tol2, int max_iter, int smem_entries, RcgState s) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
+  cl.barrier_arrive();  // waited for before the first store to another CTA's shared memory
   extern __shared__ __align__(16) unsigned char rcg_raw[];
   __shared__ RcgClusterSums<16> sums;
   __shared__ int s_steps[16], s_fit[kRcgCluster];
@@ -301,6 +302,7 @@ __global__ void __launch_bounds__(512)
   __syncthreads();
   int most = 0;
   for (int w = 0; w < nw; ++w) most = max(most, s_steps[w]);
+  cl.barrier_wait();  // every CTA of the cluster has started
   if (tid < G) *cl.map_shared_rank(&s_fit[rank], tid) = (int64_t)most * nth <= smem_entries;
   cl.sync();
   bool fit = true;
