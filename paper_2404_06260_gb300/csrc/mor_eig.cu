@@ -10,10 +10,12 @@
 // touches two columns instead of two rows, two columns and two more of V, and the pivoted
 // factor starts nearly orthogonal: 4 to 7 sweeps.
 //  - Scaling: G by a power of two to a largest diagonal entry in [1, 2).
-//  - A column whose pivot falls below n 2^-53 of its own diagonal entry is rounding noise:
-//    it becomes 2^-40 e_j (times the root of its entry), which the iteration turns into
-//    the completion of the eigenvectors; its eigenvalue (below 2^-70) is returned as 0.
-//    Columns with a zero diagonal entry stay out: eigenvalue 0, eigenvector e_j.
+//  - A column whose pivot falls below n 2^-53 of its own diagonal entry (or below kEigTiny)
+//    is rounding noise and takes no part.  The r columns of the factor give the r largest
+//    eigenvalues, however small; the others are 0, and their eigenvectors complete the basis:
+//    the unit vectors e_j of the columns left out, made orthogonal to all before them by
+//    Gram-Schmidt, repeated while a pass takes half of the vector (Giraud, Langou, Rozloznik
+//    & van den Eshof, Numer. Math. 101, 2005).
 //  - A pair rotates while |w_p.w_q| > sqrt(n) 2^-53 |w_p| |w_q| (the rounding level of the
 //    product); the iteration stops after a sweep without rotations (at most 40).
 //  - The tangent is formed in binary32 and only the orthogonality of the rotation in
@@ -42,6 +44,8 @@ constexpr int kEigSmem = 128;  // largest order of k_sym_eig (128^2 binary64 in 
 constexpr int kEigMax = 1024;
 constexpr int kEigSweeps = 40;
 constexpr int kEigLanes = 8;  // lanes per column pair in k_sym_eig
+// smallest pivot: products of two columns at the rounding level stay normal numbers
+constexpr double kEigTiny = 0x1p-600;
 
 // d^(-1/2) for d in [2^-100, 2^100]: Householder's third-order iteration from binary32
 __device__ __forceinline__ double inv_sqrt(double d) {
@@ -73,24 +77,46 @@ struct JPair {
   double dd;       // d_p d_q
   double diff;     // |q|^2 - |p|^2
   double rp, rq;   // d_p / d_q, d_q / d_p
-  float level;     // |d_p d_q pq| above which the pair rotates
+  float level;     // |d_p d_q pq| 2^k above which the pair rotates
+  int k;           // |p| |q| 2^k lies in [1, 4)
+  bool far;        // norms more than 2^50 apart
 };
+// x 2^k by the exponent bits (no binary64 operation); 0 below the normal range, huge above
+__device__ __forceinline__ double times_pow2(double x, int k) {
+  const int hi = __double2hiint(x), e = ((hi >> 20) & 0x7FF) + k;
+  if (((hi >> 20) & 0x7FF) == 0 || e <= 0) return 0.0;
+  return __hiloint2double(e < 2047 ? hi + k * (1 << 20) : (hi & 0x800FFFFF) | 0x7FE00000,
+                          __double2loint(x));
+}
+// norm^2 = m 4^e with m in [1, 4); a square lost to cancellation counts as the smallest number
+__device__ __forceinline__ float norm_split(double sq, int& e) {
+  const int hi = max(__double2hiint(sq), 0x00100000);
+  e = ((hi >> 20) - 1023) >> 1;
+  return (float)__hiloint2double(hi - e * (1 << 21), __double2loint(sq));
+}
 __device__ __forceinline__ JPair jacobi_prepare(const JCol& p, const JCol& q, float tol) {
   JPair s;
   s.dd = p.d * q.d;
   s.diff = q.sq - p.sq;
   s.rp = p.d * q.di;
   s.rq = q.d * p.di;
-  s.level = tol * (fast_sqrt((float)p.sq) * fast_sqrt((float)q.sq));
+  int ep, eq;
+  const float mp = norm_split(p.sq, ep), mq = norm_split(q.sq, eq);
+  s.level = tol * (fast_sqrt(mp) * fast_sqrt(mq));
+  s.k = -(ep + eq);
+  s.far = abs(ep - eq) > 50;
   return s;
 }
 // the tangent, 0 when the product is at the rounding level (only the angle: binary32 roots
-// and quotients by the fast instructions are exact enough); apq = d_p d_q pq
+// and quotients by the fast instructions are exact enough); apq = d_p d_q pq.  Product and
+// norms go to binary32 relative to |p| |q|: columns of a graded or rank-deficient matrix
+// have norms whose products binary32 does not hold.
 __device__ __forceinline__ double jacobi_tangent(const JPair& s, double pq, double& apq) {
   apq = s.dd * pq;
-  const float o = (float)apq;
+  const float o = (float)times_pow2(apq, s.k);
   if (!(fabsf(o) > s.level)) return 0.0;
-  const float tau = 0.5f * __fdividef((float)s.diff, o);
+  if (s.far) return apq / s.diff;  // the tangent to 2^-90
+  const float tau = 0.5f * __fdividef((float)times_pow2(s.diff, s.k), o);
   const float a = fabsf(tau);
   const float tt = a > 1e8f ? __fdividef(0.5f, a)
                             : __fdividef(1.0f, a + fast_sqrt(fmaf(a, a, 1.0f)));
@@ -117,9 +143,9 @@ __device__ __forceinline__ void circle_pair(int m, int round, int k, int& p, int
   q = b + 1;
 }
 
-// rank by descending value (ties by index) of the n values in ev
+// rank by descending value (ties by index) of ev[i] >= 0 among the n values (negative: last)
 __device__ __forceinline__ int rank_of(const double* ev, int n, int i) {
-  const long long li = __double_as_longlong(ev[i]);  // values >= 0 order like their bits
+  const long long li = __double_as_longlong(ev[i]);  // they order like their bits
   int r = 0;
   for (int j = 0; j < n; ++j) {
     const long long lj = __double_as_longlong(ev[j]);
@@ -184,7 +210,7 @@ __global__ void __launch_bounds__(E <= 12 ? 384 : 512)
       long long best = 0;
       for (int j = lane; j < n; j += 32) {
         const double d = w[j * lds + j];
-        if (nrm[j] < 0.0 && d > noise * g0[j] && d > 0x1p-120) {
+        if (nrm[j] < 0.0 && d > noise * g0[j] && d > kEigTiny) {
           const long long key = (__double_as_longlong(d) & ~255LL) | j;
           best = best > key ? best : key;
         }
@@ -215,24 +241,22 @@ __global__ void __launch_bounds__(E <= 12 ? 384 : 512)
     }
     __syncthreads();
   }
-  // noise columns, and the list of columns that take part
+  // the columns left out become unit vectors, behind the pivots in the list
+  const int m = s_m, me = m + (m & 1);
   for (int j = 0; j < n; ++j)
     if (nrm[j] < 0.0)
-      for (int i = tid; i < lds; i += nth)
-        w[j * lds + i] = i == j ? 0x1p-40 * sqrt(fmax(g0[j], 0x1p-53)) : 0.0;
+      for (int i = tid; i < lds; i += nth) w[j * lds + i] = i == j ? 1.0 : 0.0;
   if (tid < 32) {
-    int c = s_m;
+    int c = m;
     for (int j0 = 0; j0 < n; j0 += 32) {
-      const bool in = j0 + lane < n && nrm[j0 + lane] < 0.0 && g0[j0 + lane] > 0.0;
+      const bool in = j0 + lane < n && nrm[j0 + lane] < 0.0;
       const unsigned b = __ballot_sync(0xffffffffu, in);
       if (in) act[c + __popc(b & ((1u << lane) - 1))] = j0 + lane;
       c += __popc(b);
     }
-    if (lane == 0) s_m = c;
   }
   __syncthreads();
   // ---- one-sided Jacobi ----
-  const int m = s_m, me = m + (m & 1);
   const int grp = tid / kEigLanes, gl = tid % kEigLanes, ngrp = nth / kEigLanes;
   const float tol = sqrtf((float)n) * 0x1p-53f;
   auto squares = [&](int j) {  // squared norm of column j by the 8 lanes of a group
@@ -305,24 +329,64 @@ __global__ void __launch_bounds__(E <= 12 ? 384 : 512)
     __syncthreads();
     if (!rotated) break;
   }
-  // ---- eigenvalues in descending order, normalised columns ----
+  // ---- normalised columns, and the completion of the basis ----
   for (int k0 = 0; k0 < n; k0 += ngrp) {
-    const int j = min(k0 + grp, n - 1);
+    const int j = act[min(k0 + grp, n - 1)];
     const double d = jc[j].d;  // 1 unless the last sweep still rotated
     const double s = d * d * squares(j);
-    const bool in = k0 + grp < n;
-    __syncthreads();
-    if (gl == 0 && in) {
-      nrm[j] = s >= 0x1p-70 && g0[j] > 0.0 ? s : 0.0;
-      g0[j] = s > 0.0 ? d / sqrt(s) : 0.0;  // from here the column's scale
-    }
+    const bool in = k0 + grp < m;
+    const double f = in ? d / sqrt(s) : 1.0;
+    __syncwarp();
+    if (in)
+#pragma unroll
+      for (int e = 0; e < E; ++e) w[j * lds + gl + kEigLanes * e] *= f;
+    if (gl == 0 && k0 + grp < n) g0[j] = in ? s : -1.0;  // from here the eigenvalues
   }
   __syncthreads();
-  for (int i = tid; i < n; i += nth) act[i] = rank_of(nrm, n, i);
+  double* cf = reinterpret_cast<double*>(jc);  // coefficients on the columns before
+  int* rk = reinterpret_cast<int*>(cf + n);
+  for (int t = m; t < n; ++t) {
+    const int j = act[t];
+    double* wj = w + j * lds;
+    bool any = false;
+    for (int k = tid; k < t; k += nth) {
+      cf[k] = w[act[k] * lds + j];
+      any = any || nonzero(cf[k]);
+    }
+    if (!__syncthreads_or(any)) continue;  // a null column: e_j as it is
+    double s0 = 1.0, s1 = 1.0;
+    for (int pass = 0; pass < 4; ++pass) {
+      if (pass > 0) {
+        for (int k0 = 0; k0 < t; k0 += ngrp) {
+          const double* wk = w + act[min(k0 + grp, t - 1)] * lds;
+          double s = 0.0;
+#pragma unroll
+          for (int e = 0; e < E; ++e) s = fma(wk[gl + kEigLanes * e], wj[gl + kEigLanes * e], s);
+          for (int o = 1; o < kEigLanes; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+          if (gl == 0 && k0 + grp < t) cf[k0 + grp] = s;
+        }
+        __syncthreads();
+      }
+      for (int x = tid; x < n; x += nth) {
+        double v = wj[x];
+        for (int k = 0; k < t; ++k) v = fma(-cf[k], w[act[k] * lds + x], v);
+        wj[x] = v;
+      }
+      __syncthreads();
+      s0 = s1;
+      s1 = squares(j);
+      if (pass > 0 && s1 >= 0.25 * s0) break;
+    }
+    __syncthreads();
+    for (int x = tid; x < n; x += nth) wj[x] *= 1.0 / sqrt(s1);
+    __syncthreads();
+  }
+  // ---- eigenvalues in descending order ----
+  for (int k = tid; k < n; k += nth) rk[act[k]] = k < m ? rank_of(g0, n, act[k]) : k;
   __syncthreads();
   for (int i = tid; i < ld; i += nth) {
     if (i < n)
-      ev[act[i]] = nrm[i] / scale;
+      ev[rk[i]] = g0[i] > 0.0 ? g0[i] / scale : 0.0;
     else
       ev[i] = 0.0;
   }
@@ -331,7 +395,7 @@ __global__ void __launch_bounds__(E <= 12 ? 384 : 512)
     if (r >= n || j >= n)
       V[idx] = 0.0;
     else
-      V[(int64_t)r * ld + act[j]] = w[j * lds + r] * g0[j];
+      V[(int64_t)r * ld + rk[j]] = w[j * lds + r];
   }
 }
 
@@ -419,7 +483,7 @@ __global__ void __launch_bounds__(768)
       for (int k = lane; k < own; k += 32) {
         const int j = c + C * k;
         const double d = F[(int64_t)k * n + j];
-        if (__ldcg(gn + j) < 0.0 && d > noise * __ldcg(gd + j) && d > 0x1p-120) {
+        if (__ldcg(gn + j) < 0.0 && d > noise * __ldcg(gd + j) && d > kEigTiny) {
           const long long key = (__double_as_longlong(d) & ~2047LL) | j;
           best = best > key ? best : key;
         }
@@ -456,20 +520,16 @@ __global__ void __launch_bounds__(768)
     }
     __syncthreads();
   }
-  // the columns left open, behind the pivots in index order; those with a zero diagonal entry
-  // last (column m on): they are e_j already and take no part
-  int m = r;
-  for (int zero = 0, at = r; zero < 2 && at < n; ++zero) {
-    for (int j = 0; j < n; ++j) {
-      const double d = __ldcg(gd + j);
-      if (!(__ldcg(gn + j) < 0.0) || (d > 0.0) != (zero == 0)) continue;
-      if (at % C == c) {
-        const double v = 0x1p-40 * sqrt(fmax(d, 0x1p-53));
-        for (int i = tid; i < n; i += nth) __stcg(W + (int64_t)at * n + i, i == j ? v : 0.0);
-      }
-      ++at;
+  // the columns left out, behind the pivots in index order: e_j for now
+  const int m = r;
+  int* left = gturn + n;
+  for (int j = 0, at = r; j < n; ++j) {
+    if (!(__ldcg(gn + j) < 0.0)) continue;
+    if (at % C == c) {
+      for (int i = tid; i < n; i += nth) __stcg(W + (int64_t)at * n + i, i == j ? 1.0 : 0.0);
+      if (tid == 0) __stcg(left + at, j);
     }
-    if (zero == 0) m = at;
+    ++at;
   }
   cl.sync();
   // ---- one-sided Jacobi on block pairs ----
@@ -619,34 +679,99 @@ __global__ void __launch_bounds__(768)
     for (int g = 0; g < C; ++g) any |= s_rot[sweep & 1][g];
     if (!any) break;
   }
-  // ---- eigenvalues in descending order, normalised columns (CTA c: columns c, c + C, ...)
-  double* gs = gd + n;  // squared norms as they are
+  // ---- normalised columns (CTA c: columns c, c + C, ...) ----
   for (int k = warp; k < own; k += nw) {
     const int j = c + C * k;
+    double* wj = W + (int64_t)j * n;
     double s = 0.0;
     for (int i = lane; i < n; i += 32) {
-      const double v = __ldcg(W + (int64_t)j * n + i);
+      const double v = __ldcg(wj + i);
       s = fma(v, v, s);
     }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-      __stcg(gn + j, s >= 0x1p-70 ? s : 0.0);
-      __stcg(gs + j, s);
+    s = warp_sum(s);
+    if (lane == 0) __stcg(gn + j, j < m ? s : -1.0);  // from here the eigenvalues
+    if (j < m) {
+      const double f = 1.0 / sqrt(s);
+      for (int i = lane; i < n; i += 32) __stcg(wj + i, __ldcg(wj + i) * f);
     }
   }
   cl.sync();
+  // ---- completion of the basis: CTA c forms rows x0 to x1 of the vector, a warp every nw-th
+  // column's share; the coefficients of a repeated pass and the norms are summed over the
+  // cluster in `parts` ----
+  double* cf = eig_sh;                    // coefficients on the columns before
+  double* acc = cf + n;                   // 32 rows per warp
+  double* vown = acc + 32 * nw;           // own rows of the vector
+  double* parts = base + (int64_t)n * n + 4 * n;
+  const int x0 = n * c / C, nx = n * (c + 1) / C - x0;
+  for (int t = m; t < n; ++t) {
+    const int j = __ldcg(left + t);
+    bool any = false;
+    for (int k = tid; k < t; k += nth) {
+      cf[k] = __ldcg(W + (int64_t)k * n + j);
+      any = any || nonzero(cf[k]);
+    }
+    for (int x = tid; x < nx; x += nth) vown[x] = x0 + x == j ? 1.0 : 0.0;
+    if (!__syncthreads_or(any)) continue;  // a null column: e_j as it is (for every CTA)
+    double s0 = 1.0, s1 = 1.0;
+    for (int pass = 0; pass < 4; ++pass) {
+      if (pass > 0) {
+        for (int k = warp; k < t; k += nw) {
+          double s = 0.0;
+          for (int x = lane; x < nx; x += 32)
+            s = fma(__ldcg(W + (int64_t)k * n + x0 + x), vown[x], s);
+          s = warp_sum(s);
+          if (lane == 0) __stcg(parts + (int64_t)c * n + k, s);
+        }
+        cl.sync();
+        for (int k = tid; k < t; k += nth) {
+          double s = 0.0;
+          for (int g = 0; g < C; ++g) s += __ldcg(parts + (int64_t)g * n + k);
+          cf[k] = s;
+        }
+        __syncthreads();
+      }
+      for (int xb = 0; xb < nx; xb += 32) {
+        double s = 0.0;
+        if (xb + lane < nx)
+          for (int k = warp; k < t; k += nw)
+            s = fma(cf[k], __ldcg(W + (int64_t)k * n + x0 + xb + lane), s);
+        acc[warp * 32 + lane] = s;
+        __syncthreads();
+        if (warp == 0 && xb + lane < nx) {
+          for (int u = 1; u < nw; ++u) s += acc[u * 32 + lane];
+          vown[xb + lane] -= s;
+        }
+        __syncthreads();
+      }
+      if (warp == 0) {
+        double s = 0.0;
+        for (int x = lane; x < nx; x += 32) s = fma(vown[x], vown[x], s);
+        s = warp_sum(s);
+        if (lane == 0) __stcg(parts + (int64_t)C * n + c, s);
+      }
+      cl.sync();
+      s0 = s1;
+      s1 = 0.0;
+      for (int g = 0; g < C; ++g) s1 += __ldcg(parts + (int64_t)C * n + g);
+      if (pass > 0 && s1 >= 0.25 * s0) break;
+    }
+    const double f = 1.0 / sqrt(s1);
+    for (int x = tid; x < nx; x += nth) __stcg(W + (int64_t)t * n + x0 + x, vown[x] * f);
+    cl.sync();
+  }
+  // ---- eigenvalues in descending order ----
   double* evs = eig_sh;
   for (int i = tid; i < n; i += nth) evs[i] = __ldcg(gn + i);
   __syncthreads();
   for (int k = warp; k < own; k += nw) {
     const int j = c + C * k;
-    int rank = 0;
-    if (lane == 0) rank = rank_of(evs, n, j);
+    int rank = j;
+    if (lane == 0 && j < m) rank = rank_of(evs, n, j);
     rank = __shfl_sync(0xffffffffu, rank, 0);
-    const double inv = 1.0 / sqrt(__ldcg(gs + j));
-    if (lane == 0) ev[rank] = evs[j] / scale;
+    if (lane == 0) ev[rank] = j < m ? evs[j] / scale : 0.0;
     for (int i = lane; i < n; i += 32)
-      V[(int64_t)i * ld + rank] = __ldcg(W + (int64_t)j * n + i) * inv;
+      V[(int64_t)i * ld + rank] = __ldcg(W + (int64_t)j * n + i);
   }
   if (c == 0) {
     for (int i = n + tid; i < ld; i += nth) ev[i] = 0.0;
@@ -703,7 +828,10 @@ void launch_sym_eig(int n_sd, const double* A, int ld, int n, double* evals, dou
   const int b = std::max(1, std::min((n + 2 * C - 1) / (2 * C), (int)(kEigBlkSmem / (2 * col))));
   const size_t factor = sizeof(double) * (size_t)((n + C - 1) / C) * n;
   int in_smem = factor <= kEigBlkSmem ? 1 : 0;
-  const size_t sm = std::max(2 * b * col, (in_smem ? factor : 0) + sizeof(double) * (size_t)n);
+  // the staged blocks; the factor and a column; the completion's coefficients, 32 rows for
+  // each of at most 24 warps, and a vector's share
+  const size_t sm = std::max({2 * b * col, (in_smem ? factor : 0) + sizeof(double) * (size_t)n,
+                              sizeof(double) * (2 * (size_t)n + 32 * 24)});
   // row segments of a product by the binary64 issue of the busiest quarter of the SM: each
   // warp takes n / 8R multiply-adds and four additions
   const int PG = (b + 3) / 4;
