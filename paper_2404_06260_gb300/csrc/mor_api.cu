@@ -594,6 +594,7 @@ struct Build {
   // h_poll[3])
   int poll(const DTiles& tl, const int* active, const int* second = nullptr) {
     launch_count_active(tl, active, d_poll, st, second);
+    CK(cudaGetLastError());  // a refused launch leaves counters that read as "nothing open"
     CK(cudaMemcpyAsync(h_poll, d_poll, 4 * sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     return h_poll[0];
@@ -867,7 +868,7 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
   int kq = round_up4((tol_mode ? k : m_max) + 1);
   int mcols = tol_mode ? k : m_max;
   const bool wide = kp > 80;
-  if (kp > 512)
+  if (kp > kMaxCols)
     return fail(MOR_ERR_ARG, "mor_build_bases: sketch width must be <= 511 columns");
   if (!tol_mode && kq > 128)
     return fail(MOR_ERR_ARG, "mor_build_bases: rank + 1 must be <= 128 basis columns");

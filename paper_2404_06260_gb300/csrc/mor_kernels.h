@@ -108,6 +108,7 @@ struct CgState {
 // rows of one subdomain (rows are in Morton order, so a run is a spatial box);
 // E = Z^T A Z per subdomain, inverted once per matrix.  With aloc = null the
 // preconditioner is D^{-1} alone.
+constexpr int kMaxCols = 512;  // columns of a row block: the sketch, the load, padding to 4
 constexpr int kMaxSlots = 32;  // aggregates meeting one row tile (host-enforced)
 constexpr int kMaxAgg = 1024;  // aggregates per subdomain and matrix (host-enforced)
 constexpr int kCoarseRowsMin = 256;  // fewest rows of E^{-1} per row block of the SIMT product

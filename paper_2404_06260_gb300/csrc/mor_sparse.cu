@@ -68,7 +68,9 @@ struct Smem {
   double* sums;
   Slot2<T>* slots;
 };
-__host__ __device__ __forceinline__ size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
+__host__ __device__ constexpr __forceinline__ size_t align16(size_t x) {
+  return (x + 15) & ~(size_t)15;
+}
 template <typename T>
 __device__ __forceinline__ Smem<T> smem_layout(const Geo& g, int kp, int W) {
   extern __shared__ __align__(16) unsigned char raw[];
@@ -83,7 +85,7 @@ __device__ __forceinline__ Smem<T> smem_layout(const Geo& g, int kp, int W) {
   return s;
 }
 template <typename T>
-__host__ __device__ __forceinline__ size_t smem_bytes(int nch, int rb, int kp, int W) {
+__host__ __device__ constexpr __forceinline__ size_t smem_bytes(int nch, int rb, int kp, int W) {
   size_t nth = (size_t)nch * rb;
   return align16(16 * nth) + align16(sizeof(double) * (nth + 3 * kp)) +
          sizeof(Slot2<T>) * (size_t)kTileRows * ((W + 1) / 2);
@@ -550,7 +552,7 @@ __global__ void k_residual64(DTiles tl, EllView<double> A, const double* __restr
 // rows lie 23 apart, made the x/r update of the 64^3 workload 217 us a launch, now 203.)
 constexpr size_t kRestrictWhole = 32 * 1024;  // a whole tile of r up to this, else equal
 constexpr size_t kRestrictBytes = 24 * 1024;  // parts of at most this (or RB rows)
-__host__ __device__ __forceinline__ int restrict_rows(int rb, int kp, size_t tsz) {
+__host__ __device__ constexpr __forceinline__ int restrict_rows(int rb, int kp, size_t tsz) {
   const size_t tile = (size_t)kTileRows * kp * tsz;
   if (tile <= kRestrictWhole) return kTileRows;
   const int parts = (int)((tile + kRestrictBytes - 1) / kRestrictBytes);
@@ -636,12 +638,12 @@ struct TileRestrict {
 };
 // k_cg_start has a binary64 column-sum area behind the usual layout
 template <typename T>
-__host__ __device__ __forceinline__ size_t start_smem_base(int nch, int rb, int kp) {
+__host__ __device__ constexpr __forceinline__ size_t start_smem_base(int nch, int rb, int kp) {
   return align16(smem_bytes<T>(nch, rb, kp, 0)) +
          sizeof(double) * Pack<T>::N * (size_t)nch * rb;
 }
 template <typename T>
-size_t restrict_smem_bytes(int rb, int kp) {
+constexpr size_t restrict_smem_bytes(int rb, int kp) {
   const int SB = restrict_rows(rb, kp, sizeof(T));
   return align16(sizeof(T) * (size_t)SB * kp) +
          (SB < kTileRows ? align16(sizeof(T) * (size_t)kMaxSlots * kp) : 0) +
@@ -1665,12 +1667,15 @@ __global__ void k_row_abs_max(DTiles tl, EllView<double> A, unsigned long long* 
   if ((threadIdx.x & 31) == 0) atomicMax(out + sd, (unsigned long long)__double_as_longlong(sum));
 }
 
+// rows per pass of a tile kernel's block of about `threads` threads, a pack of columns each
+template <typename T>
+constexpr int block_rows(int kp, int threads) {
+  const int rb = threads / (kp / Pack<T>::N);
+  return rb < 1 ? 1 : rb < kTileRows ? rb : kTileRows;
+}
 template <typename T>
 dim3 block_of(int kp, int threads = 256) {
-  int nch = kp / Pack<T>::N;
-  int rb = std::min(threads / nch, kTileRows);
-  if (rb < 1) rb = 1;
-  return dim3(nch, rb);
+  return dim3(kp / Pack<T>::N, block_rows<T>(kp, threads));
 }
 
 // Threads per block of a step's tile kernels by the row tiles of the subdomains still
@@ -1687,9 +1692,11 @@ int light_threads(int open_tiles) {
 
 }  // namespace
 
+constexpr size_t kSmemSlots = 160 * 1024;  // kernels that stage a tile's slots
+constexpr size_t kSmemRows = 180 * 1024;   // kernels that stage a tile's rows of r
 template <typename T>
-void set_smem_attr(const void* fn) {
-  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+void set_smem_attr(const void* fn, size_t bytes = kSmemSlots) {
+  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 template <typename T>
@@ -1715,9 +1722,26 @@ bool wide_rows(dim3 bl) {
 }
 
 template <typename T>
-size_t slot_kernel_smem(dim3 bl, int kp) {
-  return align16(smem_bytes<T>(bl.x, bl.y, kp, 0)) + restrict_smem_bytes<T>(bl.y, kp);
+constexpr size_t slot_kernel_smem(int nch, int rb, int kp) {
+  return align16(smem_bytes<T>(nch, rb, kp, 0)) + restrict_smem_bytes<T>(rb, kp);
 }
+template <typename T>
+constexpr size_t start_kernel_smem(int nch, int rb, int kp) {
+  return align16(start_smem_base<T>(nch, rb, kp)) + restrict_smem_bytes<T>(rb, kp);
+}
+// every column count a build can have stays within the kernels' limit (the most: 179,712
+// bytes, k_cg_start in binary64 at 512 columns)
+template <typename T>
+constexpr bool rows_smem_fits() {
+  for (int kp = 4; kp <= kMaxCols; kp += 4) {
+    const int nch = kp / Pack<T>::N;
+    for (int threads = 256; threads <= (sizeof(T) == 4 ? 1024 : 256); threads *= 4)
+      if (slot_kernel_smem<T>(nch, block_rows<T>(kp, threads), kp) > kSmemRows) return false;
+    if (start_kernel_smem<T>(nch, block_rows<T>(kp, 256), kp) > kSmemRows) return false;
+  }
+  return true;
+}
+static_assert(rows_smem_fits<float>() && rows_smem_fits<double>(), "shared-memory limit");
 
 template <typename T>
 void launch_coarse_then_p(const DTiles& tiles, int n_sd, const T* r, T* p, const T* dinv,
@@ -1803,11 +1827,11 @@ void launch_cg_start(const DTiles& tiles, const double* b64, double* x64, T* x, 
   if (tiles.n <= 0) return;
   static bool attr = false;
   if (!attr) {
-    set_smem_attr<T>((const void*)k_cg_start<T>);
+    set_smem_attr<T>((const void*)k_cg_start<T>, kSmemRows);
     attr = true;
   }
   dim3 bl = block_of<T>(kp);
-  const size_t sm = align16(start_smem_base<T>(bl.x, bl.y, kp)) + restrict_smem_bytes<T>(bl.y, kp);
+  const size_t sm = start_kernel_smem<T>(bl.x, bl.y, kp);
   count_launch();
   k_cg_start<T><<<tiles.n, bl, sm, st>>>(tiles, b64, x64, x, r, dinv, kp, nc, ncn, rtol2, s, rs,
                                          co);
@@ -1905,9 +1929,9 @@ void launch_cg_step(const DTiles& tiles, const EllView<T>& A, T* x, T* r, T* p, 
     set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 1, 128>);
     set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 2, 128>);
     set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 2, 1024>);
-    set_smem_attr<T>((const void*)k_cg_update_xr<T, 256>);
-    set_smem_attr<T>((const void*)k_cg_update_xr<T, 256, 2>);
-    set_smem_attr<T>((const void*)k_cg_update_xr<T, 1024>);
+    set_smem_attr<T>((const void*)k_cg_update_xr<T, 256>, kSmemRows);
+    set_smem_attr<T>((const void*)k_cg_update_xr<T, 256, 2>, kSmemRows);
+    set_smem_attr<T>((const void*)k_cg_update_xr<T, 1024>, kSmemRows);
     attr = true;
   }
   const int th = light_threads<T>(open_tiles);
@@ -1923,7 +1947,7 @@ void launch_cg_step(const DTiles& tiles, const EllView<T>& A, T* x, T* r, T* p, 
   if (ev) cudaEventRecord(ev[1], st);
   auto fn = th == 1024 ? k_cg_update_xr<T, 1024>
             : wide_rows<T>(bl) ? k_cg_update_xr<T, 256, 2> : k_cg_update_xr<T, 256>;
-  fn<<<tiles.n, bl, slot_kernel_smem<T>(bl, kp), st>>>(tiles, x, r, p, q, dinv, kp, s, co);
+  fn<<<tiles.n, bl, slot_kernel_smem<T>(bl.x, bl.y, kp), st>>>(tiles, x, r, p, q, dinv, kp, s, co);
   if (ev) cudaEventRecord(ev[2], st);
   launch_coarse_then_p<T>(tiles, tiles.n_sd, r, p, dinv, kp, tol2, kCoarseStep, open_tiles, s, co,
                           st, ev ? &ev[3] : nullptr);
@@ -1961,12 +1985,12 @@ void launch_cg_replace(const DTiles& tiles, const double* r64, T* rT, T* pT, con
   if (tiles.n <= 0) return;
   static bool attr = false;
   if (!attr) {
-    set_smem_attr<T>((const void*)k_cg_replace<T>);
+    set_smem_attr<T>((const void*)k_cg_replace<T>, kSmemRows);
     attr = true;
   }
   dim3 bl = block_of<T>(kp);
   count_launch();
-  k_cg_replace<T><<<tiles.n, bl, slot_kernel_smem<T>(bl, kp), st>>>(
+  k_cg_replace<T><<<tiles.n, bl, slot_kernel_smem<T>(bl.x, bl.y, kp), st>>>(
       tiles, r64, rT, dinv, kp, drift * drift, s, rs, co);
   launch_coarse_then_p<T>(tiles, tiles.n_sd, rT, pT, dinv, kp, 0.0, kCoarseReplace,
                           tiles.n, s, co, st, nullptr);
