@@ -284,9 +284,10 @@ typedef struct {
  * launch: a small system in one thread-block cluster, a larger one cooperatively on
  * every SM, where the blocks exchange their partial sums twice per iteration.  Every
  * wait of such an exchange is bounded by the wait budget (mor_set_wait_budget), and a
- * wait that runs out ends the kernel with MOR_ERR_TIMEOUT instead of hanging.  Where a
- * cooperative launch is not possible the same iteration runs as three launches per
- * step. */
+ * wait that runs out ends the kernel with MOR_ERR_TIMEOUT instead of hanging; the blocks of
+ * a cluster, which the hardware starts together, meet at its barrier and need no budget.
+ * Where a cooperative launch is not possible the same iteration runs as three launches
+ * per step. */
 int mor_solve_reduced(const mor_reduced* h, double rtol, int32_t max_iter, void* stream,
                       double* x_dev, mor_solve_info* info);
 
@@ -336,11 +337,11 @@ int mor_solve_reduced_noalloc(int32_t n_sub, int32_t kq, const int32_t* nbr_ptr_
  * Process-wide, not thread-safe.  The paper has no counterpart. */
 int mor_set_wait_budget(double seconds);
 
-/* Test of the timeout path: one thread waits, with the given budget in seconds, on a
- * device flag that nothing sets.  *timed_out [host] = 1 when the wait ran out and the
- * kernel returned (the expected outcome), 0 otherwise; returns MOR_ERR_TIMEOUT in the
- * first case and MOR_OK in the second.  Allocates 16 bytes of device memory for the
- * flag.  The paper has no counterpart. */
+/* Test of the timeout path: four blocks run one exchange of the reduced solve (the same
+ * device code), with the given budget in seconds, and wait for one arrival more than they
+ * make.  *timed_out [host] = 1 when every block's wait ran out and the kernel returned (the
+ * expected outcome), 0 otherwise; returns MOR_ERR_TIMEOUT in the first case and MOR_OK in
+ * the second.  Allocates a few bytes of device memory.  The paper has no counterpart. */
 int mor_debug_wait_timeout(double seconds, int32_t* timed_out);
 
 /* u~ = sum_i S_i Q_i x_i on all nodes (zero on the Dirichlet boundary):

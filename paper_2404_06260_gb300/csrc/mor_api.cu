@@ -1910,19 +1910,22 @@ int mor_debug_wait_timeout(double seconds, int32_t* timed_out) {
   if (!timed_out || !(seconds >= 0.0) || seconds > 10.0)
     return fail(MOR_ERR_ARG, "mor_debug_wait_timeout: bad argument");
   Allocs A;
-  unsigned* sync;
-  int* status;
-  TRY(A.alloc(&sync, 4, true));
-  TRY(A.alloc(&status, 1, true));
+  double* part;
+  int* flag;  // arrivals, error, blocks that gave up
+  TRY(A.alloc(&part, 2 * kTimeoutBlocks, true));
+  TRY(A.alloc(&flag, 3, true));
   const double keep = g_wait_budget_s;
   g_wait_budget_s = seconds;
   const long long cycles = wait_budget_cycles();
   g_wait_budget_s = keep;
-  launch_wait_unset_flag(sync, cycles, status, nullptr);
-  int h = -1;
-  CK(cudaMemcpy(&h, status, sizeof(int), cudaMemcpyDeviceToHost));
-  *timed_out = h == 1 ? 1 : 0;
-  if (h == 1) return fail(MOR_ERR_TIMEOUT, "mor_debug_wait_timeout: the wait ran out");
+  launch_exchange_timeout(part, reinterpret_cast<unsigned*>(flag), flag + 1, cycles, flag + 2,
+                          nullptr);
+  CK(cudaGetLastError());
+  int h[3] = {0, 0, 0};
+  CK(cudaMemcpy(h, flag, sizeof(h), cudaMemcpyDeviceToHost));
+  // every block arrived, waited, and left
+  *timed_out = h[0] == kTimeoutBlocks && h[1] == 1 && h[2] == kTimeoutBlocks ? 1 : 0;
+  if (*timed_out) return fail(MOR_ERR_TIMEOUT, "mor_debug_wait_timeout: the wait ran out");
   return MOR_OK;
 }
 

@@ -165,23 +165,24 @@ __device__ __forceinline__ bool nonzero(double x) {
   return (__double2loint(x) | (__double2hiint(x) << 1)) != 0;
 }
 
-// Bounded wait of one thread until *gen differs from `seen` (any flag that another block
-// or the host sets).  It gives up after
+// Bounded wait of one thread until the arrivals counted in *count (modulo 2^32) reach
+// `want`; an acquire, so that what the arrivals released is visible.  It gives up after
 // `budget` clock cycles, or as soon as *err is non-zero (another block gave up), sets
-// *err to 1 when it is the one that ran out, and returns false; true when the flag
-// moved.  The caller's block then leaves its kernel, so no wait is unbounded.
-__device__ __forceinline__ bool bounded_wait(const volatile unsigned* gen, unsigned seen,
-                                             volatile int* err, long long budget) {
+// *err to 1 when it is the one that ran out, and returns false.  The caller's block then
+// leaves its kernel, so no wait is unbounded.
+__device__ __forceinline__ bool wait_arrivals(const unsigned* count, unsigned want, int* err,
+                                              long long budget) {
   const long long t0 = clock64();
-  while (*gen == seen) {
-    if (*err) return false;
+  while (true) {
+    unsigned c;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(count) : "memory");
+    if ((int)(c - want) >= 0) return true;
+    if (*(volatile int*)err) return false;
     if (clock64() - t0 > budget) {
-      atomicExch((int*)err, 1);
+      atomicExch(err, 1);
       return false;
     }
-    __nanosleep(100);
   }
-  return true;
 }
 
 }  // namespace mor

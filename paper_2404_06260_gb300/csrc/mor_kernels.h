@@ -382,7 +382,11 @@ RcgLaunch launch_rcg_solve(int n_sd, int kq, const int32_t* nbr_ptr, const int32
                            cudaStream_t st);
 // the budget of every bounded wait in SM clock cycles of the current device
 long long wait_budget_cycles();
-void launch_wait_unset_flag(unsigned* sync, long long budget, int* status, cudaStream_t st);
+// test of the wait in that solve's exchange: kTimeoutBlocks blocks and one arrival that never
+// comes; part: 2 * kTimeoutBlocks doubles, count, err and status zeroed by the caller
+constexpr int kTimeoutBlocks = 4;
+void launch_exchange_timeout(double* part, unsigned* count, int* err, long long budget,
+                             int* status, cudaStream_t st);
 void launch_rcg_init(int n_sd, int kq, const double* bt, const RcgState& s,
                      cudaStream_t st);
 void launch_rcg_step(int n_sd, int kq, const int32_t* nbr_ptr, const int32_t* nbr_sd,

@@ -416,6 +416,7 @@ struct RcgXch {
   int* err;
   long long budget;
   unsigned epoch;
+  unsigned peers;  // arrivals per sum: gridDim.x
   int n;        // threads with a value: those below n
   double* red;  // 32 warp sums, [40] status, [41..] results
 };
@@ -443,19 +444,7 @@ __device__ bool rcg_exchange(RcgXch& x, double v, F fin) {
       for (int w = 0; w < nw; ++w) t += red[w];
       __stcg(P + blockIdx.x, t);
       asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(x.count) : "memory");
-      const unsigned want = x.epoch * (unsigned)G;
-      const long long t0 = clock64();
-      unsigned c;
-      while (true) {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(x.count) : "memory");
-        if ((int)(c - want) >= 0) break;
-        if (*(volatile int*)x.err) ok = 0;
-        if (clock64() - t0 > x.budget) {
-          atomicExch(x.err, 1);
-          ok = 0;
-        }
-        if (!ok) break;
-      }
+      ok = wait_arrivals(x.count, x.epoch * x.peers, x.err, x.budget);
     }
     __syncwarp();
     double w[5], t = 0.0;
@@ -533,7 +522,7 @@ __global__ void __launch_bounds__(kRcgThreads)
   const int t_lo = nbr_ptr[sd_lo], t_hi = nbr_ptr[sd_hi];
   const int tcap = kRcgCap / kq;
   const float inv_kq = 1.0f / (float)kq;
-  RcgXch x{part, reinterpret_cast<unsigned*>(s.flag + 3), s.flag + 2, budget, 0u, live, red};
+  RcgXch x{part, reinterpret_cast<unsigned*>(s.flag + 3), s.flag + 2, budget, 0u, gridDim.x, live, red};
   const double* res = red + 41;
   double loc = 0.0;
   for (int i = tid; i < rows; i += kRcgThreads) {
@@ -682,11 +671,14 @@ __global__ void __launch_bounds__(kRcgThreads)
   }
 }
 
-// a bounded wait on a flag that nothing sets (the timeout path of the grid barrier)
-__global__ void k_wait_unset_flag(unsigned* sync, long long budget, int* status) {
-  volatile unsigned* gen = sync + 1;
-  volatile int* err = reinterpret_cast<volatile int*>(sync + 2);
-  if (threadIdx.x == 0) *status = bounded_wait(gen, *gen, err, budget) ? 0 : 1;
+// the timeout path of the solve's exchange: a sum that waits for one arrival more than there
+// are CTAs.  *status: CTAs that gave up
+__global__ void k_exchange_timeout(double* part, unsigned* count, int* err, long long budget,
+                                   int* status) {
+  __shared__ double red[48];
+  RcgXch x{part, count, err, budget, 0u, gridDim.x + 1, (int)blockDim.x, red};
+  if (!rcg_exchange(x, 1.0, [](double t, double* o) { o[0] = t; }) && threadIdx.x == 0)
+    atomicAdd(status, 1);
 }
 
 __global__ void k_lift(int64_t n_o, const int32_t* __restrict__ o_node,
@@ -811,9 +803,10 @@ RcgLaunch launch_rcg_solve(int n_sd, int kq, const int32_t* nbr_ptr, const int32
   return RcgLaunch::kGrid;
 }
 
-void launch_wait_unset_flag(unsigned* sync, long long budget, int* status, cudaStream_t st) {
+void launch_exchange_timeout(double* part, unsigned* count, int* err, long long budget,
+                             int* status, cudaStream_t st) {
   count_launch();
-  k_wait_unset_flag<<<1, 32, 0, st>>>(sync, budget, status);
+  k_exchange_timeout<<<kTimeoutBlocks, 64, 0, st>>>(part, count, err, budget, status);
 }
 
 void launch_lift(int64_t n_o, const int32_t* o_node, const int32_t* o_sd, const double* Q,

@@ -357,7 +357,7 @@ def set_wait_budget(seconds: float):
 
 
 def debug_wait_timeout(seconds: float) -> bool:
-    """True when a bounded wait on a flag nothing sets ran out and returned."""
+    """True when the reduced solve's exchange, one arrival short, ran out and returned."""
     t = _i32()
     rc = _lib.mor_debug_wait_timeout(float(seconds), ctypes.byref(t))
     if rc not in (MOR_OK, MOR_ERR_TIMEOUT):
