@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cmath>
 #include <atomic>
+#include <system_error>
 #include <thread>
 
 #include "../../include/mor.h"
@@ -18,12 +19,18 @@ void parallel_for(int n, int n_threads, F f) {
   if (n <= 0) return;
   int nt = std::max(1, std::min(n_threads, n));
   std::atomic<int> next(0);
+  auto work = [&](int t) {
+    int i;
+    while ((i = next.fetch_add(1)) < n) f(i, t);
+  };
   std::vector<std::thread> th;
-  for (int t = 0; t < nt; ++t)
-    th.emplace_back([&, t] {
-      int i;
-      while ((i = next.fetch_add(1)) < n) f(i, t);
-    });
+  th.reserve(nt);
+  try {
+    for (int t = 0; t < nt; ++t) th.emplace_back(work, t);
+  } catch (const std::system_error&) {
+    // no more threads to be had: the calling one takes the place of the first that is missing
+    work((int)th.size());
+  }
   for (auto& x : th) x.join();
 }
 
