@@ -649,9 +649,9 @@ struct Build {
     bool seen = false;  // a residual sweep of this solve has marked what it settled
     const int check = 8;
     const int every = std::max(check, o->replace_every / check * check);
-    int it = 0, open_tiles = tl.n;
+    int it = 0, first = 0, open_tiles = tl.n;  // first: the streaming steps start there
     // the kernel times of the roofline are those of the streaming kernels
-    const ResidentPlan rp =
+    ResidentPlan rp =
         g_prof.on ? ResidentPlan() : resident_plan<T>(n_sd, n_rows[set], AT.W, co.n_max, kp);
     while (true) {
       int act = 0;
@@ -660,8 +660,9 @@ struct Build {
         // contract: every shape the process meets has an entry)
         if (it == 0) tune_spmm<T>(tl, AT, p, q, kp, cs, st);
         CK(cudaMemsetAsync(d_poll + 3, 0, sizeof(int), st));
-        launch_cg_resident<T>(rp, tl, AT, x, r, p, dinvT, kp, rtol2,
-                              std::min(every, o->max_iter - it), cs, co, d_poll + 3, st);
+        if (!launch_cg_resident<T>(rp, tl, AT, x, r, p, dinvT, kp, rtol2,
+                                   std::min(every, o->max_iter - it), cs, co, d_poll + 3, st))
+          rp.S = 0, first = it;  // refused: streaming steps from here
       }
       int chunk = rp.S > 0 ? 0 : std::min(check, o->max_iter - it);
       for (int c = 0; c < chunk; ++c) {
@@ -679,7 +680,7 @@ struct Build {
         act = poll(tl, cs.active);
         open_tiles = h_poll[2];
       }
-      if (rp.S > 0 || act == 0 || it % every == 0 || it >= o->max_iter) {
+      if (rp.S > 0 || act == 0 || (it - first) % every == 0 || it >= o->max_iter) {
         launch_accum_reset<T>(tl, x, x64, kp, seen, rs, st);
         launch_residual64(tl, A.e64(), b64, x64, vR64, kp, nc, rtol2, seen, false, anorm[set],
                           rs, st);
@@ -1168,6 +1169,7 @@ static int build_bases_core(const mor_subdomains* sd, const mor_basis_opts* opts
   TRY(M.alloc(&B.cs.counter, n_sd, true, st));
   TRY(M.alloc(&B.cs.iters, n_sd, true, st));
   TRY(M.alloc(&B.cs.active, n_sd, true, st));
+  TRY(M.alloc(&B.cs.active_next, n_sd, true, st));
   TRY(M.alloc(&B.rs.obb, (size_t)n_sd * kp, true, st));
   TRY(M.alloc(&B.rs.orr, (size_t)n_sd * kp, true, st));
   TRY(M.alloc(&B.rs.scale, (size_t)n_sd * kp, true, st));

@@ -93,6 +93,7 @@ struct CgState {
   int* counter;                     // n_sd
   int* iters;                       // n_sd
   int* active;                      // n_sd: active columns after the last update
+  int* active_next;                 // n_sd: the same while an on-chip launch counts them
   // work counters of the algorithmic-bytes model, kept by the coarse kernel (once per
   // subdomain and step; null: not counted): work[k * n_sd + sd] with k = [0] stored
   // entries read by the sparse product, [1] (row, open pack) pairs of the sparse
@@ -173,8 +174,10 @@ void tune_spmm(const DTiles& tiles, const EllView<T>& A, const T* p, T* q, int k
                const CgState& s, cudaStream_t st);
 // Small subdomains: up to `steps` CG steps in one launch with the data on chip
 // (mor_resident.cu).  resident_plan: S = 0 where the largest subdomain (n_max rows, nc_max
-// aggregates, slot stride W) does not fit.  Zeroes s.active and fills it with the open
-// columns; steps_run takes the largest number of steps (zeroed by the caller).
+// aggregates, slot stride W) does not fit.  The launch counts the open columns into
+// s.active_next, which becomes s.active; steps_run takes the largest number of steps (zeroed
+// by the caller).  False where the launch is refused: nothing has changed, and the streaming
+// steps can go on from the same state.
 struct ResidentPlan {
   int S = 0;
   size_t smem = 0;
@@ -182,9 +185,9 @@ struct ResidentPlan {
 template <typename T>
 ResidentPlan resident_plan(int n_sd, int n_max, int W, int nc_max, int kp);
 template <typename T>
-void launch_cg_resident(const ResidentPlan& rp, const DTiles& tiles, const EllView<T>& A, T* x,
+bool launch_cg_resident(const ResidentPlan& rp, const DTiles& tiles, const EllView<T>& A, T* x,
                         const T* r, T* p, const T* dinv, int kp, double tol2, int steps,
-                        const CgState& s, const Coarse<T>& co, int* steps_run, cudaStream_t st);
+                        CgState& s, const Coarse<T>& co, int* steps_run, cudaStream_t st);
 // out[0] = sum of active[0..n_sd), out[1] = sum of second (0 if null), out[2] = row tiles of
 // the subdomains with active > 0
 void launch_count_active(const DTiles& tiles, const int* active, int* out, cudaStream_t st,

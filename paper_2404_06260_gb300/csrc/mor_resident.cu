@@ -18,6 +18,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <utility>
 
 #include "mor_kernels.h"
 
@@ -373,7 +374,7 @@ __global__ void __launch_bounds__(ResThreads<T>::n, 1)
     const int i = sd * kp + c0 + tid;
     s.rr[i] = res[0][tid];
     s.done[i] = c_done[tid];
-    if (!c_done[tid]) atomicAdd(s.active + sd, 1);
+    if (!c_done[tid]) atomicAdd(s.active_next + sd, 1);
     if (tid == 0) {
       atomicMax(s.iters + sd, it);
       atomicMax(steps_run, it);
@@ -415,13 +416,14 @@ ResidentPlan resident_plan(int n_sd, int n_max, int W, int nc_max, int kp) {
 }
 
 template <typename T>
-void launch_cg_resident(const ResidentPlan& rp, const DTiles& tiles, const EllView<T>& A, T* x,
+bool launch_cg_resident(const ResidentPlan& rp, const DTiles& tiles, const EllView<T>& A, T* x,
                         const T* r, T* p, const T* dinv, int kp, double tol2, int steps,
-                        const CgState& s, const Coarse<T>& co, int* steps_run, cudaStream_t st) {
-  cudaMemsetAsync(s.active, 0, sizeof(int) * (size_t)tiles.n_sd, st);
+                        CgState& s, const Coarse<T>& co, int* steps_run, cudaStream_t st) {
+  cudaMemsetAsync(s.active_next, 0, sizeof(int) * (size_t)tiles.n_sd, st);
   // (one limit for every shape: threads may launch different ones at the same time)
-  cudaFuncSetAttribute((const void*)k_cg_resident<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)ResThreads<T>::smem);
+  cudaError_t e = cudaFuncSetAttribute((const void*)k_cg_resident<T>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)ResThreads<T>::smem);
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
   at.val.clusterDim.x = (unsigned)rp.S;
@@ -433,20 +435,26 @@ void launch_cg_resident(const ResidentPlan& rp, const DTiles& tiles, const EllVi
   cfg.stream = st;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
+  if (e == cudaSuccess)
+    e = cudaLaunchKernelEx(&cfg, k_cg_resident<T>, tiles, A, x, r, p, dinv, kp, tol2, steps, s,
+                           co, steps_run);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
   count_launch();
-  cudaLaunchKernelEx(&cfg, k_cg_resident<T>, tiles, A, x, r, p, dinv, kp, tol2, steps, s, co,
-                     steps_run);
+  std::swap(s.active, s.active_next);
+  return true;
 }
 
 template ResidentPlan resident_plan<float>(int, int, int, int, int);
 template ResidentPlan resident_plan<double>(int, int, int, int, int);
-template void launch_cg_resident<float>(const ResidentPlan&, const DTiles&, const EllView<float>&,
+template bool launch_cg_resident<float>(const ResidentPlan&, const DTiles&, const EllView<float>&,
                                         float*, const float*, float*, const float*, int, double,
-                                        int, const CgState&, const Coarse<float>&, int*,
-                                        cudaStream_t);
-template void launch_cg_resident<double>(const ResidentPlan&, const DTiles&,
+                                        int, CgState&, const Coarse<float>&, int*, cudaStream_t);
+template bool launch_cg_resident<double>(const ResidentPlan&, const DTiles&,
                                          const EllView<double>&, double*, const double*, double*,
-                                         const double*, int, double, int, const CgState&,
+                                         const double*, int, double, int, CgState&,
                                          const Coarse<double>&, int*, cudaStream_t);
 
 }  // namespace mor
