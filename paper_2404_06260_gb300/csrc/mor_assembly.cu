@@ -22,12 +22,15 @@ __global__ void k_elem_stiff(int64_t n_tets, const double* __restrict__ xyz,
     for (int b = 0; b <= a; ++b) e[1 + a * (a + 1) / 2 + b] = dot3(G[a], G[b]) * vol;
 }
 
-// One thread per row.  Both spaces of the 64^3 workload: 6.8 ms with the geometry worked out
-// per (row, element), 2.8 from the element table.
+// One thread per row.  kTable: the geometry from the element table, else worked out per (row,
+// element), with the same operations.  Both spaces of the 64^3 workload: 6.8 ms without the
+// table, 2.8 with it.
+template <bool kTable>
 __global__ void k_assemble(int64_t n_rows, const int64_t* __restrict__ inc_ptr,
                            const int32_t* __restrict__ inc_tet,
                            const uint32_t* __restrict__ inc_code, int W,
-                           const double* __restrict__ elem, const double* __restrict__ kappa,
+                           const double* __restrict__ elem, const double* __restrict__ xyz,
+                           const int32_t* __restrict__ tets, const double* __restrict__ kappa,
                            int h1w, double* valA, double* valH, double* load, int* err) {
   int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (r >= n_rows) return;
@@ -37,7 +40,11 @@ __global__ void k_assemble(int64_t n_rows, const int64_t* __restrict__ inc_ptr,
     uint32_t code = inc_code[q];
     int a = code & 3u;
     const double* e = elem + kElemDoubles * (int64_t)t;
-    const double vol = e[0];
+    double G[4][3], vol;
+    if constexpr (kTable)
+      vol = e[0];
+    else if (!tet_gradients(xyz, tets, t, G, vol))
+      vol = -1.0;
     if (!(vol >= 0.0)) {
       atomicExch(err, 1);
       return;
@@ -49,7 +56,11 @@ __global__ void k_assemble(int64_t n_rows, const int64_t* __restrict__ inc_ptr,
       uint32_t slot = (code >> (2 + 7 * b)) & 127u;
       if (slot == 127u) continue;
       const int hi = max(a, b), lo = min(a, b);
-      double g = e[1 + hi * (hi + 1) / 2 + lo];
+      double g;
+      if constexpr (kTable)
+        g = e[1 + hi * (hi + 1) / 2 + lo];
+      else  // (dot3 is the same either way round)
+        g = dot3(G[a], G[b]) * vol;
       int64_t at = ell_at(r, (int)slot, W);
       valA[at] += kap * g;
       valH[at] += hk * g + vol * (a == b ? 0.1 : 0.05);
@@ -68,14 +79,16 @@ void launch_elem_stiff(int64_t n_tets, const double* xyz, const int32_t* tets, d
 }
 
 void launch_assemble(int64_t n_rows, const int64_t* inc_ptr, const int32_t* inc_tet,
-                     const uint32_t* inc_code, int W, const double* elem, const double* kappa,
-                     int h1_weighted, double* valA, double* valH, double* load, int* err,
-                     cudaStream_t st) {
+                     const uint32_t* inc_code, int W, const double* elem, const double* xyz,
+                     const int32_t* tets, const double* kappa, int h1_weighted, double* valA,
+                     double* valH, double* load, int* err, cudaStream_t st) {
   if (n_rows <= 0) return;
   int bs = 128;
   count_launch();
-  k_assemble<<<(unsigned)((n_rows + bs - 1) / bs), bs, 0, st>>>(
-      n_rows, inc_ptr, inc_tet, inc_code, W, elem, kappa, h1_weighted, valA, valH, load, err);
+  auto fn = elem ? k_assemble<true> : k_assemble<false>;
+  fn<<<(unsigned)((n_rows + bs - 1) / bs), bs, 0, st>>>(n_rows, inc_ptr, inc_tet, inc_code, W,
+                                                        elem, xyz, tets, kappa, h1_weighted, valA,
+                                                        valH, load, err);
 }
 
 // element H1 matrix H_T = w_T |T| grad.grad + |T|(1 + d_ab)/20 (w_T = k_T when the H1

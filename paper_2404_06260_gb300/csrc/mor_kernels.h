@@ -27,10 +27,11 @@ int set_error(int code, const std::string& msg);
 // into valH (w_T = k_T if h1_weighted, else 1), load |T|/4 into load[row].  err is set
 // to 1 on det <= 0.
 void launch_assemble(int64_t n_rows, const int64_t* inc_ptr, const int32_t* inc_tet,
-                     const uint32_t* inc_code, int W, const double* elem, const double* kappa,
-                     int h1_weighted, double* valA, double* valH, double* load, int* err,
-                     cudaStream_t st);
-// the element table `elem` of the assembly: kElemDoubles per element
+                     const uint32_t* inc_code, int W, const double* elem, const double* xyz,
+                     const int32_t* tets, const double* kappa, int h1_weighted, double* valA,
+                     double* valH, double* load, int* err, cudaStream_t st);
+// the element table `elem` of the assembly: kElemDoubles per element (null: no table, the
+// geometry is worked out per row and element)
 constexpr int kElemDoubles = 11;
 void launch_elem_stiff(int64_t n_tets, const double* xyz, const int32_t* tets, double* elem,
                        cudaStream_t st);
