@@ -365,6 +365,7 @@ void launch_pair_blocks(int n_pairs, const int64_t* pair_ptr, const int32_t* uro
                         double* blocks, cudaStream_t st);
 struct RcgState {
   double *x, *r, *p, *q;    // dim
+  double* w;                // rcg_grid_work() doubles, or null
   double* part;             // n_sd x 2 (three-launch iteration)
   int* counter;             // 1
   double* scal;             // [0] rz, [1] bb, [2] alpha, [3] beta, [4] rr, [6] b~.x
@@ -378,6 +379,9 @@ struct RcgState {
 // flag[2] = 2 says that the matrix did not fit into one cluster: launch again with
 // try_cluster = false.
 constexpr int kRcgMaxGrid = 512;
+// doubles of s.w that the launch on every SM needs beside r, p and q: none while a CTA's rows
+// fit in shared memory
+size_t rcg_grid_work(int n_sd, int kq);
 enum class RcgLaunch { kNone, kCluster, kGrid };
 RcgLaunch launch_rcg_solve(int n_sd, int kq, const int32_t* nbr_ptr, const int32_t* nbr_sd,
                            const int32_t* nbr_blk, int64_t n_blocks, const double* blocks,

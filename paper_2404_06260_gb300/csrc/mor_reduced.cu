@@ -404,6 +404,8 @@ __global__ void __launch_bounds__(512)
 constexpr int kRcgThreads = 512;
 constexpr int kRcgCap = 3072;  // neighbour columns staged at a time
 constexpr size_t kRcgStageBytes = kRcgCap * (sizeof(double) + sizeof(int64_t));
+size_t rcg_grid_smem(int64_t rows) { return 4 * sizeof(double) * (size_t)rows + kRcgStageBytes; }
+size_t rcg_smem_cap(int smem_max) { return std::min<size_t>(200 * 1024, (size_t)smem_max); }
 
 // part: 2 parities x gridDim.x partial sums; *count: arrivals since the launch (zeroed
 // before it).  A CTA rewrites a parity only after every CTA has arrived with the other one,
@@ -496,6 +498,9 @@ __device__ int rcg_first_unit(int b, int G, int n_sd, int upb, const int32_t* nb
   return (int)min(units, (int64_t)lo * upb + min(k, (int64_t)upb));
 }
 
+// kShared: the CTA's rows of x, r, p and q in shared memory; else in x, s.r and s.w (each row
+// is read and written by its CTA alone, r and p by the neighbours as ever).
+template <bool kShared>
 __global__ void __launch_bounds__(kRcgThreads)
     k_rcg_grid(int n_sd, int kq, const int32_t* __restrict__ nbr_ptr,
                const int32_t* __restrict__ nbr_sd, const int32_t* __restrict__ nbr_blk,
@@ -503,11 +508,7 @@ __global__ void __launch_bounds__(kRcgThreads)
                int max_iter, int rows_max, int weighted, RcgState s, double* part,
                long long budget) {
   extern __shared__ __align__(16) unsigned char rcg_raw[];
-  double* xs = reinterpret_cast<double*>(rcg_raw);
-  double* rs = xs + rows_max;
-  double* ps = rs + rows_max;
-  double* qs = ps + rows_max;
-  double* pj = qs + rows_max;
+  double* pj = reinterpret_cast<double*>(rcg_raw);
   int64_t* off = reinterpret_cast<int64_t*>(pj + kRcgCap);
   __shared__ double red[48];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -516,6 +517,18 @@ __global__ void __launch_bounds__(kRcgThreads)
   const int u1 = rcg_first_unit(blockIdx.x + 1, gridDim.x, n_sd, upb, nbr_ptr, weighted);
   const int64_t row0 = rcg_row(u0, upb, kq), row1 = rcg_row(u1, upb, kq);
   const int rows = (int)(row1 - row0);
+  double *xs, *rs, *ps, *qs;
+  if constexpr (kShared) {
+    xs = reinterpret_cast<double*>(off + kRcgCap);
+    rs = xs + rows_max;
+    ps = rs + rows_max;
+    qs = ps + rows_max;
+  } else {
+    xs = s.x + row0;
+    rs = s.r + row0;
+    ps = s.w + row0;
+    qs = s.w + (int64_t)n_sd * kq + row0;
+  }
   const int live = min(rows, kRcgThreads);
   // the neighbour entries of the block rows this CTA touches
   const int sd_lo = u0 / upb, sd_hi = u1 > u0 ? (u1 - 1) / upb + 1 : sd_lo;
@@ -657,7 +670,7 @@ __global__ void __launch_bounds__(kRcgThreads)
   // x and E = b~.x
   loc = 0.0;
   for (int i = tid; i < rows; i += kRcgThreads) {
-    s.x[row0 + i] = xs[i];
+    if constexpr (kShared) s.x[row0 + i] = xs[i];
     loc += bt[row0 + i] * xs[i];
   }
   if (!rcg_exchange(x, loc, [](double t, double* o) { o[0] = t; })) return;
@@ -726,6 +739,44 @@ void launch_rcg_step(int n_sd, int kq, const int32_t* nbr_ptr, const int32_t* nb
   k_rcg_update_p<<<n_sd, 128, 0, st>>>(kq, s);
 }
 
+// shape of k_rcg_grid on nsm SMs: CTAs, rows of the largest run and whether runs are weighted;
+// rows = 0: more than shared memory holds (at 152 SMs above 739,000 rows of K~)
+struct RcgGrid {
+  int G, rows, weighted;
+};
+static RcgGrid rcg_grid_shape(int64_t units, int nsm, size_t smem_max) {
+  RcgGrid g;
+  g.G = (int)std::min<int64_t>(std::min(nsm, kRcgMaxGrid), units);
+  // weighted runs hold at most five times the mean number of units; where that does not
+  // fit in shared memory, runs of equal length
+  const int64_t mean = (units + g.G - 1) / g.G;
+  for (g.weighted = 1; g.weighted >= 0; --g.weighted) {
+    const int64_t rows = g.weighted ? 4 * (5 * mean + 2) : 4 * mean;
+    if (rcg_grid_smem(rows) <= smem_max) {
+      g.rows = (int)rows;
+      return g;
+    }
+  }
+  g.rows = 0;
+  g.weighted = 1;
+  return g;
+}
+static int rcg_units(int n_sd, int kq) {
+  const int64_t units = (int64_t)n_sd * ((kq + 3) / 4);
+  return units > INT32_MAX ? 0 : (int)units;
+}
+
+size_t rcg_grid_work(int n_sd, int kq) {
+  int dev = 0, nsm = 0, smem_max = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  const int units = rcg_units(n_sd, kq);
+  if (units < 1 || nsm < 1) return 0;
+  const bool shared = rcg_grid_shape(units, nsm, rcg_smem_cap(smem_max)).rows > 0;
+  return shared ? 0 : 2 * (size_t)n_sd * kq;
+}
+
 RcgLaunch launch_rcg_solve(int n_sd, int kq, const int32_t* nbr_ptr, const int32_t* nbr_sd,
                            const int32_t* nbr_blk, int64_t n_blocks, const double* blocks,
                            const double* bt, double tol2, int max_iter, const RcgState& s,
@@ -769,32 +820,22 @@ RcgLaunch launch_rcg_solve(int n_sd, int kq, const int32_t* nbr_ptr, const int32
     }
     cudaGetLastError();
   }
-  const int64_t units = (int64_t)n_sd * ((kq + 3) / 4);
-  if (!coop || kq > kRcgCap || units > INT32_MAX || nsm < 1) return RcgLaunch::kNone;
-  const int G = (int)std::min<int64_t>(std::min(nsm, kRcgMaxGrid), units);
-  // weighted runs hold at most five times the mean number of units; where that does not
-  // fit in shared memory, runs of equal length
-  const int64_t mean = (units + G - 1) / G;
-  int weighted = 1;
-  int64_t rows = 4 * (5 * mean + 2);
-  const auto smem = [&](int64_t r) { return 4 * sizeof(double) * (size_t)r + kRcgStageBytes; };
-  const size_t cap = std::min<size_t>(200 * 1024, (size_t)smem_max);
-  if (smem(rows) > cap) {
-    weighted = 0;
-    rows = 4 * mean;
-  }
-  if (smem(rows) > cap) return RcgLaunch::kNone;
-  int rows_max = (int)rows;
-  const void* fn = (const void*)k_rcg_grid;
+  const int units = rcg_units(n_sd, kq);
+  if (!coop || kq > kRcgCap || units < 1 || nsm < 1) return RcgLaunch::kNone;
+  const size_t cap = rcg_smem_cap(smem_max);
+  const RcgGrid g = rcg_grid_shape(units, nsm, cap);
+  if (g.rows == 0 && !s.w) return RcgLaunch::kNone;
+  int rows_max = g.rows, weighted = g.weighted;
+  const void* fn = g.rows > 0 ? (const void*)k_rcg_grid<true> : (const void*)k_rcg_grid<false>;
   // (one limit for every size: threads may launch different ones at the same time)
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) !=
       cudaSuccess)
     return RcgLaunch::kNone;
   at.id = cudaLaunchAttributeCooperative;
   at.val.cooperative = 1;
-  cfg.gridDim = dim3((unsigned)G);
+  cfg.gridDim = dim3((unsigned)g.G);
   cfg.blockDim = dim3(kRcgThreads);
-  cfg.dynamicSmemBytes = smem(rows);
+  cfg.dynamicSmemBytes = rcg_grid_smem(rows_max);
   void* args[] = {&n_sd, &kq, (void*)&nbr_ptr, (void*)&nbr_sd, (void*)&nbr_blk,
                   (void*)&blocks, (void*)&bt, &tol2, &max_iter, &rows_max, &weighted, &sc,
                   &part, &budget};
