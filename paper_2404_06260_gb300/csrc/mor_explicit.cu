@@ -56,10 +56,20 @@ __global__ void k_ell_to_dense(int64_t n_rows, const int32_t* __restrict__ row_s
   }
 }
 
-// b / d from r = 1 / d rounded: the quotient b r with one correction step, faithful to the
-// last bit; the reciprocal of a pivot is formed once for all the entries it divides
+// b / d within one unit in the last place from r = 1 / d rounded: the product b r and one
+// step of Markstein's correction, whose remainder is exact (P. Markstein, IBM J. Res. Dev.
+// 34, 1990).  The reciprocal of a pivot is formed once for all the entries it divides.  That
+// holds while r is a normal number, the remainder does not underflow (b = 0 or above 2^-959)
+// and the quotient does not overflow; elsewhere, and for infinities and NaN, it divides: in a
+// function of its own, as the compiler would otherwise run the division beside the product.
+// (Division everywhere: diagonal block 49 -> 76 us, panel 42 -> 82, column solve 261 -> 355.)
+__device__ __noinline__ double div_slow(double b, double d) { return b / d; }
 __device__ __forceinline__ double div_by(double b, double d, double r) {
   const double q = b * r;
+  const int eb = (__double2hiint(b) >> 20) & 0x7FF, ed = (__double2hiint(d) >> 20) & 0x7FF;
+  const bool safe = (unsigned)(ed - 2) <= 2042u && eb - ed < 1000 && (eb >= 64 || !nonzero(b)) &&
+                    eb < 2047;
+  if (!safe) return div_slow(b, d);
   return fma(fma(-d, q, b), r, q);
 }
 
@@ -67,7 +77,7 @@ __device__ __forceinline__ double div_by(double b, double d, double r) {
 // L D L^T in registers (lower triangle, one multiply-add per entry and column), the square
 // roots of the pivots at the end, in parallel.  A non-positive pivot sets *bad.  A chain of
 // nb steps: a square root in front of every division and the update's index arithmetic
-// made a step 4,500 clocks.  8 blocks of 64: 46 us, with the panel below 81 instead of 300.
+// made a step 4,500 clocks.  8 blocks of 64: 49 us, with the panel below 91 instead of 300.
 constexpr int kPotrfOwn = (kNB * (kNB + 1) / 2 + 255) / 256;  // entries per thread
 __global__ void __launch_bounds__(256)
     k_potrf_diag(double* D, const int64_t* __restrict__ doff, const int32_t* __restrict__ nn,
@@ -141,7 +151,7 @@ __global__ void __launch_bounds__(256)
 // A[i, j0:j0+nb].  32 rows per block, four lanes per row, each with every fourth column in
 // registers: x_c comes by shuffle and its multiply-adds on the columns behind it are
 // independent.  grid (n_sd, row chunks).  One thread per row and one block per subdomain
-// cost most of 300 us a panel; 35 now (8 subdomains of order up to 340).
+// cost most of 300 us a panel; 42 now (8 subdomains of order up to 340).
 constexpr int kPanelRows = 32;
 __global__ void __launch_bounds__(4 * kPanelRows)
     k_potrf_panel(double* D, const int64_t* __restrict__ doff, const int32_t* __restrict__ nn,
@@ -264,7 +274,7 @@ __global__ void k_transpose_block(const double* __restrict__ In, const int64_t* 
 // are columns `col` of rows [roff[sd], roff[sd] + n) of X (leading dimension ldx), solved in
 // place, staged in shared memory beside the reciprocals of the diagonal.  Bound by binary64
 // issue: with one vector per block its eight warps each repeated the division of every step,
-// 8 of its 9 operations: 1.14 -> 0.25 ms a solve (8 subdomains of order about 250, 100
+// 8 of its 9 operations: 1.14 -> 0.26 ms a solve (8 subdomains of order about 250, 100
 // to 160 vectors each).  grid (n_sd, columns / (2 warps)).
 __global__ void __launch_bounds__(128)
     k_trsv_cols(const double* __restrict__ Tm, const int64_t* __restrict__ toff,
