@@ -316,8 +316,11 @@ int mor_solve_reduced(const mor_reduced* h, double rtol, int32_t max_iter, void*
  * CUDA runtime: make it once at initialisation, before any stream capture.  Later
  * calls on that device allocate nothing.
  * The solve is one launch (as in mor_solve_reduced); the call waits for its stream once,
- * to read the flags, the residual and the energy.  Without cooperative launches it
- * waits every 16 iterations to read the convergence flag.
+ * to read the flags, the residual and the energy.  The neighbour lists are on the device, so
+ * a system of at most 1,024 rows is tried in one cluster where nine neighbours per block
+ * row would fit; one that has more and does not fit takes a second launch, on every SM, and
+ * a second wait.  Without cooperative launches the call waits every 16 iterations to read
+ * the convergence flag.
  * Every call shares the one array and leaves its contents behind; the call clears the
  * state that must start at zero.  Calls whose GPU work overlaps (for example on two
  * streams, or two host threads) race on the array: serialise them.
