@@ -12,9 +12,9 @@
 // barriers: after p.q, after the restriction with r.r and r.D^{-1}r, after p with p.r.
 //
 // What bounds it: the chain of a step (six short phases between barriers), no longer
-// five launches of latency-bound kernels with their tile sums.  16^3 workload: 40 us a step there,
-// 7 here with the launch (binary64: 46 and 20, bound by binary64 issue).  Larger subdomains do not fit; they have work enough to hide
-// the launches.
+// five launches of latency-bound kernels with their tile sums.  16^3 workload: 40 us a step
+// there, 7 here with the launch (binary64: 46 and 20, bound by binary64 issue).  Larger
+// subdomains do not fit; they have work enough to hide the launches.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -407,9 +407,14 @@ ResidentPlan resident_plan(int n_sd, int n_max, int W, int nc_max, int kp) {
   // 47.6; S = 4, 6.7 waves 47.6 and 43.0, 13.5 waves 61.5 and 70.5; S = 2, 13.5 waves 39.9
   // and 38.6, 22 waves 61.9 and 67.9.  Binary32 at S = 8 and 5.7 waves 21.5 and 16.8 ms, 11.4
   // waves 26.6 and 28.2; S = 4, 13.5 waves 35.2 and 29.1, 22 waves 51.5 and 51.6; S = 2, 23
-  // waves 57.8 and 45.9, 37 waves 89.3 and 86.7
+  // waves 57.8 and 45.9, 37 waves 89.3 and 86.7.  One CTA each (398 and 724 rows): binary64
+  // 11.4 waves 35.7 and 34.2, 13.2 waves 37.4 and 37.9, 18 waves 29.0 and 34.2, 27 waves 39.1
+  // and 51.1; binary32 10.7 waves 28.3 and 25.2, 13.5 waves 24.0 and 21.3, 18 waves 26.3
+  // and 27.1, 29 waves 44.7 and 55.8, 44 waves 61.5 and 81.6
   const double waves = (double)S * tasks / 152.0;
-  if (sizeof(T) == 8 ? waves * std::min(S, 5) > 30.0 : waves * S > 48.0) return rp;
+  const double most = sizeof(T) == 8 ? (S == 1 ? 12.0 : S == 2 ? 15.0 : S == 4 ? 7.5 : 6.0)
+                                     : (S == 1 ? 16.0 : 48.0 / S);
+  if (waves > most) return rp;
   rp.S = S;
   rp.smem = res_smem<T>(n_max, (n_max + S - 1) / S, W, nc_max, S);
   return rp;
