@@ -599,6 +599,19 @@ struct Build {
     CK(cudaStreamSynchronize(st));
     return h_poll[0];
   }
+  // MOR_DEBUG: the steps and open columns of the last on-chip launch, which leaves its own
+  // largest step count per subdomain
+  int add_chip_steps(std::vector<int>& its, int& act) {
+    std::vector<int> h(n_sd);
+    CK(cudaMemcpyAsync(h.data(), cs.iters, n_sd * sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaMemsetAsync(cs.iters, 0, n_sd * sizeof(int), st));
+    CK(cudaStreamSynchronize(st));
+    for (int i = 0; i < n_sd; ++i) its[i] += h[i];
+    CK(cudaMemcpyAsync(h.data(), cs.active, n_sd * sizeof(int), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    for (int v : h) act += v;
+    return MOR_OK;
+  }
   // per matrix set: max row sum of |A| per subdomain (rounding-level bound)
   double* anorm[2] = {nullptr, nullptr};
   // per matrix set (profiling only): rows and stored entries of each subdomain
@@ -650,6 +663,7 @@ struct Build {
     const int check = 8;
     const int every = std::max(check, o->replace_every / check * check);
     int it = 0, first = 0, open_tiles = tl.n;  // first: the streaming steps start there
+    std::vector<int> chip_its(debug ? n_sd : 0, 0);
     // the kernel times of the roofline are those of the streaming kernels
     ResidentPlan rp =
         g_prof.on ? ResidentPlan() : resident_plan<T>(n_sd, n_rows[set], AT.W, co.n_max, kp);
@@ -663,6 +677,8 @@ struct Build {
         if (!launch_cg_resident<T>(rp, tl, AT, x, r, p, dinvT, kp, rtol2,
                                    std::min(every, o->max_iter - it), cs, co, d_poll + 3, st))
           rp.S = 0, first = it;  // refused: streaming steps from here
+        else if (debug)
+          TRY(add_chip_steps(chip_its, act));
       }
       int chunk = rp.S > 0 ? 0 : std::min(check, o->max_iter - it);
       for (int c = 0; c < chunk; ++c) {
@@ -716,6 +732,7 @@ struct Build {
         if (debug && (ract == 0 || it >= o->max_iter)) {
           std::vector<int> its(n_sd);
           cudaMemcpy(its.data(), cs.iters, n_sd * sizeof(int), cudaMemcpyDeviceToHost);
+          for (int i = 0; i < n_sd; ++i) its[i] += chip_its[i];
           std::sort(its.begin(), its.end());
           long tot = 0;
           for (int v : its) tot += v;
