@@ -1716,10 +1716,7 @@ void launch_spmm(const DTiles& tiles, const EllView<T>& A, const T* X, T* Y, int
 // Two rows in flight per thread in the updates where a block holds up to eight (more than 28
 // packs of columns): its threads walk 16 or more rows one after another (wide sketches on
 // 25^3: x/r update 47 -> 40 us, p update 26 -> 22).
-template <typename T>
-bool wide_rows(dim3 bl) {
-  return sizeof(T) == 4 && bl.y <= 8;
-}
+bool wide_rows(dim3 bl) { return bl.y <= 8; }  // (binary32)
 
 template <typename T>
 constexpr size_t slot_kernel_smem(int nch, int rb, int kp) {
@@ -1815,8 +1812,9 @@ void launch_coarse_then_p(const DTiles& tiles, int n_sd, const T* r, T* p, const
   const int th = light_threads<T>(open_tiles);
   const dim3 bl = block_of<T>(kp, th);
   const size_t sm = smem_bytes<T>(bl.x, bl.y, kp, 0);
-  auto fn = th == 1024 ? k_cg_update_p<T, 1024>
-            : wide_rows<T>(bl) ? k_cg_update_p<T, 256, 2> : k_cg_update_p<T, 256>;
+  auto fn = k_cg_update_p<T, 256>;
+  if constexpr (sizeof(T) == 4)
+    fn = th == 1024 ? k_cg_update_p<T, 1024> : wide_rows(bl) ? k_cg_update_p<T, 256, 2> : fn;
   fn<<<tiles.n, bl, sm, st>>>(tiles, r, p, dinv, kp, s, co);
 }
 
@@ -1928,10 +1926,12 @@ void launch_cg_step(const DTiles& tiles, const EllView<T>& A, T* x, T* r, T* p, 
     set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 2, 256>);
     set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 1, 128>);
     set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 2, 128>);
-    set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 2, 1024>);
     set_smem_attr<T>((const void*)k_cg_update_xr<T, 256>, kSmemRows);
-    set_smem_attr<T>((const void*)k_cg_update_xr<T, 256, 2>, kSmemRows);
-    set_smem_attr<T>((const void*)k_cg_update_xr<T, 1024>, kSmemRows);
+    if constexpr (sizeof(T) == 4) {
+      set_smem_attr<T>((const void*)k_cg_spmm_pq<T, 2, 1024>);
+      set_smem_attr<T>((const void*)k_cg_update_xr<T, 256, 2>, kSmemRows);
+      set_smem_attr<T>((const void*)k_cg_update_xr<T, 1024>, kSmemRows);
+    }
     attr = true;
   }
   const int th = light_threads<T>(open_tiles);
@@ -1939,14 +1939,15 @@ void launch_cg_step(const DTiles& tiles, const EllView<T>& A, T* x, T* r, T* p, 
   const int variant = spmm_variant<T>(tiles, A, p, q, kp, s, st);
   count_launch(2);
   if (ev) cudaEventRecord(ev[0], st);
-  if (th == 256) {
+  if (th == 256)
     launch_spmm_pq_variant<T>(variant, tiles, A, p, q, kp, s, st);
-  } else {
-    k_cg_spmm_pq<T, 2, 1024><<<tiles.n, bl, smem_bytes<T>(bl.x, bl.y, kp, A.W), st>>>(tiles, A, p, q, kp, s);
-  }
+  else if constexpr (sizeof(T) == 4)
+    k_cg_spmm_pq<T, 2, 1024><<<tiles.n, bl, smem_bytes<T>(bl.x, bl.y, kp, A.W), st>>>(
+        tiles, A, p, q, kp, s);
   if (ev) cudaEventRecord(ev[1], st);
-  auto fn = th == 1024 ? k_cg_update_xr<T, 1024>
-            : wide_rows<T>(bl) ? k_cg_update_xr<T, 256, 2> : k_cg_update_xr<T, 256>;
+  auto fn = k_cg_update_xr<T, 256>;
+  if constexpr (sizeof(T) == 4)
+    fn = th == 1024 ? k_cg_update_xr<T, 1024> : wide_rows(bl) ? k_cg_update_xr<T, 256, 2> : fn;
   fn<<<tiles.n, bl, slot_kernel_smem<T>(bl.x, bl.y, kp), st>>>(tiles, x, r, p, q, dinv, kp, s, co);
   if (ev) cudaEventRecord(ev[2], st);
   launch_coarse_then_p<T>(tiles, tiles.n_sd, r, p, dinv, kp, tol2, kCoarseStep, open_tiles, s, co,
