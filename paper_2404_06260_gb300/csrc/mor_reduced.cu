@@ -508,7 +508,10 @@ __global__ void __launch_bounds__(kRcgThreads)
                int max_iter, int rows_max, int weighted, RcgState s, double* part,
                long long budget) {
   extern __shared__ __align__(16) unsigned char rcg_raw[];
-  double* pj = reinterpret_cast<double*>(rcg_raw);
+  // the own rows of x, r, p and q (none of them unless kShared: rows_max = 0), then the staged
+  // neighbour columns
+  double* sh = reinterpret_cast<double*>(rcg_raw);
+  double* pj = sh + 4 * (size_t)rows_max;
   int64_t* off = reinterpret_cast<int64_t*>(pj + kRcgCap);
   __shared__ double red[48];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -519,7 +522,7 @@ __global__ void __launch_bounds__(kRcgThreads)
   const int rows = (int)(row1 - row0);
   double *xs, *rs, *ps, *qs;
   if constexpr (kShared) {
-    xs = reinterpret_cast<double*>(off + kRcgCap);
+    xs = sh;
     rs = xs + rows_max;
     ps = rs + rows_max;
     qs = ps + rows_max;
