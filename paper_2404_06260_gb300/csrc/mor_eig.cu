@@ -8,7 +8,8 @@
 // gives eigenvalue sigma_j^2 and eigenvector u_j, accurate relative to themselves as those
 // of the two-sided threshold iteration.  The eigenvectors need no accumulation, a rotation
 // touches two columns instead of two rows, two columns and two more of V, and the pivoted
-// factor starts nearly orthogonal: 4 to 7 sweeps.
+// factor starts nearly orthogonal: 6 to 9 sweeps with the last, which finds nothing to rotate,
+// at the orders and conditions of the workloads (4 at order 13).
 //  - Scaling: G by a power of two to a largest diagonal entry in [1, 2).
 //  - A column whose pivot falls below n 2^-53 of its own diagonal entry (or below kEigTiny)
 //    is rounding noise and takes no part.  The r columns of the factor give the r largest
@@ -24,13 +25,14 @@
 //
 // What bounds it: binary64 issue (a warp instruction keeps a quarter of the SM busy for 64
 // clocks) and, for small orders, the chain product -> tangent -> rotation of each round.
-// Orders up to kEigSmem: one CTA per subdomain, the factor in shared memory, 8 lanes per
-// pair (k_sym_eig).  Larger ones: a cluster per subdomain works on pairs of column blocks
-// staged from L2 (k_sym_eig_blocks).
+// Orders up to 48, and up to kEigSmem where the subdomains alone fill the chip: one CTA per
+// subdomain, the factor in shared memory, 8 lanes per pair (k_sym_eig).  Others: a cluster per
+// subdomain works on pairs of column blocks staged from L2 (k_sym_eig_blocks).
 // Per batch, against the two-sided iteration with the matrix in shared memory (up to 80) or
 // in L2 and one CTA per subdomain: 64 matrices of order 42 2.13 -> 1.06 ms, 40 of 74 8.5 ->
-// 2.0 ms, 14 of 203 145 -> 8 ms, 8 of 127 169 -> 5.4 ms (the noise directions of an
-// explicit Gram never met the two-sided threshold and ran all 40 sweeps).
+// 2.0 ms, 14 of 203 145 -> 8 ms, 8 of 127 and rank about 60 169 -> 4.0 ms (the noise directions of
+// an explicit Gram never met the two-sided threshold and ran all 40 sweeps; here they take no
+// part in the sweeps).
 #include <cooperative_groups.h>
 
 #include <algorithm>

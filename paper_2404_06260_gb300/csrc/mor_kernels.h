@@ -282,7 +282,7 @@ void launch_gram_vec(const DTiles& tiles, int n_sd, const double* X, int ldx, in
 // eigen-decomposition of the positive semidefinite leading n x n block (n <= 1024) of
 // A[sd] (stride ld), symmetrised (mor_eig.cu): evals descending (n_sd x ld, noise and null
 // directions 0), evecs orthonormal columns (n_sd x ld x ld), both zero beyond n.  work:
-// n_sd * sym_eig_work(n) doubles (none for n <= 160).
+// n_sd * sym_eig_work(n) doubles (used above order 48).
 size_t sym_eig_work(int n);
 void launch_sym_eig(int n_sd, const double* A, int ld, int n, double* evals, double* evecs,
                     double* work, cudaStream_t st);

@@ -242,7 +242,8 @@ __global__ void k_rcg_update_p(int kq, RcgState s) {
 // about 100 clocks apart), and every iteration needs two sums over all rows.  So the
 // matrix is spread as far as the sums allow: up to kRcgClusterFma multiply-adds and
 // kRcgClusterDim rows one cluster of 8 CTAs keeps matrix and vectors in shared memory
-// and sums through distributed shared memory (k_rcg_cluster, about 1.5 us a sum); above,
+// and sums through distributed shared memory (k_rcg_cluster, 0.9 to 1.5 us a sum by the
+// cluster's threads, 64 to 512 a CTA); above,
 // every SM takes part and sums through global memory (k_rcg_grid, 3.5 us).  Whole calls
 // measured on both, cluster | every SM: 5 k multiply-adds 137 | 248 us, 28 k 221 | 346,
 // 50 k 267 | 370, 78 k 425 | 407, 80 k (more rows) 369 | 457, 109 k 500 | 480, 254 k

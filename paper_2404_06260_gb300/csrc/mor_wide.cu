@@ -16,7 +16,8 @@ constexpr int kWRows = 16;   // rows staged per step of the Gram
 
 // part[(sd * S + s)][i * n + j] = sum over the rows of chunk s of subdomain sd of
 // X[r, i] Y[r, j] for the 64 x 64 tiles on and below the diagonal: every product here is
-// symmetric up to rounding (X^T X, X^T H X, V^T A V) and its reader symmetrises.  Block
+// symmetric, up to rounding (X^T X, X^T H X, V^T A V) or to the tolerance of the adjoint
+// solves, where the whole square averaged was measured no more accurate.  Block
 // (16, 16), thread (tx, ty) rows ty + 16 a and columns tx + 16 b of the tile; the 16-wide
 // strips past n are left out.  Bound by binary64 issue, so by what is multiplied: the whole
 // square in tiles padded to 64 took 1.95 ms for 14 subdomains of up to 261 columns, 0.91 now.
