@@ -1855,9 +1855,9 @@ int mor_solve_reduced(const mor_reduced* h, double rtol, int32_t max_iter, void*
   // r, p, q, and a zeroed tail: the partial sums of either iteration, the scalars and the
   // flags
   const size_t n_part = std::max(2 * (size_t)h->n_sd, 2 * (size_t)kRcgMaxGrid);
-  const size_t n_tail = n_part + 16, n_work = rcg_grid_work(h->n_sd, h->kq);
+  const size_t n_tail = n_part + 16;
   double* ws;
-  TRY(A.alloc(&ws, 3 * (size_t)h->dim + n_tail + n_work, false, st));
+  TRY(A.alloc(&ws, 3 * (size_t)h->dim + n_tail, false, st));
   double* tail = ws + 3 * (size_t)h->dim;
   CK(cudaMemsetAsync(tail, 0, n_tail * sizeof(double), st));
   RcgState s{};
@@ -1869,7 +1869,6 @@ int mor_solve_reduced(const mor_reduced* h, double rtol, int32_t max_iter, void*
   s.scal = tail + n_part;
   s.flag = reinterpret_cast<int*>(s.scal + 8);
   s.counter = s.flag + 4;
-  if (n_work) s.w = tail + n_tail;
   struct {
     double sc[8];
     int flag[4];
@@ -1886,6 +1885,14 @@ int mor_solve_reduced(const mor_reduced* h, double rtol, int32_t max_iter, void*
                             s.part, wait_budget_cycles(), cluster, st);
   };
   RcgLaunch how = launch(true);
+  if (how == RcgLaunch::kNone) {
+    // more rows than the SMs' shared memory holds
+    const size_t n_work = rcg_grid_work(h->n_sd, h->kq);
+    if (n_work > 0) {
+      TRY(A.alloc(&s.w, n_work, false, st));
+      how = launch(false);
+    }
+  }
   if (how != RcgLaunch::kNone) TRY(fetch());
   if (how == RcgLaunch::kCluster && out.flag[2] == 2) {
     CK(cudaMemsetAsync(s.flag, 0, 4 * sizeof(int), st));
